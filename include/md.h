@@ -412,7 +412,7 @@ void md_destroy(md_system *sys);
  * recomputing positions from (x, v) checkpoints taken every checkpoint_every
  * steps.  Pairs crossing rc are invisible to it (the truncated force jumps
  * there by F(rc)).
- * Device memory: about 8 * 3N * (2 * ceil(K / C) + C + 8) bytes, allocated
+ * Device memory: about 8 * 3N * (2 * ceil(K / C) + C + 18) bytes, allocated
  * by md_adj_create.  Errors: MD_E* codes with md_last_error(NULL).
  * ------------------------------------------------------------------------ */
 typedef struct md_adj md_adj;          /* opaque, owned by the library */
