@@ -409,79 +409,127 @@ void launch_energy_reduce(const double* lj_part, const double* b_part, const Rep
 }
 
 // ------------------------------------------------------------ chain observables
-// One thread per chain (the structural observables of the paper's Sec. 5):
-// the chain is made continuous by adding minimum-image bond vectors from site
-// 0; R_ee = x_last - x_first (Fig. 8), R_g^2 = sum m |x - x_cm|^2 / sum m
-// (mass-weighted, from sums relative to site 0), and the number of backbone
-// dihedrals in the trans state, |phi| > 120 deg, i.e. cos(phi) =
-// n1.n2 / (|n1||n2|) < -1/2 with n1 = b1 x b2, n2 = b2 x b3 (IUPAC, trans at
-// 180 deg).  The trans counts of a replica are added as integers.
+// One warp per chain (the structural observables of the paper's Sec. 5):
+// the chain is made continuous by minimum-image bonds, R_ee = x_last -
+// x_first (Fig. 8), R_g^2 = sum m |x - x_cm|^2 / sum m (mass-weighted, from
+// sums relative to site 0), and the number of backbone dihedrals in the trans
+// state, |phi| > 120 deg, i.e. cos(phi) = n1.n2 / (|n1||n2|) < -1/2 with n1 =
+// b1 x b2, n2 = b2 x b3 (IUPAC, trans at 180 deg).  The trans counts of a
+// replica are added as integers.
+// Lane l of a warp takes sites l, l + 32, ...: a thread per chain walked 150
+// sites alone, with 1,000 threads on the GPU and loads 1,200 bytes apart.
+// A site's whole-box shift is the number of face crossings up to it, counted
+// by ballots, so the continuous position is one FMA and no serial sum.
+// 150k sites: 383 -> 27 us.
+constexpr int kObsWarps = 4;
+
 template <class T>
-__global__ void __launch_bounds__(128) k_chain_observables(const T* __restrict__ x, int N,
-                                                           const RepDev* __restrict__ reps, int n_reps,
-                                                           const ForceParams fp, int n_chains_total,
-                                                           double* __restrict__ ree, double* __restrict__ rg2,
-                                                           unsigned long long* __restrict__ trans) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= n_chains_total) return;
-  int r = 0;
-  while (r + 1 < n_reps && reps[r + 1].chain_off <= c) ++r;
+__global__ void __launch_bounds__(32 * kObsWarps) k_chain_observables(const T* __restrict__ x, int N,
+                                                                      const RepDev* __restrict__ reps, int n_reps,
+                                                                      const ForceParams fp, int n_chains_total,
+                                                                      double* __restrict__ ree,
+                                                                      double* __restrict__ rg2,
+                                                                      unsigned long long* __restrict__ trans) {
+  const int c = blockIdx.x * kObsWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (c >= n_chains_total) return;   // the whole warp leaves together
+  int lo = 0, hi = n_reps - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (reps[mid].chain_off <= c) lo = mid; else hi = mid - 1;
+  }
+  const int r = lo;
   const RepDev& R = reps[r];
   const int S = fp.sites;
   const int o = R.atom_off + (c - R.chain_off) * S;
-  const double L = R.L;
-  double p[3] = {0.0, 0.0, 0.0};                       // site position relative to site 0
-  double m_sum = 0.0, s1[3] = {0.0, 0.0, 0.0}, s2 = 0.0;
-  double b[3][3] = {{0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}};   // the last three bond vectors
-  unsigned long long nt = 0;
-  for (int k = 0; k < S; ++k) {
-    if (k > 0) {
-      double d[3];
+  const double L = R.L, hL = R.half_L;
+  const double x0[3] = {(double)x[o], (double)x[N + o], (double)x[2 * N + o]};
+  const unsigned le = 0xffffffffu >> (31 - lane);   // this lane and those before it
+  int shift[3] = {0, 0, 0};                         // whole boxes up to the previous chunk's last site
+  double px[3] = {x0[0], x0[1], x0[2]};             // that site's position
+  double pb[3] = {0.0, 0.0, 0.0}, pn[3] = {0.0, 0.0, 0.0};   // its bond and normal (used from site 3 on)
+  double m_sum = 0.0, s1[3] = {0.0, 0.0, 0.0}, s2 = 0.0, end[3] = {0.0, 0.0, 0.0};
+  int nt = 0;
+  for (int k0 = 0; k0 < S; k0 += 32) {
+    const int k = k0 + lane;
+    const bool on = k < S;
+    double b[3], p[3], xk[3];
 #pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        double e = (double)x[a * N + o + k] - (double)x[a * N + o + k - 1];
-        e -= L * rint(e / L);
-        d[a] = e;
-        p[a] += e;
-      }
-#pragma unroll
-      for (int a = 0; a < 3; ++a) { b[0][a] = b[1][a]; b[1][a] = b[2][a]; b[2][a] = d[a]; }
-      if (k >= 3) {
-        const double n1[3] = {b[0][1] * b[1][2] - b[0][2] * b[1][1], b[0][2] * b[1][0] - b[0][0] * b[1][2],
-                              b[0][0] * b[1][1] - b[0][1] * b[1][0]};
-        const double n2[3] = {b[1][1] * b[2][2] - b[1][2] * b[2][1], b[1][2] * b[2][0] - b[1][0] * b[2][2],
-                              b[1][0] * b[2][1] - b[1][1] * b[2][0]};
-        const double dn = n1[0] * n2[0] + n1[1] * n2[1] + n1[2] * n2[2];
-        const double l1 = n1[0] * n1[0] + n1[1] * n1[1] + n1[2] * n1[2];
-        const double l2 = n2[0] * n2[0] + n2[1] * n2[1] + n2[2] * n2[2];
-        // cos(phi) < -1/2  <=>  n1.n2 < 0 and (n1.n2)^2 > |n1|^2 |n2|^2 / 4
-        nt += (dn < 0.0 && 4.0 * dn * dn > l1 * l2) ? 1ull : 0ull;
-      }
+    for (int a = 0; a < 3; ++a) {
+      xk[a] = on ? (double)x[a * N + o + k] : px[a];
+      double prev = __shfl_up_sync(0xffffffffu, xk[a], 1);
+      if (lane == 0) prev = px[a];
+      double e = xk[a] - prev;
+      const bool dn = e > hL, up = e < -hL;         // crossed the lower / upper face
+      if (dn) e -= L; else if (up) e += L;
+      b[a] = e;
+      const unsigned bu = __ballot_sync(0xffffffffu, up && on), bd = __ballot_sync(0xffffffffu, dn && on);
+      const int sh = shift[a] + __popc(bu & le) - __popc(bd & le);
+      shift[a] += __popc(bu) - __popc(bd);
+      p[a] = fma((double)sh, L, xk[a]) - x0[a];
+      px[a] = __shfl_sync(0xffffffffu, xk[a], 31);
     }
-    const double m = fp.mass[(k == 0 || k == S - 1) ? 1 : 0];
-    m_sum += m;
+    double q[3], n[3], nq[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) s1[a] += m * p[a];
-    s2 += m * (p[0] * p[0] + p[1] * p[1] + p[2] * p[2]);
+    for (int a = 0; a < 3; ++a) {
+      q[a] = __shfl_up_sync(0xffffffffu, b[a], 1);
+      if (lane == 0) q[a] = pb[a];
+      pb[a] = __shfl_sync(0xffffffffu, b[a], 31);
+    }
+    n[0] = q[1] * b[2] - q[2] * b[1];
+    n[1] = q[2] * b[0] - q[0] * b[2];
+    n[2] = q[0] * b[1] - q[1] * b[0];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      nq[a] = __shfl_up_sync(0xffffffffu, n[a], 1);
+      if (lane == 0) nq[a] = pn[a];
+      pn[a] = __shfl_sync(0xffffffffu, n[a], 31);
+    }
+    const double dn = nq[0] * n[0] + nq[1] * n[1] + nq[2] * n[2];
+    const double l2 = n[0] * n[0] + n[1] * n[1] + n[2] * n[2];
+    const double l1 = nq[0] * nq[0] + nq[1] * nq[1] + nq[2] * nq[2];
+    // cos(phi) < -1/2  <=>  n1.n2 < 0 and (n1.n2)^2 > |n1|^2 |n2|^2 / 4
+    const bool tr = on && k >= 3 && dn < 0.0 && 4.0 * dn * dn > l1 * l2;
+    nt += __popc(__ballot_sync(0xffffffffu, tr));
+    if (on) {
+      const double m = fp.mass[(k == 0 || k == S - 1) ? 1 : 0];
+      m_sum += m;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) s1[a] += m * p[a];
+      s2 += m * (p[0] * p[0] + p[1] * p[1] + p[2] * p[2]);
+      if (k == S - 1)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) end[a] = p[a];
+    }
   }
+  const int last = (S - 1) & 31;
 #pragma unroll
-  for (int a = 0; a < 3; ++a) ree[3 * c + a] = p[a];
+  for (int a = 0; a < 3; ++a) end[a] = __shfl_sync(0xffffffffu, end[a], last);
+#pragma unroll
+  for (int m = 16; m >= 1; m >>= 1) {
+    m_sum += __shfl_xor_sync(0xffffffffu, m_sum, m);
+    s2 += __shfl_xor_sync(0xffffffffu, s2, m);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) s1[a] += __shfl_xor_sync(0xffffffffu, s1[a], m);
+  }
+  if (lane != 0) return;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) ree[3 * c + a] = end[a];
   const double cx = s1[0] / m_sum, cy = s1[1] / m_sum, cz = s1[2] / m_sum;
   rg2[c] = s2 / m_sum - (cx * cx + cy * cy + cz * cz);
-  atomicAdd(trans + r, nt);
+  if (nt) atomicAdd(trans + r, (unsigned long long)nt);
 }
 
 void launch_chain_observables(bool mixed, const void* x, int N, const RepDev* reps, int n_reps,
                               const ForceParams& fp, int n_chains_total, double* ree, double* rg2,
                               unsigned long long* trans, cudaStream_t st) {
-  const int blocks = (n_chains_total + 127) / 128;
+  const int blocks = (n_chains_total + kObsWarps - 1) / kObsWarps;
   if (blocks == 0) return;
   if (mixed)
-    k_chain_observables<double><<<blocks, 128, 0, st>>>((const double*)x, N, reps, n_reps, fp, n_chains_total,
-                                                        ree, rg2, trans);
+    k_chain_observables<double><<<blocks, 32 * kObsWarps, 0, st>>>((const double*)x, N, reps, n_reps, fp,
+                                                                   n_chains_total, ree, rg2, trans);
   else
-    k_chain_observables<float><<<blocks, 128, 0, st>>>((const float*)x, N, reps, n_reps, fp, n_chains_total,
-                                                       ree, rg2, trans);
+    k_chain_observables<float><<<blocks, 32 * kObsWarps, 0, st>>>((const float*)x, N, reps, n_reps, fp,
+                                                                  n_chains_total, ree, rg2, trans);
 }
 
 // ------------------------------------------------------------------ output state
