@@ -269,7 +269,7 @@ int md_observables(md_system *sys, double *r_ee, double *rg2, double *trans_frac
  * dy^2 + dz^2), each operation rounded once, left to right) on the state's
  * positions, so the counts equal that definition's.  Re-bins the current
  * positions first.  counts: host or device pointer, int64.  Allocates and
- * frees two small device buffers.  Synchronous.  g(r) = counts / (n_pairs *
+ * frees two device buffers when the histogram exceeds the staging memory.  Synchronous.  g(r) = counts / (n_pairs *
  * shell volume / L^3) with n_pairs = N (N - 1) / 2 - n_chains (2 S - 3). */
 int md_rdf(md_system *sys, int32_t n_bins, const double *edges, int64_t *counts);
 

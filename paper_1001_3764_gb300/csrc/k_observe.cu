@@ -2,10 +2,10 @@
 // distribution function of non-bonded site pairs and the end-to-end vector
 // autocorrelation function (Fig. 8).
 //
-// RDF: one block per cell; its atoms pair with the later atoms of the cell and
-// with every atom of the 13 forward cells of a half shell, so each pair within
-// one cell side is met once.  The distance is the plain definition in FP64
-// with every operation explicitly rounded (d = x_j - x_i, d -= L rint(d / L),
+// RDF: a cell's atoms pair with the later atoms of the cell and with every
+// atom of the 13 forward cells of a half shell, so each pair within one cell
+// side is met once.  The distance is the plain definition in FP64 with every
+// operation explicitly rounded (d = x_j - x_i, d -= L rint(d / L),
 // r = sqrt(dx^2 + dy^2 + dz^2), summed left to right), and the bin is the k
 // with edges[k] <= r < edges[k + 1] (the last bin closed), so the integer
 // counts equal those of the FP64 definition on the same positions.  Counts
@@ -17,13 +17,34 @@
 // every replica, sum_c R_c(s) . R_c(s - tau) to acc[r][tau], one block per
 // (replica, tau) with a fixed-order reduction over the replica's chains.
 // After n samples acc[r][tau] = sum_{t < n - tau} sum_c R_c(t + tau) . R_c(t).
+#include <cmath>
 #include <type_traits>
 
 #include "md_kernels.cuh"
 
 namespace mdg {
 
+// The FP64 pipe of this GPU issues about 2 operations per clock and SM, and
+// the definition costs some 60 of them per candidate pair (three divisions,
+// a square root).  So a pair's bin is taken from the FP32 cell-unit
+// positions of the fresh bins wherever that cannot differ: the FP32 distance
+// is within kRdfMargin cell sides of the FP64 one, and a pair whose FP32
+// distance lies further than that inside a bin's edges (or beyond the last
+// one) has that bin by the definition too.  The few others (0.1% of the
+// pairs in range at 200 bins) are evaluated by the definition.
+//
+// A lane holds one atom j of the 14 cells, moved to the home cell's frame,
+// and a warp walks the home atoms in shared memory (one broadcast load per
+// 32 pairs).  Blocks take runs of consecutive cells, so that a histogram is
+// flushed once per run and not once per cell.  150k sites, r_max 1.0 nm,
+// 200 bins: 9,824 -> 251 us (FP64 for every candidate, one block per cell).
 constexpr int kRdfThreads = 128;
+constexpr int kRdfStage = 128;       // home atoms staged at a time
+constexpr int kRdfBlocks = 152 * 16;
+// FP32 cell units: each position is rounded by at most 2^-25 (FP32 master:
+// 2^-24.6), the offset and the difference add 2^-24 each, so a component is
+// off by at most 1.9e-7 and r <= 1 by 3.3e-7; r^2, rsqrt.approx and the scaling by h add 5e-7
+constexpr float kRdfMargin = 1.0e-6f;
 
 __device__ __forceinline__ int rdf_find_rep(const RepDev* reps, int n_reps, int c) {
   int lo = 0, hi = n_reps - 1;
@@ -34,72 +55,163 @@ __device__ __forceinline__ int rdf_find_rep(const RepDev* reps, int n_reps, int 
   return lo;
 }
 
+// bin of the pair (i, j) by the FP64 definition, or -1
+template <class T>
+__device__ __noinline__ int rdf_exact_bin(const T* __restrict__ x, int N, int i, int j, double L,
+                                          const double* __restrict__ edges, int n_bins, double norm) {
+  double d2 = 0.0;
+#pragma unroll
+  for (int ax = 0; ax < 3; ++ax) {
+    double d = __dsub_rn((double)x[ax * N + j], (double)x[ax * N + i]);
+    d = __dsub_rn(d, __dmul_rn(L, rint(__ddiv_rn(d, L))));
+    d2 = ax == 0 ? __dmul_rn(d, d) : __dadd_rn(d2, __dmul_rn(d, d));
+  }
+  const double rr = __dsqrt_rn(d2);
+  if (!(rr <= edges[n_bins]) || rr < edges[0]) return -1;
+  int k = (int)((rr - edges[0]) * norm);
+  k = k < 0 ? 0 : (k > n_bins - 1 ? n_bins - 1 : k);
+  if (rr < edges[k]) --k;
+  else if (k < n_bins - 1 && rr >= edges[k + 1]) ++k;
+  return k;
+}
+
 template <class T>
 __global__ void __launch_bounds__(kRdfThreads) k_rdf(const T* __restrict__ x, int N, const int* __restrict__ cell_start,
-                                                     const int* __restrict__ perm, const RepDev* __restrict__ reps,
-                                                     int n_reps, int sites, const double* __restrict__ edges,
-                                                     int n_bins, double norm, unsigned long long* __restrict__ counts) {
+                                                     const int* __restrict__ perm, const float4* __restrict__ pos,
+                                                     const int* __restrict__ tag, const RepDev* __restrict__ reps,
+                                                     int n_reps, int C, const double* __restrict__ edges,
+                                                     const float2* __restrict__ inner, int n_bins, double norm,
+                                                     unsigned long long* __restrict__ counts) {
   extern __shared__ unsigned int hist[];
-  const int c = blockIdx.x;
-  for (int k = threadIdx.x; k < n_bins; k += blockDim.x) hist[k] = 0u;
-  __syncthreads();
-  const int r = rdf_find_rep(reps, n_reps, c);
-  const RepDev& R = reps[r];
-  const int M = R.M, lc = c - R.cell_base;
-  const int cx = lc % M, cy = (lc / M) % M, cz = lc / (M * M);
-  const int b = cell_start[c], n = cell_start[c + 1] - b;
-  const double L = R.L, r_max = edges[n_bins];
-  // the cell itself, then its 13 forward neighbours
-  for (int o = 0; o < 14; ++o) {
-    int ox = 0, oy = 0, oz = 0;
-    if (o > 0) {
-      const int q = o - 1;                  // 9 cells of the z + 1 layer, 3 of y + 1, then x + 1
-      if (q < 9) { oz = 1; oy = q / 3 - 1; ox = q % 3 - 1; }
-      else if (q < 12) { oy = 1; ox = q - 10; }
-      else { ox = 1; }
-    }
-    const int nc = R.cell_base + (((cz + oz + M) % M) * M + ((cy + oy + M) % M)) * M + ((cx + ox + M) % M);
-    const int jb = cell_start[nc], jn = cell_start[nc + 1] - jb;
-    const long long pairs = (long long)n * jn;
-    for (long long p = threadIdx.x; p < pairs; p += blockDim.x) {
-      const int a = (int)(p / jn), q = (int)(p % jn);
-      if (o == 0 && q <= a) continue;       // the cell itself: each pair once
-      const int i = perm[b + a], j = perm[jb + q];
-      const int ci = (i - R.atom_off) / sites, cj = (j - R.atom_off) / sites;
-      const int si = (i - R.atom_off) - ci * sites, sj = (j - R.atom_off) - cj * sites;
-      if (ci == cj && abs(si - sj) <= 2) continue;   // 1-2 and 1-3 neighbours (Sec. 3.1)
-      double d2 = 0.0;
-#pragma unroll
-      for (int ax = 0; ax < 3; ++ax) {
-        double d = __dsub_rn((double)x[ax * N + j], (double)x[ax * N + i]);
-        d = __dsub_rn(d, __dmul_rn(L, rint(__ddiv_rn(d, L))));
-        d2 = ax == 0 ? __dmul_rn(d, d) : __dadd_rn(d2, __dmul_rn(d, d));
+  __shared__ float4 si[kRdfStage];          // home atoms: cell units, w = chain/site tag
+  __shared__ int s_start[14], s_pre[15];
+  __shared__ float s_off[14][3];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int c0 = (int)((long long)C * blockIdx.x / gridDim.x), c1 = (int)((long long)C * (blockIdx.x + 1) / gridDim.x);
+  if (c0 >= c1) return;
+  for (int k = threadIdx.x; k < n_bins; k += kRdfThreads) hist[k] = 0u;
+  int r = rdf_find_rep(reps, n_reps, c0);
+  const float e0 = (float)edges[0], fnorm = (float)norm, r_top = (float)edges[n_bins];
+  for (int c = c0; c < c1; ++c) {
+    __syncthreads();   // the previous cell's tables are no longer read
+    if (r + 1 < n_reps && reps[r + 1].cell_base <= c) {   // the next replica begins: its histogram is another
+      for (int k = threadIdx.x; k < n_bins; k += kRdfThreads) {
+        if (hist[k]) atomicAdd(counts + (size_t)r * n_bins + k, (unsigned long long)hist[k]);
+        hist[k] = 0u;
       }
-      const double rr = __dsqrt_rn(d2);
-      if (!(rr <= r_max) || rr < edges[0]) continue;
-      int k = (int)((rr - edges[0]) * norm);
-      k = k < 0 ? 0 : (k > n_bins - 1 ? n_bins - 1 : k);
-      if (rr < edges[k]) --k;
-      else if (k < n_bins - 1 && rr >= edges[k + 1]) ++k;
-      if (k >= 0) atomicAdd(hist + k, 1u);
+      ++r;
+    }
+    const RepDev& R = reps[r];
+    const int M = R.M, b = cell_start[c], n = cell_start[c + 1] - b;
+    if (warp == 0) {
+      int len = 0;
+      if (lane < 14) {   // the cell itself, then its 13 forward neighbours
+        int ox = 0, oy = 0, oz = 0;
+        if (lane > 0) {
+          const int q = lane - 1;           // 9 cells of the z + 1 layer, 3 of y + 1, then x + 1
+          if (q < 9) { oz = 1; oy = q / 3 - 1; ox = q % 3 - 1; }
+          else if (q < 12) { oy = 1; ox = q - 10; }
+          else { ox = 1; }
+        }
+        const int lc = c - R.cell_base;
+        const int cx = lc % M, cy = (lc / M) % M, cz = lc / (M * M);
+        const int nc = R.cell_base + (((cz + oz + M) % M) * M + ((cy + oy + M) % M)) * M + ((cx + ox + M) % M);
+        s_start[lane] = cell_start[nc];
+        len = cell_start[nc + 1] - cell_start[nc];
+        s_off[lane][0] = (float)ox; s_off[lane][1] = (float)oy; s_off[lane][2] = (float)oz;
+      }
+#pragma unroll
+      for (int o = 1; o < 16; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, len, o);
+        if (lane >= o) len += v;
+      }
+      if (lane == 0) s_pre[0] = 0;
+      if (lane < 14) s_pre[lane + 1] = len;
+    }
+    const float hf = R.hf, Mf = R.Mf;
+    // beyond this squared FP32 distance (cell units) a pair is out of range by the definition
+    const float rt = r_top / hf + 2.f * kRdfMargin;
+    const float far2 = rt * rt;
+    const float low = e0 - 4.f * kRdfMargin * hf;   // below this one, out of range as well
+    const bool fold = M == 3;   // two images of a pair can both be near a cell side away
+    for (int i0 = 0; i0 < n; i0 += kRdfStage) {
+      const int ni = min(kRdfStage, n - i0);
+      __syncthreads();
+      for (int k = threadIdx.x; k < ni; k += kRdfThreads) {
+        float4 p = pos[b + i0 + k];
+        p.w = __int_as_float(tag[b + i0 + k] & (int)kTagMask);
+        si[k] = p;
+      }
+      __syncthreads();
+      const int total = s_pre[14];
+      int o = 0;
+      for (int q = 32 * warp + lane; q - lane < total; q += kRdfThreads) {
+        const bool on = q < total;
+        int sj = b;
+        float4 pj = make_float4(0.f, 0.f, 0.f, 0.f);
+        int tj = 0, last = ni;   // home atoms i0 .. i0 + last - 1 pair with j
+        if (on) {
+          while (q >= s_pre[o + 1]) ++o;
+          sj = s_start[o] + (q - s_pre[o]);
+          pj = pos[sj];
+          pj.x += s_off[o][0]; pj.y += s_off[o][1]; pj.z += s_off[o][2];
+          tj = tag[sj] & (int)kTagMask;
+          if (o == 0) last = min(ni, sj - b - i0);   // the cell itself: each pair once, i before j
+        } else {
+          last = 0;
+        }
+        for (int k = 0; k < ni; ++k) {
+          const float4 p = si[k];
+          float dx = pj.x - p.x, dy = pj.y - p.y, dz = pj.z - p.z;
+          if (fold) {
+            dx -= Mf * rintf(dx / Mf); dy -= Mf * rintf(dy / Mf); dz -= Mf * rintf(dz / Mf);
+          }
+          const float r2 = dx * dx + dy * dy + dz * dz;
+          // |i - j| <= 2 within one chain: 1-2 and 1-3 neighbours (Sec. 3.1)
+          if (k < last && r2 <= far2 && (unsigned)(__float_as_int(p.w) - tj + 2) > 4u) {
+            const float rr = r2 * rsqrtf(r2) * hf;
+            if (rr < low) continue;
+            int g = (int)((rr - e0) * fnorm);
+            g = g < 0 ? 0 : (g > n_bins - 1 ? n_bins - 1 : g);
+            const float2 in = __ldg(inner + g);
+            if (!(rr >= in.x && rr < in.y))
+              g = rdf_exact_bin<T>(x, N, perm[b + i0 + k], perm[sj], R.L, edges, n_bins, norm);
+            if (g >= 0) atomicAdd(hist + g, 1u);
+          }
+        }
+      }
     }
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < n_bins; k += blockDim.x)
+  for (int k = threadIdx.x; k < n_bins; k += kRdfThreads)
     if (hist[k]) atomicAdd(counts + (size_t)r * n_bins + k, (unsigned long long)hist[k]);
 }
 
-void launch_rdf(bool mixed, const void* x, int N, const int* cell_start, const int* perm, const RepDev* reps,
-                int n_reps, int C, int sites, const double* edges, int n_bins, double norm,
-                unsigned long long* counts, cudaStream_t st) {
+// the part of each bin further than the FP32 distance's error from its edges
+// (h_max: the largest cell side), edges rounded outward
+void rdf_inner_edges(const double* edges, int n_bins, double h_max, float2* inner) {
+  const double m = (double)kRdfMargin * h_max;
+  for (int k = 0; k < n_bins; ++k)
+    inner[k] = make_float2(std::nextafterf((float)(edges[k] + m), INFINITY),
+                           std::nextafterf((float)(edges[k + 1] - m), -INFINITY));
+}
+
+void launch_rdf(bool mixed, const void* x, int N, const int* cell_start, const int* perm, const float4* pos,
+                const int* tag, const RepDev* reps, int n_reps, int C, const double* edges, const float2* inner,
+                int n_bins, double norm, unsigned long long* counts, cudaStream_t st) {
   if (C <= 0) return;
   const size_t sm = (size_t)n_bins * sizeof(unsigned int);
+  const int grid = C < kRdfBlocks ? C : kRdfBlocks;
+  if (sm > 40000) {   // the histogram and the staged atoms exceed 48 KB
+    cudaFuncSetAttribute(k_rdf<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaFuncSetAttribute(k_rdf<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  }
   if (mixed)
-    k_rdf<double><<<C, kRdfThreads, sm, st>>>((const double*)x, N, cell_start, perm, reps, n_reps, sites, edges,
-                                                n_bins, norm, counts);
+    k_rdf<double><<<grid, kRdfThreads, sm, st>>>((const double*)x, N, cell_start, perm, pos, tag, reps, n_reps, C,
+                                                 edges, inner, n_bins, norm, counts);
   else
-    k_rdf<float><<<C, kRdfThreads, sm, st>>>((const float*)x, N, cell_start, perm, reps, n_reps, sites, edges,
-                                               n_bins, norm, counts);
+    k_rdf<float><<<grid, kRdfThreads, sm, st>>>((const float*)x, N, cell_start, perm, pos, tag, reps, n_reps, C,
+                                                edges, inner, n_bins, norm, counts);
 }
 
 // ------------------------------------------------------------------ ACF

@@ -1015,11 +1015,22 @@ int md_rdf(md_system* s, int32_t n_bins, const double* edges, int64_t* counts) {
     if (!(edges[k + 1] > edges[k])) return fail(s, MD_EINVAL, "edges must increase");
   for (const RepDev& q : s->reps_h)
     if (edges[n_bins] > q.h) return fail(s, MD_EINVAL, "r_max beyond the cell side of a replica");
-  double* ed = nullptr;
+  double* ed = nullptr;          // the edges, then the inner part of each bin (two floats)
   unsigned long long* cnt = nullptr;
   const size_t nc = (size_t)s->n_reps * n_bins;
-  if (cudaMalloc(&ed, sizeof(double) * (n_bins + 1)) != cudaSuccess ||
-      cudaMalloc(&cnt, sizeof(unsigned long long) * nc) != cudaSuccess) {
+  double h_max = 0.0;
+  for (const RepDev& q : s->reps_h) h_max = std::max(h_max, q.h);
+  std::vector<double> table(2 * (size_t)n_bins + 1);
+  std::copy(edges, edges + n_bins + 1, table.begin());
+  rdf_inner_edges(edges, n_bins, h_max, reinterpret_cast<float2*>(table.data() + n_bins + 1));
+  // table and counts in the staging buffer (6 N doubles) where
+  // they fit, else allocated for the call (allocating and freeing takes longer than the histogram)
+  const bool own = table.size() + nc > 6 * (size_t)s->N;
+  if (!own) {
+    ed = s->stage;
+    cnt = reinterpret_cast<unsigned long long*>(s->stage + table.size());
+  } else if (cudaMalloc(&ed, sizeof(double) * table.size()) != cudaSuccess ||
+             cudaMalloc(&cnt, sizeof(unsigned long long) * nc) != cudaSuccess) {
     cudaGetLastError();
     if (ed) cudaFree(ed);
     return fail(s, MD_ENOMEM, "device memory for the histogram");
@@ -1030,13 +1041,13 @@ int md_rdf(md_system* s, int32_t n_bins, const double* edges, int64_t* counts) {
   s->profile = false;
   enqueue_rebin(s);
   s->profile = p;
-  if (cudaMemcpyAsync(ed, edges, sizeof(double) * (n_bins + 1), cudaMemcpyHostToDevice, s->st) != cudaSuccess ||
+  if (cudaMemcpyAsync(ed, table.data(), sizeof(double) * table.size(), cudaMemcpyHostToDevice, s->st) != cudaSuccess ||
       cudaMemsetAsync(cnt, 0, sizeof(unsigned long long) * nc, s->st) != cudaSuccess) {
     rc = fail(s, MD_ECUDA, "histogram set-up failed");
   } else {
     const double norm = (double)n_bins / (edges[n_bins] - edges[0]);
-    launch_rdf(s->mixed, s->x, (int)s->N, s->cell_start, s->perm, s->reps, s->n_reps, s->C, s->S, ed, n_bins, norm,
-               cnt, s->st);
+    launch_rdf(s->mixed, s->x, (int)s->N, s->cell_start, s->perm, s->pos, s->tag, s->reps, s->n_reps, s->C, ed,
+               reinterpret_cast<const float2*>(ed + n_bins + 1), n_bins, norm, cnt, s->st);
     if (cudaGetLastError() != cudaSuccess ||
         cudaMemcpyAsync(counts, cnt, sizeof(unsigned long long) * nc, cudaMemcpyDefault, s->st) != cudaSuccess)
       rc = fail(s, MD_ECUDA, "histogram kernel failed");
@@ -1047,8 +1058,10 @@ int md_rdf(md_system* s, int32_t n_bins, const double* edges, int64_t* counts) {
   } else {
     cudaStreamSynchronize(s->st);
   }
-  cudaFree(ed);
-  cudaFree(cnt);
+  if (own) {
+    cudaFree(ed);
+    cudaFree(cnt);
+  }
   return rc;
 }
 

@@ -312,10 +312,13 @@ void launch_integrate(bool mixed, IntegMode mode, bool ke, int thermostat, void*
                       cudaStream_t st);
 // RDF of non-bonded pairs (k_observe.cu): counts[r * n_bins + k] += pairs of
 // replica r with edges[k] <= r < edges[k + 1] (last bin closed); norm =
-// n_bins / (edges[n_bins] - edges[0]) gives the first guess of k
-void launch_rdf(bool mixed, const void* x, int N, const int* cell_start, const int* perm, const RepDev* reps,
-                int n_reps, int C, int sites, const double* edges, int n_bins, double norm,
-                unsigned long long* counts, cudaStream_t st);
+// n_bins / (edges[n_bins] - edges[0]) gives the first guess of k.  pos and tag
+// are those of a rebin of the current positions; inner[k] (device) is filled
+// by rdf_inner_edges (host) with h_max the largest cell side of the replicas
+void rdf_inner_edges(const double* edges, int n_bins, double h_max, float2* inner);
+void launch_rdf(bool mixed, const void* x, int N, const int* cell_start, const int* perm, const float4* pos,
+                const int* tag, const RepDev* reps, int n_reps, int C, const double* edges, const float2* inner,
+                int n_bins, double norm, unsigned long long* counts, cudaStream_t st);
 // ACF: add sample s (ring slot s % (max_lag + 1)) to acc[r][tau], tau <= min(s, max_lag)
 void launch_acf_add(const double* ring, int n_chains_total, const RepDev* reps, int n_reps, long long s, int max_lag,
                     double* acc, cudaStream_t st);
