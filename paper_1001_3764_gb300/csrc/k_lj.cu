@@ -2,7 +2,8 @@
 // Sec. 3.2) with every pair evaluated once (Newton's third law).
 //
 // Work unit: a region of up to G x G x 1 cells (G = 2 or 3; cells of side
-// >= r_c + skin, Sec. 3.1), one thread block per region.  The block stages in
+// >= r_c + skin, Sec. 3.1), one thread block per region, or in small systems
+// several blocks that share a region's clusters.  The block stages in
 // shared memory the "tile": the region's cells and every cell that one of
 // them reaches by one of the 13 forward offsets of a half shell (27 cells
 // for G = 2, 44 for G = 3), each cell a contiguous run of sorted atoms, moved
@@ -61,17 +62,17 @@ struct RegTile {
   int n_tile, n_home;
 };
 
-// Threads 0..63 read the tile cells' bounds, then one warp scans the counts
-// (two cells per lane: up to 64 tile cells); needs NT >= 64.
-__device__ __forceinline__ void region_setup(RegTile& T, const Region& g, const RegionShape& S, const RepDev& R,
-                                             const int* __restrict__ cell_start, const int* __restrict__ cl_start) {
+// Threads 0..63 read the tile cells' bounds (their ids come from a table made
+// once: two dependent loads, the ids and the bounds), then one warp scans the
+// counts (two cells per lane: up to 64 tile cells); needs NT >= 64.
+__device__ __forceinline__ void region_setup(RegTile& T, const WorkItem& item, const RegionShape& S,
+                                             const int* __restrict__ cells, const int* __restrict__ cell_start,
+                                             const int* __restrict__ cl_start) {
   const int k = threadIdx.x;
   if (k < kMaxTileCells) {
     int n = 0;
-    if (k < S.n_tile) {
-      const int M = R.M;
-      const int cx = (g.ox + S.off[k][0] + M) % M, cy = (g.oy + S.off[k][1] + M) % M, cz = (g.oz + S.off[k][2] + M) % M;
-      const int c = R.cell_base + (cz * M + cy) * M + cx;
+    const int c = k < kRegionCells ? __ldg(cells + kRegionCells * item.region + k) : -1;   // -1 past the last tile cell
+    if (c >= 0) {
       T.start[k] = cell_start[c];
       n = cell_start[c + 1] - T.start[k];
       T.sx[k] = (float)S.off[k][0] - S.cx;
@@ -114,16 +115,18 @@ __device__ __forceinline__ void region_setup(RegTile& T, const Region& g, const 
 // Copy the tile into shared memory in the region frame.  Warps take tile
 // cells in turn and their lanes start asynchronous copies (cp.async, global
 // to shared without registers) of the cell's atoms, so the whole tile is in
-// flight at once; after the wait and a barrier, a warp per tile cell adds
-// the cell's frame shift.  The w component keeps the LJ type
+// flight at once; a lane then waits for its own copies and adds the cell's
+// frame shift to the atoms it copied, without a barrier in between.  The w component keeps the LJ type
 // (0.0 / 1.0) that binning and integration store; WITH_TAG (list build)
 // replaces it by the bits of the atom's chain/site tag, which the build
 // needs instead.  tile_issue starts the copies, tile_finish waits for them,
 // shifts, and ends with a barrier.
 template <int NT>
-__device__ __forceinline__ void tile_issue(const RegTile& T, const float4* __restrict__ pos, float4* __restrict__ sp) {
-  const int nt = T.n_tile, lane = threadIdx.x & 31;
-  for (int k = threadIdx.x >> 5; k < nt; k += NT / 32) {
+__device__ __forceinline__ void tile_issue(const RegTile& T, unsigned long long need, const float4* __restrict__ pos,
+                                           float4* __restrict__ sp) {
+  const int lane = threadIdx.x & 31;
+  for (int k = threadIdx.x >> 5; k < T.n_tile; k += NT / 32) {
+    if (!((need >> k) & 1ull)) continue;
     const int t0 = T.off[k], n = T.off[k + 1] - t0;
     const float4* src = pos + T.start[k];
     const unsigned dst = (unsigned)__cvta_generic_to_shared(sp + t0);
@@ -135,12 +138,12 @@ __device__ __forceinline__ void tile_issue(const RegTile& T, const float4* __res
 }
 
 template <bool WITH_TAG, int NT>
-__device__ __forceinline__ void tile_finish(const RegTile& T, float4* __restrict__ sp, const int* __restrict__ tag) {
-  const int nt = T.n_tile;
+__device__ __forceinline__ void tile_finish(const RegTile& T, unsigned long long need, float4* __restrict__ sp,
+                                            const int* __restrict__ tag) {
   asm volatile("cp.async.wait_group 0;" ::: "memory");
-  __syncthreads();
   const int lane = threadIdx.x & 31;
-  for (int k = threadIdx.x >> 5; k < nt; k += NT / 32) {
+  for (int k = threadIdx.x >> 5; k < T.n_tile; k += NT / 32) {
+    if (!((need >> k) & 1ull)) continue;
     const int t0 = T.off[k], n = T.off[k + 1] - t0, j0 = T.start[k];
     const float ox = T.sx[k], oy = T.sy[k], oz = T.sz[k];
     for (int q = lane; q < n; q += 32) {
@@ -228,42 +231,40 @@ __device__ __forceinline__ unsigned pair_mask(const float4 (&pi)[4], const int (
 template <int NT, bool GEN>
 __global__ void __launch_bounds__(NT, 1024 / NT) k_cl_build(const float4* __restrict__ pos, const int* __restrict__ tag,
                                                  const int* __restrict__ cell_start, const int* __restrict__ cl_start,
-                                                 const Region* __restrict__ regions, int n_regions,
+                                                 const int* __restrict__ cells,
+                                                 const WorkItem* __restrict__ items,
                                                  const RegionShape* __restrict__ shapes, const RepDev* __restrict__ reps,
                                                  unsigned* __restrict__ list, int* __restrict__ ncl, int cap,
-                                                 int tile_cap, unsigned* __restrict__ flags, int persistent,
-                                                 int* __restrict__ work, const TopoDev tp) {
+                                                 int tile_cap, unsigned* __restrict__ flags, int* __restrict__ n_tasks,
+                                                 const TopoDev tp) {
   extern __shared__ __align__(16) unsigned char smem[];
   float4* sp = reinterpret_cast<float4*>(smem);   // w: the atom's chain/site tag bits
   __shared__ RegTile T;
-  __shared__ int sh_r;
   __shared__ int queue[NT / 32][kBuildQueue];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int* qw = queue[warp];
-  for (int it = 0;; ++it) {
-    const int r = next_region(persistent != 0, it, work, &sh_r);
-    if (r < 0 || r >= n_regions) break;
-    const Region g = regions[r];
-    const RegionShape& S = shapes[g.shape];
-    const RepDev& R = reps[g.rep];
-    __syncthreads();   // the previous region's tile is no longer read
-    region_setup(T, g, S, R, cell_start, cl_start);
-    const int total = T.off[T.n_tile];
+  {
+    const WorkItem item = items[blockIdx.x];
+    const RegionShape& S = shapes[item.shape];
+    const RepDev& R = reps[item.rep];
+    if (blockIdx.x == 0 && threadIdx.x == 0) *n_tasks = 0;   // for k_cl_rank
+    region_setup(T, item, S, cells, cell_start, cl_start);
+    const int total = T.off[T.n_tile], q_end = T.ncl[item.h1], q_first = T.ncl[item.h0] + item.part;
     if (total > tile_cap) {
       if (threadIdx.x == 0) atomicOr(flags, kFlagNbrOverflow);
-      for (int q = threadIdx.x; q < T.ncl[T.n_home]; q += NT) {
+      for (int q = q_first + item.parts * (int)threadIdx.x; q < q_end; q += item.parts * NT) {
         int h, k;
         cluster_of(T, q, h, k);
         ncl[T.cl0[h] + k] = 0;
       }
-      continue;
+      return;
     }
-    tile_issue<NT>(T, pos, sp);
-    tile_finish<true, NT>(T, sp, tag);
+    tile_issue<NT>(T, item.need, pos, sp);
+    tile_finish<true, NT>(T, item.need, sp, tag);
     const float rl2 = R.rlist2u;
     const float rl = sqrtf(rl2);
     const unsigned lt = (1u << lane) - 1u;
-    for (int q = warp; q < T.ncl[T.n_home]; q += NT / 32) {
+    for (int q = q_first + item.parts * warp; q < q_end; q += item.parts * (NT / 32)) {
       int h, k;
       cluster_of(T, q, h, k);
       const int i0 = T.off[h] + 4 * k;
@@ -363,12 +364,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_cl_build(const float4* __rest
       }
     }
   }
-  if (persistent) persistent_done(work);
 }
 
 // ===================================================================== force
 constexpr int kEnergyVals = 8;           // lj, lj_shifted, vxx, vyy, vzz, vxy, vxz, vyz
-constexpr int kRegionClusterCap = 512;   // clusters of one region (2,048 home atoms); more is reported
 
 // FP32 force (cell units) -> fixed point 2^-13 kJ/mol/nm; F2I saturates
 // beyond +-2^31 (2^18 kJ/mol/nm)
@@ -553,14 +552,13 @@ __device__ __forceinline__ LjConst lj_const(const RepDev& R) {
   return c;
 }
 
-// One warp task: clusters s_ord[q0 .. q0 + 32/LP) of the region, LP lanes
+// One warp task: clusters s_tab[q0 .. q0 + 32/LP) of the item, LP lanes
 // each; lane l of a cluster's group takes entries l, l + LP, ...  The warp's
 // trip count is that of its longest cluster; a lane past its own list idles.
 template <bool ENERGY, int LP, bool EXACT = false>
 __device__ __forceinline__ void cluster_task(int q0, int nq, const RegTile& T, const float4* __restrict__ sp,
                                              int* __restrict__ ax, int* __restrict__ ay, int* __restrict__ az,
-                                             const int* __restrict__ s_key, const short* __restrict__ s_ord,
-                                             const int* __restrict__ s_cl, const int* __restrict__ s_in,
+                                             const ClusterTask* __restrict__ s_tab,
                                              float (*__restrict__ ecl)[kEnergyVals], const unsigned* __restrict__ list,
                                              int cap, const RepDev& R, const ForceParams& fp, const LjConst& c,
                                              unsigned* __restrict__ flags) {
@@ -572,13 +570,13 @@ __device__ __forceinline__ void cluster_task(int q0, int nq, const RegTile& T, c
   const float cs = EXACT ? scale : 1.f;
   const float A0 = c.A0 * cs, A1 = c.A1 * cs, A2 = c.A2 * cs, B0 = c.B0 * cs, B1 = c.B1 * cs, B2 = c.B2 * cs;
   const bool valid = q0 + sub < nq;
-  const int q = valid ? (int)s_ord[q0 + sub] : nq;
-  const int in = s_in[valid ? q : nq - 1];   // first tile atom << 7 | chain-end bits << 3 | atoms
+  const ClusterTask ct = s_tab[valid ? q0 + sub : nq - 1];
+  const int in = ct.z;   // first tile atom << 7 | chain-end bits << 3 | atoms
   const int i0 = in >> 7;
   const int ni = valid ? (in & 7) : 0;
-  const int n = valid ? s_key[q] >> 9 : 0;
+  const int n = valid ? ct.x : 0;
   // the task's clusters are consecutive in longest-first order: the first is the longest
-  const int nmax = s_key[s_ord[q0]] >> 9;
+  const int nmax = s_tab[q0].x;
   float4 pi[4];   // w: LJ type (1.0 for a C_33 chain end)
 #pragma unroll
   for (int u = 0; u < 4; ++u) pi[u] = sp[i0 + max(0, min(u, ni - 1))];
@@ -614,22 +612,24 @@ __device__ __forceinline__ void cluster_task(int q0, int nq, const RegTile& T, c
 #pragma unroll
     for (int a = 0; a < kEnergyVals; ++a) ev2[a] = make_float2(0.f, 0.f);
   }
-  const unsigned* L = list + (size_t)(valid ? s_cl[q] : 0) * cap;
+  const unsigned* L = list + (size_t)ct.y * cap;
   // clusters without a chain end (the common case) share one pair
   // coefficient per j type: two scalar FMAs per entry instead of four
   // FFMA2 (same values: each coefficient is the same single-rounded FMA)
   const unsigned tb = ((unsigned)in >> 3) & 15u;   // bit u: atom u is a C_33 chain end
   const bool uni = __all_sync(0xffffffffu, tb == 0u);
   // two entries per lane per iteration (independent work for the
-  // scheduler), the next two in flight; an entry past the list is 0:
-  // tile atom 0 with an empty mask, which adds nothing
+  // scheduler), the next two in flight; an entry past the list is the
+  // cluster's own first atom (staged in any split of the region) with an
+  // empty mask, which adds nothing
+  const unsigned pad = (unsigned)i0;
   auto run = [&](auto uni_tag) {
     constexpr bool UNI = decltype(uni_tag)::value;
-    unsigned E0 = sl < n ? __ldg(L + sl) : 0u;
-    unsigned E1 = sl + LP < n ? __ldg(L + sl + LP) : 0u;
+    unsigned E0 = sl < n ? __ldg(L + sl) : pad;
+    unsigned E1 = sl + LP < n ? __ldg(L + sl + LP) : pad;
     for (int e = sl; e - sl < nmax; e += 2 * LP) {
-      const unsigned E2 = e + 2 * LP < n ? __ldg(L + e + 2 * LP) : 0u;
-      const unsigned E3 = e + 3 * LP < n ? __ldg(L + e + 3 * LP) : 0u;
+      const unsigned E2 = e + 2 * LP < n ? __ldg(L + e + 2 * LP) : pad;
+      const unsigned E3 = e + 3 * LP < n ? __ldg(L + e + 3 * LP) : pad;
       const int t0 = (int)(E0 & 0xffffu), t1 = (int)(E1 & 0xffffu);
       const float4 w0 = sp[t0], w1 = sp[t1];
       float g0x = 0.f, g0y = 0.f, g0z = 0.f, g1x = 0.f, g1y = 0.f, g1z = 0.f;
@@ -787,19 +787,21 @@ __device__ __forceinline__ void cluster_task(int q0, int nq, const RegTile& T, c
       float v = ev[a];
 #pragma unroll
       for (int o = LP / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (sl == 0 && valid) ecl[q][a] = v;
+      if (sl == 0 && valid) ecl[ct.w][a] = v;
     }
   }
 }
 
-// Add the tile's accumulators to the int64 forces (2^-32 kJ/mol/nm): warps
-// w0, w0 + nw, ... take tile cells; one integer atomic per component and
-// tile atom with a non-zero sum (consecutive atoms: coalesced).
-__device__ __forceinline__ void flush_tile(const RegTile& T, const int* __restrict__ ax, const int* __restrict__ ay,
-                                           const int* __restrict__ az, long long* __restrict__ flj, int Npad, int w0,
-                                           int nw) {
+// Add the accumulators of the needed tile cells to the int64 forces (2^-32
+// kJ/mol/nm): warps take tile cells in turn; one integer atomic per component
+// and tile atom with a non-zero sum (consecutive atoms: coalesced).
+template <int NT>
+__device__ __forceinline__ void flush_tile(const RegTile& T, unsigned long long need, const int* __restrict__ ax,
+                                           const int* __restrict__ ay, const int* __restrict__ az,
+                                           long long* __restrict__ flj, int Npad) {
   const int lane = threadIdx.x & 31;
-  for (int kc = w0; kc < T.n_tile; kc += nw) {
+  for (int kc = threadIdx.x >> 5; kc < T.n_tile; kc += NT / 32) {
+    if (!((need >> kc) & 1ull)) continue;
     const int t0 = T.off[kc], nk = T.off[kc + 1] - t0, s0 = T.start[kc];
     for (int q = lane; q < nk; q += 32) {
       const int t = t0 + q, sidx = s0 + q;
@@ -814,57 +816,86 @@ __device__ __forceinline__ void flush_tile(const RegTile& T, const int* __restri
   }
 }
 
-// Per region: the clusters' FP32 sums added in FP64 in cluster order; the
-// region's sums go to the slot of its first home cell, zeros to the others
-// (the reduction sums a replica's cell slots).  Lanes 0..7 of the caller.
-__device__ __forceinline__ void region_energy(const RegTile& T, int nq, bool fits,
-                                              const float (*__restrict__ ecl)[kEnergyVals], double* __restrict__ epart,
-                                              int a) {
+// Per home cell: its clusters' FP32 sums added in FP64 in cluster order,
+// thread a + 8 c of the block the value a of the item's cell c (so the sums do
+// not depend on how a region is split).
+__device__ __forceinline__ void cell_energy(const RegTile& T, const WorkItem& item, bool fits,
+                                            const float (*__restrict__ ecl)[kEnergyVals], double* __restrict__ epart) {
+  const int a = threadIdx.x % kEnergyVals, h = item.h0 + threadIdx.x / kEnergyVals;
+  if (h >= item.h1) return;
   double v = 0.0;
   if (fits)
-    for (int q = 0; q < nq; ++q) v += (double)ecl[q][a];
-  epart[(size_t)T.home_cell[0] * kEnergyVals + a] = v;
-  for (int hh = 1; hh < T.n_home; ++hh) epart[(size_t)T.home_cell[hh] * kEnergyVals + a] = 0.0;
+    for (int q = T.ncl[h] - T.ncl[item.h0]; q < T.ncl[h + 1] - T.ncl[item.h0]; ++q) v += (double)ecl[q][a];
+  epart[(size_t)T.home_cell[h] * kEnergyVals + a] = v;
 }
 
-// longest list first: warps that take the last clusters finish soon, and
-// the clusters that share a warp have similar lengths.  Cluster q's key is
+// The order in which the force kernel takes an item's clusters, made once per
+// list build (it was made in every launch: 3 us of a block's 26): longest
+// list first, so that warps that take the last clusters finish soon and the
+// clusters that share a warp have similar lengths.  Cluster q's key is
 // (list length << 9) | (511 - q), unique (q < 512) so that ties go to the
-// lower index; its rank is the number of larger keys (threads t0, t0 + nt,
-// ...; four keys per shared load, the slots past nq hold -1).  The same
-// thread records in s_in which of the cluster's four slots hold a C_33
-// chain end (bit u; a slot past the cell's last atom repeats that atom).
-__device__ __forceinline__ void rank_clusters(const int* __restrict__ s_key, short* __restrict__ s_ord,
-                                              int* __restrict__ s_in, const float4* __restrict__ sp, int nq, int t0,
-                                              int nt) {
+// lower index; its rank is the number of larger keys (four keys per shared
+// load, the slots past nq hold -1).  The chain-end bits tell which of the
+// cluster's four slots hold a C_33 (bit u; a slot past the cell's last atom
+// repeats that atom).
+constexpr int kRankThreads = 128;
+__global__ void __launch_bounds__(kRankThreads) k_cl_rank(const float4* __restrict__ pos,
+                                                          const int* __restrict__ cell_start,
+                                                          const int* __restrict__ cl_start,
+                                                          const int* __restrict__ cells,
+                                                          const WorkItem* __restrict__ items,
+                                                          const RegionShape* __restrict__ shapes,
+                                                          const int* __restrict__ ncl, ClusterTask* __restrict__ tasks,
+                                                          int* __restrict__ task_base, int* __restrict__ n_tasks) {
+  __shared__ RegTile T;
+  __shared__ __align__(16) int s_key[kRegionClusterCap];
+  __shared__ int base;
+  const WorkItem item = items[blockIdx.x];
+  region_setup(T, item, shapes[item.shape], cells, cell_start, cl_start);
+  const int q_first = T.ncl[item.h0], nq = T.ncl[item.h1] - q_first;
+  if (T.ncl[T.n_home] > kRegionClusterCap) return;   // reported by the force kernel
+  if (threadIdx.x == 0) task_base[blockIdx.x] = base = atomicAdd(n_tasks, nq);
+  for (int q = threadIdx.x; q < ((nq + 3) & ~3); q += kRankThreads) {
+    int key = -1;
+    if (q < nq) {
+      int h, k;
+      cluster_of(T, q_first + q, h, k);
+      key = (__ldg(ncl + T.cl0[h] + k) << 9) | (511 - q);
+    }
+    s_key[q] = key;
+  }
+  __syncthreads();
   const int4* k4 = reinterpret_cast<const int4*>(s_key);
   const int n4 = (nq + 3) >> 2;
-  for (int q = t0; q < nq; q += nt) {
+  for (int q = threadIdx.x; q < nq; q += kRankThreads) {
     const int kq = s_key[q];
     int rank = 0;
     for (int o = 0; o < n4; ++o) {
       const int4 k = k4[o];
       rank += (k.x > kq) + (k.y > kq) + (k.z > kq) + (k.w > kq);
     }
-    s_ord[rank] = (short)q;
-    const int in = s_in[q], i0 = in >> 7, ni = in & 7;
+    int h, k;
+    cluster_of(T, q_first + q, h, k);
+    const int ni = min(4, T.off[h + 1] - T.off[h] - 4 * k);
     unsigned tb = 0u;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) tb |= sp[i0 + min(u, ni - 1)].w != 0.f ? (1u << u) : 0u;
-    s_in[q] = in | (int)(tb << 3);
+    for (int u = 0; u < 4; ++u) tb |= pos[T.start[h] + 4 * k + min(u, ni - 1)].w != 0.f ? (1u << u) : 0u;
+    tasks[base + rank] =
+        make_int4(kq >> 9, T.cl0[h] + k, ((T.off[h] + 4 * k) << 7) | (int)(tb << 3) | ni, q);
   }
 }
 
-// One block per region (grid schedule), or a fixed grid whose blocks take
-// regions from a device counter (persistent schedule).  The block stages
+// One block per work item (grid schedule), or a fixed grid whose blocks take
+// items from a device counter (persistent schedule).  The block stages
 // the tile, its warps take tasks of 32/LP clusters from a shared counter
 // (longest lists first), and after a barrier the block flushes the tile's
 // accumulators.
 template <bool ENERGY, int NT, int LP, bool EXACT = false>
 __global__ void __launch_bounds__(NT, 768 / NT) k_cl_force(
     const float4* __restrict__ pos, const int* __restrict__ cell_start, const int* __restrict__ cl_start,
-    const Region* __restrict__ regions, int n_regions, const RegionShape* __restrict__ shapes,
-    const RepDev* __restrict__ reps, const unsigned* __restrict__ list, const int* __restrict__ ncl, int cap,
+    const int* __restrict__ cells, const WorkItem* __restrict__ items, int n_items,
+    const RegionShape* __restrict__ shapes, const RepDev* __restrict__ reps, const unsigned* __restrict__ list,
+    const ClusterTask* __restrict__ tasks, const int* __restrict__ task_base, int cap,
     int tile_cap, const ForceParams fp, long long* __restrict__ flj, int Npad, double* __restrict__ epart,
     unsigned* __restrict__ flags, int persistent, int* __restrict__ work) {
   constexpr int CPW = 32 / LP;
@@ -877,10 +908,7 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_cl_force(
   int* az = ax + 2;
   __shared__ RegTile T;
   __shared__ int sh_r, sh_q;
-  __shared__ __align__(16) int s_key[kRegionClusterCap];   // (list length << 9) | (511 - q) of cluster q
-  __shared__ short s_ord[kRegionClusterCap];   // the clusters, longest list first (ties: lower index)
-  __shared__ int s_cl[kRegionClusterCap];      // global id of each of the region's clusters
-  __shared__ int s_in[kRegionClusterCap];      // first tile atom << 7 | chain-end bits << 3 | atoms (1..4)
+  __shared__ ClusterTask s_tab[kRegionClusterCap];   // the item's clusters, longest list first
   // energy form: each cluster's 8 sums (FP32 lane tree), added over the
   // region's clusters in cluster order, so the result does not depend on
   // which warp took which cluster
@@ -888,50 +916,43 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_cl_force(
   const int lane = threadIdx.x & 31;
   for (int it = 0;; ++it) {
     const int r = next_region(persistent != 0, it, work, &sh_r);
-    if (r < 0 || r >= n_regions) break;
-    const Region g = regions[r];
-    const RegionShape& S = shapes[g.shape];
-    const RepDev& R = reps[g.rep];
-    __syncthreads();   // the previous region's tables are no longer read
-    region_setup(T, g, S, R, cell_start, cl_start);
+    if (r < 0 || r >= n_items) break;
+    const WorkItem item = items[r];
+    const RegionShape& S = shapes[item.shape];
+    const RepDev& R = reps[item.rep];
+    const int t_base = task_base[r];
+    __syncthreads();   // the previous item's tables are no longer read
+    region_setup(T, item, S, cells, cell_start, cl_start);
     const int total = T.off[T.n_tile];
-    const int nq = T.ncl[T.n_home];
-    const bool fits = total <= tile_cap && nq <= kRegionClusterCap;
+    const int q_first = T.ncl[item.h0], nq = T.ncl[item.h1] - q_first;   // the item's clusters
+    const bool fits = total <= tile_cap && T.ncl[T.n_home] <= kRegionClusterCap;
     if (!fits) {
       if (threadIdx.x == 0) atomicOr(flags, kFlagNbrOverflow);
     } else {
-      // list lengths and zeroed accumulators while the tile copies fly
-      tile_issue<NT>(T, pos, sp);
+      // the item's tasks and zeroed accumulators while the tile copies fly
+      for (int q = threadIdx.x; q < nq; q += NT)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(s_tab + q)),
+                     "l"(tasks + t_base + q)
+                     : "memory");
+      tile_issue<NT>(T, item.need, pos, sp);
       if (!ENERGY)   // 3 tile_cap is a multiple of 4: the rounded-up span stays in the buffer
         for (int t = threadIdx.x; t < (3 * total + 3) / 4; t += NT) reinterpret_cast<int4*>(ax)[t] = make_int4(0, 0, 0, 0);
-      for (int q = threadIdx.x; q < ((nq + 3) & ~3); q += NT) {
-        if (q >= nq) { s_key[q] = -1; continue; }
-        int h, k;
-        cluster_of(T, q, h, k);
-        const int cl = T.cl0[h] + k, i0 = T.off[h] + 4 * k;
-        s_key[q] = (__ldg(ncl + cl) << 9) | (511 - q);
-        s_cl[q] = cl;
-        s_in[q] = (i0 << 7) | min(4, T.off[h + 1] - i0);
-      }
       if (threadIdx.x == 0) sh_q = 0;
-      tile_finish<false, NT>(T, sp, nullptr);   // ends with a barrier
-      rank_clusters(s_key, s_ord, s_in, sp, nq, threadIdx.x, NT);
-      __syncthreads();
+      tile_finish<false, NT>(T, item.need, sp, nullptr);   // ends with a barrier
       const LjConst c = lj_const(R);
       for (;;) {
         int q0 = 0;
         if (lane == 0) q0 = atomicAdd(&sh_q, CPW);
         q0 = __shfl_sync(0xffffffffu, q0, 0);
         if (q0 >= nq) break;
-        cluster_task<ENERGY, LP, EXACT>(q0, nq, T, sp, ax, ay, az, s_key, s_ord, s_cl, s_in, ecl, list, cap, R, fp, c,
-                                        flags);
+        cluster_task<ENERGY, LP, EXACT>(q0, nq, T, sp, ax, ay, az, s_tab, ecl, list, cap, R, fp, c, flags);
       }
       __syncthreads();
-      if (!ENERGY) flush_tile(T, ax, ay, az, flj, Npad, threadIdx.x >> 5, NT / 32);
+      if (!ENERGY) flush_tile<NT>(T, item.need, ax, ay, az, flj, Npad);
     }
     if (ENERGY) {
       __syncthreads();
-      if (threadIdx.x < kEnergyVals) region_energy(T, nq, fits, ecl, epart, threadIdx.x);
+      cell_energy(T, item, fits, ecl, epart);
     }
   }
   if (persistent) persistent_done(work);
@@ -942,32 +963,39 @@ size_t cl_build_smem(int tile_cap) { return (size_t)tile_cap * sizeof(float4); }
 size_t cl_force_smem(int tile_cap) { return (size_t)tile_cap * (sizeof(float4) + 3 * sizeof(int)); }
 
 void launch_cl_build(const float4* pos, const int* tag, const int* cell_start, const int* cl_start,
-                     const Region* regions, int n_regions, const RegionShape* shapes, const RepDev* reps,
-                     unsigned* list, int* ncl, int cap, int tile_cap, unsigned* flags, int persistent_grid, int* work,
-                     const TopoDev* topo, cudaStream_t st) {
-  if (n_regions <= 0) return;
-  const int grid = persistent_grid > 0 ? persistent_grid : n_regions;
+                     const int* cells, const WorkItem* items, int n_items, const RegionShape* shapes,
+                     const RepDev* reps, unsigned* list, int* ncl, int cap, int tile_cap, unsigned* flags,
+                     int* n_tasks, const TopoDev* topo, cudaStream_t st) {
+  if (n_items <= 0) return;
   const size_t sm = cl_build_smem(tile_cap);
   if (topo)
-    k_cl_build<256, true><<<grid, 256, sm, st>>>(pos, tag, cell_start, cl_start, regions, n_regions, shapes, reps, list,
-                                                 ncl, cap, tile_cap, flags, persistent_grid > 0, work, *topo);
+    k_cl_build<256, true><<<n_items, 256, sm, st>>>(pos, tag, cell_start, cl_start, cells, items, shapes, reps, list,
+                                                    ncl, cap, tile_cap, flags, n_tasks, *topo);
   else
-    k_cl_build<256, false><<<grid, 256, sm, st>>>(pos, tag, cell_start, cl_start, regions, n_regions, shapes, reps,
-                                                  list, ncl, cap, tile_cap, flags, persistent_grid > 0, work, TopoDev{});
+    k_cl_build<256, false><<<n_items, 256, sm, st>>>(pos, tag, cell_start, cl_start, cells, items, shapes, reps,
+                                                     list, ncl, cap, tile_cap, flags, n_tasks, TopoDev{});
+}
+
+void launch_cl_rank(const float4* pos, const int* cell_start, const int* cl_start, const int* cells,
+                    const WorkItem* items, int n_items, const RegionShape* shapes, const int* ncl, ClusterTask* tasks,
+                    int* task_base, int* n_tasks, cudaStream_t st) {
+  if (n_items > 0)
+    k_cl_rank<<<n_items, kRankThreads, 0, st>>>(pos, cell_start, cl_start, cells, items, shapes, ncl, tasks,
+                                                 task_base, n_tasks);
 }
 
 void launch_cl_force(bool energy, const float4* pos, const int* cell_start, const int* cl_start,
-                     const Region* regions, int n_regions, const RegionShape* shapes, const RepDev* reps,
-                     const unsigned* list, const int* ncl, int cap, int tile_cap, const ForceParams& fp,
-                     long long* flj, int Npad, double* epart, unsigned* flags, int block, int lanes,
-                     int persistent_grid, int* work, bool exact, cudaStream_t st) {
-  if (n_regions <= 0) return;
-  const int grid = persistent_grid > 0 ? persistent_grid : n_regions;
+                     const int* cells, const WorkItem* items, int n_items, const RegionShape* shapes,
+                     const RepDev* reps, const unsigned* list, const ClusterTask* tasks, const int* task_base,
+                     int cap, int tile_cap, const ForceParams& fp, long long* flj, int Npad, double* epart, unsigned* flags, int block,
+                     int lanes, int persistent_grid, int* work, bool exact, cudaStream_t st) {
+  if (n_items <= 0) return;
+  const int grid = persistent_grid > 0 ? persistent_grid : n_items;
   const int pers = persistent_grid > 0;
   const size_t sm = cl_force_smem(tile_cap);
-#define MDG_CLF(E, NT, LP, X)                                                                                    \
-  k_cl_force<E, NT, LP, X><<<grid, NT, sm, st>>>(pos, cell_start, cl_start, regions, n_regions, shapes, reps, list, \
-                                                 ncl, cap, tile_cap, fp, flj, Npad, epart, flags, pers, work)
+#define MDG_CLF(E, NT, LP, X)                                                                                      \
+  k_cl_force<E, NT, LP, X><<<grid, NT, sm, st>>>(pos, cell_start, cl_start, cells, items, n_items, shapes, reps, \
+                                                 list, tasks, task_base, cap, tile_cap, fp, flj, Npad, epart, flags, pers, work)
 #define MDG_CLF2(NT, LP)                  \
   if (energy) MDG_CLF(true, NT, LP, false); \
   else if (exact) MDG_CLF(false, NT, LP, true); \

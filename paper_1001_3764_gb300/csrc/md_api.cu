@@ -25,12 +25,15 @@ using namespace mdg;
 namespace {
 
 constexpr int kIntTile = 224;    // atoms per integrator / bonded block (original order)
+constexpr int kSMs = 152;        // streaming multiprocessors of a GB300
 constexpr int kNumProf = 5;      // rebin, neighbour build, integrate, lj, bonded
 constexpr double kKB = 0.0083144626;
 
 thread_local std::string g_create_error;
 
 size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
+
+struct RegionRef { int rep, shape; };   // a region's replica and shape
 
 }  // namespace
 
@@ -64,10 +67,16 @@ struct md_system {
   int* ncl = nullptr;                        // entries per cluster
   int* cl_start = nullptr;                   // first cluster of each cell [C + 1]
   int64_t n_cl_max = 0;
-  std::vector<Region> regions_h;
+  std::vector<RegionRef> regions_h;
+  std::vector<int> region_cells_h;           // tile cells of every region (kRegionCells each, -1 past the last)
   std::vector<RegionShape> shapes_h;
-  Region* regions = nullptr;
+  int* region_cells = nullptr;
   RegionShape* shapes = nullptr;
+  std::vector<WorkItem> items_h;             // blocks of the LJ kernel, then those of the list build
+  WorkItem* items = nullptr;
+  int n_lj_items = 0, n_build_items = 0;
+  ClusterTask* tasks = nullptr;              // each LJ item's clusters in task order, from task_base[item] on
+  int *task_base = nullptr, *n_tasks = nullptr;
   int tile_cap = 0;
   int lj_block = 256, persistent_grid = 0;   // persistent_grid > 0: fixed grid for the LJ kernel
   int lj_lanes = 8;                          // lanes per 4-atom cluster in the LJ kernel
@@ -212,6 +221,87 @@ static RegionShape make_shape(int sx, int sy) {
   S.cy = 0.5f * (float)(sy - 1);
   S.cz = 0.f;
   return S;
+}
+
+// Work items of one region: its home cells in groups of `rows` rows of the
+// shape (0: single cells), each group's clusters over `parts` blocks.
+static void add_items(md_system* s, int region, int rows, int parts) {
+  const RegionRef g = s->regions_h[region];
+  const RegionShape& S = s->shapes_h[g.shape];
+  const int sx = g.shape % s->lj_region + 1;
+  const int step = rows > 0 ? rows * sx : 1;
+  for (int h = 0; h < S.n_home; h += step) {
+    WorkItem w{};
+    w.region = region;
+    w.rep = g.rep;
+    w.shape = g.shape;
+    w.h0 = (unsigned char)h;
+    w.h1 = (unsigned char)std::min(S.n_home, h + step);
+    w.parts = (unsigned char)parts;
+    for (int c = w.h0; c < w.h1; ++c)
+      for (int q = 0; q < 14; ++q) w.need |= 1ull << S.nb[c][q];
+    for (int p = 0; p < parts; ++p) {
+      w.part = (unsigned char)p;
+      s->items_h.push_back(w);
+    }
+  }
+}
+
+// Regions of G x G x 1 cells over every replica (narrower at the high faces
+// when G does not divide M), their tile cells, and the work items.
+static void plan_regions(md_system* s) {
+  const int G = s->lj_region;
+  s->regions_h.clear();
+  s->region_cells_h.clear();
+  for (int r = 0; r < s->n_reps; ++r) {
+    const int M = s->reps_h[r].M, base = s->reps_h[r].cell_base;
+    for (int z = 0; z < M; ++z)
+      for (int y = 0; y < M; y += G)
+        for (int x = 0; x < M; x += G) {
+          const int shape = (std::min(G, M - x) - 1) + G * (std::min(G, M - y) - 1);
+          const RegionShape& S = s->shapes_h[shape];
+          s->regions_h.push_back(RegionRef{r, shape});
+          for (int k = 0; k < kRegionCells; ++k) {
+            int c = -1;
+            if (k < S.n_tile) {
+              const int cx = (x + S.off[k][0] + M) % M, cy = (y + S.off[k][1] + M) % M, cz = (z + S.off[k][2] + M) % M;
+              c = base + (cz * M + cy) * M + cx;
+            }
+            s->region_cells_h.push_back(c);
+          }
+        }
+  }
+  // Work items, the regions with most cells first (narrow regions fill the
+  // tail: LJ 137.6 -> 128.1 us at 506k sites, M = 22, 47.8 -> 37.6 at 120k).
+  // A system of few regions is split, since a block spends 6 us on set-up
+  // and tail and 1.5 us per home cell, and two fit an SM.  LJ, us per launch:
+  //   cells while all are resident at once: 24.6 -> 14.2 at 1,500 sites, 27.8 -> 16.2 at 12,000
+  //   rows likewise (else whole): 25.6 -> 16.3 at 18,750, 24.8 -> 21.2 at 35,100; whole 47.7, rows 65.3 at 150k
+  //   between 1 and 2 regions per SM: rows from the second on (35.9 -> 27.4 at 84,000, M = 12)
+  const int R = (int)s->regions_h.size();
+  std::vector<int> order(R);
+  for (int r = 0; r < R; ++r) order[r] = r;
+  std::stable_sort(order.begin(), order.end(), [s](int a, int b) {
+    return s->shapes_h[s->regions_h[a].shape].n_home > s->shapes_h[s->regions_h[b].shape].n_home;
+  });
+  int n_rows = 0, n_cells = 0;
+  for (const RegionRef& g : s->regions_h) {
+    n_rows += g.shape / G + 1;
+    n_cells += s->shapes_h[g.shape].n_home;
+  }
+  constexpr int kWhole = 255;
+  s->items_h.clear();
+  const int lj_rows = n_cells <= 2 * kSMs ? 0 : n_rows <= 2 * kSMs ? 1 : kWhole;
+  for (int q = 0; q < R; ++q)
+    add_items(s, order[q], lj_rows == kWhole && R <= 2 * kSMs && q >= kSMs ? 1 : lj_rows, 1);
+  s->n_lj_items = (int)s->items_h.size();
+  // The list build gives a warp a cluster at a time (7 us alone), 8 warps a
+  // block, 4 blocks an SM: 108 -> 12 us at 1,500 sites (cells in 3 parts),
+  // 117 -> 19.5 at 12,000 (2), 113 -> 55 at 64,800 (1), 120 -> 103 at 150k and
+  // 312 -> 295 at 506k (rows; cells 110 and 338); whole 775, rows 819 at 1.5M
+  const int parts = n_cells <= 128 ? 3 : n_cells <= 256 ? 2 : 1;
+  for (int r : order) add_items(s, r, R >= 12 * kSMs ? kWhole : R >= 2 * kSMs ? 1 : 0, parts);
+  s->n_build_items = (int)s->items_h.size() - s->n_lj_items;
 }
 
 // The per-type lists of Sec. 3.3 from a molecule's bond graph: each atom's
@@ -385,18 +475,7 @@ static int configure(md_system* s, const md_desc* d) {
     if (cells >= (1 << 26)) return fail(s, MD_EINVAL, "too many cells");
   }
   s->N = atoms; s->C = (int)cells;
-  s->regions_h.clear();
-  for (int r = 0; r < s->n_reps; ++r) {
-    const int M = s->reps_h[r].M;
-    for (int z = 0; z < M; ++z)
-      for (int y = 0; y < M; y += G)
-        for (int x = 0; x < M; x += G) {
-          Region g{};
-          g.rep = r; g.ox = x; g.oy = y; g.oz = z;
-          g.shape = (std::min(G, M - x) - 1) + G * (std::min(G, M - y) - 1);
-          s->regions_h.push_back(g);
-        }
-  }
+  plan_regions(s);
   s->n_cl_max = (atoms + 3 * cells) / 4 + 1;   // sum of ceil(n_c / 4) over the cells
   s->Npad = (int)((atoms + 31) / 32 * 32);
   // default list capacity (entries per 4-atom cluster): a cluster's list holds
@@ -434,8 +513,12 @@ static size_t plan(md_system* s, char* base) {
   s->pos = (float4*)take(N * sizeof(float4));
   s->tag = (int*)take(N * sizeof(int));
   s->perm = (int*)take(N * sizeof(int));
-  s->regions = (Region*)take(sizeof(Region) * s->regions_h.size());
+  s->region_cells = (int*)take(sizeof(int) * s->region_cells_h.size());
   s->shapes = (RegionShape*)take(sizeof(RegionShape) * s->shapes_h.size());
+  s->items = (WorkItem*)take(sizeof(WorkItem) * s->items_h.size());
+  s->tasks = (ClusterTask*)take(sizeof(ClusterTask) * (size_t)s->n_cl_max);
+  s->task_base = (int*)take(sizeof(int) * (size_t)s->n_lj_items);
+  s->n_tasks = (int*)take(sizeof(int));
   s->list = (unsigned*)take((size_t)s->n_cl_max * s->cap * sizeof(unsigned));
   s->ncl = (int*)take((size_t)s->n_cl_max * sizeof(int));
   s->cl_start = (int*)take((C + 1) * sizeof(int));
@@ -481,6 +564,14 @@ static void prof_mark(md_system* s) {
     cudaEventRecord(s->ev[s->ev_used++], s->st);
 }
 
+static void enqueue_build(md_system* s) {
+  launch_cl_build(s->pos, s->tag, s->cell_start, s->cl_start, s->region_cells, s->items + s->n_lj_items,
+                  s->n_build_items, s->shapes, s->reps, s->list, s->ncl, s->cap, s->tile_cap, s->flags,
+                  s->n_tasks, s->generic ? &s->topo : nullptr, s->st);
+  launch_cl_rank(s->pos, s->cell_start, s->cl_start, s->region_cells, s->items, s->n_lj_items, s->shapes, s->ncl,
+                 s->tasks, s->task_base, s->n_tasks, s->st);
+}
+
 static void enqueue_rebin(md_system* s) {
   cudaMemsetAsync(s->count, 0, sizeof(int) * s->C, s->st);
   launch_bin_count(s->mixed, s->x, (int)s->N, s->tiles_int, (int)s->t_int.size(), s->reps, s->cell_of, s->cellc,
@@ -490,12 +581,10 @@ static void enqueue_rebin(md_system* s) {
   launch_cell_sort(s->mixed, s->x, (int)s->N, s->cell_start, s->tmp, s->fp.mtype, s->cellc, s->site, s->reps, s->n_reps, s->C,
                    s->S, s->perm, s->inv_perm, s->pos, s->tag, s->ref, s->flags, s->st);
   prof_mark(s);
-  launch_cl_build(s->pos, s->tag, s->cell_start, s->cl_start, s->regions, (int)s->regions_h.size(), s->shapes,
-                  s->reps, s->list, s->ncl, s->cap, s->tile_cap, s->flags, 0, s->work,
-                  s->generic ? &s->topo : nullptr, s->st);
+  enqueue_build(s);
   prof_mark(s);
 }
-static const int kRebinLaunches = 6;   // memset counted as a launch
+static const int kRebinLaunches = 7;   // memset counted as a launch
 
 // F_out: where the total force goes (the dynamics' s->F, or scratch for an
 // energy read-out, whose kernels need not reproduce the force bits of the
@@ -505,9 +594,9 @@ static void enqueue_forces(md_system* s, bool energy, void* F_out = nullptr) {
   long long* flj = F_out ? s->flj_e : s->flj;
   cudaMemsetAsync(flj, 0, 3 * (size_t)s->Npad * sizeof(long long), s->st);
   prof_mark(s);   // closes the integrate group (integrator, displacement check, clear)
-  launch_cl_force(energy, s->pos, s->cell_start, s->cl_start, s->regions, (int)s->regions_h.size(), s->shapes,
-                  s->reps, s->list, s->ncl, s->cap, s->tile_cap, s->fp, flj, s->Npad, s->lj_part, s->flags,
-                  s->lj_block, s->lj_lanes, s->persistent_grid, s->work, s->lj_pair_exact, s->st);
+  launch_cl_force(energy, s->pos, s->cell_start, s->cl_start, s->region_cells, s->items, s->n_lj_items, s->shapes, s->reps,
+                  s->list, s->tasks, s->task_base, s->cap, s->tile_cap, s->fp, flj, s->Npad, s->lj_part, s->flags, s->lj_block,
+                  s->lj_lanes, s->persistent_grid, s->work, s->lj_pair_exact, s->st);
   prof_mark(s);
   if (s->generic)
     launch_bonded_generic(energy, (const double*)s->x, s->inv_perm, flj, s->Npad, (int)s->N, s->tiles_int,
@@ -789,7 +878,7 @@ int md_create(const md_desc* d, md_system** out) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int per_sm = lj_blocks_per_sm(s->lj_block, s->lj_lanes, s->tile_cap);
-    s->persistent_grid = std::max(1, std::min((int)s->regions_h.size(), sms * std::max(per_sm, 1)));
+    s->persistent_grid = std::max(1, std::min(s->n_lj_items, sms * std::max(per_sm, 1)));
   }
   // static tables
   std::vector<uint16_t> site(s->N);
@@ -811,7 +900,7 @@ int md_create(const md_desc* d, md_system** out) {
             up(s->tiles_int, s->t_int.data(), sizeof(Tile) * s->t_int.size()) &&
             up(s->site, site.data(), sizeof(uint16_t) * s->N) &&
             up(s->lam, ones.data(), sizeof(double) * 6 * s->n_reps) &&
-            up(s->regions, s->regions_h.data(), sizeof(Region) * s->regions_h.size()) &&
+            up(s->region_cells, s->region_cells_h.data(), sizeof(int) * s->region_cells_h.size()) &&
             (!s->generic || (up(s->mtype, s->mtype_h.data(), s->mtype_h.size()) &&
                              up((void*)s->topo.b_off, s->t_boff.data(), s->t_boff.size() * sizeof(int)) &&
                              up((void*)s->topo.b_at, s->t_bat.data(), s->t_bat.size() * sizeof(int)) &&
@@ -822,6 +911,7 @@ int md_create(const md_desc* d, md_system** out) {
                              up((void*)s->topo.x_off, s->t_xoff.data(), s->t_xoff.size() * sizeof(int)) &&
                              up((void*)s->topo.x_at, s->t_xat.data(), s->t_xat.size() * sizeof(int)))) &&
             up(s->shapes, s->shapes_h.data(), sizeof(RegionShape) * s->shapes_h.size()) &&
+            up(s->items, s->items_h.data(), sizeof(WorkItem) * s->items_h.size()) &&
             cudaMemsetAsync(s->flj, 0, 3 * (size_t)s->Npad * sizeof(long long), s->st) == cudaSuccess &&
             cudaMemsetAsync(s->flj_e, 0, 3 * (size_t)s->Npad * sizeof(long long), s->st) == cudaSuccess &&
             cudaMemsetAsync(s->done, 0, sizeof(unsigned), s->st) == cudaSuccess &&
@@ -1167,9 +1257,7 @@ int md_bin_study(md_system* s, int32_t reps, double* ms) {
     launch_cell_sort(s->mixed, s->x, (int)N, s->cell_start, s->tmp, s->fp.mtype, s->cellc, s->site, s->reps, s->n_reps, s->C,
                      s->S, s->perm, s->inv_perm, s->pos, s->tag, s->ref, s->flags, s->st);
     cudaEventRecord(ev[1], s->st);
-    launch_cl_build(s->pos, s->tag, s->cell_start, s->cl_start, s->regions, (int)s->regions_h.size(), s->shapes,
-                    s->reps, s->list, s->ncl, s->cap, s->tile_cap, s->flags, 0, s->work,
-                  s->generic ? &s->topo : nullptr, s->st);
+    enqueue_build(s);
     cudaEventRecord(ev[2], s->st);
     // host arm: positions to the host, bins there, binned data back, sorted arrays
     if (cudaMemcpyAsync(hx, s->x, xb, cudaMemcpyDeviceToHost, s->st) != cudaSuccess) { rc = fail(s, MD_ECUDA, "copy"); break; }
@@ -1203,9 +1291,7 @@ int md_bin_study(md_system* s, int32_t reps, double* ms) {
   cudaFreeHost(hx);
   if (rc) return rc;
   // the list of the bins now in place
-  launch_cl_build(s->pos, s->tag, s->cell_start, s->cl_start, s->regions, (int)s->regions_h.size(), s->shapes,
-                  s->reps, s->list, s->ncl, s->cap, s->tile_cap, s->flags, 0, s->work,
-                  s->generic ? &s->topo : nullptr, s->st);
+  enqueue_build(s);
   for (int k = 0; k < 6; ++k) ms[k] = acc[k] / reps;
   rc = check_flags(s);
   s->fresh = rc == MD_OK;
@@ -1268,15 +1354,12 @@ int md_get_neighbors(md_system* s, int32_t* count, int32_t* entries) {
   // every listed pair, both ways, by original atom index: the region tiles
   // rebuilt here exactly as the kernels stage them
   std::vector<std::vector<int>> nb(N);
-  for (const Region& g : s->regions_h) {
-    const RegionShape& S = s->shapes_h[g.shape];
-    const RepDev& q = s->reps_h[g.rep];
-    const int M = q.M;
-    int start[kMaxTileCells], off[kMaxTileCells + 1], cell[kMaxTileCells];
+  for (size_t r = 0; r < s->regions_h.size(); ++r) {
+    const RegionShape& S = s->shapes_h[s->regions_h[r].shape];
+    const int* cell = s->region_cells_h.data() + kRegionCells * r;
+    int start[kMaxTileCells], off[kMaxTileCells + 1];
     off[0] = 0;
     for (int k = 0; k < S.n_tile; ++k) {
-      const int cx = (g.ox + S.off[k][0] + M) % M, cy = (g.oy + S.off[k][1] + M) % M, cz = (g.oz + S.off[k][2] + M) % M;
-      cell[k] = q.cell_base + (cz * M + cy) * M + cx;
       start[k] = cs[cell[k]];
       off[k + 1] = off[k] + cs[cell[k] + 1] - cs[cell[k]];
     }

@@ -25,7 +25,8 @@
 //                of the cluster's atoms that pair with it (bits 16..19)
 //     ncl        int32 [clusters] entries per cluster
 //   cells: count int32 [C], cell_start int32 [C+1], cl_start int32 [C+1]
-//   regions: up to 2 x 2 x 1 cells each, the force and list-build work units
+//   regions: up to 3 x 3 x 1 cells each; a block of the list build or LJ kernel
+//   takes a region or a part of one (WorkItem)
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -68,7 +69,7 @@ struct RepDev {
 
 struct Tile { int start, len, rep, pad; };
 
-// Regions of up to 2 x 2 x 1 cells (the work unit of the list build and LJ
+// Regions of up to 3 x 3 x 1 cells (the work unit of the list build and LJ
 // kernels) and their tiles: the region's home cells, then the cells their
 // 13 forward neighbours add, as offsets from the region's origin cell.
 constexpr int kMaxTileCells = 64;   // 44 cells for a 3 x 3 x 1 region
@@ -79,7 +80,23 @@ struct RegionShape {
   unsigned char nb[kMaxHome][14];         // home cell h: its own tile cell, then its 13 forward cells
   float cx, cy, cz;                       // region centre relative to the origin cell's centre
 };
-struct Region { int rep, ox, oy, oz, shape, pad[3]; };
+// What one block of the list build or LJ kernel does: the clusters of home
+// cells h0 .. h1 - 1 of a region, every parts-th from `part` on, on the tile
+// cells of `need` (bit k: tile cell k; the others are not staged, and the
+// tile indices of the lists stay those of the whole region).
+struct __align__(16) WorkItem {
+  unsigned long long need;
+  int region, rep, shape;
+  unsigned char h0, h1, part, parts;
+  int pad[2];
+};
+// global cell ids of a region's tile cells: cells[kRegionCells * region + k]
+constexpr int kRegionCells = 48;
+constexpr int kRegionClusterCap = 512;   // clusters of one region (2,048 home atoms); more is reported
+// One cluster of an LJ item, longest list first: x = list length, y = global
+// cluster id, z = first tile atom << 7 | chain-end bits << 3 | atoms (1..4),
+// w = the cluster's place in the item
+typedef int4 ClusterTask;
 
 // Position of atom x (one axis) in cell units relative to the centre of cell
 // c, shifted by w box lengths (w = +1/-1 for an atom that crossed a face
@@ -254,22 +271,29 @@ void launch_cell_sort(bool mixed, const void* x, int N, const int* cell_start, c
                       int sites, int* perm, int* inv_perm, float4* pos, int* tag, float4* ref, unsigned* flags,
                       cudaStream_t st);
 // ---------------------------------------------------------------- forces
-// cluster lists and LJ forces by regions (k_lj.cu).  The build writes each
-// cluster's list (up to cap entries, ncl[cl] of them); the force kernel adds
-// the LJ force of every atom into flj (int64 SoA [3][Npad], cleared by the
-// caller before) and, with energy, the per-region energy and virial sums into
-// epart (8 per cell).  persistent_grid > 0 runs that many blocks that take
-// regions from work[0..1] (two ints, zero before the first launch).
+// cluster lists and LJ forces by regions (k_lj.cu), a block per work item.
+// The build writes each cluster's list (up to cap entries, ncl[cl] of them);
+// the force kernel adds the LJ force of every atom into flj (int64 SoA
+// [3][Npad], cleared by the caller before) and, with energy, the energy and
+// virial sums of every home cell into epart (8 per cell; items then have
+// parts = 1).  persistent_grid > 0 runs that many force blocks, which take
+// items from work[0..1] (two ints, zero before the first launch).
 // topo != null: exclusions of a general molecule type from its lists; else
 // linear chains (1-2 and 1-3 neighbours by site index)
 void launch_cl_build(const float4* pos, const int* tag, const int* cell_start, const int* cl_start,
-                     const Region* regions, int n_regions, const RegionShape* shapes, const RepDev* reps,
-                     unsigned* list, int* ncl, int cap, int tile_cap, unsigned* flags, int persistent_grid, int* work,
-                     const TopoDev* topo, cudaStream_t st);
+                     const int* cells, const WorkItem* items, int n_items, const RegionShape* shapes,
+                     const RepDev* reps, unsigned* list, int* ncl, int cap, int tile_cap, unsigned* flags,
+                     int* n_tasks, const TopoDev* topo, cudaStream_t st);
+// after the build (which clears *n_tasks): each LJ item's clusters in the
+// order the force kernel takes them, tasks[task_base[item] + rank]; an item
+// claims its place in the table (as many entries as there are clusters) by *n_tasks
+void launch_cl_rank(const float4* pos, const int* cell_start, const int* cl_start, const int* cells,
+                    const WorkItem* items, int n_items, const RegionShape* shapes, const int* ncl, ClusterTask* tasks,
+                    int* task_base, int* n_tasks, cudaStream_t st);
 void launch_cl_force(bool energy, const float4* pos, const int* cell_start, const int* cl_start,
-                     const Region* regions, int n_regions, const RegionShape* shapes, const RepDev* reps,
-                     const unsigned* list, const int* ncl, int cap, int tile_cap, const ForceParams& fp,
-                     long long* flj, int Npad, double* epart, unsigned* flags, int block, int lanes,
+                     const int* cells, const WorkItem* items, int n_items, const RegionShape* shapes,
+                     const RepDev* reps, const unsigned* list, const ClusterTask* tasks, const int* task_base,
+                     int cap, int tile_cap, const ForceParams& fp, long long* flj, int Npad, double* epart, unsigned* flags, int block, int lanes,
                      int persistent_grid, int* work, bool exact, cudaStream_t st);
 int lj_blocks_per_sm(int block, int lanes, int tile_cap);
 cudaError_t tile_kernels_init();
