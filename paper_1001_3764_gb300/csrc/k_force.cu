@@ -14,7 +14,7 @@
 // then FP64 across warps, in a fixed order.
 #include <type_traits>
 
-#include "md_kernels.cuh"
+#include "bonded.cuh"
 
 namespace mdg {
 
@@ -51,75 +51,10 @@ __device__ __forceinline__ void block_sum(const float (&v)[NV], double* out) {
   }
 }
 
-// FP32 force -> int64 fixed point (2^-32 kJ/mol/nm); each part below 2^18
-__device__ __forceinline__ long long to_fix(float f, unsigned* flags) {
-  if (!(fabsf(f) < 262144.0f)) { atomicOr(flags, kFlagFixOverflow); return 0; }
-  return fix_round_int(f);   // = __float2ll_rn(f * 2^32), on the integer pipe
-}
-
 // ======================================================================= bonded
 constexpr int kBondedBlock = 256;
 constexpr int kHalo = 3;
 constexpr int kBondedVals = 9;   // bond, angle, dihedral, vxx, vyy, vzz, vxy, vxz, vyz
-
-struct f3 { float x, y, z; };
-__device__ __forceinline__ f3 mk(float x, float y, float z) { return {x, y, z}; }
-__device__ __forceinline__ f3 operator+(f3 a, f3 b) { return {a.x + b.x, a.y + b.y, a.z + b.z}; }
-__device__ __forceinline__ f3 operator-(f3 a, f3 b) { return {a.x - b.x, a.y - b.y, a.z - b.z}; }
-__device__ __forceinline__ f3 operator-(f3 a) { return {-a.x, -a.y, -a.z}; }
-__device__ __forceinline__ f3 operator*(float s, f3 a) { return {s * a.x, s * a.y, s * a.z}; }
-__device__ __forceinline__ float dot(f3 a, f3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
-__device__ __forceinline__ f3 cross(f3 a, f3 b) {
-  return {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
-}
-
-// bond vector x_{m+1} - x_m under the minimum image (FP64 master); |d| > L/2
-// is tested on the bit patterns (integer pipe), which order like the values
-__device__ __forceinline__ double bond_diff(double a, double b, double L, double hL) {
-  double d = b - a;
-  const long long bd = __double_as_longlong(d);
-  if ((bd & 0x7fffffffffffffffll) > __double_as_longlong(hL)) d = bd < 0 ? d + L : d - L;
-  return d;
-}
-
-// |b|^2 - b0^2 for an exact FP32 vector b: each square is split into its
-// rounded value and exact error (FMA), the rounded parts are summed with
-// error-free two-sums, and b0^2 = c_hi + c_lo is subtracted from the
-// leading part, where the two nearly cancel without rounding.
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-  s = a + b;
-  const float bb = s - a;
-  e = (a - (s - bb)) + (b - bb);
-}
-__device__ __forceinline__ float sq_minus(f3 b, float c_hi, float c_lo) {
-  const float px = b.x * b.x, py = b.y * b.y, pz = b.z * b.z;
-  const float ex = fmaf(b.x, b.x, -px), ey = fmaf(b.y, b.y, -py), ez = fmaf(b.z, b.z, -pz);
-  float s1, e1, s2, e2;
-  two_sum(px, py, s1, e1);
-  two_sum(s1, pz, s2, e2);
-  return (s2 - c_hi) + ((e1 + e2) + (ex + ey + ez) - c_lo);
-}
-// FP32 master: the difference of two nearby floats is exact; across a face the
-// partner is first moved by L (exact when it lies near the face, L being an
-// FP32 number), so the result is again the exact difference.
-__device__ __forceinline__ float bond_comp(float a, float b, float L, float hL) {
-  float d = b - a;
-  if (d > hL) d = (b - L) - a; else if (d < -hL) d = b - (a - L);
-  return d;
-}
-
-__device__ __forceinline__ void add_vir(float (&W)[6], f3 r, f3 f) {
-  W[0] += r.x * f.x; W[1] += r.y * f.y; W[2] += r.z * f.z;
-  W[3] += r.x * f.y; W[4] += r.x * f.z; W[5] += r.y * f.z;
-}
-
-// int64 fixed point (2^-32 kJ/mol/nm) -> FP32 on the 32-bit pipes: the high
-// word (|hi| < 2^24, exact) plus the low word scaled by 2^-32
-__device__ __forceinline__ float fix_to_float(long long q) {
-  const int hi = (int)(q >> 32);
-  const unsigned lo = (unsigned)q;
-  return fmaf((float)lo, 2.3283064365386963e-10f, (float)hi);
-}
 
 template <bool MIXED, bool ENERGY>
 __global__ void __launch_bounds__(kBondedBlock) k_bonded(const void* __restrict__ xv, const uint16_t* __restrict__ site,
@@ -145,18 +80,8 @@ __global__ void __launch_bounds__(kBondedBlock) k_bonded(const void* __restrict_
     f3 b = mk(0.f, 0.f, 0.f);
     float D = 0.f;
     if (m >= lo && m + 1 < hi && site[m] < S - 1) {
-      if (MIXED) {
-        const double dx = bond_diff((double)x[m], (double)x[m + 1], R.L, R.half_L);
-        const double dy = bond_diff((double)x[N + m], (double)x[N + m + 1], R.L, R.half_L);
-        const double dz = bond_diff((double)x[2 * N + m], (double)x[2 * N + m + 1], R.L, R.half_L);
-        b = mk(d2f_rn_int(dx), d2f_rn_int(dy), d2f_rn_int(dz));
-        D = d2f_rn_int(fma(dx, dx, fma(dy, dy, fma(dz, dz, -fp.b0sq))));
-      } else {
-        b.x = bond_comp((float)x[m], (float)x[m + 1], R.Lf, R.half_Lf);
-        b.y = bond_comp((float)x[N + m], (float)x[N + m + 1], R.Lf, R.half_Lf);
-        b.z = bond_comp((float)x[2 * N + m], (float)x[2 * N + m + 1], R.Lf, R.half_Lf);
-        D = sq_minus(b, fp.b0sq_hi, fp.b0sq_lo);
-      }
+      const T xa[3] = {x[m], x[N + m], x[2 * N + m]}, xb[3] = {x[m + 1], x[N + m + 1], x[2 * N + m + 1]};
+      bond_vector<MIXED>(xa, xb, R, fp, b, D);
     }
     bv[q] = b;
     bD[q] = D;
@@ -173,66 +98,19 @@ __global__ void __launch_bounds__(kBondedBlock) k_bonded(const void* __restrict_
     if (q < t.len + kHalo && m >= lo && m < hi) {
       const int sm = site[m];
       const bool own = m >= t.start;   // energy/virial counted once, by the owning tile
-      if (sm <= S - 2) {               // bond (m, m+1), Eq. (4)
-        const f3 b = bv[q];
-        const float r = sqrtf(dot(b, b));
-        const float dr = bD[q] / (r + fp.b0);   // r - b0 without cancellation
-        const float g = fp.kb * dr / r;
-        fb = g * b;                    // force on atom m
-        if (ENERGY && own) { Eb += 0.5f * fp.kb * dr * dr; add_vir(W, b, -fb); }
-      }
-      if (sm <= S - 3) {               // angle (m, m+1, m+2), vertex m+1, Eq. (5)
-        const f3 u = -bv[q], w = bv[q + 1];
-        const float lu = sqrtf(dot(u, u)), lw = sqrtf(dot(w, w));
-        const f3 cr = cross(u, w);
-        const float sn = sqrtf(dot(cr, cr)), cs = dot(u, w);
-        const float th = atan2f(sn, cs);
-        const float dth = th - fp.theta0;
-        const float inv = 1.0f / (lu * lw);
-        const float sin_t = sn * inv, cos_t = cs * inv;
-        if (sin_t > 1e-6f) {
-          const float g = fp.ka * dth / sin_t;
-          const f3 uh = (1.0f / lu) * u, wh = (1.0f / lw) * w;
-          fa = (g / lu) * (wh - cos_t * uh);
-          fc = (g / lw) * (uh - cos_t * wh);
-        }
-        if (ENERGY && own) { Ea += 0.5f * fp.ka * dth * dth; add_vir(W, u, fa); add_vir(W, w, fc); }
-      }
-      if (sm <= S - 4) {               // dihedral (m .. m+3), Eq. (6), IUPAC phi
-        const f3 b1 = bv[q], b2 = bv[q + 1], b3 = bv[q + 2];
-        const f3 mm = cross(b1, b2), nn = cross(b2, b3);
-        const float lb2 = sqrtf(dot(b2, b2)), m2 = dot(mm, mm), n2 = dot(nn, nn);
-        const float phi = atan2f(lb2 * dot(b1, nn), dot(mm, nn));
-        const float arg = (float)fp.n_mult * phi - fp.phis;
-        float sa, ca;
-        sincosf(arg, &sa, &ca);
-        if (m2 > 1e-24f && n2 > 1e-24f) {
-          const float dEdphi = -fp.kphi * (float)fp.n_mult * sa;
-          const float cam = -lb2 / m2, cdn = lb2 / n2;
-          const float cbm = lb2 / m2 + dot(b1, b2) / (lb2 * m2), cbn = dot(b2, b3) / (lb2 * n2);
-          const f3 ga = cam * mm, gd = cdn * nn, gb = cbm * mm + cbn * nn;
-          const f3 gc = -(ga + gb + gd);
-          f1 = -dEdphi * ga; f2 = -dEdphi * gb; f3v = -dEdphi * gc;
-          if (ENERGY && own) {
-            const f3 f4 = -(f1 + f2 + f3v);
-            add_vir(W, b1, f2); add_vir(W, b1 + b2, f3v); add_vir(W, b1 + b2 + b3, f4);
-          }
-        }
-        if (ENERGY && own) Ed += fp.kphi * (1.0f + ca);
-      }
+      chain_terms<ENERGY>(fp, sm, S, bv, bD, q, own, fb, fa, fc, f1, f2, f3v, Eb, Ea, Ed, W);
     }
     if (q < kBondedBlock) {
       fbd[q] = fb; fan_a[q] = fa; fan_c[q] = fc; fdi1[q] = f1; fdi2[q] = f2; fdi3[q] = f3v;
     }
   }
   __syncthreads();
-  // 3. sum the contributions on each home atom in a fixed order
-  if ((int)threadIdx.x < t.len) {
+  // 3. sum the contributions on each home atom in a fixed order (an energy
+  // read-out passes no Fout: it has no use for them)
+  if (Fout && (int)threadIdx.x < t.len) {
     const int q = threadIdx.x + kHalo;
     const int i = t.start + threadIdx.x;
-    f3 F = fbd[q] - fbd[q - 1];
-    F = F + fan_a[q] - (fan_a[q - 1] + fan_c[q - 1]) + fan_c[q - 2];
-    F = F + fdi1[q] + fdi2[q - 1] + fdi3[q - 2] - (fdi1[q - 3] + fdi2[q - 3] + fdi3[q - 3]);
+    const f3 F = chain_force(fbd, fan_a, fan_c, fdi1, fdi2, fdi3, q);
     // the LJ force of the atom (sorted slot s)
     const int s = inv_perm[i];
     const long long lx = __ldg(flj + s), ly = __ldg(flj + Npad + s), lz = __ldg(flj + 2 * (size_t)Npad + s);

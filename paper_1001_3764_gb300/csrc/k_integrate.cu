@@ -10,15 +10,14 @@
 //
 // The paper's Nose-Hoover coupling needs the whole-system kinetic energy,
 // which it sums through a per-atom array and a tree reduction (Sec. 3.4).
-// Here each block writes one FP64 partial; the last block to finish (ticket
-// counter, no waiting) sums the partials of each replica in a fixed order
-// (one warp per replica and summed value, see below) and computes that
-// replica's rescaling factor.
+// Here each block writes one FP64 partial; the last block of a replica to
+// finish (a ticket per replica, no waiting) sums the replica's partials in a
+// fixed order and computes its rescaling factor.
 // The factor computed at step k is applied at step k+1 (one-step lag).
 //
 // Nose-Hoover (TH = 2; the paper's NVT ensemble with Leap-Frog, Sec. 2 and
-// 3.4): per replica, lam[6r..6r+5] = (xi_k, 1 - c_k, 1/(1 + c_k), V_com),
-// c_k = dt xi_k / 2.  A step closes v_k = (v_{k-1/2} - V_com + dt F/(2m)) /
+// 3.4): per replica xi_k, 1 - c_k, 1/(1 + c_k), V_com (kNhDoubles in
+// md_kernels.cuh), c_k = dt xi_k / 2.  A step closes v_k = (v_{k-1/2} - V_com + dt F/(2m)) /
 // (1 + c_k), opens v_{k+1/2} = (1 - c_k) v_k + dt F/(2m) and drifts; the
 // last block takes T_{k+1/2} and the momentum of v_{k+1/2} and leaves
 // xi_{k+1} = xi_k + dt (T_{k+1/2} - T0)/Q, Q = tau^2 T0/(4 pi^2), and the
@@ -28,24 +27,19 @@
 // The drift also refreshes the FP32 cell-unit positions in sorted order for
 // the force kernels, wraps positions into [0, L) with image counters, and
 // flags atoms that moved more than skin/2 since the last rebin.
+//
+// The update of an atom and the thermostats' sums are in integrate.cuh,
+// shared with the fused step kernel of linear chains (k_step.cu), which does
+// every inner and closing update of a block of steps; this kernel opens a
+// block, reads out the kinetic energy, and does all updates of general
+// molecules.
 #include <type_traits>
 
-#include "md_kernels.cuh"
+#include "integrate.cuh"
 
 namespace mdg {
 
-__device__ __forceinline__ double warp_sum_i(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  return v;
-}
-
 constexpr int kIntBlock = 256;
-
-__device__ __forceinline__ bool past_box(double x, double L) { return __double_as_longlong(x) >= __double_as_longlong(L); }
-__device__ __forceinline__ bool past_box(float x, float L) { return __float_as_int(x) >= __float_as_int(L); }
-__device__ __forceinline__ bool negative(double x) { return __double_as_longlong(x) < 0; }
-__device__ __forceinline__ bool negative(float x) { return __float_as_int(x) < 0; }
 
 template <bool MIXED, int MODE, bool KE, int TH>
 __global__ void __launch_bounds__(kIntBlock) k_integrate(void* __restrict__ xv, void* __restrict__ vv,
@@ -54,28 +48,25 @@ __global__ void __launch_bounds__(kIntBlock) k_integrate(void* __restrict__ xv, 
                                                          const int* __restrict__ cellc,
                                                          const int* __restrict__ inv_perm,
                                                          const float4* __restrict__ ref, float4* __restrict__ pos,
-                                                         int N, const Tile* __restrict__ tiles,
-                                                         const RepDev* __restrict__ reps, int n_reps,
-                                                         const ForceParams fp, double* __restrict__ kepart,
-                                                         unsigned* __restrict__ done, double* __restrict__ ke_out,
-                                                         double* __restrict__ lam, double tau,
-                                                         unsigned* __restrict__ flags) {
+                                                         long long* __restrict__ flj_next, int Npad, int N,
+                                                         const Tile* __restrict__ tiles,
+                                                         const RepDev* __restrict__ reps, const ForceParams fp,
+                                                         double* __restrict__ kepart, unsigned* __restrict__ done,
+                                                         double* __restrict__ ke_out, double* __restrict__ lam,
+                                                         double tau, unsigned* __restrict__ flags,
+                                                         const MoveReport mr) {
   using T = typename std::conditional<MIXED, double, float>::type;
   T* x = reinterpret_cast<T*>(xv);
   T* v = reinterpret_cast<T*>(vv);
   const Tile t = tiles[blockIdx.x];
   const RepDev& R = reps[t.rep];
   const int i = t.start + threadIdx.x;
-  double ke = 0.0;
-  double mom[3] = {0.0, 0.0, 0.0};   // Nose-Hoover: momentum of v_{k+1/2}
+  AtomOut o;
+  o.ke = 0.0;
+  o.mom[0] = o.mom[1] = o.mom[2] = 0.0;
   if ((int)threadIdx.x < t.len) {
-    const int sm = site[i];
-    const int type = atom_type(sm, fp);
-    // mixed form: F stays in fixed-point units (int64 -> FP64 is a fast
-    // conversion) and 2^-32 is folded into dt / 2m
-    T hdt_m;
-    if constexpr (MIXED) hdt_m = fp.hdt_m_fix[type]; else hdt_m = fp.hdt_m_f[type];
-    T F[3] = {(T)0, (T)0, (T)0};
+    const int type = atom_type(site[i], fp);
+    T F[3] = {(T)0, (T)0, (T)0}, xi[3] = {(T)0, (T)0, (T)0}, vi[3] = {v[i], v[N + i], v[2 * N + i]};
     if (MODE == kKineticOnly) {
     } else if (MIXED) {
       const F4i f = reinterpret_cast<const F4i*>(Fv)[i];
@@ -84,193 +75,44 @@ __global__ void __launch_bounds__(kIntBlock) k_integrate(void* __restrict__ xv, 
       const float4 f = reinterpret_cast<const float4*>(Fv)[i];
       F[0] = f.x; F[1] = f.y; F[2] = f.z;
     }
-    T vi[3] = {v[i], v[N + i], v[2 * N + i]};
-    // Without a kinetic-energy read-out the two half kicks of KKD are one
-    // kick of dt F/m (the full-step velocity is never needed in between).
-    constexpr bool kMerged = MODE == kKickKickDrift && !KE;
-    if ((MODE == kKickKickDrift && KE) || MODE == kKickOnly) {
-      if constexpr (TH == 2) {
-        const double* nh = lam + 6 * t.rep;
-        const T fc = (T)nh[2];
+    int cc = 0;
+    float4 r0 = make_float4(0.f, 0.f, 0.f, 0.f);
+    constexpr bool kDrift = MODE == kKickDrift || MODE == kKickKickDrift;
+    if (kDrift) {
+      cc = cellc[i];
+      r0 = ref[i];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) vi[a] = (vi[a] - (T)nh[3 + a] + hdt_m * F[a]) * fc;   // v_k
-      } else {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) vi[a] += hdt_m * F[a];   // v(t): close the previous step
-      }
+      for (int a = 0; a < 3; ++a) xi[a] = x[a * N + i];
     }
-    if (KE && TH != 2) {
-      const double m = fp.mass[type];
-      ke = 0.5 * m * ((double)vi[0] * vi[0] + (double)vi[1] * vi[1] + (double)vi[2] * vi[2]);
+    integrate_atom<MIXED, MODE, KE, TH>(F, xi, vi, img, i, N, type, cc, r0, R, t.rep, fp, lam, o);
+    if (MODE == kKickOnly || kDrift) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) v[a * N + i] = vi[a];
     }
-    if (MODE == kKickOnly) {
-      v[i] = vi[0]; v[N + i] = vi[1]; v[2 * N + i] = vi[2];
-    } else if (MODE == kKickDrift || MODE == kKickKickDrift) {
-      if (TH == 1) {
-        const T l = (T)lam[t.rep];
+    if (kDrift) {
 #pragma unroll
-        for (int a = 0; a < 3; ++a) vi[a] *= l;
-      }
-      T dt, L;
-      if constexpr (MIXED) { dt = fp.dt; L = R.L; } else { dt = fp.dt_f; L = R.Lf; }
-      const int cc = cellc[i];
-      const float4 r0 = ref[i];
-      const float r0a[3] = {r0.x, r0.y, r0.z};
-      const float halfM = 0.5f * R.Mf;
-      float loc[3], d2 = 0.f;
-      bool bad = false;
-      T fo = (T)1;
-      if constexpr (TH == 2) fo = (T)lam[6 * t.rep + 1];
+      for (int a = 0; a < 3; ++a) x[a * N + i] = xi[a];
+      if (flj_next) {
 #pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        if constexpr (TH == 2) vi[a] = vi[a] * fo + hdt_m * F[a];   // v_{k+1/2}
-        else vi[a] = kMerged ? vi[a] + (hdt_m + hdt_m) * F[a] : vi[a] + hdt_m * F[a];
-        T xa = x[a * N + i] + dt * vi[a];
-        // wrap into [0, L): for non-negative IEEE numbers the bit patterns
-        // order like the values, so the tests run on the integer pipe
-        if (past_box(xa, L)) { xa -= L; img[a * N + i] += 1; }
-        else if (negative(xa)) { xa += L; img[a * N + i] -= 1; if (past_box(xa, L)) xa = (T)0; }
-        x[a * N + i] = xa;
-        v[a * N + i] = vi[a];
-        // cell units in the frame of the rebin cell; an atom that crossed a
-        // face since the rebin is moved back by one box (M cell units)
-        const int c = (cc >> (10 * a)) & 1023;
-        float ua;
-        if constexpr (MIXED) ua = cell_unit_t(xa, c, R); else ua = cell_unit(xa, c, 0, R);
-        const float du = ua - r0a[a];
-        if (du > halfM || du < -halfM) {
-          if constexpr (MIXED) ua = cell_unit_tw(xa, c, du > halfM ? -1 : 1, R);
-          else ua = cell_unit(xa, c, du > halfM ? -1 : 1, R);
-        }
-        loc[a] = ua;
-        const float d = ua - r0a[a];
-        d2 += d * d;
-        bad |= !isfinite(ua);          // a non-finite x or v reaches u
+        for (int a = 0; a < 3; ++a) flj_next[(size_t)a * Npad + i] = 0ll;
       }
-      if (d2 > R.hs2u) atomicOr(flags, kFlagDisplacement);
-      if (bad) atomicOr(flags, kFlagNaN);
-      if constexpr (TH == 2) {
-        const double m = fp.mass[type];
-        ke = 0.5 * m * ((double)vi[0] * vi[0] + (double)vi[1] * vi[1] + (double)vi[2] * vi[2]);
-#pragma unroll
-        for (int a = 0; a < 3; ++a) mom[a] = m * (double)vi[a];
-      }
-      pos[inv_perm[i]] = make_float4(loc[0], loc[1], loc[2], (float)type);   // w: LJ type, as the sort writes it
+      if (o.moved) report_move(mr, flags);
+      if (o.bad) atomicOr(flags, kFlagNaN);
+      pos[inv_perm[i]] = make_float4(o.loc[0], o.loc[1], o.loc[2], (float)type);   // w: LJ type, as the sort writes it
     }
   }
-  if (KE) {
-    // block sums in FP64 through shared memory: thread q < 8 NV adds the 32
-    // values of warp q % 8 in order, thread 0 the 8 warp sums in order (a
-    // fixed order; 255 FP64 adds per value and block, where a shuffle tree
-    // per warp would issue five on every lane: this GPU's FP64 pipe is narrow)
-    constexpr int NV = TH == 2 ? 4 : 1;
-    constexpr int NW = kIntBlock / 32;
-    __shared__ double vals[NV][kIntBlock];
-    __shared__ double wsum[NV][NW];
-    __shared__ bool last;
-    vals[0][threadIdx.x] = ke;
-    if constexpr (TH == 2) {
-#pragma unroll
-      for (int a = 0; a < 3; ++a) vals[1 + a][threadIdx.x] = mom[a];
-    }
-    __syncthreads();
-    if (threadIdx.x < NV * NW) {
-      const int a = threadIdx.x / NW, w = threadIdx.x % NW;
-      double b = 0.0;
-#pragma unroll 8
-      for (int k = 0; k < 32; ++k) b += vals[a][32 * w + k];
-      wsum[a][w] = b;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double b = 0.0;
-      for (int q = 0; q < NW; ++q) b += wsum[0][q];
-      kepart[blockIdx.x] = b;
-      if constexpr (TH == 2) {
-        for (int a = 0; a < 3; ++a) {
-          double bm = 0.0;
-          for (int q = 0; q < NW; ++q) bm += wsum[1 + a][q];
-          kepart[gridDim.x + 3 * blockIdx.x + a] = bm;   // momentum partials follow the energy partials
-        }
-      }
-      __threadfence();
-      last = atomicAdd(done, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    if (last) {
-      __threadfence();
-      // a warp per (replica, value): lane l keeps eight chains P_m (m = 0..7), P_m
-      // adding the replica's partials l + 32 m, l + 32 m + 256, ... in order
-      // (eight loads in flight); then each P_m is summed over the lanes by a
-      // fixed tree and the eight results in m order.  The order depends only
-      // on the replica's own tile count.
-      auto replica_sum = [&](const double* base, int stride, int n) {
-        double P[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-        for (int k0 = 0; k0 < n; k0 += 256) {
-#pragma unroll
-          for (int m = 0; m < 8; ++m) {
-            const int q = k0 + lane + 32 * m;
-            if (q < n) P[m] += __ldcg(base + (size_t)q * stride);
-          }
-        }
-        double sum = 0.0;
-#pragma unroll
-        for (int m = 0; m < 8; ++m) sum += warp_sum_i(P[m]);
-        return sum;
-      };
-      // (replica, value) jobs over the warps: 8 replicas per round for the
-      // kinetic energy alone, 2 for energy and momentum; then one thread per
-      // replica forms its thermostat factors
-      constexpr int RPR = NW / NV;
-      __shared__ double res[RPR][NV];
-      const int w = threadIdx.x >> 5;
-      for (int r0 = 0; r0 < n_reps; r0 += RPR) {
-        const int r = r0 + w / NV, a = w % NV;
-        if (r < n_reps) {
-          const RepDev& Q = reps[r];
-          const double sum = a == 0 ? replica_sum(kepart + Q.tile_off, 1, Q.n_tiles)
-                                    : replica_sum(kepart + gridDim.x + 3 * Q.tile_off + (a - 1), 3, Q.n_tiles);
-          if (lane == 0) res[w / NV][a] = sum;
-        }
-        __syncthreads();
-        if ((int)threadIdx.x < RPR && r0 + (int)threadIdx.x < n_reps) {
-          const int rr = r0 + threadIdx.x;
-          const RepDev& Q = reps[rr];
-          const double sum = res[threadIdx.x][0];
-          ke_out[rr] = sum;
-          if (TH == 1) {
-            const double T_inst = 2.0 * sum / (Q.dof * 0.0083144626);
-            lam[rr] = sqrt(1.0 + fp.dt / tau * (Q.T0 / T_inst - 1.0));
-          }
-          if constexpr (TH == 2) {
-            const double T_half = 2.0 * sum / (Q.dof * 0.0083144626);
-            const double Qm = tau * tau * Q.T0 / (4.0 * 3.14159265358979323846 * 3.14159265358979323846);
-            double* nh = lam + 6 * rr;
-            const double xi = nh[0] + fp.dt * (T_half - Q.T0) / Qm;
-            const double c = 0.5 * fp.dt * xi;
-            const double M = (double)Q.n_chains * fp.mol_mass;
-            nh[0] = xi; nh[1] = 1.0 - c; nh[2] = 1.0 / (1.0 + c);
-            nh[3] = res[threadIdx.x][1] / M; nh[4] = res[threadIdx.x][2] / M; nh[5] = res[threadIdx.x][3] / M;
-          }
-        }
-        __syncthreads();
-      }
-      if (threadIdx.x == 0) *done = 0u;
-    }
-  }
+  if constexpr (KE)
+    replica_kinetic<TH, kIntBlock>(o, t.rep, blockIdx.x, R.tile_off, R.n_tiles, reps, fp, kepart, done, ke_out, lam, tau);
 }
 
 template <bool MIXED>
-static void launch_int_t(IntegMode mode, bool ke, int th, void* x, void* v, int* img, const void* F,
-                         const uint16_t* site, const int* cellc, const int* inv_perm, const float4* ref, float4* pos,
-                         int N, const Tile* tiles, int n_tiles, const RepDev* reps, int n_reps,
-                         const ForceParams& fp, double* kepart, unsigned* done, double* ke_out, double* lam,
-                         double tau, unsigned* flags, cudaStream_t st) {
+static void launch_int_t(IntegMode mode, int th, const StepArgs& a, const ForceParams& fp,
+                         const MoveReport& mr, cudaStream_t st) {
 #define MDG_INT(MODE, KE, TH)                                                                                   \
-  k_integrate<MIXED, MODE, KE, TH><<<n_tiles, kIntBlock, 0, st>>>(x, v, img, F, site, cellc, inv_perm, ref,     \
-                                                                  pos, N, tiles, reps, n_reps, fp, kepart, done, \
-                                                                  ke_out, lam, tau, flags)
+  k_integrate<MIXED, MODE, KE, TH><<<a.n_tiles, kIntBlock, 0, st>>>(a.x, a.v, a.img, a.F, a.site, a.cellc,      \
+                                                                    a.inv_perm, a.ref, a.pos, a.flj_next, a.Npad, a.N, \
+                                                                    a.tiles, a.reps, fp, a.kepart, a.done, a.ke_out,   \
+                                                                    a.lam, a.tau, a.flags, mr)
   // With the weak-coupling thermostat (th = 1), every step that starts (KD,
   // KKD) takes the temperature of the unscaled v(t_k), scales v(t_k) by the
   // factor of the previous step and leaves the factor of step k for the next
@@ -285,11 +127,9 @@ static void launch_int_t(IntegMode mode, bool ke, int th, void* x, void* v, int*
   } else if (mode == kKickKickDrift) {
     if (th == 2) MDG_INT(kKickKickDrift, true, 2);
     else if (th == 1) MDG_INT(kKickKickDrift, true, 1);
-    else if (ke) MDG_INT(kKickKickDrift, true, 0);
     else MDG_INT(kKickKickDrift, false, 0);
   } else if (mode == kKickOnly) {
     if (th == 2) MDG_INT(kKickOnly, false, 2);
-    else if (ke) MDG_INT(kKickOnly, true, 0);
     else MDG_INT(kKickOnly, false, 0);
   } else {
     MDG_INT(kKineticOnly, true, 0);
@@ -297,39 +137,11 @@ static void launch_int_t(IntegMode mode, bool ke, int th, void* x, void* v, int*
 #undef MDG_INT
 }
 
-void launch_integrate(bool mixed, IntegMode mode, bool ke, int thermostat, void* x, void* v, int* img,
-                      const void* F, const uint16_t* site, const int* cellc, const int* inv_perm, const float4* ref,
-                      float4* pos, int N, const Tile* tiles, int n_tiles, const RepDev* reps, int n_reps,
-                      const ForceParams& fp, double* kepart, unsigned* done, double* ke_out, double* lam,
-                      double tau, unsigned* flags, cudaStream_t st) {
-  if (mixed)
-    launch_int_t<true>(mode, ke, thermostat, x, v, img, F, site, cellc, inv_perm, ref, pos, N, tiles, n_tiles, reps,
-                       n_reps, fp, kepart, done, ke_out, lam, tau, flags, st);
-  else
-    launch_int_t<false>(mode, ke, thermostat, x, v, img, F, site, cellc, inv_perm, ref, pos, N, tiles, n_tiles, reps,
-                        n_reps, fp, kepart, done, ke_out, lam, tau, flags, st);
-}
-
-// ---------------------------------------------------------------- early rebin
-// After a drift: if an atom has moved more than skin/2 since the rebin (the
-// integrator raised kFlagDisplacement), open the conditional rebin that
-// follows in the step graph, clear the flag (the new bins reset the
-// reference) and count the event; else keep it closed.  One thread, so the
-// condition is set once.
-__global__ void __launch_bounds__(32) k_disp_check(cudaGraphConditionalHandle h, unsigned* __restrict__ flags,
-                                                   unsigned long long* __restrict__ events) {
-  if (threadIdx.x != 0) return;
-  const unsigned f = *(volatile unsigned*)flags;
-  const bool moved = (f & kFlagDisplacement) != 0u;
-  if (moved) {
-    atomicAnd(flags, ~kFlagDisplacement);
-    *events += 1ull;
-  }
-  cudaGraphSetConditional(h, moved ? 1u : 0u);
-}
-
-void launch_disp_check(cudaGraphConditionalHandle h, unsigned* flags, unsigned long long* events, cudaStream_t st) {
-  k_disp_check<<<1, 32, 0, st>>>(h, flags, events);
+void launch_integrate(bool mixed, IntegMode mode, int thermostat, const StepArgs& a, const ForceParams& fp,
+                      const MoveReport& mr, cudaStream_t st) {
+  if (a.n_tiles <= 0) return;
+  if (mixed) launch_int_t<true>(mode, thermostat, a, fp, mr, st);
+  else launch_int_t<false>(mode, thermostat, a, fp, mr, st);
 }
 
 // ---------------------------------------------------------------- energy reduction

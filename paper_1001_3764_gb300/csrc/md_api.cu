@@ -19,6 +19,7 @@
 
 #include "../../include/md.h"
 #include "md_kernels.cuh"
+#include "integrate.cuh"
 
 using namespace mdg;
 
@@ -48,17 +49,18 @@ struct md_system {
   md_params params{};
   ForceParams fp{};
   std::vector<RepDev> reps_h;
-  std::vector<Tile> t_int;
+  std::vector<Tile> t_int;                   // kIntTile atoms each
+  std::vector<Tile> t_chain;                 // whole chains (fused step kernel; empty for general molecules)
   std::vector<double> T0;
   // memory
   char* base = nullptr;
   size_t bytes = 0;
   bool own_mem = false;
   RepDev* reps = nullptr;
-  Tile* tiles_int = nullptr;
+  Tile *tiles_int = nullptr, *tiles_chain = nullptr;
   void *x = nullptr, *v = nullptr, *F = nullptr;
-  long long* flj = nullptr;                  // LJ force, int64 SoA [3][Npad], sorted order
-  long long* flj_e = nullptr;                // the same for energy read-outs (kept apart from the dynamics)
+  long long* flj[2] = {nullptr, nullptr};    // LJ force, int64 SoA [3][Npad], sorted order: a step adds to one
+                                             // while the other is cleared for the next
   int* img = nullptr;
   uint16_t* site = nullptr;
   int *cellc = nullptr, *inv_perm = nullptr, *tag = nullptr, *perm = nullptr;
@@ -103,6 +105,7 @@ struct md_system {
   std::vector<cudaGraphExec_t> rem_graphs;   // blocks of k < R steps (remainders), captured on first use
   cudaStream_t side = nullptr;               // captures the bodies of the conditional rebins
   unsigned long long* early = nullptr;       // early rebins (displacement beyond skin/2) so far
+  unsigned* moved = nullptr;                 // an atom of this step is beyond skin/2 (cleared with the cell counts)
   // a general molecule type (md_desc.topology), or linear chains
   bool generic = false;
   int disp = MD_DISP_REBUILD;                // what a displacement beyond skin/2 does
@@ -169,6 +172,7 @@ static void fill_force_params(md_system* s) {
   for (int a = 0; a < 2; ++a) {
     f.mass[a] = p.mass[a];
     f.inv_mass[a] = 1.0 / p.mass[a];
+    f.mass_ratio = p.mass[1] / p.mass[0];
     f.hdt_m[a] = 0.5 * s->dt / p.mass[a];
     f.hdt_m_fix[a] = f.hdt_m[a] * kFixInv;
     f.hdt_m_f[a] = (float)f.hdt_m[a];
@@ -440,6 +444,7 @@ static int configure(md_system* s, const md_desc* d) {
     for (int sx = 1; sx <= G; ++sx) s->shapes_h.push_back(make_shape(sx, sy));
   const double tile_cells = (double)s->shapes_h.back().n_tile;
   s->t_int.clear();
+  s->t_chain.clear();
   for (int r = 0; r < s->n_reps; ++r) {
     const int nc = d->n_chains[r];
     const double L = d->box[r];
@@ -463,6 +468,13 @@ static int configure(md_system* s, const md_desc* d) {
     q.tile_off = (int)s->t_int.size();
     for (int o = 0; o < q.n_atoms; o += kIntTile) s->t_int.push_back(Tile{q.atom_off + o, std::min(kIntTile, q.n_atoms - o), r, 0});
     q.n_tiles = (int)s->t_int.size() - q.tile_off;
+    q.ctile_off = (int)s->t_chain.size();
+    if (!s->generic) {
+      const int per = step_chains_per_block(s->S) * s->S;
+      for (int o = 0; o < q.n_atoms; o += per)
+        s->t_chain.push_back(Tile{q.atom_off + o, std::min(per, q.n_atoms - o), r, 0});
+    }
+    q.n_ctiles = (int)s->t_chain.size() - q.ctile_off;
     // chains are locally as dense as a melt even in a sparse box, so the
     // density used for the capacity is at least that of a dense melt
     const double rho = std::max(q.n_atoms / (L * L * L), 40.0);
@@ -500,12 +512,12 @@ static size_t plan(md_system* s, char* base) {
   const size_t fsz = s->mixed ? sizeof(double) : sizeof(float);
   s->reps = (RepDev*)take(sizeof(RepDev) * s->n_reps);
   s->tiles_int = (Tile*)take(sizeof(Tile) * s->t_int.size());
+  s->tiles_chain = (Tile*)take(sizeof(Tile) * s->t_chain.size());
   s->x = take(3 * N * fsz);
   s->v = take(3 * N * fsz);
   s->img = (int*)take(3 * N * sizeof(int));
   s->F = take(N * (s->mixed ? sizeof(F4i) : sizeof(float4)));
-  s->flj = (long long*)take(3 * (size_t)s->Npad * sizeof(long long));
-  s->flj_e = (long long*)take(3 * (size_t)s->Npad * sizeof(long long));
+  for (long long*& f : s->flj) f = (long long*)take(3 * (size_t)s->Npad * sizeof(long long));
   s->site = (uint16_t*)take(N * sizeof(uint16_t));
   s->cellc = (int*)take(N * sizeof(int));
   s->ref = (float4*)take(N * sizeof(float4));
@@ -522,19 +534,21 @@ static size_t plan(md_system* s, char* base) {
   s->list = (unsigned*)take((size_t)s->n_cl_max * s->cap * sizeof(unsigned));
   s->ncl = (int*)take((size_t)s->n_cl_max * sizeof(int));
   s->cl_start = (int*)take((C + 1) * sizeof(int));
-  s->count = (int*)take(C * sizeof(int));
+  s->count = (int*)take((C + 1) * sizeof(int));
+  s->moved = (unsigned*)(s->count + C);
   s->cell_start = (int*)take((C + 1) * sizeof(int));
   s->cell_of = (int*)take(N * sizeof(int));
   s->slot = (int*)take(N * sizeof(int));
   s->tmp = (int*)take(N * sizeof(int));
   s->lj_part = (double*)take(C * 8 * sizeof(double));
   s->b_part = (double*)take(s->t_int.size() * 9 * sizeof(double));
-  s->kepart = (double*)take(4 * s->t_int.size() * sizeof(double));   // kinetic energy, then momentum (x, y, z) per tile
+  // kinetic energy (and momentum) per tile of either kind
+  s->kepart = (double*)take(4 * std::max(s->t_int.size(), s->t_chain.size()) * sizeof(double));
   s->ke_out = (double*)take(s->n_reps * sizeof(double));
-  s->lam = (double*)take(6 * s->n_reps * sizeof(double));   // rescale factor, or the Nose-Hoover state (6 per replica)
+  s->lam = (double*)take((size_t)kNhDoubles * s->n_reps * sizeof(double));   // rescale factor, or the Nose-Hoover state
   s->e_out = (double*)take((size_t)s->n_reps * 16 * sizeof(double));
   s->e_slices = (double*)take((size_t)s->n_reps * s->max_slices * 11 * sizeof(double));
-  s->done = (unsigned*)take(sizeof(unsigned));
+  s->done = (unsigned*)take(s->n_reps * sizeof(unsigned));
   s->work = (int*)take(2 * sizeof(int));
   s->flags = (unsigned*)take(sizeof(unsigned));
   s->early = (unsigned long long*)take(sizeof(unsigned long long));
@@ -573,7 +587,7 @@ static void enqueue_build(md_system* s) {
 }
 
 static void enqueue_rebin(md_system* s) {
-  cudaMemsetAsync(s->count, 0, sizeof(int) * s->C, s->st);
+  cudaMemsetAsync(s->count, 0, sizeof(int) * (s->C + 1), s->st);   // the cell counts and *moved
   launch_bin_count(s->mixed, s->x, (int)s->N, s->tiles_int, (int)s->t_int.size(), s->reps, s->cell_of, s->cellc,
                    s->count, s->slot, s->st);
   launch_scan2(s->count, s->cell_start, s->cl_start, s->C, s->st);
@@ -586,50 +600,70 @@ static void enqueue_rebin(md_system* s) {
 }
 static const int kRebinLaunches = 7;   // memset counted as a launch
 
-// F_out: where the total force goes (the dynamics' s->F, or scratch for an
-// energy read-out, whose kernels need not reproduce the force bits of the
-// force-only kernels: the compiler may fuse their arithmetic differently)
-static void enqueue_forces(md_system* s, bool energy, void* F_out = nullptr) {
-  // an energy read-out accumulates its LJ forces apart from the dynamics'
-  long long* flj = F_out ? s->flj_e : s->flj;
-  cudaMemsetAsync(flj, 0, 3 * (size_t)s->Npad * sizeof(long long), s->st);
-  prof_mark(s);   // closes the integrate group (integrator, displacement check, clear)
-  launch_cl_force(energy, s->pos, s->cell_start, s->cl_start, s->region_cells, s->items, s->n_lj_items, s->shapes, s->reps,
-                  s->list, s->tasks, s->task_base, s->cap, s->tile_cap, s->fp, flj, s->Npad, s->lj_part, s->flags, s->lj_block,
-                  s->lj_lanes, s->persistent_grid, s->work, s->lj_pair_exact, s->st);
-  prof_mark(s);
+static void enqueue_lj(md_system* s, bool energy, long long* flj) {
+  launch_cl_force(energy, s->pos, s->cell_start, s->cl_start, s->region_cells, s->items, s->n_lj_items, s->shapes,
+                  s->reps, s->list, s->tasks, s->task_base, s->cap, s->tile_cap, s->fp, flj, s->Npad, s->lj_part,
+                  s->flags, s->lj_block, s->lj_lanes, s->persistent_grid, s->work, s->lj_pair_exact, s->st);
+}
+
+static void enqueue_bonded(md_system* s, bool energy, const long long* flj, void* F_out) {
   if (s->generic)
     launch_bonded_generic(energy, (const double*)s->x, s->inv_perm, flj, s->Npad, (int)s->N, s->tiles_int,
-                          (int)s->t_int.size(), s->reps, s->fp, s->topo, F_out ? F_out : s->F, s->b_part, s->flags,
-                          s->st);
+                          (int)s->t_int.size(), s->reps, s->fp, s->topo, F_out, s->b_part, s->flags, s->st);
   else
     launch_bonded(s->mixed, energy, s->x, s->site, s->inv_perm, flj, s->Npad, (int)s->N, s->tiles_int,
-                  (int)s->t_int.size(), s->reps, s->fp, F_out ? F_out : s->F, s->b_part, s->flags, s->st);
+                  (int)s->t_int.size(), s->reps, s->fp, F_out, s->b_part, s->flags, s->st);
+}
+
+// the total force into s->F
+static void enqueue_forces(md_system* s) {
+  cudaMemsetAsync(s->flj[0], 0, 3 * (size_t)s->Npad * sizeof(long long), s->st);
+  prof_mark(s);   // closes the integrate group (integrator, early rebin, clear)
+  enqueue_lj(s, false, s->flj[0]);
+  prof_mark(s);
+  enqueue_bonded(s, false, s->flj[0], s->F);
   prof_mark(s);
 }
 
-// Inside a step-graph capture, after a drift: a one-thread check of the
-// displacement flag sets the condition of an IF node whose body re-bins and
-// rebuilds the list, so a step whose atoms moved more than skin/2 since the
-// last rebin computes its forces from fresh bins (and is counted), instead of
-// the run stopping.  No-op outside a capture.
-static void enqueue_cond_rebin(md_system* s) {
-  if (s->disp != MD_DISP_REBUILD) return;
+// energies and virial into lj_part and b_part; the force form's kernels and
+// buffers are left alone (the energy kernels' LJ form accumulates no forces,
+// the general molecules' bonded form leaves its own in scratch memory)
+static void enqueue_energy(md_system* s) {
+  enqueue_lj(s, true, s->flj[1]);
+  enqueue_bonded(s, true, s->flj[1], s->generic ? s->stage : nullptr);
+}
+
+// Inside a step-graph capture, around a drift: a condition that the drift's
+// kernel sets when an atom has moved more than skin/2 since the last rebin
+// (before), and an IF node whose body re-bins and rebuilds the list (after), so
+// such a step computes its forces from fresh bins (and is counted), instead of
+// the run stopping.  The kernel sets the condition itself: a check in a kernel
+// of its own cost 1.5 us and a launch per step.  No-op outside a capture.
+static MoveReport begin_cond_rebin(md_system* s) {
+  MoveReport mr{};
+  if (s->disp != MD_DISP_REBUILD) return mr;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  cudaGraph_t g = nullptr;
+  if (cudaStreamGetCaptureInfo(s->st, &cs, nullptr, &g, nullptr, nullptr, nullptr) != cudaSuccess ||
+      cs != cudaStreamCaptureStatusActive)
+    return mr;
+  if (cudaGraphConditionalHandleCreate(&mr.handle, g, 0, cudaGraphCondAssignDefault) != cudaSuccess) return mr;
+  mr.moved = s->moved;
+  mr.events = s->early;
+  return mr;
+}
+
+static void end_cond_rebin(md_system* s, const MoveReport& mr) {
+  if (!mr.moved) return;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   cudaGraph_t g = nullptr;
   const cudaGraphNode_t* deps = nullptr;
   const cudaGraphEdgeData* ed = nullptr;
   size_t nd = 0;
-  if (cudaStreamGetCaptureInfo(s->st, &cs, nullptr, &g, &deps, &ed, &nd) != cudaSuccess ||
-      cs != cudaStreamCaptureStatusActive)
-    return;
-  cudaGraphConditionalHandle h;
-  if (cudaGraphConditionalHandleCreate(&h, g, 0, cudaGraphCondAssignDefault) != cudaSuccess) return;
-  launch_disp_check(h, s->flags, s->early, s->st);
   if (cudaStreamGetCaptureInfo(s->st, &cs, nullptr, &g, &deps, &ed, &nd) != cudaSuccess) return;
   cudaGraphNodeParams p{};
   p.type = cudaGraphNodeTypeConditional;
-  p.conditional.handle = h;
+  p.conditional.handle = mr.handle;
   p.conditional.type = cudaGraphCondTypeIf;
   p.conditional.size = 1;
   cudaGraphNode_t node;
@@ -651,32 +685,55 @@ static void enqueue_cond_rebin(md_system* s) {
   cudaStreamEndCapture(s->side, &out);
 }
 
-static void enqueue_integrate(md_system* s, IntegMode mode, bool ke, bool mark) {
-  launch_integrate(s->mixed, mode, ke, s->thermo, s->x, s->v, s->img, s->F, s->site, s->cellc,
-                   s->inv_perm, s->ref, s->pos, (int)s->N, s->tiles_int, (int)s->t_int.size(), s->reps, s->n_reps,
-                   s->fp, s->kepart, s->done, s->ke_out, s->lam, s->tau, s->flags, s->st);
-  if (mark) prof_mark(s);
+static StepArgs step_args(md_system* s, bool chain_tiles, const long long* flj, long long* flj_next) {
+  return StepArgs{s->x, s->v, s->img, s->F, s->site, s->cellc, s->inv_perm, s->ref, s->pos, flj, flj_next, s->Npad,
+                  (int)s->N, chain_tiles ? s->tiles_chain : s->tiles_int,
+                  (int)(chain_tiles ? s->t_chain.size() : s->t_int.size()), s->reps, s->kepart, s->done, s->ke_out,
+                  s->lam, s->tau, s->flags};
 }
 
 // one block of k steps: rebin + list (unless the bins and list are already
-// those of the current positions), k velocity-Verlet steps
+// those of the current positions), k velocity-Verlet steps.  Chains: the
+// block's first drift clears an LJ buffer, and between LJ launches one kernel
+// does the bonded forces, the update and the clearing of the other buffer; the
+// last one closes the step and leaves the force.  General molecules: bonded
+// forces and integrator apart.
 static void enqueue_block(md_system* s, int k, bool rebin = true) {
   s->ev_used = 0;
   prof_mark(s);
   if (rebin) enqueue_rebin(s);
-  enqueue_integrate(s, kKickDrift, false, false);
-  enqueue_cond_rebin(s);
-  enqueue_forces(s, false);
-  for (int j = 1; j < k; ++j) {
-    enqueue_integrate(s, kKickKickDrift, false, false);
-    enqueue_cond_rebin(s);
-    enqueue_forces(s, false);
+  for (int j = 0; j < k; ++j) {
+    long long* flj = s->flj[j & 1];
+    const MoveReport mr = begin_cond_rebin(s);
+    if (j == 0 || s->generic)
+      launch_integrate(s->mixed, j == 0 ? kKickDrift : kKickKickDrift, s->thermo,
+                       step_args(s, false, nullptr, s->generic ? nullptr : flj), s->fp, mr, s->st);
+    else
+      launch_step(s->mixed, kKickKickDrift, s->thermo, s->S, step_args(s, true, s->flj[(j - 1) & 1], flj), s->fp, mr,
+                  s->st);
+    if (j > 0 && !s->generic) prof_mark(s);   // closes the bonded group (bonded forces and update)
+    end_cond_rebin(s, mr);
+    if (s->generic) {
+      enqueue_forces(s);
+      continue;
+    }
+    prof_mark(s);   // closes the integrate group
+    enqueue_lj(s, false, flj);
+    prof_mark(s);
   }
-  enqueue_integrate(s, kKickOnly, false, true);
+  if (s->generic) {
+    launch_integrate(s->mixed, kKickOnly, s->thermo, step_args(s, false, nullptr, nullptr), s->fp,
+                     MoveReport{}, s->st);
+  } else {
+    launch_step(s->mixed, kKickOnly, s->thermo, s->S, step_args(s, true, s->flj[(k - 1) & 1], nullptr), s->fp,
+                MoveReport{}, s->st);
+    prof_mark(s);
+  }
+  prof_mark(s);
 }
-// per step: integrate, displacement check, memset, LJ, bonded (a memset
-// counted as a launch; an early rebin adds kRebinLaunches)
-static int64_t block_launches(int k, bool check) { return kRebinLaunches + (check ? 5LL : 4LL) * k + 1; }
+// chains, per step: LJ and one update; a closing update (an early rebin adds
+// kRebinLaunches).  General molecules: integrate, clear, LJ, two bonded
+static int64_t block_launches(int k, bool generic) { return kRebinLaunches + (generic ? 5LL : 2LL) * k + 1; }
 
 // accumulate the event timings of the last block (requires a finished stream)
 static void prof_collect(md_system* s, int k) {
@@ -772,7 +829,7 @@ static int refresh(md_system* s) {
   const bool p = s->profile;
   s->profile = false;
   enqueue_rebin(s);
-  enqueue_forces(s, false);
+  enqueue_forces(s);
   s->profile = p;
   const int rc = check_flags(s);
   s->fresh = rc == MD_OK;
@@ -868,7 +925,7 @@ int md_create(const md_desc* d, md_system** out) {
     fail(s, MD_ECUDA, "stream creation failed");
     return bail(MD_ECUDA);
   }
-  if (tile_kernels_init() != cudaSuccess) {
+  if (tile_kernels_init() != cudaSuccess || step_kernels_init() != cudaSuccess) {
     cudaGetLastError();
     fail(s, MD_ECUDA, "cannot reserve shared memory for the neighbour-tile kernels");
     return bail(MD_ECUDA);
@@ -888,18 +945,22 @@ int md_create(const md_desc* d, md_system** out) {
     for (int i = 0; i < q.n_atoms; ++i) site[q.atom_off + i] = (uint16_t)(i % s->S);
   }
   // thermostat state: the weak-coupling factor lam[r] = 1, or per replica the
-  // Nose-Hoover (xi, 1 - c, 1/(1 + c), V_com) = (0, 1, 1, 0, 0, 0)
-  std::vector<double> ones(6 * s->n_reps, 1.0);
+  // Nose-Hoover state at rest (xi = 0, V_com = 0)
+  std::vector<double> lam0((size_t)kNhDoubles * s->n_reps, 1.0);
   if (s->thermo == MD_NOSE_HOOVER)
-    for (int r = 0; r < s->n_reps; ++r)
-      for (int k = 0; k < 6; ++k) ones[6 * r + k] = (k == 1 || k == 2) ? 1.0 : 0.0;
+    for (int r = 0; r < s->n_reps; ++r) {
+      double* nh = lam0.data() + (size_t)kNhDoubles * r;
+      const double rest[12] = {0.0, 1.0, 1.0, 0.0, 0.0, 0.0, 1.0, 2.0, 0.0, 0.0, 0.0, 0.0};
+      float* nf = reinterpret_cast<float*>(nh + 12);
+      for (int k = 0; k < 12; ++k) { nh[k] = rest[k]; nf[k] = (float)rest[k]; }
+    }
   auto up = [&](void* dst, const void* src, size_t b) {
     return cudaMemcpyAsync(dst, src, b, cudaMemcpyHostToDevice, s->st) == cudaSuccess;
   };
   bool ok = up(s->reps, s->reps_h.data(), sizeof(RepDev) * s->n_reps) &&
             up(s->tiles_int, s->t_int.data(), sizeof(Tile) * s->t_int.size()) &&
             up(s->site, site.data(), sizeof(uint16_t) * s->N) &&
-            up(s->lam, ones.data(), sizeof(double) * 6 * s->n_reps) &&
+            up(s->lam, lam0.data(), sizeof(double) * lam0.size()) &&
             up(s->region_cells, s->region_cells_h.data(), sizeof(int) * s->region_cells_h.size()) &&
             (!s->generic || (up(s->mtype, s->mtype_h.data(), s->mtype_h.size()) &&
                              up((void*)s->topo.b_off, s->t_boff.data(), s->t_boff.size() * sizeof(int)) &&
@@ -912,9 +973,10 @@ int md_create(const md_desc* d, md_system** out) {
                              up((void*)s->topo.x_at, s->t_xat.data(), s->t_xat.size() * sizeof(int)))) &&
             up(s->shapes, s->shapes_h.data(), sizeof(RegionShape) * s->shapes_h.size()) &&
             up(s->items, s->items_h.data(), sizeof(WorkItem) * s->items_h.size()) &&
-            cudaMemsetAsync(s->flj, 0, 3 * (size_t)s->Npad * sizeof(long long), s->st) == cudaSuccess &&
-            cudaMemsetAsync(s->flj_e, 0, 3 * (size_t)s->Npad * sizeof(long long), s->st) == cudaSuccess &&
-            cudaMemsetAsync(s->done, 0, sizeof(unsigned), s->st) == cudaSuccess &&
+            up(s->tiles_chain, s->t_chain.data(), sizeof(Tile) * s->t_chain.size()) &&
+            cudaMemsetAsync(s->flj[0], 0, 3 * (size_t)s->Npad * sizeof(long long), s->st) == cudaSuccess &&
+            cudaMemsetAsync(s->flj[1], 0, 3 * (size_t)s->Npad * sizeof(long long), s->st) == cudaSuccess &&
+            cudaMemsetAsync(s->done, 0, s->n_reps * sizeof(unsigned), s->st) == cudaSuccess &&
             cudaMemsetAsync(s->work, 0, 2 * sizeof(int), s->st) == cudaSuccess &&
             cudaMemsetAsync(s->flags, 0, sizeof(unsigned), s->st) == cudaSuccess &&
             cudaMemsetAsync(s->early, 0, sizeof(unsigned long long), s->st) == cudaSuccess &&
@@ -982,15 +1044,12 @@ int md_energy(md_system* s, md_energy_t* out) {
   if (!s || !out) return fail(s, MD_EINVAL, "bad arguments");
   const bool p = s->profile;
   s->profile = false;
-  // energies and virial of the current state; the forces of this pass go to
-  // the staging buffer (6N doubles + 3N ints, room for either force layout),
-  // so reading energies never changes the forces the dynamics use
-  enqueue_forces(s, true, s->stage);
+  // energies and virial of the current state
+  enqueue_energy(s);
   launch_energy_reduce(s->lj_part, s->b_part, s->reps, s->n_reps, s->max_slices, s->e_slices, s->e_out, s->st);
   // kinetic energy of the current velocities (a pass that only reads v)
-  launch_integrate(s->mixed, kKineticOnly, true, false, s->x, s->v, s->img, s->F, s->site, s->cellc, s->inv_perm,
-                   s->ref, s->pos, (int)s->N, s->tiles_int, (int)s->t_int.size(), s->reps, s->n_reps, s->fp,
-                   s->kepart, s->done, s->ke_out, s->lam, s->tau, s->flags, s->st);
+  launch_integrate(s->mixed, kKineticOnly, MD_NVE, step_args(s, false, nullptr, nullptr), s->fp, MoveReport{},
+                   s->st);
   s->profile = p;
   CU(cudaGetLastError());
   std::vector<double> e((size_t)s->n_reps * 16), ke(s->n_reps);
@@ -1059,7 +1118,7 @@ int md_set_params(md_system* s, const md_params* p) {
   if (rc) return rc;
   const bool pf = s->profile;
   s->profile = false;
-  enqueue_forces(s, false);
+  enqueue_forces(s);
   s->profile = pf;
   return check_flags(s);
 }
@@ -1310,9 +1369,9 @@ int md_early_rebins(md_system* s, int64_t* count) {
 int md_get_thermostat(md_system* s, double* xi) {
   if (!s || !xi) return fail(s, MD_EINVAL, "bad arguments");
   CU(cudaStreamSynchronize(s->st));
-  std::vector<double> h(6 * (size_t)s->n_reps);
+  std::vector<double> h((size_t)kNhDoubles * s->n_reps);
   CU(cudaMemcpy(h.data(), s->lam, h.size() * sizeof(double), cudaMemcpyDeviceToHost));
-  for (int r = 0; r < s->n_reps; ++r) xi[r] = s->thermo == MD_NOSE_HOOVER ? h[6 * r] : 0.0;
+  for (int r = 0; r < s->n_reps; ++r) xi[r] = s->thermo == MD_NOSE_HOOVER ? h[(size_t)kNhDoubles * r] : 0.0;
   return MD_OK;
 }
 
@@ -1436,10 +1495,9 @@ int md_profile_reset(md_system* s) {
 }
 
 int64_t md_launches_per_call(md_system* s, int64_t n) {
-  if (!s || n <= 0) return 0;
+  if (!s || n < 0) return 0;
   const int64_t full = n / s->R, rem = n % s->R;
-  const bool check = s->disp == MD_DISP_REBUILD;
-  return full * block_launches(s->R, check) + (rem ? block_launches((int)rem, check) : 0);
+  return full * block_launches(s->R, s->generic) + (rem ? block_launches((int)rem, s->generic) : 0);
 }
 
 // ------------------------------------------------------------------ autotuner

@@ -64,8 +64,16 @@ struct RepDev {
   float pad2[2];
   int M, cell_base, atom_off, n_atoms;
   int n_chains, chain_off, tile_off, n_tiles;
+  int ctile_off, n_ctiles;      // chain tiles (blocks of the fused step kernel)
   double T0, dof;
 };
+
+// Nose-Hoover state of a replica, doubles nh[0..11]: xi, fo = 1 - c,
+// fc = 1 / (1 + c), V_com (3), then what a closing and opening kick together
+// need: A = fo fc, 1 + A, A V_com (3), unused; followed by the same as floats
+// (twelve, for the plain form: a double to float conversion would load the
+// FP64 pipe in every thread).  The weak-coupling factor of replica r is lam[r].
+constexpr int kNhDoubles = 18;
 
 struct Tile { int start, len, rep, pad; };
 
@@ -222,6 +230,7 @@ struct ForceParams {
   float b0sq_hi, b0sq_lo;         // b0^2 as a two-float sum
   double b0sq;                    // b0^2
   double mass[2], inv_mass[2];
+  double mass_ratio;              // mass[1] / mass[0]
   double dt;
   float hdt_m_f[2], dt_f;         // FP32 copies for the plain form
   float pad_f;
@@ -327,13 +336,41 @@ void launch_egress_forces(bool mixed, const void* F, int N, double scale, double
 void launch_chain_observables(bool mixed, const void* x, int N, const RepDev* reps, int n_reps,
                               const ForceParams& fp, int n_chains_total, double* ree, double* rg2,
                               unsigned long long* trans, cudaStream_t st);
-// thermostat: 0 none, 1 weak coupling, 2 Nose-Hoover
-void launch_integrate(bool mixed, IntegMode mode, bool ke, int thermostat, void* x, void* v, int* img,
-                      const void* F, const uint16_t* site, const int* cellc, const int* inv_perm,
-                      const float4* ref, float4* pos, int N, const Tile* tiles, int n_tiles,
-                      const RepDev* reps, int n_reps, const ForceParams& fp, double* kepart,
-                      unsigned* done, double* ke_out, double* lam, double tau, unsigned* flags,
-                      cudaStream_t st);
+struct MoveReport;   // where an atom beyond skin/2 is reported (integrate.cuh)
+// Arguments common to the integrator and the fused step kernel.  flj: the LJ
+// force of the step; flj_next: the buffer cleared for the next one (may be
+// null in launch_integrate).  done: one zeroed ticket per replica.
+struct StepArgs {
+  void *x, *v;
+  int* img;
+  void* F;
+  const uint16_t* site;
+  const int *cellc, *inv_perm;
+  const float4* ref;
+  float4* pos;
+  const long long* flj;
+  long long* flj_next;
+  int Npad, N;
+  const Tile* tiles;
+  int n_tiles;
+  const RepDev* reps;
+  double* kepart;               // 4 per tile
+  unsigned* done;
+  double *ke_out, *lam;
+  double tau;
+  unsigned* flags;
+};
+// thermostat: 0 none, 1 weak coupling, 2 Nose-Hoover; tiles are the
+// integrator's (RepDev::tile_off, n_tiles)
+void launch_integrate(bool mixed, IntegMode mode, int thermostat, const StepArgs& a, const ForceParams& fp,
+                      const MoveReport& mr, cudaStream_t st);
+// bonded forces and update of linear chains (k_step.cu): mode kKickKickDrift,
+// or kKickOnly, which also writes the force F; tiles hold whole chains
+// (RepDev::ctile_off, n_ctiles), step_chains_per_block(sites) of them at most
+int step_chains_per_block(int sites);
+cudaError_t step_kernels_init();
+void launch_step(bool mixed, IntegMode mode, int thermostat, int sites, const StepArgs& a, const ForceParams& fp,
+                 const MoveReport& mr, cudaStream_t st);
 // RDF of non-bonded pairs (k_observe.cu): counts[r * n_bins + k] += pairs of
 // replica r with edges[k] <= r < edges[k + 1] (last bin closed); norm =
 // n_bins / (edges[n_bins] - edges[0]) gives the first guess of k.  pos and tag
@@ -346,9 +383,6 @@ void launch_rdf(bool mixed, const void* x, int N, const int* cell_start, const i
 // ACF: add sample s (ring slot s % (max_lag + 1)) to acc[r][tau], tau <= min(s, max_lag)
 void launch_acf_add(const double* ring, int n_chains_total, const RepDev* reps, int n_reps, long long s, int max_lag,
                     double* acc, cudaStream_t st);
-// opens the conditional rebin of a step graph when kFlagDisplacement is set
-// (then cleared and counted in *events)
-void launch_disp_check(cudaGraphConditionalHandle h, unsigned* flags, unsigned long long* events, cudaStream_t st);
 // cells per slice of the first energy-reduction pass
 constexpr int kEnergySliceCells = 1024;
 int energy_slice_count(int n_cells);
