@@ -346,7 +346,8 @@ int md_profile_read(md_system *sys, double *ms_total, int64_t *launches);
 int md_profile_reset(md_system *sys);
 
 /* Kernel launches per call of md_step(n_steps) (all library kernels and
- * memsets; an early rebuild adds seven more). */
+ * memsets; an early rebuild repeats its block's launches, those before the
+ * step that triggered it without effect). */
 int64_t md_launches_per_call(md_system *sys, int64_t n_steps);
 
 /* Cell binning of one periodic box into caller-provided DEVICE arrays, with

@@ -13,19 +13,10 @@ __device__ __forceinline__ bool past_box(float x, float L) { return __float_as_i
 __device__ __forceinline__ bool negative(double x) { return __double_as_longlong(x) < 0; }
 __device__ __forceinline__ bool negative(float x) { return __float_as_int(x) < 0; }
 
-// Where an atom that moved more than skin/2 since the rebin is reported: the
-// error flag, or the condition of the early rebin that follows in the step
-// graph.  The first atom of a step to report sets the condition and counts
-// the event; the rebin clears *moved.
-struct MoveReport {
-  cudaGraphConditionalHandle handle;
-  unsigned* moved;              // null: kFlagDisplacement
-  unsigned long long* events;
-};
-__device__ __forceinline__ void report_move(const MoveReport& m, unsigned* flags) {
-  if (!m.moved) {
+__device__ __forceinline__ void report_move(const MoveReport& m, int j, unsigned* flags) {
+  if (!m.ctl) {
     atomicOr(flags, kFlagDisplacement);
-  } else if (atomicExch(m.moved, 1u) == 0u) {
+  } else if (atomicMin(m.ctl, j) == kNoMove) {
     cudaGraphSetConditional(m.handle, 1u);
     *m.events += 1ull;
   }

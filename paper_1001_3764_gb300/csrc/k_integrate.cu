@@ -54,13 +54,14 @@ __global__ void __launch_bounds__(kIntBlock) k_integrate(void* __restrict__ xv, 
                                                          double* __restrict__ kepart, unsigned* __restrict__ done,
                                                          double* __restrict__ ke_out, double* __restrict__ lam,
                                                          double tau, unsigned* __restrict__ flags,
-                                                         const MoveReport mr) {
+                                                         const StepGate gate, const MoveReport mr) {
   using T = typename std::conditional<MIXED, double, float>::type;
   T* x = reinterpret_cast<T*>(xv);
   T* v = reinterpret_cast<T*>(vv);
   const Tile t = tiles[blockIdx.x];
   const RepDev& R = reps[t.rep];
   const int i = t.start + threadIdx.x;
+  if (MODE == kKickOnly ? !lj_runs(gate) : !drift_runs(gate)) return;
   AtomOut o;
   o.ke = 0.0;
   o.mom[0] = o.mom[1] = o.mom[2] = 0.0;
@@ -96,7 +97,7 @@ __global__ void __launch_bounds__(kIntBlock) k_integrate(void* __restrict__ xv, 
 #pragma unroll
         for (int a = 0; a < 3; ++a) flj_next[(size_t)a * Npad + i] = 0ll;
       }
-      if (o.moved) report_move(mr, flags);
+      if (o.moved) report_move(mr, gate.j, flags);
       if (o.bad) atomicOr(flags, kFlagNaN);
       pos[inv_perm[i]] = make_float4(o.loc[0], o.loc[1], o.loc[2], (float)type);   // w: LJ type, as the sort writes it
     }
@@ -107,12 +108,12 @@ __global__ void __launch_bounds__(kIntBlock) k_integrate(void* __restrict__ xv, 
 
 template <bool MIXED>
 static void launch_int_t(IntegMode mode, int th, const StepArgs& a, const ForceParams& fp,
-                         const MoveReport& mr, cudaStream_t st) {
+                         const StepGate& gate, const MoveReport& mr, cudaStream_t st) {
 #define MDG_INT(MODE, KE, TH)                                                                                   \
   k_integrate<MIXED, MODE, KE, TH><<<a.n_tiles, kIntBlock, 0, st>>>(a.x, a.v, a.img, a.F, a.site, a.cellc,      \
                                                                     a.inv_perm, a.ref, a.pos, a.flj_next, a.Npad, a.N, \
                                                                     a.tiles, a.reps, fp, a.kepart, a.done, a.ke_out,   \
-                                                                    a.lam, a.tau, a.flags, mr)
+                                                                    a.lam, a.tau, a.flags, gate, mr)
   // With the weak-coupling thermostat (th = 1), every step that starts (KD,
   // KKD) takes the temperature of the unscaled v(t_k), scales v(t_k) by the
   // factor of the previous step and leaves the factor of step k for the next
@@ -138,11 +139,21 @@ static void launch_int_t(IntegMode mode, int th, const StepArgs& a, const ForceP
 }
 
 void launch_integrate(bool mixed, IntegMode mode, int thermostat, const StepArgs& a, const ForceParams& fp,
-                      const MoveReport& mr, cudaStream_t st) {
+                      const StepGate& gate, const MoveReport& mr, cudaStream_t st) {
   if (a.n_tiles <= 0) return;
-  if (mixed) launch_int_t<true>(mode, thermostat, a, fp, mr, st);
-  else launch_int_t<false>(mode, thermostat, a, fp, mr, st);
+  if (mixed) launch_int_t<true>(mode, thermostat, a, fp, gate, mr, st);
+  else launch_int_t<false>(mode, thermostat, a, fp, gate, mr, st);
 }
+
+// ---------------------------------------------------------------- early rebin
+__global__ void __launch_bounds__(32) k_resume(cudaGraphConditionalHandle h, int* __restrict__ ctl) {
+  if (threadIdx.x != 0) return;
+  ctl[1] = ctl[0];
+  ctl[0] = kNoMove;
+  cudaGraphSetConditional(h, 0u);
+}
+
+void launch_resume(cudaGraphConditionalHandle h, int* ctl, cudaStream_t st) { k_resume<<<1, 32, 0, st>>>(h, ctl); }
 
 // ---------------------------------------------------------------- energy reduction
 // LJ partials are per cell (replica r owns cells [cell_base, cell_base + M^3)),

@@ -897,7 +897,7 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_cl_force(
     const RegionShape* __restrict__ shapes, const RepDev* __restrict__ reps, const unsigned* __restrict__ list,
     const ClusterTask* __restrict__ tasks, const int* __restrict__ task_base, int cap,
     int tile_cap, const ForceParams fp, long long* __restrict__ flj, int Npad, double* __restrict__ epart,
-    unsigned* __restrict__ flags, int persistent, int* __restrict__ work) {
+    unsigned* __restrict__ flags, int persistent, int* __restrict__ work, const StepGate gate) {
   constexpr int CPW = 32 / LP;
   extern __shared__ __align__(16) unsigned char smem[];
   float4* sp = reinterpret_cast<float4*>(smem);
@@ -914,6 +914,7 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_cl_force(
   // which warp took which cluster
   __shared__ float ecl[ENERGY ? kRegionClusterCap : 1][kEnergyVals];
   const int lane = threadIdx.x & 31;
+  if (!lj_runs(gate)) return;   // the whole grid leaves together
   for (int it = 0;; ++it) {
     const int r = next_region(persistent != 0, it, work, &sh_r);
     if (r < 0 || r >= n_items) break;
@@ -988,14 +989,15 @@ void launch_cl_force(bool energy, const float4* pos, const int* cell_start, cons
                      const int* cells, const WorkItem* items, int n_items, const RegionShape* shapes,
                      const RepDev* reps, const unsigned* list, const ClusterTask* tasks, const int* task_base,
                      int cap, int tile_cap, const ForceParams& fp, long long* flj, int Npad, double* epart, unsigned* flags, int block,
-                     int lanes, int persistent_grid, int* work, bool exact, cudaStream_t st) {
+                     int lanes, int persistent_grid, int* work, bool exact, const StepGate& gate,
+                     cudaStream_t st) {
   if (n_items <= 0) return;
   const int grid = persistent_grid > 0 ? persistent_grid : n_items;
   const int pers = persistent_grid > 0;
   const size_t sm = cl_force_smem(tile_cap);
 #define MDG_CLF(E, NT, LP, X)                                                                                      \
   k_cl_force<E, NT, LP, X><<<grid, NT, sm, st>>>(pos, cell_start, cl_start, cells, items, n_items, shapes, reps, \
-                                                 list, tasks, task_base, cap, tile_cap, fp, flj, Npad, epart, flags, pers, work)
+                                                 list, tasks, task_base, cap, tile_cap, fp, flj, Npad, epart, flags, pers, work, gate)
 #define MDG_CLF2(NT, LP)                  \
   if (energy) MDG_CLF(true, NT, LP, false); \
   else if (exact) MDG_CLF(false, NT, LP, true); \

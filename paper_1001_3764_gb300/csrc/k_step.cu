@@ -31,7 +31,8 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : NT == 512 ? 2 : 1) k_step(
                                              const RepDev* __restrict__ reps, const ForceParams fp,
                                              double* __restrict__ kepart, unsigned* __restrict__ done,
                                              double* __restrict__ ke_out, double* __restrict__ lam, double tau,
-                                             unsigned* __restrict__ flags, const MoveReport mr) {
+                                             unsigned* __restrict__ flags, const StepGate gate,
+                                             const MoveReport mr) {
   using T = typename std::conditional<MIXED, double, float>::type;
   T* x = reinterpret_cast<T*>(xv);
   T* v = reinterpret_cast<T*>(vv);
@@ -46,6 +47,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : NT == 512 ? 2 : 1) k_step(
   const RepDev& R = reps[t.rep];
   const int tid = threadIdx.x, i = t.start + tid, S = fp.sites;
   const bool on = tid < t.len;
+  const bool runs = MODE == kKickOnly ? lj_runs(gate) : drift_runs(gate);   // used before the first write
   int sm = 0, slot = 0;
   T xi[3];
   if (on) {
@@ -74,6 +76,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : NT == 512 ? 2 : 1) k_step(
     fdi1[tid + 3] = f1; fdi2[tid + 3] = f2; fdi3[tid + 3] = f3v;
   }
   __syncthreads();
+  if (!runs) return;
   AtomOut o;
   o.ke = 0.0;
   o.mom[0] = o.mom[1] = o.mom[2] = 0.0;
@@ -113,7 +116,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : NT == 512 ? 2 : 1) k_step(
         x[a * N + i] = xi[a];
         flj_next[(size_t)a * Npad + i] = 0ll;   // the buffer the next step's LJ adds to
       }
-      if (o.moved) report_move(mr, flags);
+      if (o.moved) report_move(mr, gate.j, flags);
       if (o.bad) atomicOr(flags, kFlagNaN);
       pos[slot] = make_float4(o.loc[0], o.loc[1], o.loc[2], (float)type);   // w: LJ type, as the sort writes it
     }
@@ -128,12 +131,12 @@ int step_chains_per_block(int sites) { return sites >= 256 ? 1 : 256 / sites; }
 
 template <bool MIXED, int NT>
 static void launch_step_t(IntegMode mode, int th, int threads, const StepArgs& a, const ForceParams& fp,
-                          const MoveReport& mr, cudaStream_t st) {
+                          const StepGate& gate, const MoveReport& mr, cudaStream_t st) {
 #define MDG_STEP(MODE, KE, TH)                                                                                       \
   k_step<MIXED, MODE, KE, TH, NT><<<a.n_tiles, threads, step_smem_bytes(threads), st>>>(a.x, a.v, a.img, a.F, a.site, a.cellc, a.inv_perm,  \
                                                                  a.ref, a.pos, a.flj, a.flj_next, a.Npad, a.N,       \
                                                                  a.tiles, a.reps, fp, a.kepart, a.done, a.ke_out,    \
-                                                                 a.lam, a.tau, a.flags, mr)
+                                                                 a.lam, a.tau, a.flags, gate, mr)
   if (mode == kKickKickDrift) {
     if (th == 2) MDG_STEP(kKickKickDrift, true, 2);
     else if (th == 1) MDG_STEP(kKickKickDrift, true, 1);
@@ -166,18 +169,18 @@ cudaError_t step_kernels_init() {
 }
 
 void launch_step(bool mixed, IntegMode mode, int th, int sites, const StepArgs& a, const ForceParams& fp,
-                 const MoveReport& mr, cudaStream_t st) {
+                 const StepGate& gate, const MoveReport& mr, cudaStream_t st) {
   if (a.n_tiles <= 0) return;
   const int threads = (step_chains_per_block(sites) * sites + 31) / 32 * 32;
   if (threads <= 256) {
-    if (mixed) launch_step_t<true, 256>(mode, th, threads, a, fp, mr, st);
-    else launch_step_t<false, 256>(mode, th, threads, a, fp, mr, st);
+    if (mixed) launch_step_t<true, 256>(mode, th, threads, a, fp, gate, mr, st);
+    else launch_step_t<false, 256>(mode, th, threads, a, fp, gate, mr, st);
   } else if (threads <= 512) {
-    if (mixed) launch_step_t<true, 512>(mode, th, threads, a, fp, mr, st);
-    else launch_step_t<false, 512>(mode, th, threads, a, fp, mr, st);
+    if (mixed) launch_step_t<true, 512>(mode, th, threads, a, fp, gate, mr, st);
+    else launch_step_t<false, 512>(mode, th, threads, a, fp, gate, mr, st);
   } else {
-    if (mixed) launch_step_t<true, 1024>(mode, th, threads, a, fp, mr, st);
-    else launch_step_t<false, 1024>(mode, th, threads, a, fp, mr, st);
+    if (mixed) launch_step_t<true, 1024>(mode, th, threads, a, fp, gate, mr, st);
+    else launch_step_t<false, 1024>(mode, th, threads, a, fp, gate, mr, st);
   }
 }
 

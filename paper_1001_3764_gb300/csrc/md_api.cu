@@ -19,7 +19,6 @@
 
 #include "../../include/md.h"
 #include "md_kernels.cuh"
-#include "integrate.cuh"
 
 using namespace mdg;
 
@@ -105,7 +104,7 @@ struct md_system {
   std::vector<cudaGraphExec_t> rem_graphs;   // blocks of k < R steps (remainders), captured on first use
   cudaStream_t side = nullptr;               // captures the bodies of the conditional rebins
   unsigned long long* early = nullptr;       // early rebins (displacement beyond skin/2) so far
-  unsigned* moved = nullptr;                 // an atom of this step is beyond skin/2 (cleared with the cell counts)
+  int* ctl = nullptr;                        // early rebin within a block of steps (StepGate)
   // a general molecule type (md_desc.topology), or linear chains
   bool generic = false;
   int disp = MD_DISP_REBUILD;                // what a displacement beyond skin/2 does
@@ -534,8 +533,7 @@ static size_t plan(md_system* s, char* base) {
   s->list = (unsigned*)take((size_t)s->n_cl_max * s->cap * sizeof(unsigned));
   s->ncl = (int*)take((size_t)s->n_cl_max * sizeof(int));
   s->cl_start = (int*)take((C + 1) * sizeof(int));
-  s->count = (int*)take((C + 1) * sizeof(int));
-  s->moved = (unsigned*)(s->count + C);
+  s->count = (int*)take(C * sizeof(int));
   s->cell_start = (int*)take((C + 1) * sizeof(int));
   s->cell_of = (int*)take(N * sizeof(int));
   s->slot = (int*)take(N * sizeof(int));
@@ -551,6 +549,7 @@ static size_t plan(md_system* s, char* base) {
   s->done = (unsigned*)take(s->n_reps * sizeof(unsigned));
   s->work = (int*)take(2 * sizeof(int));
   s->flags = (unsigned*)take(sizeof(unsigned));
+  s->ctl = (int*)take(2 * sizeof(int));
   s->early = (unsigned long long*)take(sizeof(unsigned long long));
   s->stage = (double*)take(6 * N * sizeof(double) + 3 * N * sizeof(int));   // staging: x, v (FP64), images
   if (s->generic) {
@@ -587,7 +586,7 @@ static void enqueue_build(md_system* s) {
 }
 
 static void enqueue_rebin(md_system* s) {
-  cudaMemsetAsync(s->count, 0, sizeof(int) * (s->C + 1), s->st);   // the cell counts and *moved
+  cudaMemsetAsync(s->count, 0, sizeof(int) * s->C, s->st);
   launch_bin_count(s->mixed, s->x, (int)s->N, s->tiles_int, (int)s->t_int.size(), s->reps, s->cell_of, s->cellc,
                    s->count, s->slot, s->st);
   launch_scan2(s->count, s->cell_start, s->cl_start, s->C, s->st);
@@ -600,10 +599,10 @@ static void enqueue_rebin(md_system* s) {
 }
 static const int kRebinLaunches = 7;   // memset counted as a launch
 
-static void enqueue_lj(md_system* s, bool energy, long long* flj) {
+static void enqueue_lj(md_system* s, bool energy, long long* flj, const StepGate& gate = StepGate{}) {
   launch_cl_force(energy, s->pos, s->cell_start, s->cl_start, s->region_cells, s->items, s->n_lj_items, s->shapes,
                   s->reps, s->list, s->tasks, s->task_base, s->cap, s->tile_cap, s->fp, flj, s->Npad, s->lj_part,
-                  s->flags, s->lj_block, s->lj_lanes, s->persistent_grid, s->work, s->lj_pair_exact, s->st);
+                  s->flags, s->lj_block, s->lj_lanes, s->persistent_grid, s->work, s->lj_pair_exact, gate, s->st);
 }
 
 static void enqueue_bonded(md_system* s, bool energy, const long long* flj, void* F_out) {
@@ -616,10 +615,10 @@ static void enqueue_bonded(md_system* s, bool energy, const long long* flj, void
 }
 
 // the total force into s->F
-static void enqueue_forces(md_system* s) {
+static void enqueue_forces(md_system* s, const StepGate& gate = StepGate{}) {
   cudaMemsetAsync(s->flj[0], 0, 3 * (size_t)s->Npad * sizeof(long long), s->st);
   prof_mark(s);   // closes the integrate group (integrator, early rebin, clear)
-  enqueue_lj(s, false, s->flj[0]);
+  enqueue_lj(s, false, s->flj[0], gate);
   prof_mark(s);
   enqueue_bonded(s, false, s->flj[0], s->F);
   prof_mark(s);
@@ -633,58 +632,6 @@ static void enqueue_energy(md_system* s) {
   enqueue_bonded(s, true, s->flj[1], s->generic ? s->stage : nullptr);
 }
 
-// Inside a step-graph capture, around a drift: a condition that the drift's
-// kernel sets when an atom has moved more than skin/2 since the last rebin
-// (before), and an IF node whose body re-bins and rebuilds the list (after), so
-// such a step computes its forces from fresh bins (and is counted), instead of
-// the run stopping.  The kernel sets the condition itself: a check in a kernel
-// of its own cost 1.5 us and a launch per step.  No-op outside a capture.
-static MoveReport begin_cond_rebin(md_system* s) {
-  MoveReport mr{};
-  if (s->disp != MD_DISP_REBUILD) return mr;
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  cudaGraph_t g = nullptr;
-  if (cudaStreamGetCaptureInfo(s->st, &cs, nullptr, &g, nullptr, nullptr, nullptr) != cudaSuccess ||
-      cs != cudaStreamCaptureStatusActive)
-    return mr;
-  if (cudaGraphConditionalHandleCreate(&mr.handle, g, 0, cudaGraphCondAssignDefault) != cudaSuccess) return mr;
-  mr.moved = s->moved;
-  mr.events = s->early;
-  return mr;
-}
-
-static void end_cond_rebin(md_system* s, const MoveReport& mr) {
-  if (!mr.moved) return;
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  cudaGraph_t g = nullptr;
-  const cudaGraphNode_t* deps = nullptr;
-  const cudaGraphEdgeData* ed = nullptr;
-  size_t nd = 0;
-  if (cudaStreamGetCaptureInfo(s->st, &cs, nullptr, &g, &deps, &ed, &nd) != cudaSuccess) return;
-  cudaGraphNodeParams p{};
-  p.type = cudaGraphNodeTypeConditional;
-  p.conditional.handle = mr.handle;
-  p.conditional.type = cudaGraphCondTypeIf;
-  p.conditional.size = 1;
-  cudaGraphNode_t node;
-  if (cudaGraphAddNode(&node, g, deps, ed, nd, &p) != cudaSuccess) return;
-  cudaGraph_t body = p.conditional.phGraph_out[0];
-  if (cudaStreamUpdateCaptureDependencies(s->st, &node, nullptr, 1, cudaStreamSetCaptureDependencies) != cudaSuccess)
-    return;
-  // the body: the rebin sequence, captured on the side stream
-  if (cudaStreamBeginCaptureToGraph(s->side, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
-    return;
-  cudaStream_t main = s->st;
-  const bool prof = s->profile;
-  s->st = s->side;
-  s->profile = false;
-  enqueue_rebin(s);
-  s->st = main;
-  s->profile = prof;
-  cudaGraph_t out = nullptr;
-  cudaStreamEndCapture(s->side, &out);
-}
-
 static StepArgs step_args(md_system* s, bool chain_tiles, const long long* flj, long long* flj_next) {
   return StepArgs{s->x, s->v, s->img, s->F, s->site, s->cellc, s->inv_perm, s->ref, s->pos, flj, flj_next, s->Npad,
                   (int)s->N, chain_tiles ? s->tiles_chain : s->tiles_int,
@@ -692,44 +639,96 @@ static StepArgs step_args(md_system* s, bool chain_tiles, const long long* flj, 
                   s->lam, s->tau, s->flags};
 }
 
-// one block of k steps: rebin + list (unless the bins and list are already
-// those of the current positions), k velocity-Verlet steps.  Chains: the
-// block's first drift clears an LJ buffer, and between LJ launches one kernel
-// does the bonded forces, the update and the clearing of the other buffer; the
-// last one closes the step and leaves the force.  General molecules: bonded
-// forces and integrator apart.
+// Steps first .. k - 1 of a block of k, LJ launch first on (first = 0: from
+// the opening drift), and the closing kick.  Chains: the opening drift clears
+// an LJ buffer, and between LJ launches one kernel does the bonded forces, the
+// update and the clearing of the other buffer; the last one closes the step
+// and leaves the force.  General molecules: bonded forces and integrator apart.
+static void enqueue_steps(md_system* s, int k, bool repeat, const MoveReport& mr) {
+  for (int j = 0; j < k; ++j) {
+    long long* flj = s->flj[j & 1];
+    const StepGate gate{mr.ctl, j, repeat ? 1 : 0};
+    if (j == 0 && repeat) {
+      // a repeat resumes at an LJ launch
+    } else if (j == 0 || s->generic) {
+      launch_integrate(s->mixed, j == 0 ? kKickDrift : kKickKickDrift, s->thermo,
+                       step_args(s, false, nullptr, s->generic ? nullptr : flj), s->fp, gate, mr, s->st);
+    } else {
+      launch_step(s->mixed, kKickKickDrift, s->thermo, s->S, step_args(s, true, s->flj[(j - 1) & 1], flj), s->fp, gate,
+                  mr, s->st);
+      prof_mark(s);   // closes the bonded group (bonded forces and update)
+    }
+    if (s->generic) {
+      enqueue_forces(s, gate);
+      continue;
+    }
+    prof_mark(s);   // closes the integrate group
+    enqueue_lj(s, false, flj, gate);
+    prof_mark(s);
+  }
+  const StepGate gate{mr.ctl, k - 1, repeat ? 1 : 0};
+  if (s->generic) {
+    launch_integrate(s->mixed, kKickOnly, s->thermo, step_args(s, false, nullptr, nullptr), s->fp, gate, mr, s->st);
+  } else {
+    launch_step(s->mixed, kKickOnly, s->thermo, s->S, step_args(s, true, s->flj[(k - 1) & 1], nullptr), s->fp, gate, mr,
+                s->st);
+    prof_mark(s);
+  }
+  prof_mark(s);
+}
+
+// One block of k steps: rebin + list (unless the bins and list are already
+// those of the current positions), k velocity-Verlet steps.  Inside a capture,
+// with MD_DISP_REBUILD, a WHILE node follows whose condition the drifts' kernels
+// set when an atom has moved more than skin/2 since the last rebin: its body
+// rebins and repeats the block from that step's LJ launch (StepGate), so such a
+// step computes its forces from fresh bins (and is counted), instead of the
+// run stopping.  A conditional node per step, and a kernel to set its
+// condition, took 9 us of a 33 us step at 1,500 sites.
 static void enqueue_block(md_system* s, int k, bool rebin = true) {
   s->ev_used = 0;
   prof_mark(s);
   if (rebin) enqueue_rebin(s);
-  for (int j = 0; j < k; ++j) {
-    long long* flj = s->flj[j & 1];
-    const MoveReport mr = begin_cond_rebin(s);
-    if (j == 0 || s->generic)
-      launch_integrate(s->mixed, j == 0 ? kKickDrift : kKickKickDrift, s->thermo,
-                       step_args(s, false, nullptr, s->generic ? nullptr : flj), s->fp, mr, s->st);
-    else
-      launch_step(s->mixed, kKickKickDrift, s->thermo, s->S, step_args(s, true, s->flj[(j - 1) & 1], flj), s->fp, mr,
-                  s->st);
-    if (j > 0 && !s->generic) prof_mark(s);   // closes the bonded group (bonded forces and update)
-    end_cond_rebin(s, mr);
-    if (s->generic) {
-      enqueue_forces(s);
-      continue;
-    }
-    prof_mark(s);   // closes the integrate group
-    enqueue_lj(s, false, flj);
-    prof_mark(s);
+  MoveReport mr{};
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  cudaGraph_t g = nullptr;
+  if (s->disp == MD_DISP_REBUILD &&
+      cudaStreamGetCaptureInfo(s->st, &cs, nullptr, &g, nullptr, nullptr, nullptr) == cudaSuccess &&
+      cs == cudaStreamCaptureStatusActive &&
+      cudaGraphConditionalHandleCreate(&mr.handle, g, 0, cudaGraphCondAssignDefault) == cudaSuccess) {
+    mr.ctl = s->ctl;
+    mr.events = s->early;
   }
-  if (s->generic) {
-    launch_integrate(s->mixed, kKickOnly, s->thermo, step_args(s, false, nullptr, nullptr), s->fp,
-                     MoveReport{}, s->st);
-  } else {
-    launch_step(s->mixed, kKickOnly, s->thermo, s->S, step_args(s, true, s->flj[(k - 1) & 1], nullptr), s->fp,
-                MoveReport{}, s->st);
-    prof_mark(s);
-  }
-  prof_mark(s);
+  enqueue_steps(s, k, false, mr);
+  if (!mr.ctl) return;
+  const cudaGraphNode_t* deps = nullptr;
+  const cudaGraphEdgeData* ed = nullptr;
+  size_t nd = 0;
+  if (cudaStreamGetCaptureInfo(s->st, &cs, nullptr, &g, &deps, &ed, &nd) != cudaSuccess) return;
+  cudaGraphNodeParams p{};
+  p.type = cudaGraphNodeTypeConditional;
+  p.conditional.handle = mr.handle;
+  p.conditional.type = cudaGraphCondTypeWhile;
+  p.conditional.size = 1;
+  cudaGraphNode_t node;
+  if (cudaGraphAddNode(&node, g, deps, ed, nd, &p) != cudaSuccess) return;
+  cudaGraph_t body = p.conditional.phGraph_out[0];
+  if (cudaStreamUpdateCaptureDependencies(s->st, &node, nullptr, 1, cudaStreamSetCaptureDependencies) != cudaSuccess)
+    return;
+  // the body, captured on the side stream
+  if (cudaStreamBeginCaptureToGraph(s->side, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
+    return;
+  cudaStream_t main = s->st;
+  const bool prof = s->profile;
+  s->st = s->side;
+  s->profile = false;
+  launch_resume(mr.handle, s->ctl, s->st);
+  enqueue_rebin(s);
+  enqueue_steps(s, k, true, mr);
+  s->st = main;
+  s->profile = prof;
+  cudaGraph_t out = nullptr;
+  cudaStreamEndCapture(s->side, &out);
 }
 // chains, per step: LJ and one update; a closing update (an early rebin adds
 // kRebinLaunches).  General molecules: integrate, clear, LJ, two bonded
@@ -957,6 +956,7 @@ int md_create(const md_desc* d, md_system** out) {
   auto up = [&](void* dst, const void* src, size_t b) {
     return cudaMemcpyAsync(dst, src, b, cudaMemcpyHostToDevice, s->st) == cudaSuccess;
   };
+  const int ctl0[2] = {kNoMove, 0};
   bool ok = up(s->reps, s->reps_h.data(), sizeof(RepDev) * s->n_reps) &&
             up(s->tiles_int, s->t_int.data(), sizeof(Tile) * s->t_int.size()) &&
             up(s->site, site.data(), sizeof(uint16_t) * s->N) &&
@@ -979,6 +979,7 @@ int md_create(const md_desc* d, md_system** out) {
             cudaMemsetAsync(s->done, 0, s->n_reps * sizeof(unsigned), s->st) == cudaSuccess &&
             cudaMemsetAsync(s->work, 0, 2 * sizeof(int), s->st) == cudaSuccess &&
             cudaMemsetAsync(s->flags, 0, sizeof(unsigned), s->st) == cudaSuccess &&
+            up(s->ctl, ctl0, sizeof ctl0) &&
             cudaMemsetAsync(s->early, 0, sizeof(unsigned long long), s->st) == cudaSuccess &&
             cudaStreamSynchronize(s->st) == cudaSuccess;
   if (!ok) { fail(s, MD_ECUDA, "initial upload failed"); return bail(MD_ECUDA); }
@@ -1048,8 +1049,8 @@ int md_energy(md_system* s, md_energy_t* out) {
   enqueue_energy(s);
   launch_energy_reduce(s->lj_part, s->b_part, s->reps, s->n_reps, s->max_slices, s->e_slices, s->e_out, s->st);
   // kinetic energy of the current velocities (a pass that only reads v)
-  launch_integrate(s->mixed, kKineticOnly, MD_NVE, step_args(s, false, nullptr, nullptr), s->fp, MoveReport{},
-                   s->st);
+  launch_integrate(s->mixed, kKineticOnly, MD_NVE, step_args(s, false, nullptr, nullptr), s->fp, StepGate{},
+                   MoveReport{}, s->st);
   s->profile = p;
   CU(cudaGetLastError());
   std::vector<double> e((size_t)s->n_reps * 16), ke(s->n_reps);

@@ -260,6 +260,36 @@ struct TopoDev {
 
 struct F4i { long long x, y, z, w; };   // fixed-point force, 32 B
 
+// Early rebins (displacement beyond skin/2) inside a block of steps.  ctl[0]
+// is the drift that found such an atom (kNoMove: none) and ctl[1] the one a
+// repeat resumes at.  Drift j comes before LJ launch j.  When drift m reports,
+// everything after it in the block does nothing; the WHILE node at the block's
+// end then rebins and runs the block again from LJ launch m on.  So a step
+// costs no graph node of its own for the check.
+constexpr int kNoMove = 0x7fffffff;
+struct StepGate {
+  const int* ctl;   // null: always runs
+  int j;            // this launch's drift or LJ index
+  int repeat;       // 1 inside the WHILE body
+};
+__device__ __forceinline__ bool lj_runs(const StepGate& g) {
+  if (!g.ctl) return true;
+  const volatile int* c = g.ctl;
+  return c[0] > g.j && (!g.repeat || g.j >= c[1]);
+}
+__device__ __forceinline__ bool drift_runs(const StepGate& g) {
+  if (!g.ctl) return true;
+  const volatile int* c = g.ctl;   // c[0] == j: another block of this launch reported
+  return c[0] >= g.j && (!g.repeat || g.j > c[1]);
+}
+// where an atom beyond skin/2 is reported: ctl null, kFlagDisplacement; else
+// ctl[0] = j, and the first report sets the condition and counts the event
+struct MoveReport {
+  cudaGraphConditionalHandle handle;
+  int* ctl;
+  unsigned long long* events;
+};
+
 // ---------------------------------------------------------------- binning
 void launch_bin_count(bool mixed, const void* x, int N, const Tile* tiles, int n_tiles,
                       const RepDev* reps, int* cell_of, int* cellc, int* count, int* slot,
@@ -303,7 +333,7 @@ void launch_cl_force(bool energy, const float4* pos, const int* cell_start, cons
                      const int* cells, const WorkItem* items, int n_items, const RegionShape* shapes,
                      const RepDev* reps, const unsigned* list, const ClusterTask* tasks, const int* task_base,
                      int cap, int tile_cap, const ForceParams& fp, long long* flj, int Npad, double* epart, unsigned* flags, int block, int lanes,
-                     int persistent_grid, int* work, bool exact, cudaStream_t st);
+                     int persistent_grid, int* work, bool exact, const StepGate& gate, cudaStream_t st);
 int lj_blocks_per_sm(int block, int lanes, int tile_cap);
 cudaError_t tile_kernels_init();
 int tile_capacity_max();
@@ -336,7 +366,6 @@ void launch_egress_forces(bool mixed, const void* F, int N, double scale, double
 void launch_chain_observables(bool mixed, const void* x, int N, const RepDev* reps, int n_reps,
                               const ForceParams& fp, int n_chains_total, double* ree, double* rg2,
                               unsigned long long* trans, cudaStream_t st);
-struct MoveReport;   // where an atom beyond skin/2 is reported (integrate.cuh)
 // Arguments common to the integrator and the fused step kernel.  flj: the LJ
 // force of the step; flj_next: the buffer cleared for the next one (may be
 // null in launch_integrate).  done: one zeroed ticket per replica.
@@ -363,14 +392,16 @@ struct StepArgs {
 // thermostat: 0 none, 1 weak coupling, 2 Nose-Hoover; tiles are the
 // integrator's (RepDev::tile_off, n_tiles)
 void launch_integrate(bool mixed, IntegMode mode, int thermostat, const StepArgs& a, const ForceParams& fp,
-                      const MoveReport& mr, cudaStream_t st);
+                      const StepGate& gate, const MoveReport& mr, cudaStream_t st);
 // bonded forces and update of linear chains (k_step.cu): mode kKickKickDrift,
 // or kKickOnly, which also writes the force F; tiles hold whole chains
 // (RepDev::ctile_off, n_ctiles), step_chains_per_block(sites) of them at most
 int step_chains_per_block(int sites);
 cudaError_t step_kernels_init();
 void launch_step(bool mixed, IntegMode mode, int thermostat, int sites, const StepArgs& a, const ForceParams& fp,
-                 const MoveReport& mr, cudaStream_t st);
+                 const StepGate& gate, const MoveReport& mr, cudaStream_t st);
+// first node of the WHILE body: the repeat resumes at ctl[0]; condition off
+void launch_resume(cudaGraphConditionalHandle h, int* ctl, cudaStream_t st);
 // RDF of non-bonded pairs (k_observe.cu): counts[r * n_bins + k] += pairs of
 // replica r with edges[k] <= r < edges[k + 1] (last bin closed); norm =
 // n_bins / (edges[n_bins] - edges[0]) gives the first guess of k.  pos and tag
