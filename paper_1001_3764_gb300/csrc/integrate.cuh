@@ -38,7 +38,7 @@ struct AtomOut {
 };
 template <int TH, class T>
 __device__ __forceinline__ void kinetic_terms(const T (&vi)[3], int type, const ForceParams& fp, AtomOut& o) {
-  const double u[3] = {(double)vi[0], (double)vi[1], (double)vi[2]};
+  const double u[3] = {f2d_int(vi[0]), f2d_int(vi[1]), f2d_int(vi[2])};
   o.ke = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
   if (TH == 2)
 #pragma unroll
@@ -136,98 +136,92 @@ __device__ __forceinline__ void integrate_atom(const T (&F)[3], T (&xi)[3], T (&
   }
 }
 
-// Sums over the block's threads of NV values each, val[a][thread], left in
-// val[a][0] on return (a barrier included): every stage adds four values per
-// thread, so 256 values take 4 stages of 3 dependent additions, and the adds
-// of all NV values fill whole warps.  This GPU's FP64 pipe is narrow: a
-// shuffle tree would issue five adds on every lane, and one thread per 32
-// values (the former form) is a chain of 40.  The order depends on the block
-// size alone.
-template <int NV, int NT>
-__device__ __forceinline__ void block_sums(double (&val)[NV][NT]) {
-  int m = blockDim.x;
+// Sums over n threads' values, NV rows of val (stride `stride`), left in
+// place 0 of each row on return (a barrier included): every stage adds four
+// values per thread, so 256 values take 4 stages of 3 dependent additions, and
+// the adds of all NV values fill whole warps.  This GPU's FP64 pipe is narrow:
+// a shuffle tree would issue five adds on every lane, and one thread per 32
+// values (the former form) is a chain of 40.  The order depends on n alone.
+template <int NV>
+__device__ __forceinline__ void block_sums(double* val, int stride, int n) {
+  int m = n;
   __syncthreads();
   while (m > 1) {
     const int q = (m + 3) >> 2;
     for (int u = threadIdx.x; u < NV * q; u += blockDim.x) {
       const int a = u / q, j = u - a * q;
-      double s = val[a][j];
+      double* row = val + a * stride;
+      double s = row[j];
 #pragma unroll
       for (int k = 1; k < 4; ++k)
-        if (j + k * q < m) s += val[a][j + k * q];
-      val[a][j] = s;
+        if (j + k * q < m) s += row[j + k * q];
+      row[j] = s;
     }
     m = q;
     __syncthreads();
   }
 }
 
-// Kinetic energy (and with Nose-Hoover the momentum) of a replica: every
-// block leaves the sums of its tile, and the last block of the replica to
-// finish (a ticket per replica; no waiting) adds the replica's tiles, in an
-// order that depends only on their number, and sets the thermostat factors of
-// the next step.  One ticket per replica lets the replicas finish side by
-// side: with one for the whole launch, a single block went through 64
-// replicas one after another (100 us of a 152 us launch).
+// Kinetic energy (and with Nose-Hoover the momentum) of a tile, left in kepart
 template <int TH, int NT>
-__device__ __forceinline__ void replica_kinetic(const AtomOut& o, int rep, int tile, int first_tile, int n_tiles,
-                                                const RepDev* __restrict__ reps, const ForceParams& fp,
-                                                double* __restrict__ kepart, unsigned* __restrict__ done,
-                                                double* __restrict__ ke_out, double* __restrict__ lam, double tau) {
+__device__ __forceinline__ void tile_kinetic(const AtomOut& o, int tile, double* __restrict__ kepart) {
   constexpr int NV = TH == 2 ? 4 : 1;
   __shared__ double vals[NV][NT];
-  __shared__ bool last;
-  const int tid = threadIdx.x;
-  vals[0][tid] = o.ke;
+  vals[0][threadIdx.x] = o.ke;
   if constexpr (TH == 2) {
 #pragma unroll
-    for (int a = 0; a < 3; ++a) vals[1 + a][tid] = o.mom[a];
+    for (int a = 0; a < 3; ++a) vals[1 + a][threadIdx.x] = o.mom[a];
   }
-  block_sums<NV, NT>(vals);
-  if (tid < NV) kepart[(size_t)NV * tile + tid] = vals[tid][0];
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) last = atomicAdd(done + rep, 1u) == (unsigned)n_tiles - 1u;
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
+  block_sums<NV>(&vals[0][0], NT, blockDim.x);
+  if (threadIdx.x < NV) kepart[(size_t)NV * tile + threadIdx.x] = vals[threadIdx.x][0];
+}
+
+// A replica's sums over its tiles, in an order that depends only on their
+// number: sum of value a at val[a * blockDim.x] (a barrier included).  val
+// holds NV rows of blockDim.x doubles.
+template <int NV>
+__device__ __forceinline__ void replica_sums(const double* __restrict__ kepart, int first_tile, int n_tiles,
+                                             double* val) {
   double P[NV];
 #pragma unroll
   for (int a = 0; a < NV; ++a) P[a] = 0.0;
 #pragma unroll 4
-  for (int q = tid; q < n_tiles; q += blockDim.x)
+  for (int q = threadIdx.x; q < n_tiles; q += blockDim.x)
 #pragma unroll
     for (int a = 0; a < NV; ++a) P[a] += __ldcg(kepart + (size_t)NV * (first_tile + q) + a);
 #pragma unroll
-  for (int a = 0; a < NV; ++a) vals[a][tid] = P[a];
-  block_sums<NV, NT>(vals);
-  if (tid != 0) return;
-  done[rep] = 0u;
-  const RepDev& Q = reps[rep];
-  const double sum = 0.5 * fp.mass[0] * vals[0][0];
-  ke_out[rep] = sum;
-  if (TH == 1) {
-    const double T_inst = 2.0 * sum / (Q.dof * 0.0083144626);
-    lam[rep] = sqrt(1.0 + fp.dt / tau * (Q.T0 / T_inst - 1.0));
+  for (int a = 0; a < NV; ++a) val[a * blockDim.x + threadIdx.x] = P[a];
+  block_sums<NV>(val, blockDim.x, blockDim.x);
+}
+
+// The thermostat factors of the next drift, by a block of the LJ launch that
+// follows a drift: the sums wait for no one there, where a last block of the
+// drift's launch added a ticket, a fence and a lone block's 5 us to it (150k
+// plain: 18.4 -> 11.4 us per update; 35k Nose-Hoover 14.4 -> 8.9).
+__device__ __forceinline__ void replica_thermostat(const ThermoArgs& ta, const RepDev& Q, int rep, double* val) {
+  const int first = ta.chain ? Q.ctile_off : Q.tile_off, n = ta.chain ? Q.n_ctiles : Q.n_tiles;
+  if (ta.th == 1) {
+    replica_sums<1>(ta.kepart, first, n, val);
+    if (threadIdx.x != 0) return;
+    const double sum = val[0];
+    ta.lam[rep] = sqrt(ta.one_minus_rate + Q.vr_num / sum);
+    return;
   }
-  if constexpr (TH == 2) {
-    const double T_half = 2.0 * sum / (Q.dof * 0.0083144626);
-    const double Qm = tau * tau * Q.T0 / (4.0 * 3.14159265358979323846 * 3.14159265358979323846);
-    double* nh = lam + (size_t)kNhDoubles * rep;
-    const double xi = nh[0] + fp.dt * (T_half - Q.T0) / Qm;
-    const double c = 0.5 * fp.dt * xi;
-    const double s = fp.mass[0] / ((double)Q.n_chains * fp.mol_mass);
-    nh[0] = xi; nh[1] = 1.0 - c; nh[2] = 1.0 / (1.0 + c);
-    const double A = nh[1] * nh[2];
-    nh[6] = A; nh[7] = 1.0 + A;
+  replica_sums<4>(ta.kepart, first, n, val);
+  if (threadIdx.x != 0) return;
+  double* nh = ta.lam + (size_t)kNhDoubles * rep;
+  const double xi = nh[0] + Q.nh_rate * (Q.t_scale * val[0] - Q.T0);
+  const double c = 0.5 * ta.dt * xi;
+  nh[0] = xi; nh[1] = 1.0 - c; nh[2] = 1.0 / (1.0 + c);
+  const double A = nh[1] * nh[2];
+  nh[6] = A; nh[7] = 1.0 + A;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      nh[3 + a] = s * vals[1 + a][0];
-      nh[8 + a] = A * nh[3 + a];
-    }
-    float* nf = reinterpret_cast<float*>(nh + 12);
-    for (int k = 0; k < 11; ++k) nf[k] = (float)nh[k];
+  for (int a = 0; a < 3; ++a) {
+    nh[3 + a] = Q.com_scale * val[(1 + a) * blockDim.x];
+    nh[8 + a] = A * nh[3 + a];
   }
+  float* nf = reinterpret_cast<float*>(nh + 12);
+  for (int k = 0; k < 11; ++k) nf[k] = (float)nh[k];
 }
 
 }  // namespace mdg

@@ -10,9 +10,9 @@
 //
 // The paper's Nose-Hoover coupling needs the whole-system kinetic energy,
 // which it sums through a per-atom array and a tree reduction (Sec. 3.4).
-// Here each block writes one FP64 partial; the last block of a replica to
-// finish (a ticket per replica, no waiting) sums the replica's partials in a
-// fixed order and computes its rescaling factor.
+// Here each block writes one FP64 partial, and a block per replica of the LJ
+// launch that follows sums the replica's partials in a fixed order and
+// computes its rescaling factor.
 // The factor computed at step k is applied at step k+1 (one-step lag).
 //
 // Nose-Hoover (TH = 2; the paper's NVT ensemble with Leap-Frog, Sec. 2 and
@@ -51,10 +51,8 @@ __global__ void __launch_bounds__(kIntBlock) k_integrate(void* __restrict__ xv, 
                                                          long long* __restrict__ flj_next, int Npad, int N,
                                                          const Tile* __restrict__ tiles,
                                                          const RepDev* __restrict__ reps, const ForceParams fp,
-                                                         double* __restrict__ kepart, unsigned* __restrict__ done,
-                                                         double* __restrict__ ke_out, double* __restrict__ lam,
-                                                         double tau, unsigned* __restrict__ flags,
-                                                         const StepGate gate, const MoveReport mr) {
+                                                         double* __restrict__ kepart, const double* __restrict__ lam,
+                                                         unsigned* __restrict__ flags, const StepGate gate, const MoveReport mr) {
   using T = typename std::conditional<MIXED, double, float>::type;
   T* x = reinterpret_cast<T*>(xv);
   T* v = reinterpret_cast<T*>(vv);
@@ -102,8 +100,7 @@ __global__ void __launch_bounds__(kIntBlock) k_integrate(void* __restrict__ xv, 
       pos[inv_perm[i]] = make_float4(o.loc[0], o.loc[1], o.loc[2], (float)type);   // w: LJ type, as the sort writes it
     }
   }
-  if constexpr (KE)
-    replica_kinetic<TH, kIntBlock>(o, t.rep, blockIdx.x, R.tile_off, R.n_tiles, reps, fp, kepart, done, ke_out, lam, tau);
+  if constexpr (KE) tile_kinetic<TH, kIntBlock>(o, blockIdx.x, kepart);
 }
 
 template <bool MIXED>
@@ -112,8 +109,8 @@ static void launch_int_t(IntegMode mode, int th, const StepArgs& a, const ForceP
 #define MDG_INT(MODE, KE, TH)                                                                                   \
   k_integrate<MIXED, MODE, KE, TH><<<a.n_tiles, kIntBlock, 0, st>>>(a.x, a.v, a.img, a.F, a.site, a.cellc,      \
                                                                     a.inv_perm, a.ref, a.pos, a.flj_next, a.Npad, a.N, \
-                                                                    a.tiles, a.reps, fp, a.kepart, a.done, a.ke_out,   \
-                                                                    a.lam, a.tau, a.flags, gate, mr)
+                                                                    a.tiles, a.reps, fp, a.kepart, a.lam, a.flags,     \
+                                                                    gate, mr)
   // With the weak-coupling thermostat (th = 1), every step that starts (KD,
   // KKD) takes the temperature of the unscaled v(t_k), scales v(t_k) by the
   // factor of the previous step and leaves the factor of step k for the next
@@ -143,6 +140,22 @@ void launch_integrate(bool mixed, IntegMode mode, int thermostat, const StepArgs
   if (a.n_tiles <= 0) return;
   if (mixed) launch_int_t<true>(mode, thermostat, a, fp, gate, mr, st);
   else launch_int_t<false>(mode, thermostat, a, fp, gate, mr, st);
+}
+
+// kinetic energies of the replicas from the tiles' sums (a read-out)
+constexpr int kKineticThreads = 256;
+__global__ void __launch_bounds__(kKineticThreads) k_kinetic(const double* __restrict__ kepart,
+                                                             const RepDev* __restrict__ reps, double half_m0,
+                                                             double* __restrict__ ke_out) {
+  __shared__ double val[kKineticThreads];
+  const RepDev& Q = reps[blockIdx.x];
+  replica_sums<1>(kepart, Q.tile_off, Q.n_tiles, val);
+  if (threadIdx.x == 0) ke_out[blockIdx.x] = half_m0 * val[0];
+}
+
+void launch_kinetic(const double* kepart, const RepDev* reps, int n_reps, const ForceParams& fp, double* ke_out,
+                    cudaStream_t st) {
+  if (n_reps > 0) k_kinetic<<<n_reps, kKineticThreads, 0, st>>>(kepart, reps, 0.5 * fp.mass[0], ke_out);
 }
 
 // ---------------------------------------------------------------- early rebin

@@ -33,9 +33,10 @@
 // accumulator is added to the int64 force (2^-32 kJ/mol/nm) with one
 // integer atomic per component.  Integer sums do not depend on the order in
 // which they are made, so the forces are deterministic.
+#include <algorithm>
 #include <type_traits>
 
-#include "md_kernels.cuh"
+#include "integrate.cuh"
 
 namespace mdg {
 
@@ -165,8 +166,8 @@ __device__ __forceinline__ void cluster_of(const RegTile& T, int q, int& h, int&
 
 // next region of this block: blockIdx.x once (grid schedule), or from the
 // work counter (persistent schedule); shared broadcast
-__device__ __forceinline__ int next_region(bool persistent, int it, int* work, int* sh) {
-  if (!persistent) return it == 0 ? (int)blockIdx.x : -1;
+__device__ __forceinline__ int next_region(bool persistent, int it, int block, int* work, int* sh) {
+  if (!persistent) return it == 0 ? block : -1;
   __syncthreads();
   if (threadIdx.x == 0) *sh = atomicAdd(work, 1);
   __syncthreads();
@@ -174,10 +175,10 @@ __device__ __forceinline__ int next_region(bool persistent, int it, int* work, i
 }
 
 // the last block of a persistent launch resets the counters for the next one
-__device__ __forceinline__ void persistent_done(int* work) {
+__device__ __forceinline__ void persistent_done(int* work, int blocks) {
   if (threadIdx.x == 0) {
     __threadfence();
-    if (atomicAdd(work + 1, 1) == (int)gridDim.x - 1) {
+    if (atomicAdd(work + 1, 1) == blocks - 1) {
       work[0] = 0;
       work[1] = 0;
     }
@@ -897,7 +898,8 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_cl_force(
     const RegionShape* __restrict__ shapes, const RepDev* __restrict__ reps, const unsigned* __restrict__ list,
     const ClusterTask* __restrict__ tasks, const int* __restrict__ task_base, int cap,
     int tile_cap, const ForceParams fp, long long* __restrict__ flj, int Npad, double* __restrict__ epart,
-    unsigned* __restrict__ flags, int persistent, int* __restrict__ work, const StepGate gate) {
+    unsigned* __restrict__ flags, int persistent, int* __restrict__ work, const StepGate gate,
+    const ThermoArgs thermo) {
   constexpr int CPW = 32 / LP;
   extern __shared__ __align__(16) unsigned char smem[];
   float4* sp = reinterpret_cast<float4*>(smem);
@@ -915,8 +917,12 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_cl_force(
   __shared__ float ecl[ENERGY ? kRegionClusterCap : 1][kEnergyVals];
   const int lane = threadIdx.x & 31;
   if (!lj_runs(gate)) return;   // the whole grid leaves together
+  if (!ENERGY && (int)blockIdx.x < thermo.n_blocks) {
+    replica_thermostat(thermo, reps[blockIdx.x], blockIdx.x, reinterpret_cast<double*>(smem));
+    return;
+  }
   for (int it = 0;; ++it) {
-    const int r = next_region(persistent != 0, it, work, &sh_r);
+    const int r = next_region(persistent != 0, it, (int)blockIdx.x - thermo.n_blocks, work, &sh_r);
     if (r < 0 || r >= n_items) break;
     const WorkItem item = items[r];
     const RegionShape& S = shapes[item.shape];
@@ -956,7 +962,7 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_cl_force(
       cell_energy(T, item, fits, ecl, epart);
     }
   }
-  if (persistent) persistent_done(work);
+  if (persistent) persistent_done(work, (int)gridDim.x - thermo.n_blocks);
 }
 
 // ===================================================================== launch
@@ -990,14 +996,16 @@ void launch_cl_force(bool energy, const float4* pos, const int* cell_start, cons
                      const RepDev* reps, const unsigned* list, const ClusterTask* tasks, const int* task_base,
                      int cap, int tile_cap, const ForceParams& fp, long long* flj, int Npad, double* epart, unsigned* flags, int block,
                      int lanes, int persistent_grid, int* work, bool exact, const StepGate& gate,
-                     cudaStream_t st) {
+                     const ThermoArgs& thermo, cudaStream_t st) {
   if (n_items <= 0) return;
-  const int grid = persistent_grid > 0 ? persistent_grid : n_items;
+  const int grid = (persistent_grid > 0 ? persistent_grid : n_items) + thermo.n_blocks;
   const int pers = persistent_grid > 0;
-  const size_t sm = cl_force_smem(tile_cap);
+  // the thermostat blocks use 4 doubles per thread of the tile's memory
+  const size_t sm = std::max(cl_force_smem(tile_cap), thermo.n_blocks ? (size_t)block * 4 * sizeof(double) : 0);
 #define MDG_CLF(E, NT, LP, X)                                                                                      \
   k_cl_force<E, NT, LP, X><<<grid, NT, sm, st>>>(pos, cell_start, cl_start, cells, items, n_items, shapes, reps, \
-                                                 list, tasks, task_base, cap, tile_cap, fp, flj, Npad, epart, flags, pers, work, gate)
+                                                 list, tasks, task_base, cap, tile_cap, fp, flj, Npad, epart, flags, pers, work, gate, \
+                                                 thermo)
 #define MDG_CLF2(NT, LP)                  \
   if (energy) MDG_CLF(true, NT, LP, false); \
   else if (exact) MDG_CLF(false, NT, LP, true); \

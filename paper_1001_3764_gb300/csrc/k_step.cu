@@ -29,8 +29,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : NT == 512 ? 2 : 1) k_step(
                                              const long long* __restrict__ flj, long long* __restrict__ flj_next,
                                              int Npad, int N, const Tile* __restrict__ tiles,
                                              const RepDev* __restrict__ reps, const ForceParams fp,
-                                             double* __restrict__ kepart, unsigned* __restrict__ done,
-                                             double* __restrict__ ke_out, double* __restrict__ lam, double tau,
+                                             double* __restrict__ kepart, const double* __restrict__ lam,
                                              unsigned* __restrict__ flags, const StepGate gate,
                                              const MoveReport mr) {
   using T = typename std::conditional<MIXED, double, float>::type;
@@ -121,8 +120,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : NT == 512 ? 2 : 1) k_step(
       pos[slot] = make_float4(o.loc[0], o.loc[1], o.loc[2], (float)type);   // w: LJ type, as the sort writes it
     }
   }
-  if constexpr (KE)
-    replica_kinetic<TH, NT>(o, t.rep, blockIdx.x, R.ctile_off, R.n_ctiles, reps, fp, kepart, done, ke_out, lam, tau);
+  if constexpr (KE) tile_kinetic<TH, NT>(o, blockIdx.x, kepart);
 }
 
 static size_t step_smem_bytes(int threads) { return (size_t)(threads + 3) * (7 * sizeof(f3) + sizeof(float)); }
@@ -135,8 +133,8 @@ static void launch_step_t(IntegMode mode, int th, int threads, const StepArgs& a
 #define MDG_STEP(MODE, KE, TH)                                                                                       \
   k_step<MIXED, MODE, KE, TH, NT><<<a.n_tiles, threads, step_smem_bytes(threads), st>>>(a.x, a.v, a.img, a.F, a.site, a.cellc, a.inv_perm,  \
                                                                  a.ref, a.pos, a.flj, a.flj_next, a.Npad, a.N,       \
-                                                                 a.tiles, a.reps, fp, a.kepart, a.done, a.ke_out,    \
-                                                                 a.lam, a.tau, a.flags, gate, mr)
+                                                                 a.tiles, a.reps, fp, a.kepart, a.lam, a.flags,      \
+                                                                 gate, mr)
   if (mode == kKickKickDrift) {
     if (th == 2) MDG_STEP(kKickKickDrift, true, 2);
     else if (th == 1) MDG_STEP(kKickKickDrift, true, 1);

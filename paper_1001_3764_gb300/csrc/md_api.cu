@@ -91,7 +91,7 @@ struct md_system {
   double* e_slices = nullptr;   // first-pass energy sums, n_reps * max_slices * 11
   int max_slices = 1;
   double* stage = nullptr;                   // input staging (6N doubles)
-  unsigned *done = nullptr, *flags = nullptr;
+  unsigned* flags = nullptr;
   // end-to-end vector ACF (allocated by md_acf_reset)
   double *acf_ring = nullptr, *acf_acc = nullptr;
   int acf_lag = -1;
@@ -133,6 +133,17 @@ static int fail(md_system* s, int code, const std::string& msg) {
     cudaError_t e_ = (call);                                                                          \
     if (e_ != cudaSuccess) return fail(s, MD_ECUDA, std::string(#call ": ") + cudaGetErrorString(e_)); \
   } while (0)
+
+// constants of the replicas' thermostats (T0, dt, tau, masses)
+static void fill_thermostats(md_system* s) {
+  for (RepDev& q : s->reps_h) {
+    const double m0 = s->params.mass[0], Qm = s->tau * s->tau * q.T0 / (4.0 * M_PI * M_PI);
+    q.t_scale = m0 / (q.dof * kKB);
+    q.vr_num = s->dt / s->tau * q.T0 * q.dof * kKB / m0;
+    q.nh_rate = s->dt / Qm;
+    q.com_scale = m0 / ((double)q.n_chains * s->fp.mol_mass);
+  }
+}
 
 static void fill_force_params(md_system* s) {
   const md_params& p = s->params;
@@ -186,6 +197,7 @@ static void fill_force_params(md_system* s) {
     f.mol_mass = (double)(s->S - 2) * p.mass[0] + 2.0 * p.mass[1];
   }
   f.mtype = s->generic ? s->mtype : nullptr;
+  fill_thermostats(s);
 }
 
 // Region shapes: sx x sy x 1 home cells (sx, sy in {1, 2}; shape id
@@ -546,7 +558,6 @@ static size_t plan(md_system* s, char* base) {
   s->lam = (double*)take((size_t)kNhDoubles * s->n_reps * sizeof(double));   // rescale factor, or the Nose-Hoover state
   s->e_out = (double*)take((size_t)s->n_reps * 16 * sizeof(double));
   s->e_slices = (double*)take((size_t)s->n_reps * s->max_slices * 11 * sizeof(double));
-  s->done = (unsigned*)take(s->n_reps * sizeof(unsigned));
   s->work = (int*)take(2 * sizeof(int));
   s->flags = (unsigned*)take(sizeof(unsigned));
   s->ctl = (int*)take(2 * sizeof(int));
@@ -599,10 +610,12 @@ static void enqueue_rebin(md_system* s) {
 }
 static const int kRebinLaunches = 7;   // memset counted as a launch
 
-static void enqueue_lj(md_system* s, bool energy, long long* flj, const StepGate& gate = StepGate{}) {
+static void enqueue_lj(md_system* s, bool energy, long long* flj, const StepGate& gate = StepGate{},
+                       const ThermoArgs& thermo = ThermoArgs{}) {
   launch_cl_force(energy, s->pos, s->cell_start, s->cl_start, s->region_cells, s->items, s->n_lj_items, s->shapes,
                   s->reps, s->list, s->tasks, s->task_base, s->cap, s->tile_cap, s->fp, flj, s->Npad, s->lj_part,
-                  s->flags, s->lj_block, s->lj_lanes, s->persistent_grid, s->work, s->lj_pair_exact, gate, s->st);
+                  s->flags, s->lj_block, s->lj_lanes, s->persistent_grid, s->work, s->lj_pair_exact, gate,
+                  thermo, s->st);
 }
 
 static void enqueue_bonded(md_system* s, bool energy, const long long* flj, void* F_out) {
@@ -615,10 +628,10 @@ static void enqueue_bonded(md_system* s, bool energy, const long long* flj, void
 }
 
 // the total force into s->F
-static void enqueue_forces(md_system* s, const StepGate& gate = StepGate{}) {
+static void enqueue_forces(md_system* s, const StepGate& gate = StepGate{}, const ThermoArgs& thermo = ThermoArgs{}) {
   cudaMemsetAsync(s->flj[0], 0, 3 * (size_t)s->Npad * sizeof(long long), s->st);
   prof_mark(s);   // closes the integrate group (integrator, early rebin, clear)
-  enqueue_lj(s, false, s->flj[0], gate);
+  enqueue_lj(s, false, s->flj[0], gate, thermo);
   prof_mark(s);
   enqueue_bonded(s, false, s->flj[0], s->F);
   prof_mark(s);
@@ -635,8 +648,7 @@ static void enqueue_energy(md_system* s) {
 static StepArgs step_args(md_system* s, bool chain_tiles, const long long* flj, long long* flj_next) {
   return StepArgs{s->x, s->v, s->img, s->F, s->site, s->cellc, s->inv_perm, s->ref, s->pos, flj, flj_next, s->Npad,
                   (int)s->N, chain_tiles ? s->tiles_chain : s->tiles_int,
-                  (int)(chain_tiles ? s->t_chain.size() : s->t_int.size()), s->reps, s->kepart, s->done, s->ke_out,
-                  s->lam, s->tau, s->flags};
+                  (int)(chain_tiles ? s->t_chain.size() : s->t_int.size()), s->reps, s->kepart, s->lam, s->flags};
 }
 
 // Steps first .. k - 1 of a block of k, LJ launch first on (first = 0: from
@@ -658,12 +670,15 @@ static void enqueue_steps(md_system* s, int k, bool repeat, const MoveReport& mr
                   mr, s->st);
       prof_mark(s);   // closes the bonded group (bonded forces and update)
     }
+    ThermoArgs thermo{};
+    if (s->thermo != MD_NVE)
+      thermo = ThermoArgs{s->n_reps, s->thermo, j > 0 && !s->generic, s->kepart, s->lam, 1.0 - s->dt / s->tau, s->dt};
     if (s->generic) {
-      enqueue_forces(s, gate);
+      enqueue_forces(s, gate, thermo);
       continue;
     }
     prof_mark(s);   // closes the integrate group
-    enqueue_lj(s, false, flj, gate);
+    enqueue_lj(s, false, flj, gate, thermo);
     prof_mark(s);
   }
   const StepGate gate{mr.ctl, k - 1, repeat ? 1 : 0};
@@ -976,7 +991,6 @@ int md_create(const md_desc* d, md_system** out) {
             up(s->tiles_chain, s->t_chain.data(), sizeof(Tile) * s->t_chain.size()) &&
             cudaMemsetAsync(s->flj[0], 0, 3 * (size_t)s->Npad * sizeof(long long), s->st) == cudaSuccess &&
             cudaMemsetAsync(s->flj[1], 0, 3 * (size_t)s->Npad * sizeof(long long), s->st) == cudaSuccess &&
-            cudaMemsetAsync(s->done, 0, s->n_reps * sizeof(unsigned), s->st) == cudaSuccess &&
             cudaMemsetAsync(s->work, 0, 2 * sizeof(int), s->st) == cudaSuccess &&
             cudaMemsetAsync(s->flags, 0, sizeof(unsigned), s->st) == cudaSuccess &&
             up(s->ctl, ctl0, sizeof ctl0) &&
@@ -1051,6 +1065,7 @@ int md_energy(md_system* s, md_energy_t* out) {
   // kinetic energy of the current velocities (a pass that only reads v)
   launch_integrate(s->mixed, kKineticOnly, MD_NVE, step_args(s, false, nullptr, nullptr), s->fp, StepGate{},
                    MoveReport{}, s->st);
+  launch_kinetic(s->kepart, s->reps, s->n_reps, s->fp, s->ke_out, s->st);
   s->profile = p;
   CU(cudaGetLastError());
   std::vector<double> e((size_t)s->n_reps * 16), ke(s->n_reps);
@@ -1128,6 +1143,7 @@ int md_set_temperature(md_system* s, const double* T) {
   if (!s || !T) return fail(s, MD_EINVAL, "bad arguments");
   CU(cudaStreamSynchronize(s->st));
   for (int r = 0; r < s->n_reps; ++r) { s->reps_h[r].T0 = T[r]; s->T0[r] = T[r]; }
+  fill_thermostats(s);
   CU(cudaMemcpy(s->reps, s->reps_h.data(), sizeof(RepDev) * s->n_reps, cudaMemcpyHostToDevice));
   return MD_OK;
 }

@@ -66,6 +66,9 @@ struct RepDev {
   int n_chains, chain_off, tile_off, n_tiles;
   int ctile_off, n_ctiles;      // chain tiles (blocks of the fused step kernel)
   double T0, dof;
+  // thermostats: T = t_scale sum(m v^2 / m_0); weak coupling lam^2 = 1 - dt/tau
+  // + vr_num / sum; Nose-Hoover dxi = nh_rate (T - T0), V_com = com_scale sum(m v / m_0)
+  double t_scale, vr_num, nh_rate, com_scale;
 };
 
 // Nose-Hoover state of a replica, doubles nh[0..11]: xi, fo = 1 - c,
@@ -135,6 +138,17 @@ __device__ __forceinline__ float d2f_rn_int(double d) {
   f = (ha > 0x7ff00000u || (ha == 0x7ff00000u && lo != 0u)) ? 0x7fc00000u : f;            // NaN
   return __uint_as_float(f | sign);
 }
+
+// FP32 -> FP64 on the integer pipe from the binary32 fields: exact for normal
+// numbers, infinities and NaN; magnitudes below 2^-126 give zero.
+__device__ __forceinline__ double f2d_int(float f) {
+  const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
+  unsigned hi = (a >> 3) + (896u << 20), lo = u << 29;
+  if (a >= 0x7f800000u) hi |= 0x7ff00000u;
+  if (a < 0x00800000u) hi = lo = 0u;
+  return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)lo);
+}
+__device__ __forceinline__ double f2d_int(double d) { return d; }
 
 // c + 1/2 as an FP64 number built from its bits (no int -> FP64 conversion):
 // n = 2c + 1 is odd and below 2^12, c + 1/2 = n / 2 = 1.m * 2^(e-1), e = msb(n).
@@ -290,6 +304,15 @@ struct MoveReport {
   unsigned long long* events;
 };
 
+// Thermostat work of the LJ launch after a drift: n_blocks = 0 (none) or one
+// block per replica ahead of the items.
+struct ThermoArgs {
+  int n_blocks, th, chain;      // th: 1 weak coupling, 2 Nose-Hoover; chain: the drift's tiles
+  const double* kepart;
+  double* lam;
+  double one_minus_rate, dt;    // 1 - dt / tau
+};
+
 // ---------------------------------------------------------------- binning
 void launch_bin_count(bool mixed, const void* x, int N, const Tile* tiles, int n_tiles,
                       const RepDev* reps, int* cell_of, int* cellc, int* count, int* slot,
@@ -333,7 +356,8 @@ void launch_cl_force(bool energy, const float4* pos, const int* cell_start, cons
                      const int* cells, const WorkItem* items, int n_items, const RegionShape* shapes,
                      const RepDev* reps, const unsigned* list, const ClusterTask* tasks, const int* task_base,
                      int cap, int tile_cap, const ForceParams& fp, long long* flj, int Npad, double* epart, unsigned* flags, int block, int lanes,
-                     int persistent_grid, int* work, bool exact, const StepGate& gate, cudaStream_t st);
+                     int persistent_grid, int* work, bool exact, const StepGate& gate,
+                     const ThermoArgs& thermo, cudaStream_t st);
 int lj_blocks_per_sm(int block, int lanes, int tile_cap);
 cudaError_t tile_kernels_init();
 int tile_capacity_max();
@@ -368,7 +392,7 @@ void launch_chain_observables(bool mixed, const void* x, int N, const RepDev* re
                               unsigned long long* trans, cudaStream_t st);
 // Arguments common to the integrator and the fused step kernel.  flj: the LJ
 // force of the step; flj_next: the buffer cleared for the next one (may be
-// null in launch_integrate).  done: one zeroed ticket per replica.
+// null in launch_integrate).
 struct StepArgs {
   void *x, *v;
   int* img;
@@ -384,9 +408,7 @@ struct StepArgs {
   int n_tiles;
   const RepDev* reps;
   double* kepart;               // 4 per tile
-  unsigned* done;
-  double *ke_out, *lam;
-  double tau;
+  const double* lam;
   unsigned* flags;
 };
 // thermostat: 0 none, 1 weak coupling, 2 Nose-Hoover; tiles are the
@@ -400,6 +422,9 @@ int step_chains_per_block(int sites);
 cudaError_t step_kernels_init();
 void launch_step(bool mixed, IntegMode mode, int thermostat, int sites, const StepArgs& a, const ForceParams& fp,
                  const StepGate& gate, const MoveReport& mr, cudaStream_t st);
+// kinetic energy of every replica after a launch_integrate(kKineticOnly)
+void launch_kinetic(const double* kepart, const RepDev* reps, int n_reps, const ForceParams& fp, double* ke_out,
+                    cudaStream_t st);
 // first node of the WHILE body: the repeat resumes at ctl[0]; condition off
 void launch_resume(cudaGraphConditionalHandle h, int* ctl, cudaStream_t st);
 // RDF of non-bonded pairs (k_observe.cu): counts[r * n_bins + k] += pairs of
