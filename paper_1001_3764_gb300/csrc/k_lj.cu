@@ -975,6 +975,16 @@ void launch_cl_build(const float4* pos, const int* tag, const int* cell_start, c
                      int* n_tasks, const TopoDev* topo, cudaStream_t st) {
   if (n_items <= 0) return;
   const size_t sm = cl_build_smem(tile_cap);
+  // 32 warps an SM: four blocks of 256 threads, or where four tiles do not fit its shared memory, two of 512
+  if (4 * (sm + 3800 + 1024) > 228 * 1024) {
+    if (topo)
+      k_cl_build<512, true><<<n_items, 512, sm, st>>>(pos, tag, cell_start, cl_start, cells, items, shapes, reps, list,
+                                                      ncl, cap, tile_cap, flags, n_tasks, *topo);
+    else
+      k_cl_build<512, false><<<n_items, 512, sm, st>>>(pos, tag, cell_start, cl_start, cells, items, shapes, reps,
+                                                       list, ncl, cap, tile_cap, flags, n_tasks, TopoDev{});
+    return;
+  }
   if (topo)
     k_cl_build<256, true><<<n_items, 256, sm, st>>>(pos, tag, cell_start, cl_start, cells, items, shapes, reps, list,
                                                     ncl, cap, tile_cap, flags, n_tasks, *topo);
@@ -1012,6 +1022,8 @@ void launch_cl_force(bool energy, const float4* pos, const int* cell_start, cons
   else MDG_CLF(false, NT, LP, false);
   if (block == 128) {
     if (lanes == 8) { MDG_CLF2(128, 8) } else if (lanes == 32) { MDG_CLF2(128, 32) } else { MDG_CLF2(128, 16) }
+  } else if (block == 768) {
+    if (lanes == 8) { MDG_CLF2(768, 8) } else if (lanes == 32) { MDG_CLF2(768, 32) } else { MDG_CLF2(768, 16) }
   } else if (block == 384) {
     if (lanes == 8) { MDG_CLF2(384, 8) } else if (lanes == 32) { MDG_CLF2(384, 32) } else { MDG_CLF2(384, 16) }
   } else {
@@ -1028,6 +1040,8 @@ int lj_blocks_per_sm(int block, int lanes, int tile_cap) {
 #define MDG_OCC(NT, LP) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_cl_force<false, NT, LP>, NT, sm)
   if (block == 128) {
     if (lanes == 8) MDG_OCC(128, 8); else if (lanes == 32) MDG_OCC(128, 32); else MDG_OCC(128, 16);
+  } else if (block == 768) {
+    if (lanes == 8) MDG_OCC(768, 8); else if (lanes == 32) MDG_OCC(768, 32); else MDG_OCC(768, 16);
   } else if (block == 384) {
     if (lanes == 8) MDG_OCC(384, 8); else if (lanes == 32) MDG_OCC(384, 32); else MDG_OCC(384, 16);
   } else {
@@ -1043,19 +1057,28 @@ cudaError_t tile_kernels_init() {
   const int mb = (int)cl_build_smem(kStageCapMax), mf = (int)cl_force_smem(kStageCapMax);
   cudaError_t e = cudaFuncSetAttribute(k_cl_build<256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mb);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_cl_build<256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mb);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_cl_build<512, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mb);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_cl_build<512, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mb);
 #define MDG_ATTR(E, NT, LP)                                                                                   \
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_cl_force<E, NT, LP>, cudaFuncAttributeMaxDynamicSharedMemorySize, mf); \
   if (e == cudaSuccess && !E)                                                                                 \
     e = cudaFuncSetAttribute(k_cl_force<false, NT, LP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mf);
 #define MDG_ATTR3(E, NT) MDG_ATTR(E, NT, 8) MDG_ATTR(E, NT, 16) MDG_ATTR(E, NT, 32)
   MDG_ATTR3(false, 128) MDG_ATTR3(true, 128) MDG_ATTR3(false, 256) MDG_ATTR3(true, 256)
-  MDG_ATTR3(false, 384) MDG_ATTR3(true, 384)
+  MDG_ATTR3(false, 384) MDG_ATTR3(true, 384) MDG_ATTR3(false, 768) MDG_ATTR3(true, 768)
 #undef MDG_ATTR3
 #undef MDG_ATTR
   return e;
 }
 
 int tile_capacity_max() { return kStageCapMax; }
+
+// 227 KB of shared memory an SM and block, 1 KB of it reserved per block; the
+// force form's tables take 9.9 KB
+int lj_tiles_per_sm(int tile_cap) {
+  const int n = (int)((size_t)(228 * 1024) / (cl_force_smem(tile_cap) + 9872 + 1024));
+  return n < 1 ? 1 : n;
+}
 
 // ===================================================================== bounded wait self-test
 // One thread waits on an mbarrier that nothing arrives on, gives up after

@@ -306,9 +306,14 @@ static void plan_regions(md_system* s) {
   }
   constexpr int kWhole = 255;
   s->items_h.clear();
-  const int lj_rows = n_cells <= 2 * kSMs ? 0 : n_rows <= 2 * kSMs ? 1 : kWhole;
+  const int per_sm = lj_tiles_per_sm(s->tile_cap), slots = per_sm * kSMs;
+  const int lj_rows = n_cells <= slots ? 0 : n_rows <= slots ? 1 : kWhole;
+  // default block: 24 warps an SM, as two resident blocks where two tiles fit
+  // the shared memory of an SM, else as one (cells above 1.22 nm: LJ 565 ->
+  // 478 us for 64 replicas at skin 0.12 nm); three of 8 warps for 2 x 2 regions
+  if (!s->lj_block) s->lj_block = G == 2 ? 256 : per_sm >= 2 || lj_rows != kWhole ? 384 : 768;
   for (int q = 0; q < R; ++q)
-    add_items(s, order[q], lj_rows == kWhole && R <= 2 * kSMs && q >= kSMs ? 1 : lj_rows, 1);
+    add_items(s, order[q], lj_rows == kWhole && per_sm >= 2 && R <= slots && q >= kSMs ? 1 : lj_rows, 1);
   s->n_lj_items = (int)s->items_h.size();
   // The list build gives a warp a cluster at a time (7 us alone), 8 warps a
   // block, 4 blocks an SM: 108 -> 12 us at 1,500 sites (cells in 3 parts),
@@ -436,9 +441,7 @@ static int configure(md_system* s, const md_desc* d) {
   s->lj_region = d->lj_region ? d->lj_region : 3;
   if (d->lj_pair_exact != 0 && d->lj_pair_exact != 1) return fail(s, MD_EINVAL, "lj_pair_exact must be 0 or 1");
   s->lj_pair_exact = d->lj_pair_exact == 1;
-  // default block: two resident blocks of 12 warps for the 3 x 3 regions'
-  // larger tiles, three of 8 warps for 2 x 2
-  s->lj_block = d->lj_block ? d->lj_block : (s->lj_region == 3 ? 384 : 256);
+  s->lj_block = d->lj_block;   // 0: set with the regions
   if (d->displacement != MD_DISP_REBUILD && d->displacement != MD_DISP_ERROR)
     return fail(s, MD_EINVAL, "displacement must be MD_DISP_REBUILD or MD_DISP_ERROR");
   s->disp = d->displacement;
@@ -498,6 +501,10 @@ static int configure(md_system* s, const md_desc* d) {
     if (cells >= (1 << 26)) return fail(s, MD_EINVAL, "too many cells");
   }
   s->N = atoms; s->C = (int)cells;
+  // tile capacity (shared memory per block): 1.4x the mean tile of
+  // the densest replica (at least melt density, 33 sites/nm^3) plus 64, in
+  // multiples of 128 atoms; a larger tile is reported as MD_EOVERFLOW
+  s->tile_cap = std::min(tile_capacity_max(), ((int)std::ceil(1.4 * max_tile + 64.0) + 127) / 128 * 128);
   plan_regions(s);
   s->n_cl_max = (atoms + 3 * cells) / 4 + 1;   // sum of ceil(n_c / 4) over the cells
   s->Npad = (int)((atoms + 31) / 32 * 32);
@@ -507,10 +514,6 @@ static int configure(md_system* s, const md_desc* d) {
   s->cap = d->nbr_capacity > 0 ? d->nbr_capacity : (int)std::ceil(2.5 * 0.75 * max_expected + 64.0);
   s->cap = (s->cap + 31) / 32 * 32;
   if (s->cap > 4096) return fail(s, MD_EINVAL, "neighbour capacity above 4096");
-  // tile capacity (shared memory per block): 1.4x the mean tile of
-  // the densest replica (at least melt density, 33 sites/nm^3) plus 64, in
-  // multiples of 128 atoms; a larger tile is reported as MD_EOVERFLOW
-  s->tile_cap = std::min(tile_capacity_max(), ((int)std::ceil(1.4 * max_tile + 64.0) + 127) / 128 * 128);
   fill_force_params(s);
   return MD_OK;
 }

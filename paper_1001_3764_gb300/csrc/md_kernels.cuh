@@ -359,6 +359,7 @@ void launch_cl_force(bool energy, const float4* pos, const int* cell_start, cons
                      int persistent_grid, int* work, bool exact, const StepGate& gate,
                      const ThermoArgs& thermo, cudaStream_t st);
 int lj_blocks_per_sm(int block, int lanes, int tile_cap);
+int lj_tiles_per_sm(int tile_cap);   // force tiles that fit an SM's shared memory together (1 or more)
 cudaError_t tile_kernels_init();
 int tile_capacity_max();
 // one block waits on an mbarrier nothing arrives on, `spins` rounds, then raises kFlagTimeout
