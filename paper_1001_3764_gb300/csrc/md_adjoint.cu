@@ -34,7 +34,7 @@
 #include <type_traits>
 
 #include "../../include/md.h"
-#include "md_kernels.cuh"
+#include "cell_order.cuh"
 
 void md_set_global_error(const char* msg);   // md_api.cu: message for md_last_error(NULL)
 
@@ -229,38 +229,41 @@ constexpr int kFields = 19;
 // wrapped coordinate in [0, L) (FP64), as the cell test takes it
 __device__ __forceinline__ double wrapped(double xv, const AdjDev& P) { return xv - P.L * floor(xv * P.inv_L); }
 
-// cell of every atom and its slot in the cell
+// cell of every atom, counted
 __global__ void __launch_bounds__(256) k_adj_count(const double* __restrict__ x, AdjDev P, int* __restrict__ cell_of,
-                                                   int* __restrict__ count, int* __restrict__ slot) {
+                                                   const OrderBuf b) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= P.N) return;
-  const int c = (cell_coord(x[3 * i + 2], P) * P.M + cell_coord(x[3 * i + 1], P)) * P.M + cell_coord(x[3 * i], P);
-  cell_of[i] = c;
-  slot[i] = atomicAdd(count + c, 1);
+  int c = 0;
+  if (i < P.N)
+    c = (cell_coord(x[3 * i + 2], P) * P.M + cell_coord(x[3 * i + 1], P)) * P.M + cell_coord(x[3 * i], P);
+  if (i < P.N) cell_of[i] = c;
+  order_count(i < P.N, c, blockIdx.x * 256, b);
 }
 
-// Atoms in cell order for the pair kernel: wrapped positions (FP64), the FP32
-// copy with the atom's index in w (bit 31: chain end, C_33), and for a
-// tangent evaluation u = cu M^-1 beta.  One pass of coalesced writes here
-// turns the pair loop's two dependent gathers per candidate (perm, then the
-// position) into one contiguous read.
-__global__ void __launch_bounds__(256) k_adj_sorted(const double* __restrict__ x, const double* __restrict__ beta,
-                                                    double cu, const int* __restrict__ perm, AdjDev P,
-                                                    double* __restrict__ xs, double* __restrict__ us,
-                                                    float4* __restrict__ s32) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= P.N) return;
-  const int i = perm[s], ty = site_type(i % P.sites, P.sites);
-  float f[3];
+// Atoms in cell order for the pair kernel, written by the last pass of the
+// ordering: wrapped positions (FP64), the FP32 copy with the atom's index in w
+// (bit 31: chain end, C_33), and for a tangent evaluation u = cu M^-1 beta.  The
+// pair loop's two dependent gathers per candidate (perm, then the position)
+// become one contiguous read.
+struct EmitSorted {
+  const double *x, *beta;
+  double cu;
+  AdjDev P;
+  double *xs, *us;
+  float4* s32;
+  __device__ __forceinline__ void operator()(int s, int i) const {
+    const int ty = site_type(i % P.sites, P.sites);
+    float f[3];
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const double w = wrapped(x[3 * i + a], P);
-    xs[(size_t)a * P.N + s] = w;
-    f[a] = (float)w;
-    if (beta) us[(size_t)a * P.N + s] = cu * P.inv_mass[ty] * beta[3 * i + a];
+    for (int a = 0; a < 3; ++a) {
+      const double w = wrapped(x[3 * i + a], P);
+      xs[(size_t)a * P.N + s] = w;
+      f[a] = (float)w;
+      if (beta) us[(size_t)a * P.N + s] = cu * P.inv_mass[ty] * beta[3 * i + a];
+    }
+    s32[s] = make_float4(f[0], f[1], f[2], __uint_as_float((unsigned)i | ((unsigned)ty << 31)));
   }
-  s32[s] = make_float4(f[0], f[1], f[2], __uint_as_float((unsigned)i | ((unsigned)ty << 31)));
-}
+};
 
 // ------------------------------------------------------------------ LJ, Eq. (2): one warp per atom
 // Bound: the FP64 pipe (about 2 operations per clock and SM).  A warp scans
@@ -666,6 +669,8 @@ __global__ void __launch_bounds__(3 * kBondTerms) k_adj_bonded(const double* __r
 // one thread per field: 18.4 + 5.0 -> 7.4 us (5.8 for the five fields of a forward step) at 7,500 sites.
 constexpr int kRedBlocks = 128, kRedThreads = 320;
 
+constexpr int kOrderPad = 16;   // ints ahead of the ordering's counters (the first is the reduction's ticket)
+
 // accumulator layout
 constexpr int kAccU = 0, kAccR2 = 1;      // forward sums of U_k and R_ee^2_k
 constexpr int kAccC12 = 2, kAccC6 = 5;    // dJ/dc12_t, dJ/dc6_t (t = 0, 1, 2)
@@ -829,7 +834,7 @@ struct md_adj {
   void* mem;
   double *x, *v, *gv, *gt, *alpha, *beta, *rec, *part, *acc, *totals, *ckx, *ckv, *seg, *xk, *xs, *us;
   float4* x32;                 // cell order: FP32 wrapped position, atom index and type
-  int *count, *cell_start, *cell_of, *slot, *tmp, *perm, *rbuf, *maxm;
+  int *count, *cell_start, *cell_of, *tmp, *perm, *seg_scan, *ticket;
   bool have_forward;
   double obs[2];
 };
@@ -860,13 +865,13 @@ int evaluate(md_adj* a, const double* xp, const double* beta, double cu, int mod
   const AdjDev& P = a->P;
   cudaStream_t st = a->st;
   const int N = P.N;
-  if (cudaMemsetAsync(a->count, 0, sizeof(int) * a->C_cells, st) != cudaSuccess) return MD_ECUDA;
-  k_adj_count<<<(N + 255) / 256, 256, 0, st>>>(xp, P, a->cell_of, a->count, a->slot);
-  launch_scan(a->count, a->cell_start, a->C_cells, st);
-  launch_bin_scatter(a->cell_of, a->slot, a->cell_start, a->tmp, N, st);
-  if (cudaMemsetAsync(a->maxm, 0, 2 * sizeof(int), st) != cudaSuccess) return MD_ECUDA;   // and the reduction's ticket
-  launch_static_order(a->cell_start, a->C_cells, N, a->tmp, a->rbuf, a->slot, a->perm, a->maxm, st);
-  k_adj_sorted<<<(N + 255) / 256, 256, 0, st>>>(xp, beta, cu, a->perm, P, a->xs, a->us, a->x32);
+  const OrderBuf ob = order_buffers(a->count, N, a->C_cells);
+  // the reduction's ticket and the ordering's counters in one run
+  if (cudaMemsetAsync(a->ticket, 0, sizeof(int) * (kOrderPad + order_clear_ints(ob, a->C_cells)), st) != cudaSuccess)
+    return MD_ECUDA;
+  k_adj_count<<<(N + 255) / 256, 256, 0, st>>>(xp, P, a->cell_of, ob);
+  launch_cell_order(a->cell_of, N, a->C_cells, ob, a->cell_start, a->seg_scan, a->tmp, a->perm,
+                    EmitSorted{xp, beta, cu, P, a->xs, a->us, a->x32}, st);
   const int lj_blocks = (N + kLjWarps - 1) / kLjWarps, b_blocks = (N + kBondTile - 1) / kBondTile;
   if (beta && a->hvp32) {
     k_adj_lj<float, true><<<lj_blocks, 32 * kLjWarps, 0, st>>>(a->xs, a->us, a->x32, a->cell_start, a->cell_of, P, 1,
@@ -886,11 +891,11 @@ int evaluate(md_adj* a, const double* xp, const double* beta, double cu, int mod
   const int nb = N < kRedBlocks ? 1 : kRedBlocks;
   // without a tangent only the energies and R_ee^2 are asked for
   if (beta)
-    k_adj_reduce<0, kFields><<<nb, kRedThreads, 0, st>>>(a->rec, N, P.n_chains, mode, wu, a->part, a->maxm + 1,
+    k_adj_reduce<0, kFields><<<nb, kRedThreads, 0, st>>>(a->rec, N, P.n_chains, mode, wu, a->part, a->ticket,
                                                          a->totals, a->acc);
   else
     k_adj_reduce<kElj, kFields - kElj><<<nb, kRedThreads, 0, st>>>(a->rec, N, P.n_chains, mode, wu, a->part,
-                                                                   a->maxm + 1, a->totals, a->acc);
+                                                                   a->ticket, a->totals, a->acc);
   return cudaPeekAtLastError() == cudaSuccess ? MD_OK : MD_ECUDA;
 }
 
@@ -1012,10 +1017,10 @@ extern "C" int md_adj_create(const md_adj_desc* d, md_adj** out) {
   const size_t n3 = sizeof(double) * 3 * (size_t)N;
   const size_t sizes[] = {n3, n3, n3, n3, n3, n3, sizeof(double) * kRec * (size_t)N,
                           sizeof(double) * kRec * kRedBlocks, sizeof(double) * kAccN, sizeof(double) * kRec,
-                          n3 * a->S, n3 * a->S, n3 * (size_t)(a->C + 1), sizeof(int) * a->C_cells,
-                          sizeof(int) * (a->C_cells + 1), sizeof(int) * (size_t)N, sizeof(int) * (size_t)N,
-                          sizeof(int) * (size_t)N, sizeof(int) * (size_t)N, n3, sizeof(float4) * (size_t)N,
-                          sizeof(int) * (size_t)N, 2 * sizeof(int), n3, n3};
+                          n3 * a->S, n3 * a->S, n3 * (size_t)(a->C + 1), sizeof(int) * (kOrderPad + order_ints((int)N, a->C_cells)),
+                          sizeof(int) * (a->C_cells + 1), sizeof(int) * (size_t)N,
+                          sizeof(int) * scan_seg_ints(a->C_cells), sizeof(int) * (size_t)N, sizeof(int) * (size_t)N, n3,
+                          sizeof(float4) * (size_t)N, n3, n3};
   const int nbuf = sizeof(sizes) / sizeof(sizes[0]);
   size_t total = 0;
   for (int k = 0; k < nbuf; ++k) total += align256(sizes[k]);
@@ -1031,12 +1036,11 @@ extern "C" int md_adj_create(const md_adj_desc* d, md_adj** out) {
   a->x = (double*)ptrs[0]; a->v = (double*)ptrs[1]; a->gv = (double*)ptrs[2]; a->gt = (double*)ptrs[3];
   a->alpha = (double*)ptrs[4]; a->beta = (double*)ptrs[5]; a->rec = (double*)ptrs[6]; a->part = (double*)ptrs[7];
   a->acc = (double*)ptrs[8]; a->totals = (double*)ptrs[9]; a->ckx = (double*)ptrs[10]; a->ckv = (double*)ptrs[11];
-  a->seg = (double*)ptrs[12]; a->count = (int*)ptrs[13]; a->cell_start = (int*)ptrs[14];
-  a->cell_of = (int*)ptrs[15]; a->slot = (int*)ptrs[16]; a->tmp = (int*)ptrs[17]; a->perm = (int*)ptrs[18];
+  a->seg = (double*)ptrs[12]; a->ticket = (int*)ptrs[13]; a->count = a->ticket + kOrderPad; a->cell_start = (int*)ptrs[14];
+  a->cell_of = (int*)ptrs[15]; a->seg_scan = (int*)ptrs[16]; a->tmp = (int*)ptrs[17]; a->perm = (int*)ptrs[18];
   a->xk = (double*)ptrs[19];
   a->x32 = (float4*)ptrs[20];
-  a->rbuf = (int*)ptrs[21]; a->maxm = (int*)ptrs[22];
-  a->xs = (double*)ptrs[23]; a->us = (double*)ptrs[24];
+  a->xs = (double*)ptrs[21]; a->us = (double*)ptrs[22];
   a->have_forward = false;
   *out = a;
   return MD_OK;

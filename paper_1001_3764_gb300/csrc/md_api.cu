@@ -84,7 +84,7 @@ struct md_system {
   int lj_region = 3;                         // cells per side (x, y) of an LJ / list region
   bool lj_pair_exact = false;                // each LJ pair force converted once, +q to i and -q to j
   int* work = nullptr;                       // LJ work counters (persistent schedule)
-  int *count = nullptr, *cell_start = nullptr, *cell_of = nullptr;
+  int *count = nullptr, *cell_start = nullptr, *cell_of = nullptr, *scan_seg = nullptr;
   int *slot = nullptr, *tmp = nullptr;
   double *lj_part = nullptr, *b_part = nullptr, *kepart = nullptr, *ke_out = nullptr, *lam = nullptr;
   double* e_out = nullptr;
@@ -549,6 +549,7 @@ static size_t plan(md_system* s, char* base) {
   s->ncl = (int*)take((size_t)s->n_cl_max * sizeof(int));
   s->cl_start = (int*)take((C + 1) * sizeof(int));
   s->count = (int*)take(C * sizeof(int));
+  s->scan_seg = (int*)take(scan_seg_ints(s->C) * sizeof(int));
   s->cell_start = (int*)take((C + 1) * sizeof(int));
   s->cell_of = (int*)take(N * sizeof(int));
   s->slot = (int*)take(N * sizeof(int));
@@ -603,7 +604,7 @@ static void enqueue_rebin(md_system* s) {
   cudaMemsetAsync(s->count, 0, sizeof(int) * s->C, s->st);
   launch_bin_count(s->mixed, s->x, (int)s->N, s->tiles_int, (int)s->t_int.size(), s->reps, s->cell_of, s->cellc,
                    s->count, s->slot, s->st);
-  launch_scan2(s->count, s->cell_start, s->cl_start, s->C, s->st);
+  launch_scan2(s->count, s->cell_start, s->cl_start, s->C, s->scan_seg, s->st);
   launch_bin_scatter(s->cell_of, s->slot, s->cell_start, s->tmp, (int)s->N, s->st);
   launch_cell_sort(s->mixed, s->x, (int)s->N, s->cell_start, s->tmp, s->fp.mtype, s->cellc, s->site, s->reps, s->n_reps, s->C,
                    s->S, s->perm, s->inv_perm, s->pos, s->tag, s->ref, s->flags, s->st);
@@ -1331,7 +1332,7 @@ int md_bin_study(md_system* s, int32_t reps, double* ms) {
     cudaMemsetAsync(s->count, 0, sizeof(int) * C, s->st);
     launch_bin_count(s->mixed, s->x, (int)N, s->tiles_int, (int)s->t_int.size(), s->reps, s->cell_of, s->cellc,
                      s->count, s->slot, s->st);
-    launch_scan2(s->count, s->cell_start, s->cl_start, s->C, s->st);
+    launch_scan2(s->count, s->cell_start, s->cl_start, s->C, s->scan_seg, s->st);
     launch_bin_scatter(s->cell_of, s->slot, s->cell_start, s->tmp, (int)N, s->st);
     launch_cell_sort(s->mixed, s->x, (int)N, s->cell_start, s->tmp, s->fp.mtype, s->cellc, s->site, s->reps, s->n_reps, s->C,
                      s->S, s->perm, s->inv_perm, s->pos, s->tag, s->ref, s->flags, s->st);

@@ -150,6 +150,17 @@ __device__ __forceinline__ double f2d_int(float f) {
 }
 __device__ __forceinline__ double f2d_int(double d) { return d; }
 
+// floor(s) clamped to a cell index 0 .. M - 1 (M <= 2^20), on the integer pipe:
+// below 2^20 the integer part of a double lies in its high word.  Negative
+// numbers and NaN give 0.
+__device__ __forceinline__ int cell_floor(double s, int M) {
+  const int hi = __double2hiint(s);
+  const int e = (hi >> 20) - 1023;                                     // s >= 0: the exponent
+  int k = e < 0 ? 0 : e >= 20 ? M - 1 : ((hi & 0xfffff) | 0x100000) >> (20 - e);
+  if (!(s >= 0.0)) k = 0;
+  return k > M - 1 ? M - 1 : k;
+}
+
 // c + 1/2 as an FP64 number built from its bits (no int -> FP64 conversion):
 // n = 2c + 1 is odd and below 2^12, c + 1/2 = n / 2 = 1.m * 2^(e-1), e = msb(n).
 __device__ __forceinline__ double half_plus(int c) {
@@ -317,15 +328,15 @@ struct ThermoArgs {
 void launch_bin_count(bool mixed, const void* x, int N, const Tile* tiles, int n_tiles,
                       const RepDev* reps, int* cell_of, int* cellc, int* count, int* slot,
                       cudaStream_t st);
-void launch_scan(const int* count, int* cell_start, int C, cudaStream_t st);
-// cell_start from count, and cl_start from ceil(count / 4) (clusters per cell)
-void launch_scan2(const int* count, int* cell_start, int* cl_start, int C, cudaStream_t st);
-// stable order by atom index inside each of C cells (n atoms in all):
-// perm[cell_start[c] + rank] = atom, from the unsorted bucket contents in
-// `runs` (overwritten), in O(m log m) work for a cell of m atoms.  Scratch:
-// buf[n], pcell[n] and one int *maxm that the caller clears before the call.
-void launch_static_order(const int* cell_start, int C, int n, int* runs, int* buf, int* pcell, int* perm, int* maxm,
-                         cudaStream_t st);
+// exclusive scan of C counts (count 16-byte aligned) into cell_start[C + 1];
+// launch_scan2 also scans ceil(count / 4), the clusters per cell, into
+// cl_start.  seg: scan_seg_ints(C) ints of scratch (none for C <= 131,072).
+// tot (or null): launch_scan also sums the digit counts hist[n_tiles][2^bits]
+// over the tiles (cell_order.cuh)
+size_t scan_seg_ints(long long C);
+void launch_scan(const int* count, int* cell_start, int C, int* seg, const int* hist, int n_tiles, int bits,
+                 int* tot, cudaStream_t st);
+void launch_scan2(const int* count, int* cell_start, int* cl_start, int C, int* seg, cudaStream_t st);
 void launch_bin_scatter(const int* cell_of, const int* slot, const int* cell_start, int* tmp, int N,
                         cudaStream_t st);
 void launch_cell_sort(bool mixed, const void* x, int N, const int* cell_start, const int* tmp, const unsigned char* mtype,
