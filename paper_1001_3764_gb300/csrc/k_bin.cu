@@ -123,6 +123,7 @@ __global__ void __launch_bounds__(1024) k_scan_segments(const int* __restrict__ 
                                                         int segs, const int* __restrict__ hist, int n_tiles,
                                                         int bits, int* __restrict__ tot) {
   __shared__ int2 sh[32];
+  wait_for_predecessor();
   if ((int)blockIdx.x >= segs) {   // blocks past the segments: 32 digit totals each (cell_order.cuh)
     digit_totals(blockIdx.x - segs, bits, hist, n_tiles, tot);
     return;
@@ -179,33 +180,34 @@ size_t scan_seg_ints(long long C) { return C <= kScanDirect ? 0 : 2 * (size_t)((
 
 template <bool CL>
 static void launch_scan_t(const int* count, int* start, int* cl_start, int C, int* seg, const int* hist, int n_tiles,
-                          int bits, int* tot, cudaStream_t st) {
+                          int bits, int* tot, bool dep, cudaStream_t st) {
   const int segs = (C + kScanSeg - 1) / kScanSeg;
   int2* sg = C <= kScanDirect ? nullptr : reinterpret_cast<int2*>(seg);
   if (sg) k_scan_sums<CL><<<segs, 1024, 0, st>>>(count, C, sg);
-  k_scan_segments<CL><<<segs + (tot ? (1 << bits) / 32 : 0), 1024, 0, st>>>(count, start, cl_start, C, sg, segs,
-                                                                            hist, n_tiles, bits, tot);
+  launch_dependent(dep, k_scan_segments<CL>, segs + (tot ? (1 << bits) / 32 : 0), 1024, 0, st, count, start, cl_start, C,
+                   sg, segs, hist, n_tiles, bits, tot);
 }
 
 void launch_scan(const int* count, int* cell_start, int C, int* seg, const int* hist, int n_tiles, int bits,
-                 int* tot, cudaStream_t st) {
-  launch_scan_t<false>(count, cell_start, nullptr, C, seg, hist, n_tiles, bits, tot, st);
+                 int* tot, bool dep, cudaStream_t st) {
+  launch_scan_t<false>(count, cell_start, nullptr, C, seg, hist, n_tiles, bits, tot, dep, st);
 }
 
-void launch_scan2(const int* count, int* cell_start, int* cl_start, int C, int* seg, cudaStream_t st) {
-  launch_scan_t<true>(count, cell_start, cl_start, C, seg, nullptr, 0, 0, nullptr, st);
+void launch_scan2(const int* count, int* cell_start, int* cl_start, int C, int* seg, bool dep, cudaStream_t st) {
+  launch_scan_t<true>(count, cell_start, cl_start, C, seg, nullptr, 0, 0, nullptr, dep, st);
 }
 
 // --------------------------------------------------------------- scatter
 __global__ void __launch_bounds__(256) k_bin_scatter(const int* __restrict__ cell_of, const int* __restrict__ slot,
                                                      const int* __restrict__ cell_start, int* __restrict__ tmp, int N) {
+  wait_for_predecessor();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < N) tmp[cell_start[cell_of[i]] + slot[i]] = i;
 }
 
-void launch_bin_scatter(const int* cell_of, const int* slot, const int* cell_start, int* tmp, int N,
+void launch_bin_scatter(const int* cell_of, const int* slot, const int* cell_start, int* tmp, int N, bool dep,
                         cudaStream_t st) {
-  if (N > 0) k_bin_scatter<<<(N + 255) / 256, 256, 0, st>>>(cell_of, slot, cell_start, tmp, N);
+  if (N > 0) launch_dependent(dep, k_bin_scatter, (N + 255) / 256, 256, 0, st, cell_of, slot, cell_start, tmp, N);
 }
 
 // --------------------------------------------------------------- per-cell stable order + sorted arrays
@@ -221,6 +223,7 @@ __global__ void __launch_bounds__(128) k_cell_sort(const T* __restrict__ x, int 
                                                    int* __restrict__ tag, float4* __restrict__ ref,
                                                    unsigned* __restrict__ flags) {
   __shared__ int ids[kSortCap];
+  wait_for_predecessor();
   const int c = blockIdx.x;
   const int b = cell_start[c], n = cell_start[c + 1] - b;
   if (n == 0) return;
@@ -267,12 +270,13 @@ __global__ void __launch_bounds__(128) k_cell_sort(const T* __restrict__ x, int 
 void launch_cell_sort(bool mixed, const void* x, int N, const int* cell_start, const int* tmp,
                       const unsigned char* mtype, const int* cellc,
                       const uint16_t* site, const RepDev* reps, int n_reps, int C, int sites, int* perm,
-                      int* inv_perm, float4* pos, int* tag, float4* ref, unsigned* flags, cudaStream_t st) {
+                      int* inv_perm, float4* pos, int* tag, float4* ref, unsigned* flags, bool dep,
+                      cudaStream_t st) {
   if (mixed)
-    k_cell_sort<double><<<C, 128, 0, st>>>((const double*)x, N, cell_start, tmp, mtype, cellc, site, reps, n_reps, sites,
+    launch_dependent(dep, k_cell_sort<double>, C, 128, 0, st, (const double*)x, N, cell_start, tmp, mtype, cellc, site, reps, n_reps, sites,
                                            perm, inv_perm, pos, tag, ref, flags);
   else
-    k_cell_sort<float><<<C, 128, 0, st>>>((const float*)x, N, cell_start, tmp, mtype, cellc, site, reps, n_reps, sites,
+    launch_dependent(dep, k_cell_sort<float>, C, 128, 0, st, (const float*)x, N, cell_start, tmp, mtype, cellc, site, reps, n_reps, sites,
                                           perm, inv_perm, pos, tag, ref, flags);
 }
 

@@ -56,6 +56,7 @@ __global__ void __launch_bounds__(kIntBlock) k_integrate(void* __restrict__ xv, 
   using T = typename std::conditional<MIXED, double, float>::type;
   T* x = reinterpret_cast<T*>(xv);
   T* v = reinterpret_cast<T*>(vv);
+  wait_for_predecessor();
   const Tile t = tiles[blockIdx.x];
   const RepDev& R = reps[t.rep];
   const int i = t.start + threadIdx.x;
@@ -106,11 +107,10 @@ __global__ void __launch_bounds__(kIntBlock) k_integrate(void* __restrict__ xv, 
 template <bool MIXED>
 static void launch_int_t(IntegMode mode, int th, const StepArgs& a, const ForceParams& fp,
                          const StepGate& gate, const MoveReport& mr, cudaStream_t st) {
-#define MDG_INT(MODE, KE, TH)                                                                                   \
-  k_integrate<MIXED, MODE, KE, TH><<<a.n_tiles, kIntBlock, 0, st>>>(a.x, a.v, a.img, a.F, a.site, a.cellc,      \
-                                                                    a.inv_perm, a.ref, a.pos, a.flj_next, a.Npad, a.N, \
-                                                                    a.tiles, a.reps, fp, a.kepart, a.lam, a.flags,     \
-                                                                    gate, mr)
+#define MDG_INT(MODE, KE, TH)                                                                                        \
+  launch_dependent(gate.dep, k_integrate<MIXED, MODE, KE, TH>, a.n_tiles, kIntBlock, 0, st, a.x, a.v, a.img, a.F, a.site,      \
+                   a.cellc, a.inv_perm, a.ref, a.pos, a.flj_next, a.Npad, a.N, a.tiles, a.reps, fp, a.kepart, a.lam, \
+                   a.flags, gate, mr)
   // With the weak-coupling thermostat (th = 1), every step that starts (KD,
   // KKD) takes the temperature of the unscaled v(t_k), scales v(t_k) by the
   // factor of the previous step and leaves the factor of step k for the next

@@ -245,6 +245,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_cl_build(const float4* __rest
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int* qw = queue[warp];
   {
+    wait_for_predecessor();
     const WorkItem item = items[blockIdx.x];
     const RegionShape& S = shapes[item.shape];
     const RepDev& R = reps[item.rep];
@@ -851,6 +852,7 @@ __global__ void __launch_bounds__(kRankThreads) k_cl_rank(const float4* __restri
   __shared__ RegTile T;
   __shared__ __align__(16) int s_key[kRegionClusterCap];
   __shared__ int base;
+  wait_for_predecessor();
   const WorkItem item = items[blockIdx.x];
   region_setup(T, item, shapes[item.shape], cells, cell_start, cl_start);
   const int q_first = T.ncl[item.h0], nq = T.ncl[item.h1] - q_first;
@@ -916,10 +918,13 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_cl_force(
   // which warp took which cluster
   __shared__ float ecl[ENERGY ? kRegionClusterCap : 1][kEnergyVals];
   const int lane = threadIdx.x & 31;
-  if (!lj_runs(gate)) return;   // the whole grid leaves together
-  if (!ENERGY && (int)blockIdx.x < thermo.n_blocks) {
-    replica_thermostat(thermo, reps[blockIdx.x], blockIdx.x, reinterpret_cast<double*>(smem));
-    return;
+  if ((!ENERGY && (int)blockIdx.x < thermo.n_blocks) || persistent) {
+    wait_for_predecessor();
+    if (!lj_runs(gate)) return;   // the whole grid leaves together
+    if (!ENERGY && (int)blockIdx.x < thermo.n_blocks) {
+      replica_thermostat(thermo, reps[blockIdx.x], blockIdx.x, reinterpret_cast<double*>(smem));
+      return;
+    }
   }
   for (int it = 0;; ++it) {
     const int r = next_region(persistent != 0, it, (int)blockIdx.x - thermo.n_blocks, work, &sh_r);
@@ -933,18 +938,28 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_cl_force(
     const int total = T.off[T.n_tile];
     const int q_first = T.ncl[item.h0], nq = T.ncl[item.h1] - q_first;   // the item's clusters
     const bool fits = total <= tile_cap && T.ncl[T.n_home] <= kRegionClusterCap;
-    if (!fits) {
-      if (threadIdx.x == 0) atomicOr(flags, kFlagNbrOverflow);
-    } else {
-      // the item's tasks and zeroed accumulators while the tile copies fly
+    // the item's tasks and zeroed accumulators: like the tables above the work
+    // of the last rebin, not of the predecessor
+    if (fits) {
       for (int q = threadIdx.x; q < nq; q += NT)
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(s_tab + q)),
                      "l"(tasks + t_base + q)
                      : "memory");
-      tile_issue<NT>(T, item.need, pos, sp);
       if (!ENERGY)   // 3 tile_cap is a multiple of 4: the rounded-up span stays in the buffer
         for (int t = threadIdx.x; t < (3 * total + 3) / 4; t += NT) reinterpret_cast<int4*>(ax)[t] = make_int4(0, 0, 0, 0);
       if (threadIdx.x == 0) sh_q = 0;
+    }
+    if (!persistent) {
+      wait_for_predecessor();
+      if (!lj_runs(gate)) {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        return;
+      }
+    }
+    if (!fits) {
+      if (threadIdx.x == 0) atomicOr(flags, kFlagNbrOverflow);
+    } else {
+      tile_issue<NT>(T, item.need, pos, sp);
       tile_finish<false, NT>(T, item.need, sp, nullptr);   // ends with a barrier
       const LjConst c = lj_const(R);
       for (;;) {
@@ -972,32 +987,32 @@ size_t cl_force_smem(int tile_cap) { return (size_t)tile_cap * (sizeof(float4) +
 void launch_cl_build(const float4* pos, const int* tag, const int* cell_start, const int* cl_start,
                      const int* cells, const WorkItem* items, int n_items, const RegionShape* shapes,
                      const RepDev* reps, unsigned* list, int* ncl, int cap, int tile_cap, unsigned* flags,
-                     int* n_tasks, const TopoDev* topo, cudaStream_t st) {
+                     int* n_tasks, const TopoDev* topo, bool dep, cudaStream_t st) {
   if (n_items <= 0) return;
   const size_t sm = cl_build_smem(tile_cap);
   // 32 warps an SM: four blocks of 256 threads, or where four tiles do not fit its shared memory, two of 512
   if (4 * (sm + 3800 + 1024) > 228 * 1024) {
     if (topo)
-      k_cl_build<512, true><<<n_items, 512, sm, st>>>(pos, tag, cell_start, cl_start, cells, items, shapes, reps, list,
-                                                      ncl, cap, tile_cap, flags, n_tasks, *topo);
+      launch_dependent(dep, k_cl_build<512, true>, n_items, 512, sm, st, pos, tag, cell_start, cl_start, cells, items, shapes, reps, list,
+                       ncl, cap, tile_cap, flags, n_tasks, *topo);
     else
-      k_cl_build<512, false><<<n_items, 512, sm, st>>>(pos, tag, cell_start, cl_start, cells, items, shapes, reps,
-                                                       list, ncl, cap, tile_cap, flags, n_tasks, TopoDev{});
+      launch_dependent(dep, k_cl_build<512, false>, n_items, 512, sm, st, pos, tag, cell_start, cl_start, cells, items, shapes, reps,
+                       list, ncl, cap, tile_cap, flags, n_tasks, TopoDev{});
     return;
   }
   if (topo)
-    k_cl_build<256, true><<<n_items, 256, sm, st>>>(pos, tag, cell_start, cl_start, cells, items, shapes, reps, list,
-                                                    ncl, cap, tile_cap, flags, n_tasks, *topo);
+    launch_dependent(dep, k_cl_build<256, true>, n_items, 256, sm, st, pos, tag, cell_start, cl_start, cells, items, shapes, reps, list,
+                       ncl, cap, tile_cap, flags, n_tasks, *topo);
   else
-    k_cl_build<256, false><<<n_items, 256, sm, st>>>(pos, tag, cell_start, cl_start, cells, items, shapes, reps,
-                                                     list, ncl, cap, tile_cap, flags, n_tasks, TopoDev{});
+    launch_dependent(dep, k_cl_build<256, false>, n_items, 256, sm, st, pos, tag, cell_start, cl_start, cells, items, shapes, reps,
+                       list, ncl, cap, tile_cap, flags, n_tasks, TopoDev{});
 }
 
 void launch_cl_rank(const float4* pos, const int* cell_start, const int* cl_start, const int* cells,
                     const WorkItem* items, int n_items, const RegionShape* shapes, const int* ncl, ClusterTask* tasks,
-                    int* task_base, int* n_tasks, cudaStream_t st) {
+                    int* task_base, int* n_tasks, bool dep, cudaStream_t st) {
   if (n_items > 0)
-    k_cl_rank<<<n_items, kRankThreads, 0, st>>>(pos, cell_start, cl_start, cells, items, shapes, ncl, tasks,
+    launch_dependent(dep, k_cl_rank, n_items, kRankThreads, 0, st, pos, cell_start, cl_start, cells, items, shapes, ncl, tasks,
                                                  task_base, n_tasks);
 }
 
@@ -1012,10 +1027,10 @@ void launch_cl_force(bool energy, const float4* pos, const int* cell_start, cons
   const int pers = persistent_grid > 0;
   // the thermostat blocks use 4 doubles per thread of the tile's memory
   const size_t sm = std::max(cl_force_smem(tile_cap), thermo.n_blocks ? (size_t)block * 4 * sizeof(double) : 0);
-#define MDG_CLF(E, NT, LP, X)                                                                                      \
-  k_cl_force<E, NT, LP, X><<<grid, NT, sm, st>>>(pos, cell_start, cl_start, cells, items, n_items, shapes, reps, \
-                                                 list, tasks, task_base, cap, tile_cap, fp, flj, Npad, epart, flags, pers, work, gate, \
-                                                 thermo)
+#define MDG_CLF(E, NT, LP, X)                                                                                        \
+  launch_dependent(gate.dep, k_cl_force<E, NT, LP, X>, grid, NT, sm, st, pos, cell_start, cl_start, cells, items,    \
+                   n_items, shapes, reps, list, tasks, task_base, cap, tile_cap, fp, flj, Npad, epart, flags, pers,  \
+                   work, gate, thermo)
 #define MDG_CLF2(NT, LP)                  \
   if (energy) MDG_CLF(true, NT, LP, false); \
   else if (exact) MDG_CLF(false, NT, LP, true); \

@@ -46,7 +46,6 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : NT == 512 ? 2 : 1) k_step(
   const RepDev& R = reps[t.rep];
   const int tid = threadIdx.x, i = t.start + tid, S = fp.sites;
   const bool on = tid < t.len;
-  const bool runs = MODE == kKickOnly ? lj_runs(gate) : drift_runs(gate);   // used before the first write
   int sm = 0, slot = 0;
   T xi[3];
   if (on) {
@@ -74,8 +73,11 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : NT == 512 ? 2 : 1) k_step(
     fbd[tid + 3] = fb; fan_a[tid + 3] = fa; fan_c[tid + 3] = fc;
     fdi1[tid + 3] = f1; fdi2[tid + 3] = f2; fdi3[tid + 3] = f3v;
   }
+  // all before this line reads what the update before the LJ launch left: it
+  // runs while the last LJ blocks finish
+  wait_for_predecessor();
   __syncthreads();
-  if (!runs) return;
+  if (MODE == kKickOnly ? !lj_runs(gate) : !drift_runs(gate)) return;
   AtomOut o;
   o.ke = 0.0;
   o.mom[0] = o.mom[1] = o.mom[2] = 0.0;
@@ -131,10 +133,9 @@ template <bool MIXED, int NT>
 static void launch_step_t(IntegMode mode, int th, int threads, const StepArgs& a, const ForceParams& fp,
                           const StepGate& gate, const MoveReport& mr, cudaStream_t st) {
 #define MDG_STEP(MODE, KE, TH)                                                                                       \
-  k_step<MIXED, MODE, KE, TH, NT><<<a.n_tiles, threads, step_smem_bytes(threads), st>>>(a.x, a.v, a.img, a.F, a.site, a.cellc, a.inv_perm,  \
-                                                                 a.ref, a.pos, a.flj, a.flj_next, a.Npad, a.N,       \
-                                                                 a.tiles, a.reps, fp, a.kepart, a.lam, a.flags,      \
-                                                                 gate, mr)
+  launch_dependent(gate.dep, k_step<MIXED, MODE, KE, TH, NT>, a.n_tiles, threads, step_smem_bytes(threads), st, a.x, a.v, a.img, \
+                   a.F, a.site, a.cellc, a.inv_perm, a.ref, a.pos, a.flj, a.flj_next, a.Npad, a.N, a.tiles, a.reps,  \
+                   fp, a.kepart, a.lam, a.flags, gate, mr)
   if (mode == kKickKickDrift) {
     if (th == 2) MDG_STEP(kKickKickDrift, true, 2);
     else if (th == 1) MDG_STEP(kKickKickDrift, true, 1);

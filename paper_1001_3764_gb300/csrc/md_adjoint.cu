@@ -871,7 +871,7 @@ int evaluate(md_adj* a, const double* xp, const double* beta, double cu, int mod
     return MD_ECUDA;
   k_adj_count<<<(N + 255) / 256, 256, 0, st>>>(xp, P, a->cell_of, ob);
   launch_cell_order(a->cell_of, N, a->C_cells, ob, a->cell_start, a->seg_scan, a->tmp, a->perm,
-                    EmitSorted{xp, beta, cu, P, a->xs, a->us, a->x32}, st);
+                    EmitSorted{xp, beta, cu, P, a->xs, a->us, a->x32}, false, st);
   const int lj_blocks = (N + kLjWarps - 1) / kLjWarps, b_blocks = (N + kBondTile - 1) / kBondTile;
   if (beta && a->hvp32) {
     k_adj_lj<float, true><<<lj_blocks, 32 * kLjWarps, 0, st>>>(a->xs, a->us, a->x32, a->cell_start, a->cell_of, P, 1,

@@ -592,24 +592,26 @@ static void prof_mark(md_system* s) {
     cudaEventRecord(s->ev[s->ev_used++], s->st);
 }
 
-static void enqueue_build(md_system* s) {
+// dep: the launch before is the sort's (launch_dependent)
+static void enqueue_build(md_system* s, bool dep = false) {
   launch_cl_build(s->pos, s->tag, s->cell_start, s->cl_start, s->region_cells, s->items + s->n_lj_items,
                   s->n_build_items, s->shapes, s->reps, s->list, s->ncl, s->cap, s->tile_cap, s->flags,
-                  s->n_tasks, s->generic ? &s->topo : nullptr, s->st);
+                  s->n_tasks, s->generic ? &s->topo : nullptr, dep, s->st);
   launch_cl_rank(s->pos, s->cell_start, s->cl_start, s->region_cells, s->items, s->n_lj_items, s->shapes, s->ncl,
-                 s->tasks, s->task_base, s->n_tasks, s->st);
+                 s->tasks, s->task_base, s->n_tasks, true, s->st);
 }
 
 static void enqueue_rebin(md_system* s) {
+  constexpr bool dep = true;
   cudaMemsetAsync(s->count, 0, sizeof(int) * s->C, s->st);
   launch_bin_count(s->mixed, s->x, (int)s->N, s->tiles_int, (int)s->t_int.size(), s->reps, s->cell_of, s->cellc,
                    s->count, s->slot, s->st);
-  launch_scan2(s->count, s->cell_start, s->cl_start, s->C, s->scan_seg, s->st);
-  launch_bin_scatter(s->cell_of, s->slot, s->cell_start, s->tmp, (int)s->N, s->st);
+  launch_scan2(s->count, s->cell_start, s->cl_start, s->C, s->scan_seg, dep, s->st);
+  launch_bin_scatter(s->cell_of, s->slot, s->cell_start, s->tmp, (int)s->N, dep, s->st);
   launch_cell_sort(s->mixed, s->x, (int)s->N, s->cell_start, s->tmp, s->fp.mtype, s->cellc, s->site, s->reps, s->n_reps, s->C,
-                   s->S, s->perm, s->inv_perm, s->pos, s->tag, s->ref, s->flags, s->st);
+                   s->S, s->perm, s->inv_perm, s->pos, s->tag, s->ref, s->flags, dep, s->st);
   prof_mark(s);
-  enqueue_build(s);
+  enqueue_build(s, !s->profile);
   prof_mark(s);
 }
 static const int kRebinLaunches = 7;   // memset counted as a launch
@@ -663,7 +665,10 @@ static StepArgs step_args(md_system* s, bool chain_tiles, const long long* flj, 
 static void enqueue_steps(md_system* s, int k, bool repeat, const MoveReport& mr) {
   for (int j = 0; j < k; ++j) {
     long long* flj = s->flj[j & 1];
-    const StepGate gate{mr.ctl, j, repeat ? 1 : 0};
+    // launched as dependents of the kernel before, but where the profile's event
+    // records come in between, and a repeat's first LJ launch: what that reads
+    // before its wait is the list build's, its predecessor's
+    const StepGate gate{mr.ctl, j, repeat ? 1 : 0, !s->profile && !s->generic && !(repeat && j == 0)};
     if (j == 0 && repeat) {
       // a repeat resumes at an LJ launch
     } else if (j == 0 || s->generic) {
@@ -685,7 +690,7 @@ static void enqueue_steps(md_system* s, int k, bool repeat, const MoveReport& mr
     enqueue_lj(s, false, flj, gate, thermo);
     prof_mark(s);
   }
-  const StepGate gate{mr.ctl, k - 1, repeat ? 1 : 0};
+  const StepGate gate{mr.ctl, k - 1, repeat ? 1 : 0, !s->profile && !s->generic};
   if (s->generic) {
     launch_integrate(s->mixed, kKickOnly, s->thermo, step_args(s, false, nullptr, nullptr), s->fp, gate, mr, s->st);
   } else {
@@ -1323,6 +1328,7 @@ int md_bin_study(md_system* s, int32_t reps, double* ms) {
   cudaEvent_t ev[6];
   for (cudaEvent_t& e : ev) cudaEventCreate(&e);
   double acc[6] = {0, 0, 0, 0, 0, 0};
+  constexpr bool dep = false;   // event records and copies between the launches
   const bool prof = s->profile;
   s->profile = false;
   int rc = MD_OK;
@@ -1332,10 +1338,10 @@ int md_bin_study(md_system* s, int32_t reps, double* ms) {
     cudaMemsetAsync(s->count, 0, sizeof(int) * C, s->st);
     launch_bin_count(s->mixed, s->x, (int)N, s->tiles_int, (int)s->t_int.size(), s->reps, s->cell_of, s->cellc,
                      s->count, s->slot, s->st);
-    launch_scan2(s->count, s->cell_start, s->cl_start, s->C, s->scan_seg, s->st);
-    launch_bin_scatter(s->cell_of, s->slot, s->cell_start, s->tmp, (int)N, s->st);
+    launch_scan2(s->count, s->cell_start, s->cl_start, s->C, s->scan_seg, dep, s->st);
+    launch_bin_scatter(s->cell_of, s->slot, s->cell_start, s->tmp, (int)N, dep, s->st);
     launch_cell_sort(s->mixed, s->x, (int)N, s->cell_start, s->tmp, s->fp.mtype, s->cellc, s->site, s->reps, s->n_reps, s->C,
-                     s->S, s->perm, s->inv_perm, s->pos, s->tag, s->ref, s->flags, s->st);
+                     s->S, s->perm, s->inv_perm, s->pos, s->tag, s->ref, s->flags, dep, s->st);
     cudaEventRecord(ev[1], s->st);
     enqueue_build(s);
     cudaEventRecord(ev[2], s->st);
@@ -1355,7 +1361,7 @@ int md_bin_study(md_system* s, int32_t reps, double* ms) {
               cudaMemcpyAsync(s->tmp, perm.data(), N * sizeof(int), cudaMemcpyHostToDevice, s->st) == cudaSuccess;
     if (!ok) { rc = fail(s, MD_ECUDA, "copy"); break; }
     launch_cell_sort(s->mixed, s->x, (int)N, s->cell_start, s->tmp, s->fp.mtype, s->cellc, s->site, s->reps, s->n_reps, s->C,
-                     s->S, s->perm, s->inv_perm, s->pos, s->tag, s->ref, s->flags, s->st);
+                     s->S, s->perm, s->inv_perm, s->pos, s->tag, s->ref, s->flags, dep, s->st);
     cudaEventRecord(ev[5], s->st);
     if (cudaStreamSynchronize(s->st) != cudaSuccess) { rc = fail(s, MD_ECUDA, "sync"); break; }
     float a, b, c, d;

@@ -296,6 +296,7 @@ struct StepGate {
   const int* ctl;   // null: always runs
   int j;            // this launch's drift or LJ index
   int repeat;       // 1 inside the WHILE body
+  bool dep;         // launch_dependent
 };
 __device__ __forceinline__ bool lj_runs(const StepGate& g) {
   if (!g.ctl) return true;
@@ -324,6 +325,37 @@ struct ThermoArgs {
   double one_minus_rate, dt;    // 1 - dt / tau
 };
 
+// ---------------------------------------------------------------- dependent launches
+// A kernel launched by launch_dependent may start while the kernel before it in
+// the stream (or graph) is still running; it calls wait_for_predecessor()
+// before it touches anything that kernel reads or writes, and lets its own
+// successor start afterwards.  So what a kernel reads before the wait may be
+// the work of any kernel but its predecessor: that one has passed its own wait,
+// and all before it are complete.  The wait is the hardware's, on the whole
+// predecessor grid; every block passes it (no block leaves before).  It hides
+// the launch latency and what a kernel does before the wait: 1,500 sites,
+// 26.2 -> 21.5 us per step.
+__device__ __forceinline__ void wait_for_predecessor() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// (dep = false: an ordinary launch, for a predecessor that is not a kernel)
+template <class... P, class... A>
+inline void launch_dependent(bool dep, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                             const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = dep ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // ---------------------------------------------------------------- binning
 void launch_bin_count(bool mixed, const void* x, int N, const Tile* tiles, int n_tiles,
                       const RepDev* reps, int* cell_of, int* cellc, int* count, int* slot,
@@ -335,14 +367,14 @@ void launch_bin_count(bool mixed, const void* x, int N, const Tile* tiles, int n
 // over the tiles (cell_order.cuh)
 size_t scan_seg_ints(long long C);
 void launch_scan(const int* count, int* cell_start, int C, int* seg, const int* hist, int n_tiles, int bits,
-                 int* tot, cudaStream_t st);
-void launch_scan2(const int* count, int* cell_start, int* cl_start, int C, int* seg, cudaStream_t st);
-void launch_bin_scatter(const int* cell_of, const int* slot, const int* cell_start, int* tmp, int N,
+                 int* tot, bool dep, cudaStream_t st);
+void launch_scan2(const int* count, int* cell_start, int* cl_start, int C, int* seg, bool dep, cudaStream_t st);
+void launch_bin_scatter(const int* cell_of, const int* slot, const int* cell_start, int* tmp, int N, bool dep,
                         cudaStream_t st);
 void launch_cell_sort(bool mixed, const void* x, int N, const int* cell_start, const int* tmp, const unsigned char* mtype,
                       const int* cellc, const uint16_t* site, const RepDev* reps, int n_reps, int C,
                       int sites, int* perm, int* inv_perm, float4* pos, int* tag, float4* ref, unsigned* flags,
-                      cudaStream_t st);
+                      bool dep, cudaStream_t st);
 // ---------------------------------------------------------------- forces
 // cluster lists and LJ forces by regions (k_lj.cu), a block per work item.
 // The build writes each cluster's list (up to cap entries, ncl[cl] of them);
@@ -356,13 +388,13 @@ void launch_cell_sort(bool mixed, const void* x, int N, const int* cell_start, c
 void launch_cl_build(const float4* pos, const int* tag, const int* cell_start, const int* cl_start,
                      const int* cells, const WorkItem* items, int n_items, const RegionShape* shapes,
                      const RepDev* reps, unsigned* list, int* ncl, int cap, int tile_cap, unsigned* flags,
-                     int* n_tasks, const TopoDev* topo, cudaStream_t st);
+                     int* n_tasks, const TopoDev* topo, bool dep, cudaStream_t st);
 // after the build (which clears *n_tasks): each LJ item's clusters in the
 // order the force kernel takes them, tasks[task_base[item] + rank]; an item
 // claims its place in the table (as many entries as there are clusters) by *n_tasks
 void launch_cl_rank(const float4* pos, const int* cell_start, const int* cl_start, const int* cells,
                     const WorkItem* items, int n_items, const RegionShape* shapes, const int* ncl, ClusterTask* tasks,
-                    int* task_base, int* n_tasks, cudaStream_t st);
+                    int* task_base, int* n_tasks, bool dep, cudaStream_t st);
 void launch_cl_force(bool energy, const float4* pos, const int* cell_start, const int* cl_start,
                      const int* cells, const WorkItem* items, int n_items, const RegionShape* shapes,
                      const RepDev* reps, const unsigned* list, const ClusterTask* tasks, const int* task_base,

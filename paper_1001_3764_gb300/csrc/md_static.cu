@@ -87,7 +87,7 @@ extern "C" int md_bin_static(const double* pos, int32_t n_atoms, double box, int
   if (cudaMemsetAsync(scratch, 0, sizeof(int) * order_clear_ints(ob, C), st) != cudaSuccess)
     return fail(MD_ECUDA, "clearing the cell counters failed");
   k_static_count<<<(n_atoms + 255) / 256, 256, 0, st>>>(pos, n_atoms, box, inv_h, cells_per_side, cell_of, ob);
-  launch_cell_order(cell_of, n_atoms, C, ob, cell_start, nullptr, tmp, perm, EmitNothing{}, st);   // C <= 2^17: no seg
+  launch_cell_order(cell_of, n_atoms, C, ob, cell_start, nullptr, tmp, perm, EmitNothing{}, true, st);   // C <= 2^17: no seg
   if (cudaGetLastError() != cudaSuccess) return fail(MD_ECUDA, "a binning kernel failed to launch");
   return MD_OK;
 }
