@@ -58,6 +58,7 @@ struct RegTile {
   float sx[kMaxTileCells], sy[kMaxTileCells], sz[kMaxTileCells];
   int ncl[kMaxHome + 1];          // clusters of home cells before h (ncl[n_home] = all)
   int cl0[kMaxHome];              // global id of home cell h's first cluster
+  int home[kMaxHome];             // tile cell of home cell h
   int home_cell[kMaxHome];        // global id of home cell h
   int cnt[kMaxTileCells];         // atoms of tile cell k (set-up scratch)
   int n_tile, n_home;
@@ -79,30 +80,31 @@ __device__ __forceinline__ void region_setup(RegTile& T, const WorkItem& item, c
       T.sx[k] = (float)S.off[k][0] - S.cx;
       T.sy[k] = (float)S.off[k][1] - S.cy;
       T.sz[k] = (float)S.off[k][2] - S.cz;
-      if (k < S.n_home) {
-        T.home_cell[k] = c;
-        T.cl0[k] = cl_start[c];
-      }
     }
     T.cnt[k] = n;
+  }
+  if (k >= 32 && k < 32 + S.n_home) {   // the home cells, on the second warp
+    const int h = k - 32, th = S.nb[h][0], c = __ldg(cells + kRegionCells * item.region + th);
+    T.home[h] = th;
+    T.home_cell[h] = c;
+    T.cl0[h] = cl_start[c];
   }
   __syncthreads();
   if (k < 32) {
     const int a = T.cnt[2 * k], b = T.cnt[2 * k + 1];
     int incl = a + b;
-    // clusters of the home cells (ceil(n / 4) each); home cells come first
-    const int ca = 2 * k < S.n_home ? (a + 3) >> 2 : 0, cb = 2 * k + 1 < S.n_home ? (b + 3) >> 2 : 0;
-    int ci = ca + cb;
+    // clusters of the home cells (ceil(n / 4) each)
+    const int own = k < S.n_home ? (T.cnt[T.home[k]] + 3) >> 2 : 0;
+    int ci = own;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int v = __shfl_up_sync(0xffffffffu, incl, o), w = __shfl_up_sync(0xffffffffu, ci, o);
       if (k >= o) { incl += v; ci += w; }
     }
-    const int ex = incl - a - b, cx = ci - ca - cb;
+    const int ex = incl - a - b;
     if (2 * k < S.n_tile) T.off[2 * k] = ex;
     if (2 * k + 1 < S.n_tile) T.off[2 * k + 1] = ex + a;
-    if (2 * k < S.n_home) T.ncl[2 * k] = cx;
-    if (2 * k + 1 < S.n_home) T.ncl[2 * k + 1] = cx + ca;
+    if (k < S.n_home) T.ncl[k] = ci - own;
     if (k == 31) {
       T.off[S.n_tile] = incl;
       T.ncl[S.n_home] = ci;
@@ -117,11 +119,10 @@ __device__ __forceinline__ void region_setup(RegTile& T, const WorkItem& item, c
 // cells in turn and their lanes start asynchronous copies (cp.async, global
 // to shared without registers) of the cell's atoms, so the whole tile is in
 // flight at once; a lane then waits for its own copies and adds the cell's
-// frame shift to the atoms it copied, without a barrier in between.  The w component keeps the LJ type
-// (0.0 / 1.0) that binning and integration store; WITH_TAG (list build)
-// replaces it by the bits of the atom's chain/site tag, which the build
-// needs instead.  tile_issue starts the copies, tile_finish waits for them,
-// shifts, and ends with a barrier.
+// frame shift to the atoms it copied, without a barrier in between.  The w
+// component keeps the LJ type (0.0 / 1.0) that binning and integration store.
+// tile_issue starts the copies, tile_finish waits for them, shifts, and ends
+// with a barrier.
 template <int NT>
 __device__ __forceinline__ void tile_issue(const RegTile& T, unsigned long long need, const float4* __restrict__ pos,
                                            float4* __restrict__ sp) {
@@ -138,19 +139,17 @@ __device__ __forceinline__ void tile_issue(const RegTile& T, unsigned long long 
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-template <bool WITH_TAG, int NT>
-__device__ __forceinline__ void tile_finish(const RegTile& T, unsigned long long need, float4* __restrict__ sp,
-                                            const int* __restrict__ tag) {
+template <int NT>
+__device__ __forceinline__ void tile_finish(const RegTile& T, unsigned long long need, float4* __restrict__ sp) {
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   const int lane = threadIdx.x & 31;
   for (int k = threadIdx.x >> 5; k < T.n_tile; k += NT / 32) {
     if (!((need >> k) & 1ull)) continue;
-    const int t0 = T.off[k], n = T.off[k + 1] - t0, j0 = T.start[k];
+    const int t0 = T.off[k], n = T.off[k + 1] - t0;
     const float ox = T.sx[k], oy = T.sy[k], oz = T.sz[k];
     for (int q = lane; q < n; q += 32) {
       float4 p = sp[t0 + q];
       p.x += ox; p.y += oy; p.z += oz;
-      if (WITH_TAG) p.w = __int_as_float(__ldg(tag + j0 + q) & (int)kTagMask);
       sp[t0 + q] = p;
     }
   }
@@ -197,7 +196,14 @@ __device__ __forceinline__ void persistent_done(int* work, int blocks) {
 // that pass are queued per warp in shared memory and tested 32 at a time,
 // so the lanes of a warp run the four-atom test on candidates that may pair
 // rather than on every 32nd atom of the tile.
-constexpr int kBuildQueue = 64;
+//
+// Bound: instruction issue (600 sphere tests and 190 four-atom tests a
+// cluster).  So the tile is kept as one array per coordinate: a lane takes two
+// consecutive candidates in packed FP32 (three 8-byte loads and six packed
+// operations for both), the forward cells are five runs of consecutive tile
+// cells (13 loops over 46 atoms each left 28% of the lanes without work), and the
+// four-atom test is packed as well.  1.5M sites: 780 -> 655 us.
+constexpr int kBuildQueue = 128;   // a ring: at most 31 + 64 candidates wait
 
 // is atom b of a molecule a 1-2 or 1-3 neighbour of atom a (general type)?
 __device__ __forceinline__ bool topo_excluded(int a, int b, const TopoDev& tp) {
@@ -206,27 +212,78 @@ __device__ __forceinline__ bool topo_excluded(int a, int b, const TopoDev& tp) {
   return a == b;
 }
 
-// the four-atom test of candidate t: bit u set if atom u of the cluster pairs with t
+// The list-build tile: coordinates in the region frame and chain/site tags.
+struct BuildTile {
+  float *x, *y, *z;
+  int* tag;
+};
+
+// the four-atom test of candidate t: bit u set if atom u of the cluster
+// (packed: atoms 0, 1 and 2, 3) pairs with t
 template <bool GEN>
-__device__ __forceinline__ unsigned pair_mask(const float4 (&pi)[4], const int (&ti)[4], const float4& w, float rl2,
+__device__ __forceinline__ unsigned pair_mask(const float2 (&px)[2], const float2 (&py)[2], const float2 (&pz)[2],
+                                              const int (&ti)[4], const BuildTile& B, int t, float rl2,
                                               const TopoDev& tp) {
-  const int tg = __float_as_int(w.w);   // the candidate's tag (list-build tile)
+  const float wx = B.x[t], wy = B.y[t], wz = B.z[t];
+  const int tg = B.tag[t];
   unsigned m = 0u;
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const float dx = pi[u].x - w.x, dy = pi[u].y - w.y, dz = pi[u].z - w.z;
-    bool keep = dx * dx + dy * dy + dz * dz < rl2;
-    if (GEN) {
-      // same molecule: its exclusion list (Sec. 3.1, t_exclusions)
-      if (keep && ((ti[u] ^ tg) >> kTagSiteBits) == 0)
-        keep = !topo_excluded(ti[u] & ((1 << kTagSiteBits) - 1), tg & ((1 << kTagSiteBits) - 1), tp);
-    } else {
-      // |i - j| <= 2 within one chain: 1-2 and 1-3 neighbours (and i itself)
-      keep &= (unsigned)(ti[u] - tg + 2) > 4u;
+  for (int p = 0; p < 2; ++p) {
+    const float2 dx = __fadd2_rn(px[p], make_float2(-wx, -wx)), dy = __fadd2_rn(py[p], make_float2(-wy, -wy)),
+                 dz = __fadd2_rn(pz[p], make_float2(-wz, -wz));
+    const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dx, dx, __fmul2_rn(dy, dy)));
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int u = 2 * p + e;
+      bool keep = (e ? r2.y : r2.x) < rl2;
+      if (GEN) {
+        // same molecule: its exclusion list (Sec. 3.1, t_exclusions)
+        if (keep && ((ti[u] ^ tg) >> kTagSiteBits) == 0)
+          keep = !topo_excluded(ti[u] & ((1 << kTagSiteBits) - 1), tg & ((1 << kTagSiteBits) - 1), tp);
+      } else {
+        // |i - j| <= 2 within one chain: 1-2 and 1-3 neighbours (and i itself)
+        keep &= (unsigned)(ti[u] - tg + 2) > 4u;
+      }
+      m |= keep ? (1u << u) : 0u;
     }
-    m |= keep ? (1u << u) : 0u;
   }
   return m;
+}
+
+// Stage the tile: a warp takes two tile cells at a time, up to four loads of a
+// lane in flight, adds the frame shift and stores by coordinate.
+template <int NT>
+__device__ __forceinline__ void stage_build_tile(const RegTile& T, unsigned long long need,
+                                                 const float4* __restrict__ pos, const int* __restrict__ tag,
+                                                 const BuildTile& B) {
+  constexpr int NW = NT / 32;
+  const int lane = threadIdx.x & 31;
+  for (int k = threadIdx.x >> 5; k < T.n_tile; k += 2 * NW) {
+    const int kk[2] = {k, k + NW < T.n_tile ? k + NW : k};
+    int n[2];
+    n[0] = (need >> k) & 1ull ? T.off[k + 1] - T.off[k] : 0;
+    n[1] = k + NW < T.n_tile && ((need >> (k + NW)) & 1ull) ? T.off[k + NW + 1] - T.off[k + NW] : 0;
+    for (int q0 = lane; q0 - lane < max(n[0], n[1]); q0 += 64) {
+      float4 p[4];
+      int tg[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int q = q0 + 32 * (e & 1), s = T.start[kk[e >> 1]] + q;
+        if (q < n[e >> 1]) { p[e] = __ldg(pos + s); tg[e] = __ldg(tag + s) & (int)kTagMask; }
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int c = kk[e >> 1], q = q0 + 32 * (e & 1), t = T.off[c] + q;
+        if (q < n[e >> 1]) {
+          B.x[t] = p[e].x + T.sx[c];
+          B.y[t] = p[e].y + T.sy[c];
+          B.z[t] = p[e].z + T.sz[c];
+          B.tag[t] = tg[e];
+        }
+      }
+    }
+  }
+  __syncthreads();
 }
 
 template <int NT, bool GEN>
@@ -239,131 +296,137 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_cl_build(const float4* __rest
                                                  int tile_cap, unsigned* __restrict__ flags, int* __restrict__ n_tasks,
                                                  const TopoDev tp) {
   extern __shared__ __align__(16) unsigned char smem[];
-  float4* sp = reinterpret_cast<float4*>(smem);   // w: the atom's chain/site tag bits
+  BuildTile B;
+  B.x = reinterpret_cast<float*>(smem);
+  B.y = B.x + tile_cap;
+  B.z = B.y + tile_cap;
+  B.tag = reinterpret_cast<int*>(B.z + tile_cap);
   __shared__ RegTile T;
   __shared__ int queue[NT / 32][kBuildQueue];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int* qw = queue[warp];
-  {
-    wait_for_predecessor();
-    const WorkItem item = items[blockIdx.x];
-    const RegionShape& S = shapes[item.shape];
-    const RepDev& R = reps[item.rep];
-    if (blockIdx.x == 0 && threadIdx.x == 0) *n_tasks = 0;   // for k_cl_rank
-    region_setup(T, item, S, cells, cell_start, cl_start);
-    const int total = T.off[T.n_tile], q_end = T.ncl[item.h1], q_first = T.ncl[item.h0] + item.part;
-    if (total > tile_cap) {
-      if (threadIdx.x == 0) atomicOr(flags, kFlagNbrOverflow);
-      for (int q = q_first + item.parts * (int)threadIdx.x; q < q_end; q += item.parts * NT) {
-        int h, k;
-        cluster_of(T, q, h, k);
-        ncl[T.cl0[h] + k] = 0;
-      }
-      return;
-    }
-    tile_issue<NT>(T, item.need, pos, sp);
-    tile_finish<true, NT>(T, item.need, sp, tag);
-    const float rl2 = R.rlist2u;
-    const float rl = sqrtf(rl2);
-    const unsigned lt = (1u << lane) - 1u;
-    for (int q = q_first + item.parts * warp; q < q_end; q += item.parts * (NT / 32)) {
+  wait_for_predecessor();
+  const WorkItem item = items[blockIdx.x];
+  const RegionShape& S = shapes[item.shape];
+  const RepDev& R = reps[item.rep];
+  if (blockIdx.x == 0 && threadIdx.x == 0) *n_tasks = 0;   // for k_cl_rank
+  region_setup(T, item, S, cells, cell_start, cl_start);
+  const int total = T.off[T.n_tile], q_end = T.ncl[item.h1], q_first = T.ncl[item.h0] + item.part;
+  if (total > tile_cap) {
+    if (threadIdx.x == 0) atomicOr(flags, kFlagNbrOverflow);
+    for (int q = q_first + item.parts * (int)threadIdx.x; q < q_end; q += item.parts * NT) {
       int h, k;
       cluster_of(T, q, h, k);
-      const int i0 = T.off[h] + 4 * k;
-      const int ni = min(4, T.off[h + 1] - i0);
-      float4 pi[4];
-      int ti[4];
-      float cx = 0.f, cy = 0.f, cz = 0.f;
+      ncl[T.cl0[h] + k] = 0;
+    }
+    return;
+  }
+  stage_build_tile<NT>(T, item.need, pos, tag, B);
+  const float rl2 = R.rlist2u;
+  const float rl = sqrtf(rl2);
+  const unsigned lt = (1u << lane) - 1u;
+  for (int q = q_first + item.parts * warp; q < q_end; q += item.parts * (NT / 32)) {
+    int h, k;
+    cluster_of(T, q, h, k);
+    const int th = T.home[h], cell_end = T.off[th + 1];
+    const int i0 = T.off[th] + 4 * k;
+    const int ni = min(4, cell_end - i0);
+    float4 pi[4];
+    int ti[4];
+    float cx = 0.f, cy = 0.f, cz = 0.f;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int t = i0 + min(u, ni - 1);
-        pi[u] = sp[t];
-        ti[u] = __float_as_int(pi[u].w);
-        cx += pi[u].x; cy += pi[u].y; cz += pi[u].z;
-      }
-      cx *= 0.25f; cy *= 0.25f; cz *= 0.25f;
-      float rad2 = 0.f;
+    for (int u = 0; u < 4; ++u) {
+      const int t = i0 + min(u, ni - 1);
+      pi[u] = make_float4(B.x[t], B.y[t], B.z[t], 0.f);
+      ti[u] = B.tag[t];
+      cx += pi[u].x; cy += pi[u].y; cz += pi[u].z;
+    }
+    cx *= 0.25f; cy *= 0.25f; cz *= 0.25f;
+    float rad2 = 0.f;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const float dx = pi[u].x - cx, dy = pi[u].y - cy, dz = pi[u].z - cz;
-        rad2 = fmaxf(rad2, dx * dx + dy * dy + dz * dz);
-        // a slot past the cell's last atom gets a far position: it pairs with nothing
-        if (u >= ni) pi[u] = make_float4(1e9f, 1e9f, 1e9f, 0.f);
+    for (int u = 0; u < 4; ++u) {
+      const float dx = pi[u].x - cx, dy = pi[u].y - cy, dz = pi[u].z - cz;
+      rad2 = fmaxf(rad2, dx * dx + dy * dy + dz * dz);
+      // a slot past the cell's last atom gets a far position: it pairs with nothing
+      if (u >= ni) pi[u] = make_float4(1e9f, 1e9f, 1e9f, 0.f);
+    }
+    float2 px[2], py[2], pz[2];
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      px[p] = make_float2(pi[2 * p].x, pi[2 * p + 1].x);
+      py[p] = make_float2(pi[2 * p].y, pi[2 * p + 1].y);
+      pz[p] = make_float2(pi[2 * p].z, pi[2 * p + 1].z);
+    }
+    // the sphere test is taken with a margin of 1e-5 cell units over the
+    // FP32 roundings of c and rad, so it never rejects a pair the exact
+    // test keeps
+    const float reach = rl + sqrtf(rad2) + 1e-5f;
+    const float reach2 = reach * reach;
+    const float2 ncx = make_float2(-cx, -cx), ncy = make_float2(-cy, -cy), ncz = make_float2(-cz, -cz);
+    const int cl = T.cl0[h] + k;
+    unsigned* out = list + (size_t)cl * cap;
+    int cnt = 0;
+    auto append = [&](int t, unsigned m) {
+      const unsigned b = __ballot_sync(0xffffffffu, m != 0u);
+      const int p = cnt + __popc(b & lt);
+      if (m != 0u && p < cap) out[p] = (unsigned)t | (m << 16);
+      cnt += __popc(b);
+    };
+    // own cell, from the cluster on: each pair once, i before j
+    for (int t0 = i0; t0 < cell_end; t0 += 32) {
+      const int t = t0 + lane;
+      unsigned m = 0u;
+      if (t < cell_end) {
+        m = pair_mask<GEN>(px, py, pz, ti, B, t, rl2, tp);
+        m &= ((t > i0) ? 1u : 0u) | ((t > i0 + 1) ? 2u : 0u) | ((t > i0 + 2) ? 4u : 0u) | ((t > i0 + 3) ? 8u : 0u);
       }
-      // the sphere test is taken with a margin of 1e-5 cell units over the
-      // FP32 roundings of c and rad, so it never rejects a pair the exact
-      // test keeps
-      const float reach = rl + sqrtf(rad2) + 1e-5f;
-      const float reach2 = reach * reach;
-      const int cl = T.cl0[h] + k;
-      unsigned* out = list + (size_t)cl * cap;
-      int cnt = 0;
-      // own cell, from the cluster on: each pair once, i before j
-      {
-        const int t_end = T.off[h + 1];
-        for (int t0 = i0; t0 < t_end; t0 += 32) {
-          const int t = t0 + lane;
-          unsigned m = 0u;
-          if (t < t_end) {
-            m = pair_mask<GEN>(pi, ti, sp[t], rl2, tp);
-            m &= ((t > i0) ? 1u : 0u) | ((t > i0 + 1) ? 2u : 0u) | ((t > i0 + 2) ? 4u : 0u) | ((t > i0 + 3) ? 8u : 0u);
-          }
-          const unsigned b = __ballot_sync(0xffffffffu, m != 0u);
-          const int p = cnt + __popc(b & lt);
-          if (m != 0u && p < cap) out[p] = (unsigned)t | (m << 16);
-          cnt += __popc(b);
+      append(t, m);
+    }
+    // the 13 forward cells, five runs of tile cells: sphere test of two
+    // consecutive candidates per lane, queue, four-atom test 32 at a time
+    int qn = 0, head = 0;   // waiting candidates: ring places head .. head + qn - 1
+#pragma unroll 1
+    for (int run = 0; run < 5; ++run) {
+      const int t_beg = T.off[S.nb[h][3 * run + 1]], t_end = T.off[S.nb[h][min(3 * run + 3, 13)] + 1];
+      for (int t0 = t_beg & ~1; t0 < t_end; t0 += 64) {
+        const int t = t0 + 2 * lane;
+        bool pass0 = false, pass1 = false;
+        if (t < t_end) {
+          const float2 dx = __fadd2_rn(*reinterpret_cast<const float2*>(B.x + t), ncx),
+                       dy = __fadd2_rn(*reinterpret_cast<const float2*>(B.y + t), ncy),
+                       dz = __fadd2_rn(*reinterpret_cast<const float2*>(B.z + t), ncz);
+          const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
+          pass0 = r2.x < reach2 && t >= t_beg;
+          pass1 = r2.y < reach2 && t + 1 < t_end;
         }
-      }
-      // the 13 forward cells: sphere test, queue, four-atom test 32 at a time
-      int qn = 0;
-      for (int c14 = 1; c14 < 14; ++c14) {
-        const int tc = S.nb[h][c14];
-        const int t_end = T.off[tc + 1];
-        for (int t0 = T.off[tc]; t0 < t_end; t0 += 32) {
-          const int t = t0 + lane;
-          bool pass = false;
-          if (t < t_end) {
-            const float4 w = sp[t];
-            const float dx = w.x - cx, dy = w.y - cy, dz = w.z - cz;
-            pass = dx * dx + dy * dy + dz * dz < reach2;
-          }
-          const unsigned b = __ballot_sync(0xffffffffu, pass);
-          if (pass) qw[qn + __popc(b & lt)] = t;
-          qn += __popc(b);
-          __syncwarp();
-          if (qn >= 32) {
-            const int tq = qw[lane];
-            const unsigned m = pair_mask<GEN>(pi, ti, sp[tq], rl2, tp);
-            const unsigned bm = __ballot_sync(0xffffffffu, m != 0u);
-            const int p = cnt + __popc(bm & lt);
-            if (m != 0u && p < cap) out[p] = (unsigned)tq | (m << 16);
-            cnt += __popc(bm);
-            const int rest = qn - 32;
-            const int moved = lane < rest ? qw[32 + lane] : 0;
-            __syncwarp();
-            if (lane < rest) qw[lane] = moved;
-            __syncwarp();
-            qn = rest;
-          }
+        const unsigned b0 = __ballot_sync(0xffffffffu, pass0), b1 = __ballot_sync(0xffffffffu, pass1);
+        const int at = head + qn + __popc(b0 & lt) + __popc(b1 & lt);
+        if (pass0) qw[at & (kBuildQueue - 1)] = t;
+        if (pass1) qw[(at + (pass0 ? 1 : 0)) & (kBuildQueue - 1)] = t + 1;
+        qn += __popc(b0) + __popc(b1);
+        __syncwarp();
+        while (qn >= 32) {
+          const int tq = qw[(head + lane) & (kBuildQueue - 1)];
+          append(tq, pair_mask<GEN>(px, py, pz, ti, B, tq, rl2, tp));
+          head += 32;
+          qn -= 32;
         }
+        __syncwarp();
       }
-      if (qn > 0) {
-        unsigned m = 0u;
-        int tq = 0;
-        if (lane < qn) {
-          tq = qw[lane];
-          m = pair_mask<GEN>(pi, ti, sp[tq], rl2, tp);
-        }
-        const unsigned bm = __ballot_sync(0xffffffffu, m != 0u);
-        const int p = cnt + __popc(bm & lt);
-        if (m != 0u && p < cap) out[p] = (unsigned)tq | (m << 16);
-        cnt += __popc(bm);
+    }
+    if (qn > 0) {
+      unsigned m = 0u;
+      int tq = 0;
+      if (lane < qn) {
+        tq = qw[(head + lane) & (kBuildQueue - 1)];
+        m = pair_mask<GEN>(px, py, pz, ti, B, tq, rl2, tp);
       }
-      __syncwarp();
-      if (lane == 0) {
-        ncl[cl] = min(cnt, cap);
-        if (cnt > cap) atomicOr(flags, kFlagNbrOverflow);
-      }
+      append(tq, m);
+    }
+    __syncwarp();
+    if (lane == 0) {
+      ncl[cl] = min(cnt, cap);
+      if (cnt > cap) atomicOr(flags, kFlagNbrOverflow);
     }
   }
 }
@@ -879,12 +942,12 @@ __global__ void __launch_bounds__(kRankThreads) k_cl_rank(const float4* __restri
     }
     int h, k;
     cluster_of(T, q_first + q, h, k);
-    const int ni = min(4, T.off[h + 1] - T.off[h] - 4 * k);
+    const int th = T.home[h], ni = min(4, T.off[th + 1] - T.off[th] - 4 * k);
     unsigned tb = 0u;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) tb |= pos[T.start[h] + 4 * k + min(u, ni - 1)].w != 0.f ? (1u << u) : 0u;
+    for (int u = 0; u < 4; ++u) tb |= pos[T.start[th] + 4 * k + min(u, ni - 1)].w != 0.f ? (1u << u) : 0u;
     tasks[base + rank] =
-        make_int4(kq >> 9, T.cl0[h] + k, ((T.off[h] + 4 * k) << 7) | (int)(tb << 3) | ni, q);
+        make_int4(kq >> 9, T.cl0[h] + k, ((T.off[th] + 4 * k) << 7) | (int)(tb << 3) | ni, q);
   }
 }
 
@@ -960,7 +1023,7 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_cl_force(
       if (threadIdx.x == 0) atomicOr(flags, kFlagNbrOverflow);
     } else {
       tile_issue<NT>(T, item.need, pos, sp);
-      tile_finish<false, NT>(T, item.need, sp, nullptr);   // ends with a barrier
+      tile_finish<NT>(T, item.need, sp);   // ends with a barrier
       const LjConst c = lj_const(R);
       for (;;) {
         int q0 = 0;
@@ -991,7 +1054,7 @@ void launch_cl_build(const float4* pos, const int* tag, const int* cell_start, c
   if (n_items <= 0) return;
   const size_t sm = cl_build_smem(tile_cap);
   // 32 warps an SM: four blocks of 256 threads, or where four tiles do not fit its shared memory, two of 512
-  if (4 * (sm + 3800 + 1024) > 228 * 1024) {
+  if (4 * (sm + 5800 + 1024) > 228 * 1024) {
     if (topo)
       launch_dependent(dep, k_cl_build<512, true>, n_items, 512, sm, st, pos, tag, cell_start, cl_start, cells, items, shapes, reps, list,
                        ncl, cap, tile_cap, flags, n_tasks, *topo);

@@ -200,16 +200,20 @@ static void fill_force_params(md_system* s) {
   fill_thermostats(s);
 }
 
-// Region shapes: sx x sy x 1 home cells (sx, sy in {1, 2}; shape id
-// (sx - 1) + 2 (sy - 1)).  The tile lists the home cells first, then every
-// cell that a home cell's 13 forward offsets reach, in the order first met;
-// nb[h] gives home cell h's own tile cell and its 13 forward tile cells, in
-// the offset order (dz = +1 layer, then dz = 0, dy = +1, then (+1, 0, 0)).
+// Region shapes: sx x sy x 1 home cells (sx, sy in 1 .. G; shape id
+// (sx - 1) + G (sy - 1)).  The tile lists the cells that the home cells and
+// their 13 forward offsets take up, rows of x one after another: the layer above,
+// then the home layer.  So a home cell's forward cells are five runs of
+// consecutive tile cells.  nb[h] gives home cell h's own tile cell and its 13
+// forward tile cells, in the offset order (dz = +1 layer: dy = +1, 0, -1, each
+// dx = -1, 0, 1; then dz = 0, dy = +1; then (+1, 0, 0)).
 static RegionShape make_shape(int sx, int sy) {
   RegionShape S{};
   std::vector<std::array<int, 3>> tile;
-  for (int y = 0; y < sy; ++y)
-    for (int x = 0; x < sx; ++x) tile.push_back({x, y, 0});
+  for (int y = -1; y <= sy; ++y)
+    for (int x = -1; x <= sx; ++x) tile.push_back({x, y, 1});
+  for (int y = 0; y <= sy; ++y)
+    for (int x = y == 0 ? 0 : -1; x <= sx; ++x) tile.push_back({x, y, 0});
   S.n_home = sx * sy;
   std::vector<std::array<int, 3>> fw;
   for (int dz = -1; dz <= 1; ++dz)
@@ -220,14 +224,12 @@ static RegionShape make_shape(int sx, int sy) {
     return std::make_tuple(-a[2], -a[1], a[0]) < std::make_tuple(-b[2], -b[1], b[0]);
   });
   for (int h = 0; h < S.n_home; ++h) {
-    S.nb[h][0] = (unsigned char)h;
-    for (int q = 0; q < 13; ++q) {
-      const std::array<int, 3> c = {tile[h][0] + fw[q][0], tile[h][1] + fw[q][1], tile[h][2] + fw[q][2]};
-      int k = 0;
-      while (k < (int)tile.size() && tile[k] != c) ++k;
-      if (k == (int)tile.size()) tile.push_back(c);
-      S.nb[h][q + 1] = (unsigned char)k;
-    }
+    const std::array<int, 3> home = {h % sx, h / sx, 0};
+    auto index = [&](const std::array<int, 3>& c) {
+      return (unsigned char)(std::find(tile.begin(), tile.end(), c) - tile.begin());
+    };
+    S.nb[h][0] = index(home);
+    for (int q = 0; q < 13; ++q) S.nb[h][q + 1] = index({home[0] + fw[q][0], home[1] + fw[q][1], home[2] + fw[q][2]});
   }
   S.n_tile = (int)tile.size();
   for (int k = 0; k < S.n_tile; ++k)
@@ -1450,9 +1452,9 @@ int md_get_neighbors(md_system* s, int32_t* count, int32_t* entries) {
       off[k + 1] = off[k] + cs[cell[k] + 1] - cs[cell[k]];
     }
     for (int h = 0; h < S.n_home; ++h) {
-      const int n_h = off[h + 1] - off[h];
+      const int th = S.nb[h][0], n_h = off[th + 1] - off[th];
       for (int kq = 0; kq < (n_h + 3) / 4; ++kq) {
-        const int cl = cls[cell[h]] + kq;
+        const int cl = cls[cell[th]] + kq;
         for (int e = 0; e < nc[cl]; ++e) {
           const unsigned E = lst[(size_t)cl * s->cap + e];
           const int t = (int)(E & 0xffffu);
@@ -1461,7 +1463,7 @@ int md_get_neighbors(md_system* s, int32_t* count, int32_t* entries) {
           const int j = pm[start[kc] + (t - off[kc])];
           for (int u = 0; u < 4; ++u)
             if ((E >> (16 + u)) & 1u) {
-              const int i = pm[start[h] + 4 * kq + u];
+              const int i = pm[start[th] + 4 * kq + u];
               nb[i].push_back(j);
               nb[j].push_back(i);
             }

@@ -81,8 +81,8 @@ constexpr int kNhDoubles = 18;
 struct Tile { int start, len, rep, pad; };
 
 // Regions of up to 3 x 3 x 1 cells (the work unit of the list build and LJ
-// kernels) and their tiles: the region's home cells, then the cells their
-// 13 forward neighbours add, as offsets from the region's origin cell.
+// kernels) and their tiles: the region's home cells and the cells their 13
+// forward neighbours add, as offsets from the region's origin cell.
 constexpr int kMaxTileCells = 64;   // 44 cells for a 3 x 3 x 1 region
 constexpr int kMaxHome = 9;
 struct RegionShape {
