@@ -202,8 +202,10 @@ __device__ __forceinline__ void persistent_done(int* work, int blocks) {
 // consecutive candidates in packed FP32 (three 8-byte loads and six packed
 // operations for both), the forward cells are five runs of consecutive tile
 // cells (13 loops over 46 atoms each left 28% of the lanes without work), and the
-// four-atom test is packed as well.  1.5M sites: 780 -> 655 us.
-constexpr int kBuildQueue = 128;   // a ring: at most 31 + 64 candidates wait
+// four-atom test is packed as well, and the runs' bounds are looked up once a
+// block.  1.5M sites: 780 -> 592 us.
+constexpr int kBuildQueue = 256;   // a ring: at most 31 + 64 candidates wait (why not 128: at the barrier below)
+constexpr int kBuildPad = 64;      // places past each of the tile's arrays that a round of 64 candidates may read
 
 // is atom b of a molecule a 1-2 or 1-3 neighbour of atom a (general type)?
 __device__ __forceinline__ bool topo_excluded(int a, int b, const TopoDev& tp) {
@@ -298,13 +300,14 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_cl_build(const float4* __rest
   extern __shared__ __align__(16) unsigned char smem[];
   BuildTile B;
   B.x = reinterpret_cast<float*>(smem);
-  B.y = B.x + tile_cap;
-  B.z = B.y + tile_cap;
-  B.tag = reinterpret_cast<int*>(B.z + tile_cap);
+  B.y = B.x + tile_cap + kBuildPad;
+  B.z = B.y + tile_cap + kBuildPad;
+  B.tag = reinterpret_cast<int*>(B.z + tile_cap + kBuildPad);
   __shared__ RegTile T;
-  __shared__ int queue[NT / 32][kBuildQueue];
+  __shared__ unsigned short queue[NT / 32][kBuildQueue];   // places of the tile (fewer than 2^16)
+  __shared__ int2 runs[5 * kMaxHome];   // first and end tile atom of the forward runs of each home cell
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int* qw = queue[warp];
+  unsigned short* qw = queue[warp];
   wait_for_predecessor();
   const WorkItem item = items[blockIdx.x];
   const RegionShape& S = shapes[item.shape];
@@ -320,6 +323,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_cl_build(const float4* __rest
       ncl[T.cl0[h] + k] = 0;
     }
     return;
+  }
+  if (threadIdx.x < 5 * T.n_home) {
+    const int h = threadIdx.x / 5, run = threadIdx.x % 5;
+    runs[threadIdx.x] = make_int2(T.off[S.nb[h][3 * run + 1]], T.off[S.nb[h][min(3 * run + 3, 13)] + 1]);
   }
   stage_build_tile<NT>(T, item.need, pos, tag, B);
   const float rl2 = R.rlist2u;
@@ -387,23 +394,26 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_cl_build(const float4* __rest
     int qn = 0, head = 0;   // waiting candidates: ring places head .. head + qn - 1
 #pragma unroll 1
     for (int run = 0; run < 5; ++run) {
-      const int t_beg = T.off[S.nb[h][3 * run + 1]], t_end = T.off[S.nb[h][min(3 * run + 3, 13)] + 1];
-      for (int t0 = t_beg & ~1; t0 < t_end; t0 += 64) {
-        const int t = t0 + 2 * lane;
-        bool pass0 = false, pass1 = false;
-        if (t < t_end) {
-          const float2 dx = __fadd2_rn(*reinterpret_cast<const float2*>(B.x + t), ncx),
-                       dy = __fadd2_rn(*reinterpret_cast<const float2*>(B.y + t), ncy),
-                       dz = __fadd2_rn(*reinterpret_cast<const float2*>(B.z + t), ncz);
-          const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
-          pass0 = r2.x < reach2 && t >= t_beg;
-          pass1 = r2.y < reach2 && t + 1 < t_end;
-        }
+      const int2 r = runs[5 * h + run];
+      const unsigned len = (unsigned)(r.y - r.x);
+      // d: the lane's first candidate from the run's start (the tile arrays are
+      // padded: reads past the end are in bounds and fail the range test)
+      int d = (r.x & ~1) - r.x + 2 * lane;
+#pragma unroll 1
+      for (; d - 2 * lane < (int)len; d += 64) {
+        const int t = r.x + d;
+        const float2 dx = __fadd2_rn(*reinterpret_cast<const float2*>(B.x + t), ncx),
+                     dy = __fadd2_rn(*reinterpret_cast<const float2*>(B.y + t), ncy),
+                     dz = __fadd2_rn(*reinterpret_cast<const float2*>(B.z + t), ncz);
+        const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
+        const bool pass0 = r2.x < reach2 && (unsigned)d < len, pass1 = r2.y < reach2 && (unsigned)(d + 1) < len;
         const unsigned b0 = __ballot_sync(0xffffffffu, pass0), b1 = __ballot_sync(0xffffffffu, pass1);
         const int at = head + qn + __popc(b0 & lt) + __popc(b1 & lt);
-        if (pass0) qw[at & (kBuildQueue - 1)] = t;
-        if (pass1) qw[(at + (pass0 ? 1 : 0)) & (kBuildQueue - 1)] = t + 1;
+        if (pass0) qw[at & (kBuildQueue - 1)] = (unsigned short)t;
+        if (pass1) qw[(at + (pass0 ? 1 : 0)) & (kBuildQueue - 1)] = (unsigned short)(t + 1);
         qn += __popc(b0) + __popc(b1);
+        // one barrier a round: the 64 places that a flush reads lie before head,
+        // and the next round writes at most 94 past it (256 in the ring)
         __syncwarp();
         while (qn >= 32) {
           const int tq = qw[(head + lane) & (kBuildQueue - 1)];
@@ -411,9 +421,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_cl_build(const float4* __rest
           head += 32;
           qn -= 32;
         }
-        __syncwarp();
       }
     }
+    __syncwarp();
     if (qn > 0) {
       unsigned m = 0u;
       int tq = 0;
@@ -1047,7 +1057,7 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_cl_force(
 }
 
 // ===================================================================== launch
-size_t cl_build_smem(int tile_cap) { return (size_t)tile_cap * sizeof(float4); }
+size_t cl_build_smem(int tile_cap) { return (size_t)(tile_cap + kBuildPad) * sizeof(float4); }
 size_t cl_force_smem(int tile_cap) { return (size_t)tile_cap * (sizeof(float4) + 3 * sizeof(int)); }
 
 void launch_cl_build(const float4* pos, const int* tag, const int* cell_start, const int* cl_start,
