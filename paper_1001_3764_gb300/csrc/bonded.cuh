@@ -159,4 +159,87 @@ __device__ __forceinline__ void bond_vector(const T (&a)[3], const T (&c)[3], co
   }
 }
 
+// ---------------------------------------------------------------- general molecules
+// The terms of a bond-graph topology, shared by the fused step kernel
+// (k_step.cu) and k_bonded_generic (k_force.cu).  x holds the FP64 positions as
+// three rows of N; add(i, f) adds f to the force of atom i.  The separations are
+// minimum-image differences rounded to FP32, as in the chain kernels.
+
+// FP32 separation x_b - x_a
+__device__ __forceinline__ f3 sep_ab(const double* x, int N, int a, int b, const RepDev& R) {
+  const double dx = bond_diff(x[a], x[b], R.L, R.half_L);
+  const double dy = bond_diff(x[N + a], x[N + b], R.L, R.half_L);
+  const double dz = bond_diff(x[2 * N + a], x[2 * N + b], R.L, R.half_L);
+  return mk(d2f_rn_int(dx), d2f_rn_int(dy), d2f_rn_int(dz));
+}
+
+// bond (i, j), Eq. (4); |x_j - x_i|^2 - b0^2 in FP64
+template <bool ENERGY, class Add>
+__device__ __forceinline__ void bond_term(const double* x, int N, int i, int j, const RepDev& R, const ForceParams& fp,
+                                          Add add, float& Eb, float (&W)[6]) {
+  const f3 b = sep_ab(x, N, i, j, R);
+  const double dx = bond_diff(x[i], x[j], R.L, R.half_L), dy = bond_diff(x[N + i], x[N + j], R.L, R.half_L);
+  const double dz = bond_diff(x[2 * N + i], x[2 * N + j], R.L, R.half_L);
+  const float D = d2f_rn_int(fma(dx, dx, fma(dy, dy, fma(dz, dz, -fp.b0sq))));
+  const float r = sqrtf(dot(b, b));
+  const float dr = D / (r + fp.b0);   // r - b0 without cancellation
+  const f3 fb = (fp.kb * dr / r) * b; // force on a
+  add(i, fb);
+  add(j, -fb);
+  if (ENERGY) { Eb += 0.5f * fp.kb * dr * dr; add_vir(W, b, -fb); }
+}
+
+// angle (i, jb, jc), vertex jb, Eq. (5)
+template <bool ENERGY, class Add>
+__device__ __forceinline__ void angle_term(const double* x, int N, int i, int jb, int jc, const RepDev& R,
+                                           const ForceParams& fp, Add add, float& Ea, float (&W)[6]) {
+  const f3 u = sep_ab(x, N, jb, i, R), w = sep_ab(x, N, jb, jc, R);
+  const float lu = sqrtf(dot(u, u)), lw = sqrtf(dot(w, w));
+  const f3 cr = cross(u, w);
+  const float sn = sqrtf(dot(cr, cr)), cs = dot(u, w);
+  const float th = atan2f(sn, cs);
+  const float dth = th - fp.theta0;
+  const float inv = 1.0f / (lu * lw);
+  const float sin_t = sn * inv, cos_t = cs * inv;
+  f3 fa = mk(0.f, 0.f, 0.f), fc = fa;
+  if (sin_t > 1e-6f) {
+    const float g = fp.ka * dth / sin_t;
+    const f3 uh = (1.0f / lu) * u, wh = (1.0f / lw) * w;
+    fa = (g / lu) * (wh - cos_t * uh);
+    fc = (g / lw) * (uh - cos_t * wh);
+  }
+  add(i, fa);
+  add(jc, fc);
+  add(jb, -(fa + fc));
+  if (ENERGY) { Ea += 0.5f * fp.ka * dth * dth; add_vir(W, u, fa); add_vir(W, w, fc); }
+}
+
+// dihedral (i, jb, jc, jd), Eq. (6), IUPAC phi
+template <bool ENERGY, class Add>
+__device__ __forceinline__ void dihedral_term(const double* x, int N, int i, int jb, int jc, int jd, const RepDev& R,
+                                              const ForceParams& fp, Add add, float& Ed, float (&W)[6]) {
+  const f3 b1 = sep_ab(x, N, i, jb, R), b2 = sep_ab(x, N, jb, jc, R), b3 = sep_ab(x, N, jc, jd, R);
+  const f3 mm = cross(b1, b2), nn = cross(b2, b3);
+  const float lb2 = sqrtf(dot(b2, b2)), m2 = dot(mm, mm), n2 = dot(nn, nn);
+  const float phi = atan2f(lb2 * dot(b1, nn), dot(mm, nn));
+  const float arg = (float)fp.n_mult * phi - fp.phis;
+  float sa, ca;
+  sincosf(arg, &sa, &ca);
+  if (m2 > 1e-24f && n2 > 1e-24f) {
+    const float dEdphi = -fp.kphi * (float)fp.n_mult * sa;
+    const float cam = -lb2 / m2, cdn = lb2 / n2;
+    const float cbm = lb2 / m2 + dot(b1, b2) / (lb2 * m2), cbn = dot(b2, b3) / (lb2 * n2);
+    const f3 ga = cam * mm, gd = cdn * nn, gb = cbm * mm + cbn * nn;
+    const f3 gc = -(ga + gb + gd);
+    const f3 f1 = -dEdphi * ga, f2 = -dEdphi * gb, f3v = -dEdphi * gc;
+    const f3 f4 = -(f1 + f2 + f3v);
+    add(i, f1);
+    add(jb, f2);
+    add(jc, f3v);
+    add(jd, f4);
+    if (ENERGY) { add_vir(W, b1, f2); add_vir(W, b1 + b2, f3v); add_vir(W, b1 + b2 + b3, f4); }
+  }
+  if (ENERGY) Ed += fp.kphi * (1.0f + ca);
+}
+
 }  // namespace mdg

@@ -29,10 +29,9 @@
 // flags atoms that moved more than skin/2 since the last rebin.
 //
 // The update of an atom and the thermostats' sums are in integrate.cuh,
-// shared with the fused step kernel of linear chains (k_step.cu), which does
-// every inner and closing update of a block of steps; this kernel opens a
-// block, reads out the kinetic energy, and does all updates of general
-// molecules.
+// shared with the fused step kernels (k_step.cu), which do every inner and
+// closing update of a block of steps; this kernel opens a block and reads out
+// the kinetic energy.
 #include <type_traits>
 
 #include "integrate.cuh"
@@ -60,7 +59,7 @@ __global__ void __launch_bounds__(kIntBlock) k_integrate(void* __restrict__ xv, 
   const Tile t = tiles[blockIdx.x];
   const RepDev& R = reps[t.rep];
   const int i = t.start + threadIdx.x;
-  if (MODE == kKickOnly ? !lj_runs(gate) : !drift_runs(gate)) return;
+  if (!drift_runs(gate)) return;
   AtomOut o;
   o.ke = 0.0;
   o.mom[0] = o.mom[1] = o.mom[2] = 0.0;
@@ -77,7 +76,7 @@ __global__ void __launch_bounds__(kIntBlock) k_integrate(void* __restrict__ xv, 
     }
     int cc = 0;
     float4 r0 = make_float4(0.f, 0.f, 0.f, 0.f);
-    constexpr bool kDrift = MODE == kKickDrift || MODE == kKickKickDrift;
+    constexpr bool kDrift = MODE == kKickDrift;
     if (kDrift) {
       cc = cellc[i];
       r0 = ref[i];
@@ -85,16 +84,12 @@ __global__ void __launch_bounds__(kIntBlock) k_integrate(void* __restrict__ xv, 
       for (int a = 0; a < 3; ++a) xi[a] = x[a * N + i];
     }
     integrate_atom<MIXED, MODE, KE, TH>(F, xi, vi, img, i, N, type, cc, r0, R, t.rep, fp, lam, o);
-    if (MODE == kKickOnly || kDrift) {
-#pragma unroll
-      for (int a = 0; a < 3; ++a) v[a * N + i] = vi[a];
-    }
     if (kDrift) {
 #pragma unroll
-      for (int a = 0; a < 3; ++a) x[a * N + i] = xi[a];
-      if (flj_next) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) flj_next[(size_t)a * Npad + i] = 0ll;
+      for (int a = 0; a < 3; ++a) {
+        v[a * N + i] = vi[a];
+        x[a * N + i] = xi[a];
+        flj_next[(size_t)a * Npad + i] = 0ll;
       }
       if (o.moved) report_move(mr, gate.j, flags);
       if (o.bad) atomicOr(flags, kFlagNaN);
@@ -122,13 +117,6 @@ static void launch_int_t(IntegMode mode, int th, const StepArgs& a, const ForceP
     if (th == 2) MDG_INT(kKickDrift, true, 2);
     else if (th == 1) MDG_INT(kKickDrift, true, 1);
     else MDG_INT(kKickDrift, false, 0);
-  } else if (mode == kKickKickDrift) {
-    if (th == 2) MDG_INT(kKickKickDrift, true, 2);
-    else if (th == 1) MDG_INT(kKickKickDrift, true, 1);
-    else MDG_INT(kKickKickDrift, false, 0);
-  } else if (mode == kKickOnly) {
-    if (th == 2) MDG_INT(kKickOnly, false, 2);
-    else MDG_INT(kKickOnly, false, 0);
   } else {
     MDG_INT(kKineticOnly, true, 0);
   }

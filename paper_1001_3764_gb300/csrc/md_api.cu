@@ -49,7 +49,7 @@ struct md_system {
   ForceParams fp{};
   std::vector<RepDev> reps_h;
   std::vector<Tile> t_int;                   // kIntTile atoms each
-  std::vector<Tile> t_chain;                 // whole chains (fused step kernel; empty for general molecules)
+  std::vector<Tile> t_chain;                 // whole chains or molecules (fused step kernels)
   std::vector<double> T0;
   // memory
   char* base = nullptr;
@@ -110,6 +110,7 @@ struct md_system {
   int disp = MD_DISP_REBUILD;                // what a displacement beyond skin/2 does
   std::vector<unsigned char> mtype_h;        // type of each atom of the molecule
   std::vector<int> t_boff, t_bat, t_aoff, t_aat, t_doff, t_dat, t_xoff, t_xat;   // term and exclusion lists
+  std::vector<ushort4> t_terms;
   unsigned char* mtype = nullptr;            // device copies
   TopoDev topo{};
   bool fresh = false;                        // bins, list and forces are those of the current positions
@@ -393,6 +394,16 @@ static int build_topology(md_system* s, const md_topology* t) {
   // the CSR offsets of angles and dihedrals count ints; the kernels index terms
   for (int& o : s->t_aoff) o /= 2;
   for (int& o : s->t_doff) o /= 3;
+  auto terms = [&](const std::vector<std::vector<int>>& v, size_t m) {
+    for (int a = 0; a < n; ++a)
+      for (size_t q = 0; q < v[a].size(); q += m)
+        s->t_terms.push_back({(unsigned short)a, (unsigned short)v[a][q], (unsigned short)(m > 1 ? v[a][q + 1] : 0),
+                              (unsigned short)(m > 2 ? v[a][q + 2] : 0)});
+  };
+  s->t_terms.clear();
+  terms(ob, 1);
+  terms(oa, 2);
+  terms(od, 3);
   return MD_OK;
 }
 
@@ -485,11 +496,9 @@ static int configure(md_system* s, const md_desc* d) {
     for (int o = 0; o < q.n_atoms; o += kIntTile) s->t_int.push_back(Tile{q.atom_off + o, std::min(kIntTile, q.n_atoms - o), r, 0});
     q.n_tiles = (int)s->t_int.size() - q.tile_off;
     q.ctile_off = (int)s->t_chain.size();
-    if (!s->generic) {
-      const int per = step_chains_per_block(s->S) * s->S;
-      for (int o = 0; o < q.n_atoms; o += per)
-        s->t_chain.push_back(Tile{q.atom_off + o, std::min(per, q.n_atoms - o), r, 0});
-    }
+    const int per = step_chains_per_block(s->S, s->generic) * s->S;
+    for (int o = 0; o < q.n_atoms; o += per)
+      s->t_chain.push_back(Tile{q.atom_off + o, std::min(per, q.n_atoms - o), r, 0});
     q.n_ctiles = (int)s->t_chain.size() - q.ctile_off;
     // chains are locally as dense as a melt even in a sparse box, so the
     // density used for the capacity is at least that of a dense melt
@@ -576,7 +585,11 @@ static size_t plan(md_system* s, char* base) {
     s->topo.a_off = ti(s->t_aoff); s->topo.a_at = ti(s->t_aat);
     s->topo.d_off = ti(s->t_doff); s->topo.d_at = ti(s->t_dat);
     s->topo.x_off = ti(s->t_xoff); s->topo.x_at = ti(s->t_xat);
+    s->topo.terms = (const ushort4*)take(s->t_terms.size() * sizeof(ushort4));
     s->topo.naom = s->S;
+    s->topo.n_bonds = s->t_boff[s->S];
+    s->topo.n_angles = s->t_aoff[s->S];
+    s->topo.n_dihedrals = s->t_doff[s->S];
   }
   return off;
 }
@@ -636,13 +649,10 @@ static void enqueue_bonded(md_system* s, bool energy, const long long* flj, void
 }
 
 // the total force into s->F
-static void enqueue_forces(md_system* s, const StepGate& gate = StepGate{}, const ThermoArgs& thermo = ThermoArgs{}) {
+static void enqueue_forces(md_system* s) {
   cudaMemsetAsync(s->flj[0], 0, 3 * (size_t)s->Npad * sizeof(long long), s->st);
-  prof_mark(s);   // closes the integrate group (integrator, early rebin, clear)
-  enqueue_lj(s, false, s->flj[0], gate, thermo);
-  prof_mark(s);
+  enqueue_lj(s, false, s->flj[0]);
   enqueue_bonded(s, false, s->flj[0], s->F);
-  prof_mark(s);
 }
 
 // energies and virial into lj_part and b_part; the force form's kernels and
@@ -660,46 +670,38 @@ static StepArgs step_args(md_system* s, bool chain_tiles, const long long* flj, 
 }
 
 // Steps first .. k - 1 of a block of k, LJ launch first on (first = 0: from
-// the opening drift), and the closing kick.  Chains: the opening drift clears
-// an LJ buffer, and between LJ launches one kernel does the bonded forces, the
+// the opening drift), and the closing kick.  The opening drift clears an LJ
+// buffer, and between LJ launches one kernel does the bonded forces, the
 // update and the clearing of the other buffer; the last one closes the step
-// and leaves the force.  General molecules: bonded forces and integrator apart.
+// and leaves the force.
 static void enqueue_steps(md_system* s, int k, bool repeat, const MoveReport& mr) {
+  const TopoDev* topo = s->generic ? &s->topo : nullptr;
   for (int j = 0; j < k; ++j) {
     long long* flj = s->flj[j & 1];
     // launched as dependents of the kernel before, but where the profile's event
     // records come in between, and a repeat's first LJ launch: what that reads
     // before its wait is the list build's, its predecessor's
-    const StepGate gate{mr.ctl, j, repeat ? 1 : 0, !s->profile && !s->generic && !(repeat && j == 0)};
+    const StepGate gate{mr.ctl, j, repeat ? 1 : 0, !s->profile && !(repeat && j == 0)};
     if (j == 0 && repeat) {
       // a repeat resumes at an LJ launch
-    } else if (j == 0 || s->generic) {
-      launch_integrate(s->mixed, j == 0 ? kKickDrift : kKickKickDrift, s->thermo,
-                       step_args(s, false, nullptr, s->generic ? nullptr : flj), s->fp, gate, mr, s->st);
+    } else if (j == 0) {
+      launch_integrate(s->mixed, kKickDrift, s->thermo, step_args(s, false, nullptr, flj), s->fp, gate, mr, s->st);
     } else {
-      launch_step(s->mixed, kKickKickDrift, s->thermo, s->S, step_args(s, true, s->flj[(j - 1) & 1], flj), s->fp, gate,
-                  mr, s->st);
+      launch_step(s->mixed, kKickKickDrift, s->thermo, s->S, step_args(s, true, s->flj[(j - 1) & 1], flj), s->fp, topo,
+                  gate, mr, s->st);
       prof_mark(s);   // closes the bonded group (bonded forces and update)
     }
     ThermoArgs thermo{};
     if (s->thermo != MD_NVE)
-      thermo = ThermoArgs{s->n_reps, s->thermo, j > 0 && !s->generic, s->kepart, s->lam, 1.0 - s->dt / s->tau, s->dt};
-    if (s->generic) {
-      enqueue_forces(s, gate, thermo);
-      continue;
-    }
+      thermo = ThermoArgs{s->n_reps, s->thermo, j > 0, s->kepart, s->lam, 1.0 - s->dt / s->tau, s->dt};
     prof_mark(s);   // closes the integrate group
     enqueue_lj(s, false, flj, gate, thermo);
     prof_mark(s);
   }
-  const StepGate gate{mr.ctl, k - 1, repeat ? 1 : 0, !s->profile && !s->generic};
-  if (s->generic) {
-    launch_integrate(s->mixed, kKickOnly, s->thermo, step_args(s, false, nullptr, nullptr), s->fp, gate, mr, s->st);
-  } else {
-    launch_step(s->mixed, kKickOnly, s->thermo, s->S, step_args(s, true, s->flj[(k - 1) & 1], nullptr), s->fp, gate, mr,
-                s->st);
-    prof_mark(s);
-  }
+  const StepGate gate{mr.ctl, k - 1, repeat ? 1 : 0, !s->profile};
+  launch_step(s->mixed, kKickOnly, s->thermo, s->S, step_args(s, true, s->flj[(k - 1) & 1], nullptr), s->fp, topo, gate,
+              mr, s->st);
+  prof_mark(s);
   prof_mark(s);
 }
 
@@ -756,9 +758,8 @@ static void enqueue_block(md_system* s, int k, bool rebin = true) {
   cudaGraph_t out = nullptr;
   cudaStreamEndCapture(s->side, &out);
 }
-// chains, per step: LJ and one update; a closing update (an early rebin adds
-// kRebinLaunches).  General molecules: integrate, clear, LJ, two bonded
-static int64_t block_launches(int k, bool generic) { return kRebinLaunches + (generic ? 5LL : 2LL) * k + 1; }
+// per step: LJ and one update; a closing update (an early rebin adds kRebinLaunches)
+static int64_t block_launches(int k) { return kRebinLaunches + 2LL * k + 1; }
 
 // accumulate the event timings of the last block (requires a finished stream)
 static void prof_collect(md_system* s, int k) {
@@ -996,7 +997,8 @@ int md_create(const md_desc* d, md_system** out) {
                              up((void*)s->topo.d_off, s->t_doff.data(), s->t_doff.size() * sizeof(int)) &&
                              up((void*)s->topo.d_at, s->t_dat.data(), s->t_dat.size() * sizeof(int)) &&
                              up((void*)s->topo.x_off, s->t_xoff.data(), s->t_xoff.size() * sizeof(int)) &&
-                             up((void*)s->topo.x_at, s->t_xat.data(), s->t_xat.size() * sizeof(int)))) &&
+                             up((void*)s->topo.x_at, s->t_xat.data(), s->t_xat.size() * sizeof(int)) &&
+                             up((void*)s->topo.terms, s->t_terms.data(), s->t_terms.size() * sizeof(ushort4)))) &&
             up(s->shapes, s->shapes_h.data(), sizeof(RegionShape) * s->shapes_h.size()) &&
             up(s->items, s->items_h.data(), sizeof(WorkItem) * s->items_h.size()) &&
             up(s->tiles_chain, s->t_chain.data(), sizeof(Tile) * s->t_chain.size()) &&
@@ -1526,7 +1528,7 @@ int md_profile_reset(md_system* s) {
 int64_t md_launches_per_call(md_system* s, int64_t n) {
   if (!s || n < 0) return 0;
   const int64_t full = n / s->R, rem = n % s->R;
-  return full * block_launches(s->R, s->generic) + (rem ? block_launches((int)rem, s->generic) : 0);
+  return full * block_launches(s->R) + (rem ? block_launches((int)rem) : 0);
 }
 
 // ------------------------------------------------------------------ autotuner

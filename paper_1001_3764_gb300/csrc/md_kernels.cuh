@@ -280,7 +280,9 @@ struct TopoDev {
   const int *a_off, *a_at;        // a_at[2q..2q+1] = (b, c)
   const int *d_off, *d_at;        // d_at[3q..3q+2] = (b, c, d)
   const int *x_off, *x_at;        // exclusions of a: x_at[x_off[a] .. x_off[a+1])
-  int naom, pad;
+  // every term as (a, b, c, d): n_bonds bonds, then the angles, then the dihedrals
+  const ushort4* terms;
+  int naom, n_bonds, n_angles, n_dihedrals;
 };
 
 struct F4i { long long x, y, z, w; };   // fixed-point force, 32 B
@@ -435,8 +437,7 @@ void launch_chain_observables(bool mixed, const void* x, int N, const RepDev* re
                               const ForceParams& fp, int n_chains_total, double* ree, double* rg2,
                               unsigned long long* trans, cudaStream_t st);
 // Arguments common to the integrator and the fused step kernel.  flj: the LJ
-// force of the step; flj_next: the buffer cleared for the next one (may be
-// null in launch_integrate).
+// force of the step; flj_next: the buffer cleared for the next one.
 struct StepArgs {
   void *x, *v;
   int* img;
@@ -459,13 +460,14 @@ struct StepArgs {
 // integrator's (RepDev::tile_off, n_tiles)
 void launch_integrate(bool mixed, IntegMode mode, int thermostat, const StepArgs& a, const ForceParams& fp,
                       const StepGate& gate, const MoveReport& mr, cudaStream_t st);
-// bonded forces and update of linear chains (k_step.cu): mode kKickKickDrift,
-// or kKickOnly, which also writes the force F; tiles hold whole chains
-// (RepDev::ctile_off, n_ctiles), step_chains_per_block(sites) of them at most
-int step_chains_per_block(int sites);
+// bonded forces and update of linear chains, or with topo of general molecules
+// (k_step.cu): mode kKickKickDrift, or kKickOnly, which also writes the force F;
+// tiles hold whole molecules (RepDev::ctile_off, n_ctiles),
+// step_chains_per_block(sites) of them at most
+int step_chains_per_block(int sites, bool generic);
 cudaError_t step_kernels_init();
 void launch_step(bool mixed, IntegMode mode, int thermostat, int sites, const StepArgs& a, const ForceParams& fp,
-                 const StepGate& gate, const MoveReport& mr, cudaStream_t st);
+                 const TopoDev* topo, const StepGate& gate, const MoveReport& mr, cudaStream_t st);
 // kinetic energy of every replica after a launch_integrate(kKineticOnly)
 void launch_kinetic(const double* kepart, const RepDev* reps, int n_reps, const ForceParams& fp, double* ke_out,
                     cudaStream_t st);
