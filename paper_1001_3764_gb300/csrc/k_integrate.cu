@@ -357,23 +357,21 @@ void launch_chain_observables(bool mixed, const void* x, int N, const RepDev* re
 }
 
 // ------------------------------------------------------------------ output state
-// SoA state -> AoS FP64 positions, velocities and image counters in the
-// staging buffer (one DMA each to the caller afterwards).
+// SoA state -> AoS FP64 positions, velocities and image counters (null: not
+// wanted).  One element of the AoS arrays per thread: whole lines are written (the reads, a
+// third of a line per row, meet in L1).  With an atom per thread the writes were
+// 24 bytes apart (1.5M sites: 38.6 -> 34.9 us).
 template <bool MIXED>
 __global__ void __launch_bounds__(256) k_egress_state(const void* __restrict__ xv, const void* __restrict__ vv,
                                                       const int* __restrict__ img, int N, double* __restrict__ pos,
                                                       double* __restrict__ vel, int* __restrict__ im) {
   using T = typename std::conditional<MIXED, double, float>::type;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  const T* x = reinterpret_cast<const T*>(xv);
-  const T* v = reinterpret_cast<const T*>(vv);
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    pos[3 * (size_t)i + a] = (double)x[a * N + i];
-    vel[3 * (size_t)i + a] = (double)v[a * N + i];
-    im[3 * (size_t)i + a] = img[a * N + i];
-  }
+  const unsigned e = blockIdx.x * blockDim.x + threadIdx.x;   // 3 N < 2^28
+  if (e >= 3u * (unsigned)N) return;
+  const unsigned i = e / 3u, q = (e - 3u * i) * (unsigned)N + i;
+  if (pos) pos[e] = (double)reinterpret_cast<const T*>(xv)[q];
+  if (vel) vel[e] = (double)reinterpret_cast<const T*>(vv)[q];
+  if (im) im[e] = img[q];
 }
 
 // total force (int64 fixed point or FP32) -> AoS FP64 kJ/mol/nm
@@ -396,8 +394,8 @@ __global__ void __launch_bounds__(256) k_egress_forces(const void* __restrict__ 
 void launch_egress_state(bool mixed, const void* x, const void* v, const int* img, int N, double* pos, double* vel,
                          int* im, cudaStream_t st) {
   if (N <= 0) return;
-  if (mixed) k_egress_state<true><<<(N + 255) / 256, 256, 0, st>>>(x, v, img, N, pos, vel, im);
-  else k_egress_state<false><<<(N + 255) / 256, 256, 0, st>>>(x, v, img, N, pos, vel, im);
+  if (mixed) k_egress_state<true><<<(3 * N + 255) / 256, 256, 0, st>>>(x, v, img, N, pos, vel, im);
+  else k_egress_state<false><<<(3 * N + 255) / 256, 256, 0, st>>>(x, v, img, N, pos, vel, im);
 }
 
 void launch_egress_forces(bool mixed, const void* F, int N, double scale, double* out, cudaStream_t st) {
@@ -408,7 +406,7 @@ void launch_egress_forces(bool mixed, const void* F, int N, double scale, double
 
 // ------------------------------------------------------------------ input state
 template <bool MIXED>
-__global__ void __launch_bounds__(kIntBlock) k_ingest(const double* __restrict__ stage, int N,
+__global__ void __launch_bounds__(kIntBlock) k_ingest(const double* __restrict__ pos, const double* __restrict__ vel, int N,
                                                       const Tile* __restrict__ tiles, const RepDev* __restrict__ reps,
                                                       void* __restrict__ xv, void* __restrict__ vv,
                                                       int* __restrict__ img, unsigned* __restrict__ flags) {
@@ -422,8 +420,8 @@ __global__ void __launch_bounds__(kIntBlock) k_ingest(const double* __restrict__
   bool bad = false;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    double xa = stage[3 * (size_t)i + a];
-    const double va = stage[3 * (size_t)N + 3 * (size_t)i + a];
+    double xa = pos[3 * (size_t)i + a];
+    const double va = vel[3 * (size_t)i + a];
     bad |= !isfinite(xa) || !isfinite(va);
     xa -= R.L * floor(xa / R.L);
     if (!(xa < R.L) || xa < 0.0) xa = 0.0;
@@ -435,11 +433,11 @@ __global__ void __launch_bounds__(kIntBlock) k_ingest(const double* __restrict__
   if (bad) atomicOr(flags, kFlagBadInput);
 }
 
-void launch_ingest(bool mixed, const double* stage, int N, const Tile* tiles, int n_tiles, const RepDev* reps,
+void launch_ingest(bool mixed, const double* pos, const double* vel, int N, const Tile* tiles, int n_tiles, const RepDev* reps,
                    void* x, void* v, int* img, unsigned* flags, cudaStream_t st) {
   if (n_tiles <= 0) return;
-  if (mixed) k_ingest<true><<<n_tiles, kIntBlock, 0, st>>>(stage, N, tiles, reps, x, v, img, flags);
-  else k_ingest<false><<<n_tiles, kIntBlock, 0, st>>>(stage, N, tiles, reps, x, v, img, flags);
+  if (mixed) k_ingest<true><<<n_tiles, kIntBlock, 0, st>>>(pos, vel, N, tiles, reps, x, v, img, flags);
+  else k_ingest<false><<<n_tiles, kIntBlock, 0, st>>>(pos, vel, N, tiles, reps, x, v, img, flags);
 }
 
 }  // namespace mdg

@@ -422,12 +422,12 @@ void launch_bonded(bool mixed, bool energy, const void* x, const uint16_t* site,
 
 // ---------------------------------------------------------------- integration
 enum IntegMode { kKickDrift = 0, kKickKickDrift = 1, kKickOnly = 2, kKineticOnly = 3 };
-// Input state from a staging copy of the caller's arrays (x,y,z per atom:
-// positions, then velocities): check, wrap into [0, L), write the SoA state
-// and clear the image counters, on the integrator's tiles.
-void launch_ingest(bool mixed, const double* stage, int N, const Tile* tiles, int n_tiles, const RepDev* reps,
+// Input state from the caller's arrays or a staging copy of them (x,y,z per
+// atom): check, wrap into [0, L), write the SoA state and clear the image
+// counters, on the integrator's tiles.
+void launch_ingest(bool mixed, const double* pos, const double* vel, int N, const Tile* tiles, int n_tiles, const RepDev* reps,
                    void* x, void* v, int* img, unsigned* flags, cudaStream_t st);
-// AoS FP64 copies of the state / total force in device memory (for one DMA to the caller)
+// AoS FP64 copies of the state (null: not wanted) / total force in device memory
 void launch_egress_state(bool mixed, const void* x, const void* v, const int* img, int N, double* pos, double* vel,
                          int* im, cudaStream_t st);
 void launch_egress_forces(bool mixed, const void* F, int N, double scale, double* out, cudaStream_t st);
