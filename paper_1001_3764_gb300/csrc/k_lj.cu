@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_cl_build(const float4* __rest
   const WorkItem item = items[blockIdx.x];
   const RegionShape& S = shapes[item.shape];
   const RepDev& R = reps[item.rep];
-  if (blockIdx.x == 0 && threadIdx.x == 0) *n_tasks = 0;   // for k_cl_rank
+  if (blockIdx.x == 0 && threadIdx.x < 2) n_tasks[threadIdx.x] = 0;   // for k_cl_rank
   region_setup(T, item, S, cells, cell_start, cl_start);
   const int total = T.off[T.n_tile], q_end = T.ncl[item.h1], q_first = T.ncl[item.h0] + item.part;
   if (total > tile_cap) {
@@ -910,7 +910,8 @@ __device__ __forceinline__ void cell_energy(const RegTile& T, const WorkItem& it
 // The order in which the force kernel takes an item's clusters, made once per
 // list build (it was made in every launch: 3 us of a block's 26): longest
 // list first, so that warps that take the last clusters finish soon and the
-// clusters that share a warp have similar lengths.  Cluster q's key is
+// clusters that share a warp have similar lengths.  An item whose tile exceeds
+// the force kernel's usual tile (lj_cap) is noted in `big`.  Cluster q's key is
 // (list length << 9) | (511 - q), unique (q < 512) so that ties go to the
 // lower index; its rank is the number of larger keys (four keys per shared
 // load, the slots past nq hold -1).  The chain-end bits tell which of the
@@ -924,7 +925,8 @@ __global__ void __launch_bounds__(kRankThreads) k_cl_rank(const float4* __restri
                                                           const WorkItem* __restrict__ items,
                                                           const RegionShape* __restrict__ shapes,
                                                           const int* __restrict__ ncl, ClusterTask* __restrict__ tasks,
-                                                          int* __restrict__ task_base, int* __restrict__ n_tasks) {
+                                                          int* __restrict__ task_base, int* __restrict__ n_tasks,
+                                                          int lj_cap, int* __restrict__ big) {
   __shared__ RegTile T;
   __shared__ __align__(16) int s_key[kRegionClusterCap];
   __shared__ int base;
@@ -933,7 +935,10 @@ __global__ void __launch_bounds__(kRankThreads) k_cl_rank(const float4* __restri
   region_setup(T, item, shapes[item.shape], cells, cell_start, cl_start);
   const int q_first = T.ncl[item.h0], nq = T.ncl[item.h1] - q_first;
   if (T.ncl[T.n_home] > kRegionClusterCap) return;   // reported by the force kernel
-  if (threadIdx.x == 0) task_base[blockIdx.x] = base = atomicAdd(n_tasks, nq);
+  if (threadIdx.x == 0) {
+    task_base[blockIdx.x] = base = atomicAdd(n_tasks, nq);
+    if (T.off[T.n_tile] > lj_cap) big[atomicAdd(n_tasks + 1, 1)] = blockIdx.x;
+  }
   for (int q = threadIdx.x; q < ((nq + 3) & ~3); q += kRankThreads) {
     int key = -1;
     if (q < nq) {
@@ -965,18 +970,20 @@ __global__ void __launch_bounds__(kRankThreads) k_cl_rank(const float4* __restri
 }
 
 // One block per work item (grid schedule), or a fixed grid whose blocks take
-// items from a device counter (persistent schedule).  The block stages
+// items from a device counter (persistent schedule), or the items of a list
+// dealt out over the grid (those whose tile does not fit the first launch's shared
+// memory: BigTiles).  The block stages
 // the tile, its warps take tasks of 32/LP clusters from a shared counter
 // (longest lists first), and after a barrier the block flushes the tile's
 // accumulators.
-template <bool ENERGY, int NT, int LP, bool EXACT = false>
+template <bool ENERGY, int NT, int LP, bool EXACT = false, bool BIG = false>
 __global__ void __launch_bounds__(NT, 768 / NT) k_cl_force(
     const float4* __restrict__ pos, const int* __restrict__ cell_start, const int* __restrict__ cl_start,
     const int* __restrict__ cells, const WorkItem* __restrict__ items, int n_items,
     const RegionShape* __restrict__ shapes, const RepDev* __restrict__ reps, const unsigned* __restrict__ list,
     const ClusterTask* __restrict__ tasks, const int* __restrict__ task_base, int cap,
     int tile_cap, const ForceParams fp, long long* __restrict__ flj, int Npad, double* __restrict__ epart,
-    unsigned* __restrict__ flags, int persistent, int* __restrict__ work, const StepGate gate,
+    unsigned* __restrict__ flags, int persistent, int* __restrict__ work, const BigTiles big, const StepGate gate,
     const ThermoArgs thermo) {
   constexpr int CPW = 32 / LP;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -1003,7 +1010,13 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_cl_force(
     }
   }
   for (int it = 0;; ++it) {
-    const int r = next_region(persistent != 0, it, (int)blockIdx.x - thermo.n_blocks, work, &sh_r);
+    int r;
+    if constexpr (BIG) {
+      const int q = (int)blockIdx.x + it * (int)gridDim.x;
+      r = q < *big.n_ids ? big.ids[q] : -1;
+    } else {
+      r = next_region(persistent != 0, it, (int)blockIdx.x - thermo.n_blocks, work, &sh_r);
+    }
     if (r < 0 || r >= n_items) break;
     const WorkItem item = items[r];
     const RegionShape& S = shapes[item.shape];
@@ -1033,7 +1046,9 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_cl_force(
       }
     }
     if (!fits) {
-      if (threadIdx.x == 0) atomicOr(flags, kFlagNbrOverflow);
+      // left to the launch for large tiles, or too large for the list build as well
+      if (threadIdx.x == 0 && (total > big.tile_cap || T.ncl[T.n_home] > kRegionClusterCap))
+        atomicOr(flags, kFlagNbrOverflow);
     } else {
       tile_issue<NT>(T, item.need, pos, sp);
       tile_finish<NT>(T, item.need, sp);   // ends with a barrier
@@ -1086,32 +1101,38 @@ void launch_cl_build(const float4* pos, const int* tag, const int* cell_start, c
 
 void launch_cl_rank(const float4* pos, const int* cell_start, const int* cl_start, const int* cells,
                     const WorkItem* items, int n_items, const RegionShape* shapes, const int* ncl, ClusterTask* tasks,
-                    int* task_base, int* n_tasks, bool dep, cudaStream_t st) {
+                    int* task_base, int* n_tasks, int lj_cap, int* big, bool dep, cudaStream_t st) {
   if (n_items > 0)
     launch_dependent(dep, k_cl_rank, n_items, kRankThreads, 0, st, pos, cell_start, cl_start, cells, items, shapes, ncl, tasks,
-                                                 task_base, n_tasks);
+                     task_base, n_tasks, lj_cap, big);
 }
 
 void launch_cl_force(bool energy, const float4* pos, const int* cell_start, const int* cl_start,
                      const int* cells, const WorkItem* items, int n_items, const RegionShape* shapes,
                      const RepDev* reps, const unsigned* list, const ClusterTask* tasks, const int* task_base,
                      int cap, int tile_cap, const ForceParams& fp, long long* flj, int Npad, double* epart, unsigned* flags, int block,
-                     int lanes, int persistent_grid, int* work, bool exact, const StepGate& gate,
+                     int lanes, int persistent_grid, int* work, bool exact, const BigTiles& big, const StepGate& gate,
                      const ThermoArgs& thermo, cudaStream_t st) {
   if (n_items <= 0) return;
-  const int grid = (persistent_grid > 0 ? persistent_grid : n_items) + thermo.n_blocks;
+  const int grid = big.ids ? std::min(n_items, kSMs) : (persistent_grid > 0 ? persistent_grid : n_items) + thermo.n_blocks;
   const int pers = persistent_grid > 0;
   // the thermostat blocks use 4 doubles per thread of the tile's memory
   const size_t sm = std::max(cl_force_smem(tile_cap), thermo.n_blocks ? (size_t)block * 4 * sizeof(double) : 0);
-#define MDG_CLF(E, NT, LP, X)                                                                                        \
-  launch_dependent(gate.dep, k_cl_force<E, NT, LP, X>, grid, NT, sm, st, pos, cell_start, cl_start, cells, items,    \
+#define MDG_CLF(E, NT, LP, X, ...)                                                                                   \
+  launch_dependent(gate.dep, k_cl_force<E, NT, LP, X, ##__VA_ARGS__>, grid, NT, sm, st, pos, cell_start, cl_start, cells, items,    \
                    n_items, shapes, reps, list, tasks, task_base, cap, tile_cap, fp, flj, Npad, epart, flags, pers,  \
-                   work, gate, thermo)
+                   work, big, gate, thermo)
 #define MDG_CLF2(NT, LP)                  \
   if (energy) MDG_CLF(true, NT, LP, false); \
   else if (exact) MDG_CLF(false, NT, LP, true); \
   else MDG_CLF(false, NT, LP, false);
-  if (block == 128) {
+#define MDG_CLF_BIG(LP)                                \
+  if (energy) MDG_CLF(true, 768, LP, false, true);     \
+  else if (exact) MDG_CLF(false, 768, LP, true, true); \
+  else MDG_CLF(false, 768, LP, false, true);
+  if (big.ids) {   // one block an SM
+    if (lanes == 8) { MDG_CLF_BIG(8) } else if (lanes == 32) { MDG_CLF_BIG(32) } else { MDG_CLF_BIG(16) }
+  } else if (block == 128) {
     if (lanes == 8) { MDG_CLF2(128, 8) } else if (lanes == 32) { MDG_CLF2(128, 32) } else { MDG_CLF2(128, 16) }
   } else if (block == 768) {
     if (lanes == 8) { MDG_CLF2(768, 8) } else if (lanes == 32) { MDG_CLF2(768, 32) } else { MDG_CLF2(768, 16) }
@@ -1121,6 +1142,7 @@ void launch_cl_force(bool energy, const float4* pos, const int* cell_start, cons
     if (lanes == 8) { MDG_CLF2(256, 8) } else if (lanes == 32) { MDG_CLF2(256, 32) } else { MDG_CLF2(256, 16) }
   }
 #undef MDG_CLF2
+#undef MDG_CLF_BIG
 #undef MDG_CLF
 }
 
@@ -1154,6 +1176,15 @@ cudaError_t tile_kernels_init() {
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_cl_force<E, NT, LP>, cudaFuncAttributeMaxDynamicSharedMemorySize, mf); \
   if (e == cudaSuccess && !E)                                                                                 \
     e = cudaFuncSetAttribute(k_cl_force<false, NT, LP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mf);
+#define MDG_ATTR_BIG(LP)                                                                                         \
+  if (e == cudaSuccess)                                                                                          \
+    e = cudaFuncSetAttribute(k_cl_force<true, 768, LP, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mf);  \
+  if (e == cudaSuccess)                                                                                          \
+    e = cudaFuncSetAttribute(k_cl_force<false, 768, LP, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mf); \
+  if (e == cudaSuccess)                                                                                          \
+    e = cudaFuncSetAttribute(k_cl_force<false, 768, LP, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mf);
+  MDG_ATTR_BIG(8) MDG_ATTR_BIG(16) MDG_ATTR_BIG(32)
+#undef MDG_ATTR_BIG
 #define MDG_ATTR3(E, NT) MDG_ATTR(E, NT, 8) MDG_ATTR(E, NT, 16) MDG_ATTR(E, NT, 32)
   MDG_ATTR3(false, 128) MDG_ATTR3(true, 128) MDG_ATTR3(false, 256) MDG_ATTR3(true, 256)
   MDG_ATTR3(false, 384) MDG_ATTR3(true, 384) MDG_ATTR3(false, 768) MDG_ATTR3(true, 768)
@@ -1166,6 +1197,9 @@ int tile_capacity_max() { return kStageCapMax; }
 
 // 227 KB of shared memory an SM and block, 1 KB of it reserved per block; the
 // force form's tables take 9.9 KB
+int lj_tile_cap_for(int per_sm) {
+  return std::min(kStageCapMax, (int)(((size_t)(228 * 1024) / per_sm - 9872 - 1024) / cl_force_smem(1)) / 32 * 32);
+}
 int lj_tiles_per_sm(int tile_cap) {
   const int n = (int)((size_t)(228 * 1024) / (cl_force_smem(tile_cap) + 9872 + 1024));
   return n < 1 ? 1 : n;

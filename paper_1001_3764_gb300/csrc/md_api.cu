@@ -26,7 +26,6 @@ using namespace mdg;
 namespace {
 
 constexpr int kIntTile = 224;    // atoms per integrator / bonded block (original order)
-constexpr int kSMs = 152;        // streaming multiprocessors of a GB300
 constexpr int kNumProf = 5;      // rebin, neighbour build, integrate, lj, bonded
 constexpr double kKB = 0.0083144626;
 
@@ -78,8 +77,8 @@ struct md_system {
   WorkItem* items = nullptr;
   int n_lj_items = 0, n_build_items = 0;
   ClusterTask* tasks = nullptr;              // each LJ item's clusters in task order, from task_base[item] on
-  int *task_base = nullptr, *n_tasks = nullptr;
-  int tile_cap = 0;
+  int *task_base = nullptr, *n_tasks = nullptr, *big = nullptr;
+  int tile_cap = 0, lj_cap = 0;              // atoms of a tile: list build, first force launch
   int lj_block = 256, persistent_grid = 0;   // persistent_grid > 0: fixed grid for the LJ kernel
   int lj_lanes = 8;                          // lanes per 4-atom cluster in the LJ kernel
   int lj_region = 3;                         // cells per side (x, y) of an LJ / list region
@@ -268,8 +267,31 @@ static void add_items(md_system* s, int region, int rows, int parts) {
 
 // Regions of G x G x 1 cells over every replica (narrower at the high faces
 // when G does not divide M), their tile cells, and the work items.
-static void plan_regions(md_system* s) {
+static void plan_regions(md_system* s, bool grid_schedule) {
   const int G = s->lj_region;
+  // Where two of the largest tiles do not fit an SM's shared memory (cells
+  // above 1.22 nm) but two of the usual ones do: the force kernel's tile is
+  // the one that fits twice, and items of larger tiles are left to a second
+  // launch: those of the replicas whose mean tile is within 12% of it (a melt's
+  // tiles differ by 3%), at most half of the atoms, and dense parts of an
+  // uneven box.  For systems of more rows than resident blocks; smaller ones
+  // are split.  Else one block of 24 warps an SM.  64 replicas, 1.5M sites,
+  // skin 0.12 nm: LJ 484 us with one block an SM, 357 + 19 now.
+  s->lj_cap = s->tile_cap;
+  std::vector<char> large(s->n_reps, 0);
+  if (G == 3 && !s->lj_block && grid_schedule && lj_tiles_per_sm(s->tile_cap) == 1) {
+    const int two = lj_tile_cap_for(2);
+    int64_t rows = 0, large_atoms = 0;
+    for (int r = 0; r < s->n_reps; ++r) {
+      const RepDev& q = s->reps_h[r];
+      const double cell = std::max(q.n_atoms / (q.L * q.L * q.L), 33.0) * q.h * q.h * q.h;
+      large[r] = 1.12 * s->shapes_h.back().n_tile * cell + 64.0 > two;
+      if (large[r]) large_atoms += q.n_atoms;
+      rows += (int64_t)q.M * q.M * ((q.M + G - 1) / G);
+    }
+    if (rows > 2 * kSMs && 2 * large_atoms <= s->N) s->lj_cap = two;
+    else large.assign(s->n_reps, 0);
+  }
   s->regions_h.clear();
   s->region_cells_h.clear();
   for (int r = 0; r < s->n_reps; ++r) {
@@ -310,14 +332,23 @@ static void plan_regions(md_system* s) {
   }
   constexpr int kWhole = 255;
   s->items_h.clear();
-  const int per_sm = lj_tiles_per_sm(s->tile_cap), slots = per_sm * kSMs;
+  const int per_sm = lj_tiles_per_sm(s->lj_cap), slots = per_sm * kSMs;
   const int lj_rows = n_cells <= slots ? 0 : n_rows <= slots ? 1 : kWhole;
   // default block: 24 warps an SM, as two resident blocks where two tiles fit
   // the shared memory of an SM, else as one (cells above 1.22 nm: LJ 565 ->
   // 478 us for 64 replicas at skin 0.12 nm); three of 8 warps for 2 x 2 regions
   if (!s->lj_block) s->lj_block = G == 2 ? 256 : per_sm >= 2 || lj_rows != kWhole ? 384 : 768;
-  for (int q = 0; q < R; ++q)
-    add_items(s, order[q], lj_rows == kWhole && per_sm >= 2 && R <= slots && q >= kSMs ? 1 : lj_rows, 1);
+  // the second launch takes one block of 24 warps an SM: its items are whole
+  // regions, rows or cells, by how many there are
+  int n_large = 0;
+  for (const RegionRef& g : s->regions_h)
+    if (large[g.rep] && g.shape == (int)s->shapes_h.size() - 1) ++n_large;
+  const int large_rows = 9 * n_large <= kSMs ? 0 : 3 * n_large <= kSMs ? 1 : kWhole;
+  for (int q = 0; q < R; ++q) {
+    const RegionRef& g = s->regions_h[order[q]];
+    if (large[g.rep] && g.shape == (int)s->shapes_h.size() - 1) add_items(s, order[q], large_rows, 1);
+    else add_items(s, order[q], lj_rows == kWhole && per_sm >= 2 && R <= slots && q >= kSMs ? 1 : lj_rows, 1);
+  }
   s->n_lj_items = (int)s->items_h.size();
   // The list build gives a warp a cluster at a time (7 us alone), 8 warps a
   // block, 4 blocks an SM: 108 -> 12 us at 1,500 sites (cells in 3 parts),
@@ -517,7 +548,7 @@ static int configure(md_system* s, const md_desc* d) {
   // the densest replica (at least melt density, 33 sites/nm^3) plus 64, in
   // multiples of 128 atoms; a larger tile is reported as MD_EOVERFLOW
   s->tile_cap = std::min(tile_capacity_max(), ((int)std::ceil(1.4 * max_tile + 64.0) + 127) / 128 * 128);
-  plan_regions(s);
+  plan_regions(s, d->schedule == MD_SCHED_GRID);
   s->n_cl_max = (atoms + 3 * cells) / 4 + 1;   // sum of ceil(n_c / 4) over the cells
   s->Npad = (int)((atoms + 31) / 32 * 32);
   // default list capacity (entries per 4-atom cluster): a cluster's list holds
@@ -556,7 +587,8 @@ static size_t plan(md_system* s, char* base) {
   s->items = (WorkItem*)take(sizeof(WorkItem) * s->items_h.size());
   s->tasks = (ClusterTask*)take(sizeof(ClusterTask) * (size_t)s->n_cl_max);
   s->task_base = (int*)take(sizeof(int) * (size_t)s->n_lj_items);
-  s->n_tasks = (int*)take(sizeof(int));
+  s->n_tasks = (int*)take(2 * sizeof(int));
+  s->big = (int*)take(sizeof(int) * (size_t)s->n_lj_items);
   s->list = (unsigned*)take((size_t)s->n_cl_max * s->cap * sizeof(unsigned));
   s->ncl = (int*)take((size_t)s->n_cl_max * sizeof(int));
   s->cl_start = (int*)take((C + 1) * sizeof(int));
@@ -614,7 +646,7 @@ static void enqueue_build(md_system* s, bool dep = false) {
                   s->n_build_items, s->shapes, s->reps, s->list, s->ncl, s->cap, s->tile_cap, s->flags,
                   s->n_tasks, s->generic ? &s->topo : nullptr, dep, s->st);
   launch_cl_rank(s->pos, s->cell_start, s->cl_start, s->region_cells, s->items, s->n_lj_items, s->shapes, s->ncl,
-                 s->tasks, s->task_base, s->n_tasks, true, s->st);
+                 s->tasks, s->task_base, s->n_tasks, s->lj_cap, s->big, true, s->st);
 }
 
 static void enqueue_rebin(md_system* s) {
@@ -634,10 +666,19 @@ static const int kRebinLaunches = 7;   // memset counted as a launch
 
 static void enqueue_lj(md_system* s, bool energy, long long* flj, const StepGate& gate = StepGate{},
                        const ThermoArgs& thermo = ThermoArgs{}) {
-  launch_cl_force(energy, s->pos, s->cell_start, s->cl_start, s->region_cells, s->items, s->n_lj_items, s->shapes,
-                  s->reps, s->list, s->tasks, s->task_base, s->cap, s->tile_cap, s->fp, flj, s->Npad, s->lj_part,
-                  s->flags, s->lj_block, s->lj_lanes, s->persistent_grid, s->work, s->lj_pair_exact, gate,
-                  thermo, s->st);
+  auto launch = [&](int tile_cap, int block, const BigTiles& big, const StepGate& g, const ThermoArgs& t) {
+    launch_cl_force(energy, s->pos, s->cell_start, s->cl_start, s->region_cells, s->items, s->n_lj_items, s->shapes,
+                    s->reps, s->list, s->tasks, s->task_base, s->cap, tile_cap, s->fp, flj, s->Npad, s->lj_part,
+                    s->flags, block, s->lj_lanes, s->persistent_grid, s->work, s->lj_pair_exact, big, g, t, s->st);
+  };
+  launch(s->lj_cap, s->lj_block, BigTiles{nullptr, nullptr, s->tile_cap}, gate, thermo);
+  if (s->lj_cap < s->tile_cap) {
+    // not a dependent: the kernel after it may read what the update before the
+    // first launch left while this one runs, not while that one does
+    StepGate g = gate;
+    g.dep = false;
+    launch(s->tile_cap, 768, BigTiles{s->big, s->n_tasks + 1, s->tile_cap}, g, ThermoArgs{});
+  }
 }
 
 static void enqueue_bonded(md_system* s, bool energy, const long long* flj, void* F_out) {
@@ -759,8 +800,10 @@ static void enqueue_block(md_system* s, int k, bool rebin = true) {
   cudaGraph_t out = nullptr;
   cudaStreamEndCapture(s->side, &out);
 }
-// per step: LJ and one update; a closing update (an early rebin adds kRebinLaunches)
-static int64_t block_launches(int k) { return kRebinLaunches + 2LL * k + 1; }
+// per step: LJ (two launches where tiles are large) and one update; a closing update (an early rebin adds kRebinLaunches)
+static int64_t block_launches(const md_system* s, int k) {
+  return kRebinLaunches + (s->lj_cap < s->tile_cap ? 3LL : 2LL) * k + 1;
+}
 
 // accumulate the event timings of the last block (requires a finished stream)
 static void prof_collect(md_system* s, int k) {
@@ -1574,7 +1617,7 @@ int md_profile_reset(md_system* s) {
 int64_t md_launches_per_call(md_system* s, int64_t n) {
   if (!s || n < 0) return 0;
   const int64_t full = n / s->R, rem = n % s->R;
-  return full * block_launches(s->R) + (rem ? block_launches((int)rem) : 0);
+  return full * block_launches(s, s->R) + (rem ? block_launches(s, (int)rem) : 0);
 }
 
 // ------------------------------------------------------------------ autotuner

@@ -101,6 +101,7 @@ struct __align__(16) WorkItem {
   unsigned char h0, h1, part, parts;
   int pad[2];
 };
+constexpr int kSMs = 152;             // streaming multiprocessors of a GB300
 // global cell ids of a region's tile cells: cells[kRegionCells * region + k]
 constexpr int kRegionCells = 48;
 constexpr int kRegionClusterCap = 512;   // clusters of one region (2,048 home atoms); more is reported
@@ -393,17 +394,27 @@ void launch_cl_build(const float4* pos, const int* tag, const int* cell_start, c
                      int* n_tasks, const TopoDev* topo, bool dep, cudaStream_t st);
 // after the build (which clears *n_tasks): each LJ item's clusters in the
 // order the force kernel takes them, tasks[task_base[item] + rank]; an item
-// claims its place in the table (as many entries as there are clusters) by *n_tasks
+// claims its place in the table (as many entries as there are clusters) by
+// n_tasks[0]; items with tiles of more than lj_cap atoms are listed in big[0 .. n_tasks[1])
 void launch_cl_rank(const float4* pos, const int* cell_start, const int* cl_start, const int* cells,
                     const WorkItem* items, int n_items, const RegionShape* shapes, const int* ncl, ClusterTask* tasks,
-                    int* task_base, int* n_tasks, bool dep, cudaStream_t st);
+                    int* task_base, int* n_tasks, int lj_cap, int* big, bool dep, cudaStream_t st);
+// Items whose tile exceeds the force kernel's usual one.  ids null: the usual
+// launch, which leaves items of more than its own tile_cap atoms to the other one
+// (and reports those above tile_cap here); ids, n_ids (device): the launch that
+// takes them.
+struct BigTiles {
+  const int *ids, *n_ids;
+  int tile_cap;
+};
 void launch_cl_force(bool energy, const float4* pos, const int* cell_start, const int* cl_start,
                      const int* cells, const WorkItem* items, int n_items, const RegionShape* shapes,
                      const RepDev* reps, const unsigned* list, const ClusterTask* tasks, const int* task_base,
                      int cap, int tile_cap, const ForceParams& fp, long long* flj, int Npad, double* epart, unsigned* flags, int block, int lanes,
-                     int persistent_grid, int* work, bool exact, const StepGate& gate,
+                     int persistent_grid, int* work, bool exact, const BigTiles& big, const StepGate& gate,
                      const ThermoArgs& thermo, cudaStream_t st);
 int lj_blocks_per_sm(int block, int lanes, int tile_cap);
+int lj_tile_cap_for(int per_sm);     // largest tile of which per_sm fit
 int lj_tiles_per_sm(int tile_cap);   // force tiles that fit an SM's shared memory together (1 or more)
 cudaError_t tile_kernels_init();
 int tile_capacity_max();

@@ -58,3 +58,28 @@ def test_every_split_gives_the_oracle_forces(L, n_chains):
     for k, idx in (("lj", 0), ("lj_shifted", 1), ("bond", 2), ("angle", 3), ("dihedral", 4)):
         assert abs(e[k] - en[idx]) <= 1e-5 * max(1.0, abs(en[idx]))
     s.close()
+
+
+def test_large_tiles_of_an_uneven_box():
+    """Cells of 1.31 nm (skin 0.3): in the batch (441 rows) the force kernel's tile is the one that fits an SM twice,
+    3,776 atoms, and the dense parts (42 sites/nm^3 in 44 cells: 4,200 atoms) of the first replica go to the launch for
+    large tiles.  Alone it is split into rows.  The bits are the same."""
+    L0, L, sites = 7.0, 9.2, 8
+    melts = []
+    for seed, n, side in ((5, 1800, L0), (6, 3200, L), (7, 3200, L)):
+        m = chaingen.melt(n, sites=sites, seed=seed, T=300.0, L=side)
+        x = m["pos"].reshape(n, sites, 3).copy()
+        d = np.diff(x, axis=1)
+        x[:, 1:] = x[:, :1] + np.cumsum(d - side * np.round(d / side), axis=1)
+        melts.append(dict(m, pos=np.mod(x.reshape(-1, 3) + (2.4, 2.4, 0.0), L), L=L))
+    kw = dict(precision=md.MD_MIXED, skin=0.3, rebin_every=3)
+    both, alone = md.System(melts, **kw), md.System(melts[0], **kw)
+    n = len(melts[0]["pos"])
+    for _ in range(2):
+        assert np.array_equal(alone.forces(), both.forces()[:n])
+        assert alone.energy()[0] == both.energy()[0]
+        alone.step(4)
+        both.step(4)
+    assert np.array_equal(alone.state()[0], both.state()[0][:n])
+    alone.close()
+    both.close()
