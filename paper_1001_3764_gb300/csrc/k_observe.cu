@@ -34,13 +34,18 @@ namespace mdg {
 // pairs in range at 200 bins) are evaluated by the definition.
 //
 // A lane holds one atom j of the 14 cells, moved to the home cell's frame,
-// and a warp walks the home atoms in shared memory (one broadcast load per
-// 32 pairs).  Blocks take runs of consecutive cells, so that a histogram is
-// flushed once per run and not once per cell.  150k sites, r_max 1.0 nm,
-// 200 bins: 9,824 -> 251 us (FP64 for every candidate, one block per cell).
+// and a warp walks the home atoms in shared memory, two at a time in packed
+// FP32.  9% of the candidates are in range, so nearly every round of 32 holds
+// one: they are queued and binned 32 at a time.  A block takes a cell, or
+// above 4 times the resident blocks a run of consecutive ones, so that a
+// histogram is flushed once per run.  Bound: instruction issue.  150k sites,
+// r_max 1.0 nm, 200 bins: 9,824 us (FP64 for every candidate) -> 251 (binned
+// as met, runs of one or two cells) -> 175.
 constexpr int kRdfThreads = 128;
 constexpr int kRdfStage = 128;       // home atoms staged at a time
-constexpr int kRdfBlocks = 152 * 16;
+constexpr int kRdfBlocks = kSMs * 16;
+constexpr int kRdfQueue = 256;       // a ring: at most 31 + 64 pairs wait
+constexpr int kRdfSlotBits = 26;     // atoms < 2^26; six bits of the home atom above, its seventh with r^2
 // FP32 cell units: each position is rounded by at most 2^-25 (FP32 master:
 // 2^-24.6), the offset and the difference add 2^-24 each, so a component is
 // off by at most 1.9e-7 and r <= 1 by 3.3e-7; r^2, rsqrt.approx and the scaling by h add 5e-7
@@ -83,10 +88,14 @@ __global__ void __launch_bounds__(kRdfThreads) k_rdf(const T* __restrict__ x, in
                                                      const float2* __restrict__ inner, int n_bins, double norm,
                                                      unsigned long long* __restrict__ counts) {
   extern __shared__ unsigned int hist[];
-  __shared__ float4 si[kRdfStage];          // home atoms: cell units, w = chain/site tag
+  __shared__ __align__(8) float hx[kRdfStage], hy[kRdfStage], hz[kRdfStage];   // home atoms: cell units
+  __shared__ __align__(8) int ht[kRdfStage];                                   // and chain/site tags
+  __shared__ uint2 queue[kRdfThreads / 32][kRdfQueue];
   __shared__ int s_start[14], s_pre[15];
   __shared__ float s_off[14][3];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint2* qw = queue[warp];
+  const unsigned lt = (1u << lane) - 1u;
   const int c0 = (int)((long long)C * blockIdx.x / gridDim.x), c1 = (int)((long long)C * (blockIdx.x + 1) / gridDim.x);
   if (c0 >= c1) return;
   for (int k = threadIdx.x; k < n_bins; k += kRdfThreads) hist[k] = 0u;
@@ -138,48 +147,73 @@ __global__ void __launch_bounds__(kRdfThreads) k_rdf(const T* __restrict__ x, in
       const int ni = min(kRdfStage, n - i0);
       __syncthreads();
       for (int k = threadIdx.x; k < ni; k += kRdfThreads) {
-        float4 p = pos[b + i0 + k];
-        p.w = __int_as_float(tag[b + i0 + k] & (int)kTagMask);
-        si[k] = p;
+        const float4 p = pos[b + i0 + k];
+        hx[k] = p.x; hy[k] = p.y; hz[k] = p.z;
+        ht[k] = tag[b + i0 + k] & (int)kTagMask;
       }
       __syncthreads();
+      // bin of one queued pair
+      auto take = [&](uint2 e) {
+        const int k = (int)((e.x >> 31) << 6 | e.y >> kRdfSlotBits), sj = (int)(e.y & ((1u << kRdfSlotBits) - 1u));
+        const float r2 = __uint_as_float(e.x & 0x7fffffffu);
+        const float rr = r2 * rsqrtf(r2) * hf;
+        if (rr < low) return;
+        int g = (int)((rr - e0) * fnorm);
+        g = g < 0 ? 0 : (g > n_bins - 1 ? n_bins - 1 : g);
+        const float2 in = __ldg(inner + g);
+        if (!(rr >= in.x && rr < in.y))
+          g = rdf_exact_bin<T>(x, N, perm[b + i0 + k], perm[sj], R.L, edges, n_bins, norm);
+        if (g >= 0) atomicAdd(hist + g, 1u);
+      };
       const int total = s_pre[14];
-      int o = 0;
+      int o = 0, qn = 0, head = 0;   // waiting pairs: ring places head .. head + qn - 1
       for (int q = 32 * warp + lane; q - lane < total; q += kRdfThreads) {
-        const bool on = q < total;
-        int sj = b;
+        int sj = b, tj = 0, last = 0;   // home atoms i0 .. i0 + last - 1 pair with j
         float4 pj = make_float4(0.f, 0.f, 0.f, 0.f);
-        int tj = 0, last = ni;   // home atoms i0 .. i0 + last - 1 pair with j
-        if (on) {
+        if (q < total) {
           while (q >= s_pre[o + 1]) ++o;
           sj = s_start[o] + (q - s_pre[o]);
           pj = pos[sj];
           pj.x += s_off[o][0]; pj.y += s_off[o][1]; pj.z += s_off[o][2];
           tj = tag[sj] & (int)kTagMask;
-          if (o == 0) last = min(ni, sj - b - i0);   // the cell itself: each pair once, i before j
-        } else {
-          last = 0;
+          last = o == 0 ? min(ni, sj - b - i0) : ni;   // the cell itself: each pair once, i before j
         }
-        for (int k = 0; k < ni; ++k) {
-          const float4 p = si[k];
-          float dx = pj.x - p.x, dy = pj.y - p.y, dz = pj.z - p.z;
+        const float2 jx = make_float2(pj.x, pj.x), jy = make_float2(pj.y, pj.y), jz = make_float2(pj.z, pj.z);
+        const float2 m1 = make_float2(-1.f, -1.f);
+        for (int k = 0; k < ni; k += 2) {   // a place past the last home atom is not below `last`
+          float2 dx = __ffma2_rn(*reinterpret_cast<const float2*>(hx + k), m1, jx),
+                 dy = __ffma2_rn(*reinterpret_cast<const float2*>(hy + k), m1, jy),
+                 dz = __ffma2_rn(*reinterpret_cast<const float2*>(hz + k), m1, jz);
+          const int2 t = *reinterpret_cast<const int2*>(ht + k);
           if (fold) {
-            dx -= Mf * rintf(dx / Mf); dy -= Mf * rintf(dy / Mf); dz -= Mf * rintf(dz / Mf);
+            dx.x -= Mf * rintf(dx.x / Mf); dy.x -= Mf * rintf(dy.x / Mf); dz.x -= Mf * rintf(dz.x / Mf);
+            dx.y -= Mf * rintf(dx.y / Mf); dy.y -= Mf * rintf(dy.y / Mf); dz.y -= Mf * rintf(dz.y / Mf);
           }
-          const float r2 = dx * dx + dy * dy + dz * dz;
+          const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
           // |i - j| <= 2 within one chain: 1-2 and 1-3 neighbours (Sec. 3.1)
-          if (k < last && r2 <= far2 && (unsigned)(__float_as_int(p.w) - tj + 2) > 4u) {
-            const float rr = r2 * rsqrtf(r2) * hf;
-            if (rr < low) continue;
-            int g = (int)((rr - e0) * fnorm);
-            g = g < 0 ? 0 : (g > n_bins - 1 ? n_bins - 1 : g);
-            const float2 in = __ldg(inner + g);
-            if (!(rr >= in.x && rr < in.y))
-              g = rdf_exact_bin<T>(x, N, perm[b + i0 + k], perm[sj], R.L, edges, n_bins, norm);
-            if (g >= 0) atomicAdd(hist + g, 1u);
+          const bool pass0 = k < last && r2.x <= far2 && (unsigned)(t.x - tj + 2) > 4u;
+          const bool pass1 = k + 1 < last && r2.y <= far2 && (unsigned)(t.y - tj + 2) > 4u;
+          const unsigned b0 = __ballot_sync(0xffffffffu, pass0), b1 = __ballot_sync(0xffffffffu, pass1);
+          const int at = head + qn + __popc(b0 & lt) + __popc(b1 & lt);
+          const unsigned hi = (unsigned)(k >> 6) << 31, lo = (unsigned)sj | (unsigned)(k & 63) << kRdfSlotBits;
+          if (pass0) qw[at & (kRdfQueue - 1)] = make_uint2(__float_as_uint(r2.x) | hi, lo);
+          if (pass1)
+            qw[(at + (pass0 ? 1 : 0)) & (kRdfQueue - 1)] =
+                make_uint2(__float_as_uint(r2.y) | hi, lo + (1u << kRdfSlotBits));   // k is even
+          qn += __popc(b0) + __popc(b1);
+          // one barrier a round: the 64 places that are taken lie before head,
+          // and the next round writes at most 94 past it (256 in the ring)
+          __syncwarp();
+          while (qn >= 32) {
+            take(qw[(head + lane) & (kRdfQueue - 1)]);
+            head += 32;
+            qn -= 32;
           }
         }
       }
+      __syncwarp();
+      if (lane < qn) take(qw[(head + lane) & (kRdfQueue - 1)]);
+      __syncwarp();
     }
   }
   __syncthreads();
@@ -201,8 +235,8 @@ void launch_rdf(bool mixed, const void* x, int N, const int* cell_start, const i
                 int n_bins, double norm, unsigned long long* counts, cudaStream_t st) {
   if (C <= 0) return;
   const size_t sm = (size_t)n_bins * sizeof(unsigned int);
-  const int grid = C < kRdfBlocks ? C : kRdfBlocks;
-  if (sm > 40000) {   // the histogram and the staged atoms exceed 48 KB
+  const int grid = C < 4 * kRdfBlocks ? C : kRdfBlocks;
+  if (sm > 36000) {   // the histogram, queues and staged atoms exceed 48 KB
     cudaFuncSetAttribute(k_rdf<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     cudaFuncSetAttribute(k_rdf<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   }
