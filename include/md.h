@@ -53,14 +53,15 @@ enum {
 
 enum { MD_PLAIN_FP32 = 0, MD_MIXED = 1 };   /* precision forms */
 enum { MD_NVE = 0, MD_VRESCALE = 1, MD_NOSE_HOOVER = 2 };   /* thermostat */
-/* LJ work schedule: one thread block per region of cells, or a fixed grid
- * (resident blocks x SMs) whose blocks take regions from a device counter.
- * Both give the same forces bit for bit.  The list build always runs one
- * block per region. */
+/* LJ work schedule: one thread block per work item (a region of cells, or
+ * in small systems a part of one), or a fixed grid (resident blocks x SMs)
+ * whose blocks take items from a device counter.  Both give the same forces
+ * bit for bit.  The list build always runs one block per work item. */
 enum { MD_SCHED_GRID = 0, MD_SCHED_PERSISTENT = 1 };
 /* What a step does when an atom has moved more than skin/2 since the last
  * list build: rebuild the bins and list before its forces (a conditional
- * node in the step graph), or report MD_EUNSTABLE at the next synchronising
+ * node at the end of the block's graph, which repeats the block from that
+ * step on), or report MD_EUNSTABLE at the next synchronising
  * call (graphs without conditional nodes, which profilers can take apart). */
 enum { MD_DISP_REBUILD = 0, MD_DISP_ERROR = 1 };
 
@@ -122,8 +123,9 @@ typedef struct {
                                   velocity of v_{k+1/2} removed before the next step.  xi starts
                                   at 0 and persists across md_step and md_set_state calls. */
   int32_t nbr_capacity;        /* neighbour slots per atom; 0 = chosen from density */
-  int32_t lj_block;            /* threads per block of the LJ kernel: 128, 256 or 384 (0 = 384 with
-                                  3 x 3 regions, 256 with 2 x 2) */
+  int32_t lj_block;            /* threads per block of the LJ kernel: 128, 256 or 384 (0 = 256 with
+                                  2 x 2 regions; with 3 x 3 384, or 768 where two tiles do not fit
+                                  an SM's shared memory) */
   int32_t schedule;            /* MD_SCHED_GRID or MD_SCHED_PERSISTENT (see below) */
   int32_t lj_lanes;            /* lanes of the LJ kernel that share one 4-atom cluster's list:
                                   8, 16 or 32 (0 = 8) */
@@ -201,7 +203,7 @@ int md_create(const md_desc *desc, md_system **out);
  * steps and of every call (the paper rebuilds it every 10 steps, Sec. 5),
  * and also before the force evaluation of any step in which an atom has
  * moved more than skin/2 since the last rebuild (a device-side check that
- * opens a conditional rebuild in the step graph; md_early_rebins counts
+ * opens the conditional node of the block's graph; md_early_rebins counts
  * them), so every force comes from a list that holds all pairs within rc;
  * with MD_DISP_ERROR such a step is reported as MD_EUNSTABLE instead.
  * Synchronises and reports device flags. */
@@ -339,7 +341,9 @@ int md_get_cell_units(md_system *sys, float *u);
 
 /* Per-kernel GPU time recording.  When enabled, CUDA events bracket every
  * kernel group of each step (rebin, neighbour build, integrate, LJ, bonded)
- * and md_step / md_sync accumulate their durations.  ms_total[5] and
+ * and md_step / md_sync accumulate their durations.  One kernel does the
+ * bonded forces and the update of a step and counts as bonded; integrate is
+ * a block's opening update.  ms_total[5] and
  * launches[5] are in that order; md_profile_reset clears them. */
 int md_profile_enable(md_system *sys, int32_t on);
 int md_profile_read(md_system *sys, double *ms_total, int64_t *launches);

@@ -1,4 +1,4 @@
-// k_bin.cu -- on-GPU cell binning and neighbour-list build (Sec. 3.1).
+// k_bin.cu -- on-GPU cell binning (Sec. 3.1).
 //
 // The paper's GBIN_NEW claims a slot per atom with atomicAdd into a
 // fixed-capacity bin (Sec. 3.1, GBIN_NEW listing).  Here the same histogram

@@ -1,4 +1,6 @@
-// k_force.cu -- Dreiding II bonded forces (Eqs. 4-6, Sec. 3.3) on sm_103a.
+// k_force.cu -- Dreiding II bonded forces (Eqs. 4-6, Sec. 3.3) on sm_103a for
+// the read-outs: the total force at the present positions, and the bonded
+// energies and virial.  The steps' form is in k_step.cu, the terms in bonded.cuh.
 // The Lennard-Jones force (Eq. 2) is in k_lj.cu.
 //
 // Each thread block owns a contiguous range of atoms (whole or partial
@@ -9,8 +11,7 @@
 // contributions of the (at most 2+3+4) terms that contain it in a fixed
 // order.  This removes the paper's 2x/3x/4x redundant per-home-atom flops
 // (Sec. 3.3) without atomics.  The kernel also adds the LJ force of the atom
-// (read from cell-sorted order through inv_perm) so the integrator reads one
-// force per atom.  Energies and the virial are block sums: FP32 warp trees,
+// (read from cell-sorted order through inv_perm).  Energies and the virial are block sums: FP32 warp trees,
 // then FP64 across warps, in a fixed order.
 #include <type_traits>
 

@@ -3,7 +3,7 @@
 //
 // Work unit: a region of up to G x G x 1 cells (G = 2 or 3; cells of side
 // >= r_c + skin, Sec. 3.1), one thread block per region, or in small systems
-// several blocks that share a region's clusters.  The block stages in
+// several blocks that share its cells or clusters (WorkItem).  The block stages in
 // shared memory the "tile": the region's cells and every cell that one of
 // them reaches by one of the 13 forward offsets of a half shell (27 cells
 // for G = 2, 44 for G = 3), each cell a contiguous run of sorted atoms, moved
@@ -1082,39 +1082,34 @@ void launch_cl_build(const float4* pos, const int* tag, const int* cell_start, c
   if (n_items <= 0) return;
   const size_t sm = cl_build_smem(tile_cap);
   // 32 warps an SM: four blocks of 256 threads, or where four tiles do not fit its shared memory, two of 512
-  if (4 * (sm + 5800 + 1024) > 228 * 1024) {
-    if (topo)
-      launch_dependent(dep, k_cl_build<512, true>, n_items, 512, sm, st, pos, tag, cell_start, cl_start, cells, items, shapes, reps, list,
-                       ncl, cap, tile_cap, flags, n_tasks, *topo);
-    else
-      launch_dependent(dep, k_cl_build<512, false>, n_items, 512, sm, st, pos, tag, cell_start, cl_start, cells, items, shapes, reps,
-                       list, ncl, cap, tile_cap, flags, n_tasks, TopoDev{});
-    return;
-  }
-  if (topo)
-    launch_dependent(dep, k_cl_build<256, true>, n_items, 256, sm, st, pos, tag, cell_start, cl_start, cells, items, shapes, reps, list,
-                       ncl, cap, tile_cap, flags, n_tasks, *topo);
-  else
-    launch_dependent(dep, k_cl_build<256, false>, n_items, 256, sm, st, pos, tag, cell_start, cl_start, cells, items, shapes, reps,
-                       list, ncl, cap, tile_cap, flags, n_tasks, TopoDev{});
+  const bool wide = 4 * (sm + 5800 + 1024) > 228 * 1024;
+#define MDG_CLB(NT, GEN, TOPO)                                                                                    \
+  launch_dependent(dep, k_cl_build<NT, GEN>, n_items, NT, sm, st, pos, tag, cell_start, cl_start, cells, items, \
+                   shapes, reps, list, ncl, cap, tile_cap, flags, n_tasks, TOPO)
+  if (wide && topo) MDG_CLB(512, true, *topo);
+  else if (wide) MDG_CLB(512, false, TopoDev{});
+  else if (topo) MDG_CLB(256, true, *topo);
+  else MDG_CLB(256, false, TopoDev{});
+#undef MDG_CLB
 }
 
 void launch_cl_rank(const float4* pos, const int* cell_start, const int* cl_start, const int* cells,
                     const WorkItem* items, int n_items, const RegionShape* shapes, const int* ncl, ClusterTask* tasks,
                     int* task_base, int* n_tasks, int lj_cap, int* big, bool dep, cudaStream_t st) {
   if (n_items > 0)
-    launch_dependent(dep, k_cl_rank, n_items, kRankThreads, 0, st, pos, cell_start, cl_start, cells, items, shapes, ncl, tasks,
-                     task_base, n_tasks, lj_cap, big);
+    launch_dependent(dep, k_cl_rank, n_items, kRankThreads, 0, st, pos, cell_start, cl_start, cells, items, shapes, ncl,
+                     tasks, task_base, n_tasks, lj_cap, big);
 }
 
 void launch_cl_force(bool energy, const float4* pos, const int* cell_start, const int* cl_start,
                      const int* cells, const WorkItem* items, int n_items, const RegionShape* shapes,
                      const RepDev* reps, const unsigned* list, const ClusterTask* tasks, const int* task_base,
-                     int cap, int tile_cap, const ForceParams& fp, long long* flj, int Npad, double* epart, unsigned* flags, int block,
-                     int lanes, int persistent_grid, int* work, bool exact, const BigTiles& big, const StepGate& gate,
+                     int cap, int tile_cap, const ForceParams& fp, long long* flj, int Npad, double* epart,
+                     unsigned* flags, int block, int lanes, int persistent_grid, int* work, bool exact, const BigTiles& big, const StepGate& gate,
                      const ThermoArgs& thermo, cudaStream_t st) {
   if (n_items <= 0) return;
-  const int grid = big.ids ? std::min(n_items, kSMs) : (persistent_grid > 0 ? persistent_grid : n_items) + thermo.n_blocks;
+  const int grid = big.ids ? std::min(n_items, kSMs)
+                           : (persistent_grid > 0 ? persistent_grid : n_items) + thermo.n_blocks;
   const int pers = persistent_grid > 0;
   // the thermostat blocks use 4 doubles per thread of the tile's memory
   const size_t sm = std::max(cl_force_smem(tile_cap), thermo.n_blocks ? (size_t)block * 4 * sizeof(double) : 0);

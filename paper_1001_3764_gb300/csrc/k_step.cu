@@ -45,16 +45,13 @@ __device__ __forceinline__ void update_atom(const T (&F)[3], T (&xi)[3], T (&vi)
 }
 
 template <bool MIXED, int MODE, bool KE, int TH, int NT>
-__global__ void __launch_bounds__(NT, NT == 256 ? 4 : NT == 512 ? 2 : 1) k_step(void* __restrict__ xv, void* __restrict__ vv, int* __restrict__ img,
-                                             void* __restrict__ Fv, const uint16_t* __restrict__ site,
-                                             const int* __restrict__ cellc, const int* __restrict__ inv_perm,
-                                             const float4* __restrict__ ref, float4* __restrict__ pos,
-                                             const long long* __restrict__ flj, long long* __restrict__ flj_next,
-                                             int Npad, int N, const Tile* __restrict__ tiles,
-                                             const RepDev* __restrict__ reps, const ForceParams fp,
-                                             double* __restrict__ kepart, const double* __restrict__ lam,
-                                             unsigned* __restrict__ flags, const StepGate gate,
-                                             const MoveReport mr) {
+__global__ void __launch_bounds__(NT, NT == 256 ? 4 : NT == 512 ? 2 : 1)
+    k_step(void* __restrict__ xv, void* __restrict__ vv, int* __restrict__ img, void* __restrict__ Fv,
+           const uint16_t* __restrict__ site, const int* __restrict__ cellc, const int* __restrict__ inv_perm,
+           const float4* __restrict__ ref, float4* __restrict__ pos, const long long* __restrict__ flj,
+           long long* __restrict__ flj_next, int Npad, int N, const Tile* __restrict__ tiles,
+           const RepDev* __restrict__ reps, const ForceParams fp, double* __restrict__ kepart,
+           const double* __restrict__ lam, unsigned* __restrict__ flags, const StepGate gate, const MoveReport mr) {
   using T = typename std::conditional<MIXED, double, float>::type;
   T* x = reinterpret_cast<T*>(xv);
   T* v = reinterpret_cast<T*>(vv);
@@ -256,8 +253,8 @@ template <bool MIXED, int NT>
 static void launch_step_t(IntegMode mode, int th, int threads, const StepArgs& a, const ForceParams& fp,
                           const StepGate& gate, const MoveReport& mr, cudaStream_t st) {
 #define MDG_STEP(MODE, KE, TH)                                                                                       \
-  launch_dependent(gate.dep, k_step<MIXED, MODE, KE, TH, NT>, a.n_tiles, threads, step_smem_bytes(threads), st, a.x, a.v, a.img, \
-                   a.F, a.site, a.cellc, a.inv_perm, a.ref, a.pos, a.flj, a.flj_next, a.Npad, a.N, a.tiles, a.reps,  \
+  launch_dependent(gate.dep, k_step<MIXED, MODE, KE, TH, NT>, a.n_tiles, threads, step_smem_bytes(threads), st,     \
+                   a.x, a.v, a.img, a.F, a.site, a.cellc, a.inv_perm, a.ref, a.pos, a.flj, a.flj_next, a.Npad, a.N, a.tiles, a.reps,  \
                    fp, a.kepart, a.lam, a.flags, gate, mr)
   if (mode == kKickKickDrift) {
     if (th == 2) MDG_STEP(kKickKickDrift, true, 2);

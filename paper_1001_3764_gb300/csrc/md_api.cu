@@ -3,10 +3,13 @@
 // One md_system owns: a replica table, tile tables, every device buffer (one
 // allocation, or a caller workspace), a stream, and a CUDA graph holding one
 // rebin cycle (rebin + neighbour list + rebin_every steps).  Kernels are in
-// k_bin.cu (binning), k_lj.cu (neighbour list and Lennard-Jones), k_force.cu
-// (bonded terms), k_integrate.cu (integration, kinetic energy, thermostats,
-// energy reductions, observables, state transfer) and md_adjoint.cu (the
-// adjoint); md_static.cu holds the allocation-free binning entry point.
+// k_bin.cu (binning), k_lj.cu (neighbour list and Lennard-Jones), k_step.cu
+// (bonded forces and update of a step), k_force.cu (bonded terms of the
+// read-outs), k_integrate.cu (opening update, kinetic energy, energy
+// reductions, chain observables, state transfer), k_observe.cu (RDF, ACF) and
+// md_adjoint.cu (the adjoint); md_static.cu holds the allocation-free binning
+// entry point.  bonded.cuh, integrate.cuh and cell_order.cuh hold what several
+// of them share.
 #include <algorithm>
 #include <array>
 #include <chrono>
@@ -279,7 +282,7 @@ static void plan_regions(md_system* s, bool grid_schedule) {
   // skin 0.12 nm: LJ 484 us with one block an SM, 357 + 19 now.
   s->lj_cap = s->tile_cap;
   std::vector<char> large(s->n_reps, 0);
-  if (G == 3 && !s->lj_block && grid_schedule && lj_tiles_per_sm(s->tile_cap) == 1) {
+  if (G == 3 && (!s->lj_block || s->lj_block == 384) && grid_schedule && lj_tiles_per_sm(s->tile_cap) == 1) {
     const int two = lj_tile_cap_for(2);
     int64_t rows = 0, large_atoms = 0;
     for (int r = 0; r < s->n_reps; ++r) {
@@ -744,7 +747,6 @@ static void enqueue_steps(md_system* s, int k, bool repeat, const MoveReport& mr
   launch_step(s->mixed, kKickOnly, s->thermo, s->S, step_args(s, true, s->flj[(k - 1) & 1], nullptr), s->fp, topo, gate,
               mr, s->st);
   prof_mark(s);
-  prof_mark(s);
 }
 
 // One block of k steps: rebin + list (unless the bins and list are already
@@ -807,18 +809,16 @@ static int64_t block_launches(const md_system* s, int k) {
 
 // accumulate the event timings of the last block (requires a finished stream)
 static void prof_collect(md_system* s, int k) {
-  if (!s->profile || s->ev_used < 3 + 3 * k + 1) return;
+  if (!s->profile || s->ev_used < 3 + 3 * k) return;
   float ms;
   cudaEventElapsedTime(&ms, s->ev[0], s->ev[1]); s->prof_ms[0] += ms; s->prof_n[0] += 5;
   cudaEventElapsedTime(&ms, s->ev[1], s->ev[2]); s->prof_ms[1] += ms; s->prof_n[1] += 1;
-  int e = 2;
-  for (int j = 0; j < k; ++j) {
-    cudaEventElapsedTime(&ms, s->ev[e], s->ev[e + 1]); s->prof_ms[2] += ms; s->prof_n[2] += 1;
+  // per step: the opening update (later steps have none: two records in a row), LJ, bonded and update
+  for (int j = 0, e = 2; j < k; ++j, e += 3) {
+    if (j == 0) { cudaEventElapsedTime(&ms, s->ev[e], s->ev[e + 1]); s->prof_ms[2] += ms; s->prof_n[2] += 1; }
     cudaEventElapsedTime(&ms, s->ev[e + 1], s->ev[e + 2]); s->prof_ms[3] += ms; s->prof_n[3] += 1;
     cudaEventElapsedTime(&ms, s->ev[e + 2], s->ev[e + 3]); s->prof_ms[4] += ms; s->prof_n[4] += 1;
-    e += 3;
   }
-  cudaEventElapsedTime(&ms, s->ev[e], s->ev[e + 1]); s->prof_ms[2] += ms; s->prof_n[2] += 1;
 }
 
 // the rebin cycle as a graph, and the same without its leading rebin + list
@@ -892,7 +892,8 @@ static bool usable_in_place(const md_system* s, const T* ptr, size_t n) {
   static const Fn fn = [] {
     void* f = nullptr;
     cudaDriverEntryPointQueryResult q{};
-    const bool ok = cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &q) == cudaSuccess;
+    const bool ok =
+        cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &q) == cudaSuccess;
     return ok && q == cudaDriverEntryPointSuccess ? (Fn)f : nullptr;
   }();
   if (!fn || !ptr || (uintptr_t)ptr % sizeof(T)) return false;
@@ -1108,7 +1109,7 @@ int md_step_async(md_system* s, int64_t n) {
     s->fresh = false;
     CU(cudaGraphLaunch(skip_rebin ? s->cycle_fresh : s->cycle, s->st));
     if (s->profile) {
-      s->ev_used = (int)std::min<int64_t>(s->ev.size(), 3 + 3 * s->R + 1);
+      s->ev_used = (int)std::min<int64_t>(s->ev.size(), 3 + 3 * s->R);
       CU(cudaStreamSynchronize(s->st));
       prof_collect(s, s->R);
     }
@@ -1120,7 +1121,7 @@ int md_step_async(md_system* s, int64_t n) {
       const int rc = capture_block(s, (int)rem, &gr);
       if (rc) return rc;
     }
-    if (s->profile) s->ev_used = (int)std::min<int64_t>(s->ev.size(), 3 + 3 * rem + 1);
+    if (s->profile) s->ev_used = (int)std::min<int64_t>(s->ev.size(), 3 + 3 * rem);
     CU(cudaGraphLaunch(gr, s->st));
     if (s->profile) { CU(cudaStreamSynchronize(s->st)); prof_collect(s, (int)rem); }
   }

@@ -5,20 +5,21 @@
 //   original (chain-major) order, index i:
 //     mixed form : x, v  double SoA [3][N];   plain form : float SoA [3][N]
 //     img        int32 SoA [3][N]  periodic image counters
-//     F          force, AoS 32 B/atom: int64x3 fixed point (mixed) or float x3
+//     F          force, AoS 32 B/atom: int64x3 fixed point (mixed) or float x3;
+//                written where a call ends, read where the next one begins
 //     site       uint16 [N] position of the atom in its chain (MAIDX - 1)
 //     cellc      int32 [N] packed cell coordinates at the last rebin
 //     ref        float4 [N] cell-unit position at the last rebin
 //     inv_perm   int32 [N] sorted slot of atom i
 //   sorted (cell-major) order, index s:
 //     pos        float4 [N] position in cell units relative to the centre of the
-//                atom's cell at the last rebin, u = (x - (c + 1/2) h) / h; w unused
+//                atom's cell at the last rebin, u = (x - (c + 1/2) h) / h; w: LJ type
 //     tag        int32 [N]  chain*1024 + site | type << 30 (sites < 1024, so the
 //                site fields of two chains never come within 2 of each other)
 //     perm       int32 [N]  original index of slot s
-//     Flj        int64 SoA [3][Npad]  LJ force on slot s (2^-32 kJ/mol/nm):
-//                cleared, added to by the force kernel, read by the bonded
-//                kernel
+//     flj        two int64 SoA [3][Npad]: LJ force on slot s (2^-32
+//                kJ/mol/nm); the force kernel adds to one while the step kernel
+//                that follows reads it and clears the other
 //   clusters (4 consecutive slots of a cell; cluster k of cell c is
 //   cl_start[c] + k):
 //     list       uint32 [clusters][cap]: tile index (bits 0..15) and the mask
@@ -410,8 +411,8 @@ struct BigTiles {
 void launch_cl_force(bool energy, const float4* pos, const int* cell_start, const int* cl_start,
                      const int* cells, const WorkItem* items, int n_items, const RegionShape* shapes,
                      const RepDev* reps, const unsigned* list, const ClusterTask* tasks, const int* task_base,
-                     int cap, int tile_cap, const ForceParams& fp, long long* flj, int Npad, double* epart, unsigned* flags, int block, int lanes,
-                     int persistent_grid, int* work, bool exact, const BigTiles& big, const StepGate& gate,
+                     int cap, int tile_cap, const ForceParams& fp, long long* flj, int Npad, double* epart,
+                     unsigned* flags, int block, int lanes, int persistent_grid, int* work, bool exact, const BigTiles& big, const StepGate& gate,
                      const ThermoArgs& thermo, cudaStream_t st);
 int lj_blocks_per_sm(int block, int lanes, int tile_cap);
 int lj_tile_cap_for(int per_sm);     // largest tile of which per_sm fit
