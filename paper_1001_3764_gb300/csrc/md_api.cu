@@ -353,11 +353,13 @@ static void plan_regions(md_system* s, bool grid_schedule) {
     else add_items(s, order[q], lj_rows == kWhole && per_sm >= 2 && R <= slots && q >= kSMs ? 1 : lj_rows, 1);
   }
   s->n_lj_items = (int)s->items_h.size();
-  // The list build gives a warp a cluster at a time (7 us alone), 8 warps a
-  // block, 4 blocks an SM: 108 -> 12 us at 1,500 sites (cells in 3 parts),
-  // 117 -> 19.5 at 12,000 (2), 113 -> 55 at 64,800 (1), 120 -> 103 at 150k and
-  // 312 -> 295 at 506k (rows; cells 110 and 338); whole 775, rows 819 at 1.5M
-  const int parts = n_cells <= 128 ? 3 : n_cells <= 256 ? 2 : 1;
+  // The list build gives a warp a cluster at a time (7 us alone), 32 warps an
+  // SM.  With the task order, us (whole regions / rows / cells / cells in 3 parts):
+  //   - / 31 / 21 / 18.6 at 1,500 sites, 67 / 35 / 23 / 18.8 at 6,000, 62 / 33 / 26 / 31 at 12,000 (216 cells),
+  //   82 / 56 / 54 at 64,800 (176 regions), 102 / 89 / 94 at 150k (375), 232 / 213 / 243 at 444k (1,029),
+  //   236 / 243 / 272 at 506k (1,408), 317 / 336 / 388 at 737k (2,025), 609 / 639 / 774 at 1.5M;
+  // between 600 and 1,800 regions the last wave decides, by up to 8% either way
+  const int parts = n_cells <= 128 ? 3 : 1;
   for (int r : order) add_items(s, r, R >= 12 * kSMs ? kWhole : R >= 2 * kSMs ? 1 : 0, parts);
   s->n_build_items = (int)s->items_h.size() - s->n_lj_items;
 }
