@@ -635,8 +635,8 @@ def run_gpu(args):
             "value": aggregate_rate(ws, n_atoms, md_steps, results["rebuild_policy"]["ms"] * 1e-3),
             "ms_per_step": results["rebuild_policy"]["ms"] / args.steps,
             "early_rebuilds": results["rebuild_policy"]["early"],
-            "note": "same loop with the default MD_DISP_REBUILD policy (a displacement check and a conditional "
-                    "list rebuild in every step graph); the headline uses MD_DISP_ERROR, whose graphs ncu can "
+            "note": "same loop with the default MD_DISP_REBUILD policy (a displacement check in every step, "
+                    "one conditional rebuild per block of steps); the headline uses MD_DISP_ERROR, whose graphs ncu can "
                     "profile, with the same work on this melt"},
         "roofline": {"kernel": "k_cl_force (LJ force, Eq. 2)", "bound": "alu", "achieved": achieved,
                      "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": achieved / FP32_PEAK_TFLOPS,
