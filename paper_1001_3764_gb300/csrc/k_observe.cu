@@ -35,16 +35,18 @@ namespace mdg {
 //
 // A lane holds one atom j of the 14 cells, moved to the home cell's frame,
 // and a warp walks the home atoms in shared memory, two at a time in packed
-// FP32.  9% of the candidates are in range, so nearly every round of 32 holds
-// one: they are queued and binned 32 at a time.  A block takes a cell, or
+// FP32.  40% of the candidates lie too far from the home cell for any of its
+// atoms and are left out before.  Of the rest 15% are in range, so nearly
+// every round of 32 holds one: they are queued and binned 32 at a time.  A block takes a cell, or
 // above 4 times the resident blocks a run of consecutive ones, so that a
 // histogram is flushed once per run.  Bound: instruction issue.  150k sites,
 // r_max 1.0 nm, 200 bins: 9,824 us (FP64 for every candidate) -> 251 (binned
-// as met, runs of one or two cells) -> 175.
+// as met, runs of one or two cells) -> 175 (all candidates) -> 161.
 constexpr int kRdfThreads = 128;
 constexpr int kRdfStage = 128;       // home atoms staged at a time
 constexpr int kRdfBlocks = kSMs * 16;
 constexpr int kRdfQueue = 256;       // a ring: at most 31 + 64 pairs wait
+constexpr int kRdfCand = 128;        // a ring: at most 31 + 32 candidates wait, and none is written over as it is read
 constexpr int kRdfSlotBits = 26;     // atoms < 2^26; six bits of the home atom above, its seventh with r^2
 // FP32 cell units: each position is rounded by at most 2^-25 (FP32 master:
 // 2^-24.6), the offset and the difference add 2^-24 each, so a component is
@@ -91,10 +93,12 @@ __global__ void __launch_bounds__(kRdfThreads) k_rdf(const T* __restrict__ x, in
   __shared__ __align__(8) float hx[kRdfStage], hy[kRdfStage], hz[kRdfStage];   // home atoms: cell units
   __shared__ __align__(8) int ht[kRdfStage];                                   // and chain/site tags
   __shared__ uint2 queue[kRdfThreads / 32][kRdfQueue];
+  __shared__ unsigned cand[kRdfThreads / 32][kRdfCand];
   __shared__ int s_start[14], s_pre[15];
   __shared__ float s_off[14][3];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint2* qw = queue[warp];
+  unsigned* cw = cand[warp];
   const unsigned lt = (1u << lane) - 1u;
   const int c0 = (int)((long long)C * blockIdx.x / gridDim.x), c1 = (int)((long long)C * (blockIdx.x + 1) / gridDim.x);
   if (c0 >= c1) return;
@@ -143,6 +147,8 @@ __global__ void __launch_bounds__(kRdfThreads) k_rdf(const T* __restrict__ x, in
     const float far2 = rt * rt;
     const float low = e0 - 4.f * kRdfMargin * hf;   // below this one, out of range as well
     const bool fold = M == 3;   // two images of a pair can both be near a cell side away
+    // half the home cell's side and the atoms' rounding; with folded images every candidate is near
+    const float box = fold ? 4.f : 0.5f + kRdfMargin;
     for (int i0 = 0; i0 < n; i0 += kRdfStage) {
       const int ni = min(kRdfStage, n - i0);
       __syncthreads();
@@ -165,14 +171,14 @@ __global__ void __launch_bounds__(kRdfThreads) k_rdf(const T* __restrict__ x, in
           g = rdf_exact_bin<T>(x, N, perm[b + i0 + k], perm[sj], R.L, edges, n_bins, norm);
         if (g >= 0) atomicAdd(hist + g, 1u);
       };
-      const int total = s_pre[14];
-      int o = 0, qn = 0, head = 0;   // waiting pairs: ring places head .. head + qn - 1
-      for (int q = 32 * warp + lane; q - lane < total; q += kRdfThreads) {
+      int qn = 0, head = 0;   // waiting pairs: ring places head .. head + qn - 1
+      // the home atoms against candidate e (tile slot | cell << kRdfSlotBits) of each lane
+      auto walk = [&](unsigned e, bool on) {
         int sj = b, tj = 0, last = 0;   // home atoms i0 .. i0 + last - 1 pair with j
         float4 pj = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (q < total) {
-          while (q >= s_pre[o + 1]) ++o;
-          sj = s_start[o] + (q - s_pre[o]);
+        if (on) {
+          const int o = (int)(e >> kRdfSlotBits);
+          sj = (int)(e & ((1u << kRdfSlotBits) - 1u));
           pj = pos[sj];
           pj.x += s_off[o][0]; pj.y += s_off[o][1]; pj.z += s_off[o][2];
           tj = tag[sj] & (int)kTagMask;
@@ -210,6 +216,38 @@ __global__ void __launch_bounds__(kRdfThreads) k_rdf(const T* __restrict__ x, in
             qn -= 32;
           }
         }
+      };
+      // candidates that no home atom can be in range of (further than that from
+      // the cell) are left out: the others wait until 32 can be taken together
+      const int total = s_pre[14];
+      int o = 0, cn = 0, chead = 0;
+      for (int q0 = 32 * warp;; q0 += kRdfThreads) {
+        const bool more = q0 < total;
+        if (more) {
+          const int q = q0 + lane;
+          bool near = false;
+          unsigned e = 0u;
+          if (q < total) {
+            while (q >= s_pre[o + 1]) ++o;
+            const int sj = s_start[o] + (q - s_pre[o]);
+            const float4 pj = pos[sj];
+            const float bx = fmaxf(fabsf(pj.x + s_off[o][0]) - box, 0.f), by = fmaxf(fabsf(pj.y + s_off[o][1]) - box, 0.f),
+                        bz = fmaxf(fabsf(pj.z + s_off[o][2]) - box, 0.f);
+            near = bx * bx + by * by + bz * bz <= far2;
+            e = (unsigned)sj | (unsigned)o << kRdfSlotBits;
+          }
+          const unsigned m = __ballot_sync(0xffffffffu, near);
+          if (near) cw[(chead + cn + __popc(m & lt)) & (kRdfCand - 1)] = e;
+          cn += __popc(m);
+          __syncwarp();
+        }
+        while (cn >= 32 || (!more && cn > 0)) {
+          walk(cw[(chead + lane) & (kRdfCand - 1)], lane < cn);
+          const int n = min(cn, 32);
+          chead += n;
+          cn -= n;
+        }
+        if (!more) break;
       }
       __syncwarp();
       if (lane < qn) take(qw[(head + lane) & (kRdfQueue - 1)]);
