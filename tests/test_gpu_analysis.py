@@ -45,6 +45,20 @@ def test_rdf_of_lattice_distances_on_bin_edges(precision, L, n_bins):
     s.close()
 
 
+@pytest.mark.parametrize("skin,L,n_chains", [(0.1, 4.375, 55), (0.4, 6.625, 192)])
+@pytest.mark.parametrize("r_max", [0.35, 1.0])
+def test_rdf_of_full_cells(skin, L, n_chains, r_max):
+    """Cells of about 102 atoms at 3 a side (folded images) and 150 at 4 (home atoms in two stages, the second of few
+    and odd numbers), with most of the candidates in reach and with few: counts equal to the FP64 definition's."""
+    from oracle import observables as ob
+    m = chaingen.melt(n_chains, sites=50, seed=23, T=300.0, L=L)
+    s = md.System(m, skin=skin, lj_region=2)   # 3 x 3 cells of 150 atoms do not fit a tile
+    _, _, counts = s.rdf(r_max, 200)
+    _, _, want = ob.rdf(s.state()[0], L, 50, r_max, 200)
+    assert np.array_equal(counts[0], want)
+    s.close()
+
+
 def test_rdf_from_a_positive_first_edge():
     """edges[0] > 0: nearer pairs are left out, and the first edge is inclusive."""
     import ctypes
