@@ -285,14 +285,19 @@ static void launch_molecules_t(IntegMode mode, int th, int threads, const StepAr
 #undef MDG_STEP
 }
 
-// chains of more than 512 sites (and molecules, beside the static arrays) need
-// more than 48 KB of shared memory (once per device)
+// Dynamic shared memory of a form: beside the static array of the kinetic sums
+// (tile_kinetic: up to 16 KB for 512 threads, 32 KB for 1,024) it can exceed the
+// 48 KB that need no opt-in from 353 sites a chain on, so every form opts in to
+// the most that its block size asks for (once per device)
 cudaError_t step_kernels_init() {
-  const int b = (int)step_smem_bytes(1024);
   cudaError_t e = cudaSuccess;
-#define MDG_STEP_ATTR(MIXED, MODE, KE, TH) \
-  if (e == cudaSuccess)                    \
-    e = cudaFuncSetAttribute(k_step<MIXED, MODE, KE, TH, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, b)
+  auto allow = [&](const void* kernel, size_t bytes) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  };
+#define MDG_STEP_ATTR(MIXED, MODE, KE, TH)                                     \
+  allow((const void*)k_step<MIXED, MODE, KE, TH, 256>, step_smem_bytes(256));  \
+  allow((const void*)k_step<MIXED, MODE, KE, TH, 512>, step_smem_bytes(512));  \
+  allow((const void*)k_step<MIXED, MODE, KE, TH, 1024>, step_smem_bytes(1024))
 #define MDG_STEP_ATTRS(MIXED)                     \
   MDG_STEP_ATTR(MIXED, kKickKickDrift, true, 2);  \
   MDG_STEP_ATTR(MIXED, kKickKickDrift, true, 1);  \
@@ -303,10 +308,9 @@ cudaError_t step_kernels_init() {
   MDG_STEP_ATTRS(false);
 #undef MDG_STEP_ATTRS
 #undef MDG_STEP_ATTR
-  const int m = (int)molecules_smem_bytes(1024);
-#define MDG_STEP_ATTR(MODE, KE, TH) \
-  if (e == cudaSuccess)             \
-    e = cudaFuncSetAttribute(k_step_molecules<MODE, KE, TH, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, m)
+#define MDG_STEP_ATTR(MODE, KE, TH)                                                            \
+  allow((const void*)k_step_molecules<MODE, KE, TH, 128>, molecules_smem_bytes(128));          \
+  allow((const void*)k_step_molecules<MODE, KE, TH, 1024>, molecules_smem_bytes(1024))
   MDG_STEP_ATTR(kKickKickDrift, true, 2);
   MDG_STEP_ATTR(kKickKickDrift, true, 1);
   MDG_STEP_ATTR(kKickKickDrift, false, 0);
