@@ -106,25 +106,33 @@ __global__ void __launch_bounds__(kBondedBlock) k_bonded(const void* __restrict_
     }
   }
   __syncthreads();
-  // 3. sum the contributions on each home atom in a fixed order (an energy
-  // read-out passes no Fout: it has no use for them)
-  if (Fout && (int)threadIdx.x < t.len) {
+  // 3. sum the contributions on each home atom in a fixed order.  An energy
+  // read-out passes no Fout; in the mixed form it still converts the forces, so
+  // that one beyond the fixed-point range, or not a number, is reported.
+  if ((MIXED || Fout) && (int)threadIdx.x < t.len) {
     const int q = threadIdx.x + kHalo;
     const int i = t.start + threadIdx.x;
     const f3 F = chain_force(fbd, fan_a, fan_c, fdi1, fdi2, fdi3, q);
-    // the LJ force of the atom (sorted slot s)
-    const int s = inv_perm[i];
-    const long long lx = __ldg(flj + s), ly = __ldg(flj + Npad + s), lz = __ldg(flj + 2 * (size_t)Npad + s);
+    F4i o;
     if (MIXED) {
-      F4i o;
-      o.x = lx + to_fix(F.x, flags);
-      o.y = ly + to_fix(F.y, flags);
-      o.z = lz + to_fix(F.z, flags);
+      o.x = to_fix(F.x, flags);
+      o.y = to_fix(F.y, flags);
+      o.z = to_fix(F.z, flags);
       o.w = 0;
-      reinterpret_cast<F4i*>(Fout)[i] = o;
-    } else {
-      reinterpret_cast<float4*>(Fout)[i] =
-          make_float4(fix_to_float(lx) + F.x, fix_to_float(ly) + F.y, fix_to_float(lz) + F.z, 0.f);
+    }
+    if (Fout) {
+      // the LJ force of the atom (sorted slot s)
+      const int s = inv_perm[i];
+      const long long lx = __ldg(flj + s), ly = __ldg(flj + Npad + s), lz = __ldg(flj + 2 * (size_t)Npad + s);
+      if (MIXED) {
+        o.x += lx;
+        o.y += ly;
+        o.z += lz;
+        reinterpret_cast<F4i*>(Fout)[i] = o;
+      } else {
+        reinterpret_cast<float4*>(Fout)[i] =
+            make_float4(fix_to_float(lx) + F.x, fix_to_float(ly) + F.y, fix_to_float(lz) + F.z, 0.f);
+      }
     }
   }
   if (ENERGY) {
