@@ -850,6 +850,7 @@ namespace {
 
 int adj_fail(int code, const char* msg) {
   md_set_global_error(msg);
+  if (code == MD_ECUDA || code == MD_ENOMEM) cudaGetLastError();   // reported: not left to the next call
   return code;
 }
 
@@ -936,8 +937,9 @@ bool capture(md_adj* a, cudaGraphExec_t* exec, F&& body) {
   cudaGraph_t g = nullptr;
   if (cudaStreamBeginCapture(a->st, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return false;
   const int rc = body();
+  const cudaError_t refused = cudaGetLastError();
   const cudaError_t e = cudaStreamEndCapture(a->st, &g);
-  if (rc != MD_OK || e != cudaSuccess || !g) {
+  if (rc != MD_OK || refused != cudaSuccess || e != cudaSuccess || !g) {
     if (g) cudaGraphDestroy(g);
     cudaGetLastError();
     return false;
@@ -1099,7 +1101,8 @@ extern "C" int md_adj_forward(md_adj* a, const double* pos, const double* vel, d
     cudaMemcpyAsync(a->ckv, a->v, n3, cudaMemcpyDeviceToDevice, st);
   }
   double acc[2];
-  if (cudaMemcpyAsync(acc, a->acc, sizeof(acc), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+  if (cudaGetLastError() != cudaSuccess ||
+      cudaMemcpyAsync(acc, a->acc, sizeof(acc), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess)
     return adj_fail(MD_ECUDA, "forward run failed");
   a->obs[0] = acc[0] / (double)(a->K + 1);
@@ -1178,7 +1181,8 @@ extern "C" int md_adj_backward(md_adj* a, const double weight[2], double grad[5]
     }
   }
   double acc[kAccN];
-  if (cudaMemcpyAsync(acc, a->acc, sizeof(acc), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+  if (cudaGetLastError() != cudaSuccess ||
+      cudaMemcpyAsync(acc, a->acc, sizeof(acc), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess)
     return adj_fail(MD_ECUDA, "reverse run failed");
   chain_rule(a, acc, grad);

@@ -130,6 +130,7 @@ void md_set_global_error(const char* msg) { g_create_error = msg; }
 // ------------------------------------------------------------------ helpers
 static int fail(md_system* s, int code, const std::string& msg) {
   if (s) s->err = msg; else g_create_error = msg;
+  if (code == MD_ECUDA || code == MD_ENOMEM) cudaGetLastError();   // reported: not left to the next call
   return code;
 }
 #define CU(call)                                                                                      \
@@ -758,40 +759,41 @@ static void enqueue_steps(md_system* s, int k, bool repeat, const MoveReport& mr
 // rebins and repeats the block from that step's LJ launch (StepGate), so such a
 // step computes its forces from fresh bins (and is counted), instead of the
 // run stopping.  A conditional node per step, and a kernel to set its
-// condition, took 9 us of a 33 us step at 1,500 sites.
-static void enqueue_block(md_system* s, int k, bool rebin = true) {
+// condition, took 9 us of a 33 us step at 1,500 sites.  The error of a graph
+// call is returned; a refused launch is the runtime's last error.
+static cudaError_t enqueue_block(md_system* s, int k, bool rebin) {
   s->ev_used = 0;
   prof_mark(s);
   if (rebin) enqueue_rebin(s);
   MoveReport mr{};
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   cudaGraph_t g = nullptr;
-  if (s->disp == MD_DISP_REBUILD &&
-      cudaStreamGetCaptureInfo(s->st, &cs, nullptr, &g, nullptr, nullptr, nullptr) == cudaSuccess &&
-      cs == cudaStreamCaptureStatusActive &&
-      cudaGraphConditionalHandleCreate(&mr.handle, g, 0, cudaGraphCondAssignDefault) == cudaSuccess) {
+  cudaError_t e = cudaSuccess;
+  if (s->disp == MD_DISP_REBUILD) {
+    if ((e = cudaStreamGetCaptureInfo(s->st, &cs, nullptr, &g, nullptr, nullptr, nullptr)) != cudaSuccess) return e;
+    if ((e = cudaGraphConditionalHandleCreate(&mr.handle, g, 0, cudaGraphCondAssignDefault)) != cudaSuccess) return e;
     mr.ctl = s->ctl;
     mr.events = s->early;
   }
   enqueue_steps(s, k, false, mr);
-  if (!mr.ctl) return;
+  if (!mr.ctl) return cudaSuccess;
   const cudaGraphNode_t* deps = nullptr;
   const cudaGraphEdgeData* ed = nullptr;
   size_t nd = 0;
-  if (cudaStreamGetCaptureInfo(s->st, &cs, nullptr, &g, &deps, &ed, &nd) != cudaSuccess) return;
+  if ((e = cudaStreamGetCaptureInfo(s->st, &cs, nullptr, &g, &deps, &ed, &nd)) != cudaSuccess) return e;
   cudaGraphNodeParams p{};
   p.type = cudaGraphNodeTypeConditional;
   p.conditional.handle = mr.handle;
   p.conditional.type = cudaGraphCondTypeWhile;
   p.conditional.size = 1;
   cudaGraphNode_t node;
-  if (cudaGraphAddNode(&node, g, deps, ed, nd, &p) != cudaSuccess) return;
+  if ((e = cudaGraphAddNode(&node, g, deps, ed, nd, &p)) != cudaSuccess) return e;
   cudaGraph_t body = p.conditional.phGraph_out[0];
-  if (cudaStreamUpdateCaptureDependencies(s->st, &node, nullptr, 1, cudaStreamSetCaptureDependencies) != cudaSuccess)
-    return;
+  e = cudaStreamUpdateCaptureDependencies(s->st, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
+  if (e != cudaSuccess) return e;
   // the body, captured on the side stream
-  if (cudaStreamBeginCaptureToGraph(s->side, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
-    return;
+  e = cudaStreamBeginCaptureToGraph(s->side, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
+  if (e != cudaSuccess) return e;
   cudaStream_t main = s->st;
   const bool prof = s->profile;
   s->st = s->side;
@@ -802,7 +804,7 @@ static void enqueue_block(md_system* s, int k, bool rebin = true) {
   s->st = main;
   s->profile = prof;
   cudaGraph_t out = nullptr;
-  cudaStreamEndCapture(s->side, &out);
+  return cudaStreamEndCapture(s->side, &out);
 }
 // per step: LJ (two launches where tiles are large) and one update; a closing update (an early rebin adds kRebinLaunches)
 static int64_t block_launches(const md_system* s, int k) {
@@ -831,16 +833,24 @@ static void drop_rem_graphs(md_system* s) {
     if (e) { cudaGraphExecDestroy(e); e = nullptr; }
 }
 
-// a block of k steps (leading rebin included) as a graph
-static int capture_block(md_system* s, int k, cudaGraphExec_t* out) {
-  cudaGraph_t g;
+// a block of k steps as a graph; rebin: with its leading rebin + list
+static int capture_block(md_system* s, int k, bool rebin, cudaGraphExec_t* out) {
+  cudaGraph_t g = nullptr;
   CU(cudaStreamBeginCapture(s->st, cudaStreamCaptureModeThreadLocal));
-  enqueue_block(s, k, true);
-  cudaError_t e = cudaStreamEndCapture(s->st, &g);
-  if (e != cudaSuccess) return fail(s, MD_ECUDA, std::string("graph capture: ") + cudaGetErrorString(e));
+  cudaError_t e = enqueue_block(s, k, rebin);
+  const cudaError_t refused = cudaGetLastError();   // a launch, or the graph call that e tells of
+  const cudaError_t end = cudaStreamEndCapture(s->st, &g);
+  if (e == cudaSuccess) e = refused != cudaSuccess ? refused : end;
+  if (e != cudaSuccess) {
+    if (g) cudaGraphDestroy(g);
+    return fail(s, MD_ECUDA, std::string("graph capture: ") + cudaGetErrorString(e));
+  }
   e = cudaGraphInstantiate(out, g, 0);
   cudaGraphDestroy(g);
-  if (e != cudaSuccess) return fail(s, MD_ECUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
+  if (e != cudaSuccess) {
+    *out = nullptr;
+    return fail(s, MD_ECUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
+  }
   return MD_OK;
 }
 
@@ -849,24 +859,18 @@ static int capture_cycle(md_system* s) {
   if (s->cycle_fresh) { cudaGraphExecDestroy(s->cycle_fresh); s->cycle_fresh = nullptr; }
   drop_rem_graphs(s);
   s->rem_graphs.assign(s->R, nullptr);
-  for (int pass = 0; pass < 2; ++pass) {
-    const bool prof = s->profile;
-    if (pass == 1) s->profile = false;
-    cudaGraph_t g;
-    CU(cudaStreamBeginCapture(s->st, cudaStreamCaptureModeThreadLocal));
-    enqueue_block(s, s->R, pass == 0);
-    cudaError_t e = cudaStreamEndCapture(s->st, &g);
-    s->profile = prof;
-    if (e != cudaSuccess) return fail(s, MD_ECUDA, std::string("graph capture: ") + cudaGetErrorString(e));
-    e = cudaGraphInstantiate(pass == 0 ? &s->cycle : &s->cycle_fresh, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) return fail(s, MD_ECUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
-  }
-  return MD_OK;
+  const int rc = capture_block(s, s->R, true, &s->cycle);
+  if (rc) return rc;
+  const bool prof = s->profile;
+  s->profile = false;
+  const int rc_fresh = capture_block(s, s->R, false, &s->cycle_fresh);
+  s->profile = prof;
+  return rc_fresh;
 }
 
 static int check_flags(md_system* s) {
   unsigned f = 0;
+  CU(cudaGetLastError());   // a launch that was refused
   CU(cudaStreamSynchronize(s->st));
   CU(cudaMemcpy(&f, s->flags, sizeof f, cudaMemcpyDeviceToHost));
   if (!f) return MD_OK;
@@ -1120,7 +1124,7 @@ int md_step_async(md_system* s, int64_t n) {
     s->fresh = false;
     cudaGraphExec_t& gr = s->rem_graphs[rem];
     if (!gr) {
-      const int rc = capture_block(s, (int)rem, &gr);
+      const int rc = capture_block(s, (int)rem, true, &gr);
       if (rc) return rc;
     }
     if (s->profile) s->ev_used = (int)std::min<int64_t>(s->ev.size(), 3 + 3 * rem);

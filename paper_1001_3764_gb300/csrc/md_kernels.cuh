@@ -343,7 +343,9 @@ __device__ __forceinline__ void wait_for_predecessor() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
-// (dep = false: an ordinary launch, for a predecessor that is not a kernel)
+// (dep = false: an ordinary launch, for a predecessor that is not a kernel).  A
+// refused launch is left as the runtime's last error, like one by <<<>>>: the
+// captures and the synchronising calls read it.
 template <class... P, class... A>
 inline void launch_dependent(bool dep, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                              const A&... args) {

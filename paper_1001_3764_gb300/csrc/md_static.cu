@@ -60,6 +60,7 @@ extern "C" int md_bin_static(const double* pos, int32_t n_atoms, double box, int
                              int32_t* cell_start, int32_t* perm, void* cuda_stream) {
   auto fail = [](int code, const char* msg) {
     md_set_global_error(msg);
+    if (code == MD_ECUDA) cudaGetLastError();   // reported: not left to the next call
     return code;
   };
   if (!pos || !cell_of || !cell_start || !perm) return fail(MD_EINVAL, "null pointer argument");
@@ -74,10 +75,7 @@ extern "C" int md_bin_static(const double* pos, int32_t n_atoms, double box, int
   // loaded again elsewhere.
   void* sp = nullptr;
   const cudaError_t se = cudaGetSymbolAddress(&sp, g_bin_scratch);
-  if (se != cudaSuccess || !sp) {
-    cudaGetLastError();
-    return fail(MD_ECUDA, "cudaGetSymbolAddress of the binning scratch failed");
-  }
+  if (se != cudaSuccess || !sp) return fail(MD_ECUDA, "cudaGetSymbolAddress of the binning scratch failed");
   int* scratch = (int*)sp;
   // counters and digit counts (131,072 + 2 * 513 * 512 ints at most), then n ints
   const OrderBuf ob = order_buffers(scratch, n_atoms, C);
