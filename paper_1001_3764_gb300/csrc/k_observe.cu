@@ -274,9 +274,14 @@ void launch_rdf(bool mixed, const void* x, int N, const int* cell_start, const i
   if (C <= 0) return;
   const size_t sm = (size_t)n_bins * sizeof(unsigned int);
   const int grid = C < 4 * kRdfBlocks ? C : kRdfBlocks;
-  if (sm > 36000) {   // the histogram, queues and staged atoms exceed 48 KB
-    cudaFuncSetAttribute(k_rdf<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    cudaFuncSetAttribute(k_rdf<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  // The histogram, queues and staged atoms may exceed 48 KB.  The opt-in is the
+  // kernel's, not the launch's, so it is always the one for the most bins: a
+  // smaller one would take it from another thread's call between that one's
+  // opt-in and its launch.
+  if (sm > 36000) {
+    constexpr int most = kRdfMaxBins * (int)sizeof(unsigned int);
+    cudaFuncSetAttribute(k_rdf<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    cudaFuncSetAttribute(k_rdf<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   }
   if (mixed)
     k_rdf<double><<<grid, kRdfThreads, sm, st>>>((const double*)x, N, cell_start, perm, pos, tag, reps, n_reps, C,

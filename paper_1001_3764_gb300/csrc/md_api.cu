@@ -1283,7 +1283,7 @@ int md_observables(md_system* s, double* r_ee, double* rg2, double* trans_fracti
 }
 
 int md_rdf(md_system* s, int32_t n_bins, const double* edges, int64_t* counts) {
-  if (!s || !edges || !counts || n_bins < 1 || n_bins > 16384) return fail(s, MD_EINVAL, "bad arguments (1 <= n_bins <= 16384)");
+  if (!s || !edges || !counts || n_bins < 1 || n_bins > kRdfMaxBins) return fail(s, MD_EINVAL, "bad arguments (1 <= n_bins <= 16384)");
   if (s->generic) return fail(s, MD_EINVAL, "the RDF's exclusions are those of linear chains");
   if (!(edges[0] >= 0.0)) return fail(s, MD_EINVAL, "edges[0] must be >= 0");
   for (int k = 0; k < n_bins; ++k)

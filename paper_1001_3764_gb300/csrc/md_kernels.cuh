@@ -492,6 +492,7 @@ void launch_resume(cudaGraphConditionalHandle h, int* ctl, cudaStream_t st);
 // n_bins / (edges[n_bins] - edges[0]) gives the first guess of k.  pos and tag
 // are those of a rebin of the current positions; inner[k] (device) is filled
 // by rdf_inner_edges (host) with h_max the largest cell side of the replicas
+constexpr int kRdfMaxBins = 16384;
 void rdf_inner_edges(const double* edges, int n_bins, double h_max, float2* inner);
 void launch_rdf(bool mixed, const void* x, int N, const int* cell_start, const int* perm, const float4* pos,
                 const int* tag, const RepDev* reps, int n_reps, int C, const double* edges, const float2* inner,
