@@ -668,7 +668,8 @@ static void enqueue_rebin(md_system* s) {
   enqueue_build(s, !s->profile);
   prof_mark(s);
 }
-static const int kRebinLaunches = 7;   // memset counted as a launch
+// memset counted as a launch; the scan of many cells takes two
+static int rebin_launches(const md_system* s) { return 7 + (scan_seg_ints(s->C) > 0 ? 1 : 0); }
 
 static void enqueue_lj(md_system* s, bool energy, long long* flj, const StepGate& gate = StepGate{},
                        const ThermoArgs& thermo = ThermoArgs{}) {
@@ -806,9 +807,10 @@ static cudaError_t enqueue_block(md_system* s, int k, bool rebin) {
   cudaGraph_t out = nullptr;
   return cudaStreamEndCapture(s->side, &out);
 }
-// per step: LJ (two launches where tiles are large) and one update; a closing update (an early rebin adds kRebinLaunches)
+// per step: LJ (two launches where tiles are large) and one update; a closing update (an early rebin adds rebin_launches
+// and the launches of the steps it repeats)
 static int64_t block_launches(const md_system* s, int k) {
-  return kRebinLaunches + (s->lj_cap < s->tile_cap ? 3LL : 2LL) * k + 1;
+  return rebin_launches(s) + (s->lj_cap < s->tile_cap ? 3LL : 2LL) * k + 1;
 }
 
 // accumulate the event timings of the last block (requires a finished stream)
