@@ -164,7 +164,7 @@ typedef struct {
 typedef struct {
   double skin;                 /* nm; sets the cell side (>= rc + skin) */
   int32_t rebin_every;
-  int32_t lj_block;
+  int32_t lj_block;            /* 0: the default of 768 threads (md_desc.lj_block) */
   int32_t schedule;
   int32_t lj_lanes;
   int32_t lj_region;
@@ -174,13 +174,13 @@ typedef struct {
 
 /* Autotuner: times short runs of candidate settings on the system the
  * descriptor describes -- region side and LJ block shape ((2, 128), (2, 256),
- * (3, 256), (3, 384) cells / threads) with schedule (grid, persistent),
- * lanes per cluster (8, 16, 32), then cell size via (skin, rebin_every) in
- * {(0.08, 6), (0.10, 10), (0.12, 12), (0.15, 16)} nm / steps -- and writes the
- * fastest into desc->skin, rebin_every, lj_block, schedule, lj_lanes and
- * lj_region.  Candidates that
- * raise a device flag (e.g. an atom moving more than skin/2 between rebins)
- * are rejected.  With cache_path != NULL the result is looked up in / appended
+ * (3, 256), (3, 384) cells / threads, and 3 with the default block where that
+ * is another) with schedule (grid, persistent), lanes per cluster (8, 16, 32),
+ * then cell size via (skin, rebin_every) in {(0.08, 6), (0.10, 10),
+ * (0.12, 12), (0.15, 16)} nm / steps -- and writes the fastest into
+ * desc->skin, rebin_every, lj_block, schedule, lj_lanes and lj_region.
+ * Candidates that raise a device flag (e.g. an atom moving more than skin/2
+ * between rebins) are rejected.  With cache_path != NULL the result is looked up in / appended
  * to that text file, keyed by GPU, precision, replica count and atom-count and
  * box-size buckets.  trial_cycles: rebin cycles timed per candidate (>= 1).
  * Allocates and frees its own trial systems; the caller's state is only

@@ -1686,10 +1686,11 @@ extern "C" int md_autotune(md_desc* d, int32_t trial_cycles, const char* cache_p
   const int region0 = d->lj_region ? d->lj_region : 3;
   md_tuning best{d->skin, d->rebin_every, d->lj_block ? d->lj_block : (region0 == 3 ? 384 : 256), d->schedule,
                  d->lj_lanes ? d->lj_lanes : 8, region0, 0, 1e300};
-  auto apply = [&](const md_tuning& t) {
-    d->skin = t.skin; d->rebin_every = t.rebin_every; d->lj_block = t.lj_block; d->schedule = t.schedule;
-    d->lj_lanes = t.lj_lanes; d->lj_region = t.lj_region;
+  auto apply_to = [](md_desc& c, const md_tuning& t) {
+    c.skin = t.skin; c.rebin_every = t.rebin_every; c.lj_block = t.lj_block; c.schedule = t.schedule;
+    c.lj_lanes = t.lj_lanes; c.lj_region = t.lj_region;
   };
+  auto apply = [&](const md_tuning& t) { apply_to(*d, t); };
   if (cache_path) {
     if (FILE* f = fopen(cache_path, "r")) {
       char line[512], k[256];
@@ -1711,14 +1712,22 @@ extern "C" int md_autotune(md_desc* d, int32_t trial_cycles, const char* cache_p
     }
   }
   bool any = false;
+  // the block that a descriptor's default stands for: 768 threads, which only
+  // the default gives, where one tile fills an SM (plan_regions)
+  auto default_block = [](md_desc c) {
+    md_system t;
+    c.lj_block = 0;
+    return configure(&t, &c) == MD_OK ? t.lj_block : 0;
+  };
   // region side x block shape x schedule at the descriptor's cell size
-  const int shapes[4][2] = {{2, 128}, {2, 256}, {3, 256}, {3, 384}};
+  const int shapes[5][2] = {{2, 128}, {2, 256}, {3, 256}, {3, 384}, {3, 0}};
   for (const auto& rb : shapes)
     for (int sch : {(int)MD_SCHED_GRID, (int)MD_SCHED_PERSISTENT}) {
       md_desc c = *d;
       c.lj_region = rb[0];
       c.lj_block = rb[1];
       c.schedule = sch;
+      if (!rb[1] && default_block(c) != 768) continue;   // one of the others
       c.lj_lanes = best.lj_lanes;
       double us = 0.0;
       if (tune_trial(c, trial_cycles, &us) == MD_OK && us < best.us_per_step) {
@@ -1741,20 +1750,25 @@ extern "C" int md_autotune(md_desc* d, int32_t trial_cycles, const char* cache_p
     }
   }
   // cell size through (skin, rebin interval)
+  // (a block that is the default's at one size stays the default's at the others)
+  auto at_best = [&](int block) {
+    md_desc c = *d;
+    apply_to(c, best);
+    c.lj_block = block;
+    return c;
+  };
+  const bool dflt = best.lj_block == 0 || best.lj_block == default_block(at_best(0));
   const double skins[4] = {0.08, 0.10, 0.12, 0.15};
   const int reb[4] = {6, 10, 12, 16};
   for (int k = 0; k < 4; ++k) {
     if (skins[k] == best.skin && reb[k] == best.rebin_every) continue;
-    md_desc c = *d;
-    c.lj_region = best.lj_region;
-    c.lj_block = best.lj_block;
-    c.schedule = best.schedule;
-    c.lj_lanes = best.lj_lanes;
+    md_desc c = at_best(best.lj_block);
     c.skin = skins[k];
     c.rebin_every = reb[k];
+    if (dflt) c.lj_block = default_block(c) == 768 ? 0 : default_block(c);
     double us = 0.0;
     if (tune_trial(c, trial_cycles, &us) == MD_OK && us < best.us_per_step) {
-      best = md_tuning{skins[k], reb[k], best.lj_block, best.schedule, best.lj_lanes, best.lj_region, 0, us};
+      best = md_tuning{skins[k], reb[k], c.lj_block, best.schedule, best.lj_lanes, best.lj_region, 0, us};
       any = true;
     }
   }
