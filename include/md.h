@@ -60,8 +60,8 @@ enum { MD_NVE = 0, MD_VRESCALE = 1, MD_NOSE_HOOVER = 2 };   /* thermostat */
 enum { MD_SCHED_GRID = 0, MD_SCHED_PERSISTENT = 1 };
 /* What a step does when an atom has moved more than skin/2 since the last
  * list build: rebuild the bins and list before its forces (a conditional
- * node at the end of the block's graph, which repeats the block from that
- * step on), or report MD_EUNSTABLE at the next synchronising
+ * node after every group of up to 16 steps of the block's graph, which repeats
+ * the group from that step on), or report MD_EUNSTABLE at the next synchronising
  * call (graphs without conditional nodes, which profilers can take apart). */
 enum { MD_DISP_REBUILD = 0, MD_DISP_ERROR = 1 };
 
@@ -350,8 +350,8 @@ int md_profile_read(md_system *sys, double *ms_total, int64_t *launches);
 int md_profile_reset(md_system *sys);
 
 /* Kernel launches per call of md_step(n_steps) (all library kernels and
- * memsets; an early rebuild repeats its block's launches, those before the
- * step that triggered it without effect). */
+ * memsets; an early rebuild repeats the launches of its group of up to 16
+ * steps, those before the step that triggered it without effect). */
 int64_t md_launches_per_call(md_system *sys, int64_t n_steps);
 
 /* Cell binning of one periodic box into caller-provided DEVICE arrays, with

@@ -1022,6 +1022,15 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_cl_force(
     const RegionShape& S = shapes[item.shape];
     const RepDev& R = reps[item.rep];
     const int t_base = task_base[r];
+    if (!persistent && it == 0) {
+      // (read together with the item, whose loads are asked for here, not after the branch)
+      const bool off = lj_off(gate);
+      asm volatile("" ::"r"(item.region), "r"(t_base));
+      if (off) {
+        wait_for_predecessor();
+        return;
+      }
+    }
     __syncthreads();   // the previous item's tables are no longer read
     region_setup(T, item, S, cells, cell_start, cl_start);
     const int total = T.off[T.n_tile];
@@ -1038,19 +1047,21 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_cl_force(
         for (int t = threadIdx.x; t < (3 * total + 3) / 4; t += NT) reinterpret_cast<int4*>(ax)[t] = make_int4(0, 0, 0, 0);
       if (threadIdx.x == 0) sh_q = 0;
     }
-    if (!persistent) {
-      wait_for_predecessor();
-      if (!lj_runs(gate)) {
-        asm volatile("cp.async.wait_all;" ::: "memory");
-        return;
-      }
+    // (the gate is read while the copies of the tile are under way)
+    const bool gated = !persistent && gate.ctl;
+    int2 ctl = make_int2(0, 0);
+    if (!persistent) wait_for_predecessor();
+    if (gated) ctl = gate_ctl(gate);
+    if (fits) tile_issue<NT>(T, item.need, pos, sp);
+    if (gated && !lj_runs(gate, ctl)) {
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      return;
     }
     if (!fits) {
       // left to the launch for large tiles, or too large for the list build as well
       if (threadIdx.x == 0 && (total > big.tile_cap || T.ncl[T.n_home] > kRegionClusterCap))
         atomicOr(flags, kFlagNbrOverflow);
     } else {
-      tile_issue<NT>(T, item.need, pos, sp);
       tile_finish<NT>(T, item.need, sp);   // ends with a barrier
       const LjConst c = lj_const(R);
       for (;;) {

@@ -44,6 +44,15 @@ __device__ __forceinline__ void update_atom(const T (&F)[3], T (&xi)[3], T (&vi)
   }
 }
 
+// A launch that is off passes its wait and leaves (the gate is read together with the tile)
+template <int MODE>
+__device__ __forceinline__ bool step_off(const StepGate& gate, const Tile& t) {
+  const bool off = MODE == kKickOnly ? !lj_runs(gate) : !drift_runs(gate);
+  asm volatile("" ::"r"(t.start));
+  if (off) wait_for_predecessor();
+  return off;
+}
+
 template <bool MIXED, int MODE, bool KE, int TH, int NT>
 __global__ void __launch_bounds__(NT, NT == 256 ? 4 : NT == 512 ? 2 : 1)
     k_step(void* __restrict__ xv, void* __restrict__ vv, int* __restrict__ img, void* __restrict__ Fv,
@@ -66,6 +75,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : NT == 512 ? 2 : 1)
   const RepDev& R = reps[t.rep];
   const int tid = threadIdx.x, i = t.start + tid, S = fp.sites;
   const bool on = tid < t.len;
+  if (step_off<MODE>(gate, t)) return;
   int sm = 0, slot = 0;
   T xi[3];
   if (on) {
@@ -97,7 +107,6 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : NT == 512 ? 2 : 1)
   // runs while the last LJ blocks finish
   wait_for_predecessor();
   __syncthreads();
-  if (MODE == kKickOnly ? !lj_runs(gate) : !drift_runs(gate)) return;
   AtomOut o;
   o.ke = 0.0;
   o.mom[0] = o.mom[1] = o.mom[2] = 0.0;
@@ -177,6 +186,7 @@ __global__ void __launch_bounds__(NT) k_step_molecules(double* __restrict__ x, d
   const RepDev& R = reps[t.rep];
   const int tid = threadIdx.x, i = t.start + tid;
   const bool on = tid < t.len;
+  if (step_off<MODE>(gate, t)) return;
   int type = 0, slot = 0;
   if (on) {
     type = atom_type(site[i], fp);
@@ -214,7 +224,6 @@ __global__ void __launch_bounds__(NT) k_step_molecules(double* __restrict__ x, d
   // all before this line reads what the update before the LJ launch left (k_step)
   wait_for_predecessor();
   __syncthreads();
-  if (MODE == kKickOnly ? !lj_runs(gate) : !drift_runs(gate)) return;
   AtomOut o;
   o.ke = 0.0;
   o.mom[0] = o.mom[1] = o.mom[2] = 0.0;

@@ -718,20 +718,20 @@ static StepArgs step_args(md_system* s, bool chain_tiles, const long long* flj, 
                   (int)(chain_tiles ? s->t_chain.size() : s->t_int.size()), s->reps, s->kepart, s->lam, s->flags};
 }
 
-// Steps first .. k - 1 of a block of k, LJ launch first on (first = 0: from
-// the opening drift), and the closing kick.  The opening drift clears an LJ
+// Steps first .. last - 1 of a block of k and, with the last, the closing
+// kick; repeat: from LJ launch `first` on.  The opening drift clears an LJ
 // buffer, and between LJ launches one kernel does the bonded forces, the
 // update and the clearing of the other buffer; the last one closes the step
 // and leaves the force.
-static void enqueue_steps(md_system* s, int k, bool repeat, const MoveReport& mr) {
+static void enqueue_steps(md_system* s, int first, int last, int k, bool repeat, const MoveReport& mr) {
   const TopoDev* topo = s->generic ? &s->topo : nullptr;
-  for (int j = 0; j < k; ++j) {
+  for (int j = first; j < last; ++j) {
     long long* flj = s->flj[j & 1];
     // launched as dependents of the kernel before, but where the profile's event
-    // records come in between, and a repeat's first LJ launch: what that reads
-    // before its wait is the list build's, its predecessor's
-    const StepGate gate{mr.ctl, j, repeat ? 1 : 0, !s->profile && !(repeat && j == 0)};
-    if (j == 0 && repeat) {
+    // records or a WHILE node come in between, and a repeat's first LJ launch: what
+    // that reads before its wait is the list build's, its predecessor's
+    const StepGate gate{mr.ctl, j, repeat ? 1 : 0, !s->profile && (j > first || (j == 0 && !repeat))};
+    if (j == first && repeat) {
       // a repeat resumes at an LJ launch
     } else if (j == 0) {
       launch_integrate(s->mixed, kKickDrift, s->thermo, step_args(s, false, nullptr, flj), s->fp, gate, mr, s->st);
@@ -744,40 +744,43 @@ static void enqueue_steps(md_system* s, int k, bool repeat, const MoveReport& mr
     if (s->thermo != MD_NVE)
       thermo = ThermoArgs{s->n_reps, s->thermo, j > 0, s->kepart, s->lam, 1.0 - s->dt / s->tau, s->dt};
     prof_mark(s);   // closes the integrate group
-    enqueue_lj(s, false, flj, gate, thermo);
+    StepGate lj_gate = gate;
+    lj_gate.dep = !s->profile && !(repeat && j == first);
+    enqueue_lj(s, false, flj, lj_gate, thermo);
     prof_mark(s);
   }
+  if (last < k) return;
   const StepGate gate{mr.ctl, k - 1, repeat ? 1 : 0, !s->profile};
   launch_step(s->mixed, kKickOnly, s->thermo, s->S, step_args(s, true, s->flj[(k - 1) & 1], nullptr), s->fp, topo, gate,
               mr, s->st);
   prof_mark(s);
 }
 
-// One block of k steps: rebin + list (unless the bins and list are already
-// those of the current positions), k velocity-Verlet steps.  Inside a capture,
-// with MD_DISP_REBUILD, a WHILE node follows whose condition the drifts' kernels
-// set when an atom has moved more than skin/2 since the last rebin: its body
-// rebins and repeats the block from that step's LJ launch (StepGate), so such a
-// step computes its forces from fresh bins (and is counted), instead of the
-// run stopping.  A conditional node per step, and a kernel to set its
-// condition, took 9 us of a 33 us step at 1,500 sites.  The error of a graph
-// call is returned; a refused launch is the runtime's last error.
-static cudaError_t enqueue_block(md_system* s, int k, bool rebin) {
-  s->ev_used = 0;
-  prof_mark(s);
-  if (rebin) enqueue_rebin(s);
+// Steps that share a WHILE node.  A report leaves the rest of its group without
+// effect, and its repeat the launches before, so an early rebin costs a group
+// of launches that are off, and a node that is not taken 20 us at 1,500 sites (a
+// node per step and a kernel to set its condition: 9 us of a 33 us step).  506k
+// sites, us a step, with a node per step / one per block whose launches worked
+// before they read the gate / now: 211 / 238 / 177 with 2 early rebins a block of
+// 50 steps, 286 / 766 / 272 with 16, 518 / 2,073 / 528 with one every step; 213 /
+// 174 / 174 without, in blocks of 10.
+constexpr int kGroupSteps = 10, kOneGroup = 16;
+
+// A group of steps inside a capture and the WHILE node after it, whose
+// condition the drifts' kernels set when an atom has moved more than skin/2
+// since the last rebin: its body rebins and repeats the group from that step's
+// LJ launch (StepGate), so such a step computes its forces from fresh bins (and
+// is counted), instead of the run stopping.
+static cudaError_t enqueue_group(md_system* s, int first, int last, int k) {
   MoveReport mr{};
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   cudaGraph_t g = nullptr;
-  cudaError_t e = cudaSuccess;
-  if (s->disp == MD_DISP_REBUILD) {
-    if ((e = cudaStreamGetCaptureInfo(s->st, &cs, nullptr, &g, nullptr, nullptr, nullptr)) != cudaSuccess) return e;
-    if ((e = cudaGraphConditionalHandleCreate(&mr.handle, g, 0, cudaGraphCondAssignDefault)) != cudaSuccess) return e;
-    mr.ctl = s->ctl;
-    mr.events = s->early;
-  }
-  enqueue_steps(s, k, false, mr);
-  if (!mr.ctl) return cudaSuccess;
+  cudaError_t e = cudaStreamGetCaptureInfo(s->st, &cs, nullptr, &g, nullptr, nullptr, nullptr);
+  if (e != cudaSuccess) return e;
+  if ((e = cudaGraphConditionalHandleCreate(&mr.handle, g, 0, cudaGraphCondAssignDefault)) != cudaSuccess) return e;
+  mr.ctl = s->ctl;
+  mr.events = s->early;
+  enqueue_steps(s, first, last, k, false, mr);
   const cudaGraphNode_t* deps = nullptr;
   const cudaGraphEdgeData* ed = nullptr;
   size_t nd = 0;
@@ -801,11 +804,31 @@ static cudaError_t enqueue_block(md_system* s, int k, bool rebin) {
   s->profile = false;
   launch_resume(mr.handle, s->ctl, s->st);
   enqueue_rebin(s);
-  enqueue_steps(s, k, true, mr);
+  enqueue_steps(s, first, last, k, true, mr);
   s->st = main;
   s->profile = prof;
   cudaGraph_t out = nullptr;
   return cudaStreamEndCapture(s->side, &out);
+}
+
+// One block of k steps, inside a capture: rebin + list (unless the bins and
+// list are already those of the current positions), k velocity-Verlet steps,
+// with MD_DISP_REBUILD in groups.  The error of a graph call is returned; a
+// refused launch is the runtime's last error.
+static cudaError_t enqueue_block(md_system* s, int k, bool rebin) {
+  s->ev_used = 0;
+  prof_mark(s);
+  if (rebin) enqueue_rebin(s);
+  if (s->disp != MD_DISP_REBUILD) {
+    enqueue_steps(s, 0, k, k, false, MoveReport{});
+    return cudaSuccess;
+  }
+  const int groups = k <= kOneGroup ? 1 : (k + kGroupSteps - 1) / kGroupSteps;
+  for (int q = 0; q < groups; ++q) {
+    const cudaError_t e = enqueue_group(s, (int)((int64_t)k * q / groups), (int)((int64_t)k * (q + 1) / groups), k);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 // per step: LJ (two launches where tiles are large) and one update; a closing update (an early rebin adds rebin_launches
 // and the launches of the steps it repeats)

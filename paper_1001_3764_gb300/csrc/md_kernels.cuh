@@ -289,11 +289,11 @@ struct TopoDev {
 
 struct F4i { long long x, y, z, w; };   // fixed-point force, 32 B
 
-// Early rebins (displacement beyond skin/2) inside a block of steps.  ctl[0]
+// Early rebins (displacement beyond skin/2) inside a group of steps.  ctl[0]
 // is the drift that found such an atom (kNoMove: none) and ctl[1] the one a
 // repeat resumes at.  Drift j comes before LJ launch j.  When drift m reports,
-// everything after it in the block does nothing; the WHILE node at the block's
-// end then rebins and runs the block again from LJ launch m on.  So a step
+// everything after it in the group does nothing; the WHILE node at the group's
+// end then rebins and runs the group again from LJ launch m on.  So a step
 // costs no graph node of its own for the check.
 constexpr int kNoMove = 0x7fffffff;
 struct StepGate {
@@ -302,15 +302,29 @@ struct StepGate {
   int repeat;       // 1 inside the WHILE body
   bool dep;         // launch_dependent
 };
-__device__ __forceinline__ bool lj_runs(const StepGate& g) {
-  if (!g.ctl) return true;
-  const volatile int* c = g.ctl;
-  return c[0] > g.j && (!g.repeat || g.j >= c[1]);
+__device__ __forceinline__ int2 gate_ctl(const StepGate& g) {
+  int2 c;
+  asm volatile("ld.volatile.global.v2.s32 {%0, %1}, [%2];" : "=r"(c.x), "=r"(c.y) : "l"(g.ctl) : "memory");
+  return c;
 }
+__device__ __forceinline__ bool lj_runs(const StepGate& g, int2 c) { return c.x > g.j && (!g.repeat || g.j >= c.y); }
+__device__ __forceinline__ bool lj_runs(const StepGate& g) { return !g.ctl || lj_runs(g, gate_ctl(g)); }
 __device__ __forceinline__ bool drift_runs(const StepGate& g) {
   if (!g.ctl) return true;
-  const volatile int* c = g.ctl;   // c[0] == j: another block of this launch reported
-  return c[0] >= g.j && (!g.repeat || g.j > c[1]);
+  const int2 c = gate_ctl(g);   // c.x == j: another block of this launch reported
+  return c.x >= g.j && (!g.repeat || g.j > c.y);
+}
+// What an LJ launch knows before its wait: a drift before its predecessor has
+// reported, or the repeat resumes later.  Its predecessor, drift j, may be
+// writing j, which does not change the answer, so it is the same for all
+// threads; the launch asks lj_runs after the wait.  A step launch asks before
+// its wait alone: its predecessor, an LJ launch, writes nothing here, and what
+// its own blocks write (c.x = j) leaves drift_runs as it is.  So launches that
+// are off do no work.
+__device__ __forceinline__ bool lj_off(const StepGate& g) {
+  if (!g.ctl) return false;
+  const int2 c = gate_ctl(g);
+  return c.x < g.j || (g.repeat && g.j < c.y);
 }
 // where an atom beyond skin/2 is reported: ctl null, kFlagDisplacement; else
 // ctl[0] = j, and the first report sets the condition and counts the event
