@@ -36,8 +36,6 @@ thread_local std::string g_create_error;
 
 size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
-struct RegionRef { int rep, shape; };   // a region's replica and shape
-
 }  // namespace
 
 struct md_system {
@@ -71,13 +69,13 @@ struct md_system {
   int* ncl = nullptr;                        // entries per cluster
   int* cl_start = nullptr;                   // first cluster of each cell [C + 1]
   int64_t n_cl_max = 0;
-  std::vector<RegionRef> regions_h;
-  std::vector<int> region_cells_h;           // tile cells of every region (kRegionCells each, -1 past the last)
+  int n_regions = 0;
   std::vector<RegionShape> shapes_h;
   int* region_cells = nullptr;
   RegionShape* shapes = nullptr;
-  std::vector<WorkItem> items_h;             // blocks of the LJ kernel, then those of the list build
-  WorkItem* items = nullptr;
+  std::vector<ItemRun> runs_h;               // what the items are made from (launch_plan)
+  ItemRun* runs = nullptr;
+  WorkItem* items = nullptr;                 // blocks of the LJ kernel, then those of the list build
   int n_lj_items = 0, n_build_items = 0;
   ClusterTask* tasks = nullptr;              // each LJ item's clusters in task order, from task_base[item] on
   int *task_base = nullptr, *n_tasks = nullptr, *big = nullptr;
@@ -245,32 +243,8 @@ static RegionShape make_shape(int sx, int sy) {
   return S;
 }
 
-// Work items of one region: its home cells in groups of `rows` rows of the
-// shape (0: single cells), each group's clusters over `parts` blocks.
-static void add_items(md_system* s, int region, int rows, int parts) {
-  const RegionRef g = s->regions_h[region];
-  const RegionShape& S = s->shapes_h[g.shape];
-  const int sx = g.shape % s->lj_region + 1;
-  const int step = rows > 0 ? rows * sx : 1;
-  for (int h = 0; h < S.n_home; h += step) {
-    WorkItem w{};
-    w.region = region;
-    w.rep = g.rep;
-    w.shape = g.shape;
-    w.h0 = (unsigned char)h;
-    w.h1 = (unsigned char)std::min(S.n_home, h + step);
-    w.parts = (unsigned char)parts;
-    for (int c = w.h0; c < w.h1; ++c)
-      for (int q = 0; q < 14; ++q) w.need |= 1ull << S.nb[c][q];
-    for (int p = 0; p < parts; ++p) {
-      w.part = (unsigned char)p;
-      s->items_h.push_back(w);
-    }
-  }
-}
-
 // Regions of G x G x 1 cells over every replica (narrower at the high faces
-// when G does not divide M), their tile cells, and the work items.
+// when G does not divide M) and the runs of their work items.
 static void plan_regions(md_system* s, bool grid_schedule) {
   const int G = s->lj_region;
   // Where two of the largest tiles do not fit an SM's shared memory (cells
@@ -296,26 +270,21 @@ static void plan_regions(md_system* s, bool grid_schedule) {
     if (rows > 2 * kSMs && 2 * large_atoms <= s->N) s->lj_cap = two;
     else large.assign(s->n_reps, 0);
   }
-  s->regions_h.clear();
-  s->region_cells_h.clear();
-  for (int r = 0; r < s->n_reps; ++r) {
-    const int M = s->reps_h[r].M, base = s->reps_h[r].cell_base;
-    for (int z = 0; z < M; ++z)
-      for (int y = 0; y < M; y += G)
-        for (int x = 0; x < M; x += G) {
-          const int shape = (std::min(G, M - x) - 1) + G * (std::min(G, M - y) - 1);
-          const RegionShape& S = s->shapes_h[shape];
-          s->regions_h.push_back(RegionRef{r, shape});
-          for (int k = 0; k < kRegionCells; ++k) {
-            int c = -1;
-            if (k < S.n_tile) {
-              const int cx = (x + S.off[k][0] + M) % M, cy = (y + S.off[k][1] + M) % M, cz = (z + S.off[k][2] + M) % M;
-              c = base + (cz * M + cy) * M + cx;
-            }
-            s->region_cells_h.push_back(c);
-          }
-        }
+  int n_rows = 0, n_cells = 0, R = 0;
+  for (RepDev& q : s->reps_h) {
+    const int nx = (q.M + G - 1) / G;
+    q.region_off = R;
+    R += nx * nx * q.M;
+    n_rows += nx * q.M * q.M;
+    n_cells += q.M * q.M * q.M;
   }
+  s->n_regions = R;
+  // regions of a shape in a replica
+  const int n_shapes = (int)s->shapes_h.size();
+  auto regions_of = [&](int r, int shape) {
+    auto along = [&](int side) { return side == G ? s->reps_h[r].M / G : s->reps_h[r].M % G == side ? 1 : 0; };
+    return along(shape % G + 1) * along(shape / G + 1) * s->reps_h[r].M;
+  };
   // Work items, the regions with most cells first (narrow regions fill the
   // tail: LJ 137.6 -> 128.1 us at 506k sites, M = 22, 47.8 -> 37.6 at 120k).
   // A system of few regions is split, since a block spends 6 us on set-up
@@ -323,19 +292,21 @@ static void plan_regions(md_system* s, bool grid_schedule) {
   //   cells while all are resident at once: 24.6 -> 14.2 at 1,500 sites, 27.8 -> 16.2 at 12,000
   //   rows likewise (else whole): 25.6 -> 16.3 at 18,750, 24.8 -> 21.2 at 35,100; whole 47.7, rows 65.3 at 150k
   //   between 1 and 2 regions per SM: rows from the second on (35.9 -> 27.4 at 84,000, M = 12)
-  const int R = (int)s->regions_h.size();
-  std::vector<int> order(R);
-  for (int r = 0; r < R; ++r) order[r] = r;
-  std::stable_sort(order.begin(), order.end(), [s](int a, int b) {
-    return s->shapes_h[s->regions_h[a].shape].n_home > s->shapes_h[s->regions_h[b].shape].n_home;
-  });
-  int n_rows = 0, n_cells = 0;
-  for (const RegionRef& g : s->regions_h) {
-    n_rows += g.shape / G + 1;
-    n_cells += s->shapes_h[g.shape].n_home;
-  }
+  std::vector<int> order(n_shapes);
+  for (int k = 0; k < n_shapes; ++k) order[k] = k;
+  std::stable_sort(order.begin(), order.end(),
+                   [s](int a, int b) { return s->shapes_h[a].n_home > s->shapes_h[b].n_home; });
+  s->runs_h.clear();
+  int n_items = 0;
+  // rows of home cells a block takes (0: a single cell)
+  auto add_run = [&](int r, int shape, int region0, int count, int rows, int parts) {
+    if (count <= 0) return;
+    const int n_home = s->shapes_h[shape].n_home;
+    const int step = std::min(n_home, rows > 0 ? rows * (shape % G + 1) : 1);
+    s->runs_h.push_back(ItemRun{n_items, r, shape, region0, step, parts});
+    n_items += count * ((n_home + step - 1) / step) * parts;
+  };
   constexpr int kWhole = 255;
-  s->items_h.clear();
   const int per_sm = lj_tiles_per_sm(s->lj_cap), slots = per_sm * kSMs;
   const int lj_rows = n_cells <= slots ? 0 : n_rows <= slots ? 1 : kWhole;
   // default block: 24 warps an SM, as two resident blocks where two tiles fit
@@ -345,15 +316,25 @@ static void plan_regions(md_system* s, bool grid_schedule) {
   // the second launch takes one block of 24 warps an SM: its items are whole
   // regions, rows or cells, by how many there are
   int n_large = 0;
-  for (const RegionRef& g : s->regions_h)
-    if (large[g.rep] && g.shape == (int)s->shapes_h.size() - 1) ++n_large;
+  for (int r = 0; r < s->n_reps; ++r)
+    if (large[r]) n_large += regions_of(r, n_shapes - 1);
   const int large_rows = 9 * n_large <= kSMs ? 0 : 3 * n_large <= kSMs ? 1 : kWhole;
-  for (int q = 0; q < R; ++q) {
-    const RegionRef& g = s->regions_h[order[q]];
-    if (large[g.rep] && g.shape == (int)s->shapes_h.size() - 1) add_items(s, order[q], large_rows, 1);
-    else add_items(s, order[q], lj_rows == kWhole && per_sm >= 2 && R <= slots && q >= kSMs ? 1 : lj_rows, 1);
-  }
-  s->n_lj_items = (int)s->items_h.size();
+  int q = 0;   // regions so far
+  for (int shape : order)
+    for (int r = 0; r < s->n_reps; ++r) {
+      const int n = regions_of(r, shape);
+      if (large[r] && shape == n_shapes - 1) {
+        add_run(r, shape, 0, n, large_rows, 1);
+      } else if (lj_rows == kWhole && per_sm >= 2 && R <= slots) {
+        const int whole = std::max(0, std::min(n, kSMs - q));
+        add_run(r, shape, 0, whole, kWhole, 1);
+        add_run(r, shape, whole, n - whole, 1, 1);
+      } else {
+        add_run(r, shape, 0, n, lj_rows, 1);
+      }
+      q += n;
+    }
+  s->n_lj_items = n_items;
   // The list build gives a warp a cluster at a time (7 us alone), 32 warps an
   // SM.  With the task order, us (whole regions / rows / cells / cells in 3 parts):
   //   - / 31 / 21 / 18.6 at 1,500 sites, 67 / 35 / 23 / 18.8 at 6,000, 62 / 33 / 26 / 31 at 12,000 (216 cells),
@@ -361,8 +342,10 @@ static void plan_regions(md_system* s, bool grid_schedule) {
   //   236 / 243 / 272 at 506k (1,408), 317 / 336 / 388 at 737k (2,025), 609 / 639 / 774 at 1.5M;
   // between 600 and 1,800 regions the last wave decides, by up to 8% either way
   const int parts = n_cells <= 128 ? 3 : 1;
-  for (int r : order) add_items(s, r, R >= 12 * kSMs ? kWhole : R >= 2 * kSMs ? 1 : 0, parts);
-  s->n_build_items = (int)s->items_h.size() - s->n_lj_items;
+  for (int shape : order)
+    for (int r = 0; r < s->n_reps; ++r)
+      add_run(r, shape, 0, regions_of(r, shape), R >= 12 * kSMs ? kWhole : R >= 2 * kSMs ? 1 : 0, parts);
+  s->n_build_items = n_items - s->n_lj_items;
 }
 
 // The per-type lists of Sec. 3.3 from a molecule's bond graph: each atom's
@@ -588,9 +571,10 @@ static size_t plan(md_system* s, char* base) {
   s->pos = (float4*)take(N * sizeof(float4));
   s->tag = (int*)take(N * sizeof(int));
   s->perm = (int*)take(N * sizeof(int));
-  s->region_cells = (int*)take(sizeof(int) * s->region_cells_h.size());
+  s->region_cells = (int*)take(sizeof(int) * (size_t)kRegionCells * s->n_regions);
   s->shapes = (RegionShape*)take(sizeof(RegionShape) * s->shapes_h.size());
-  s->items = (WorkItem*)take(sizeof(WorkItem) * s->items_h.size());
+  s->runs = (ItemRun*)take(sizeof(ItemRun) * s->runs_h.size());
+  s->items = (WorkItem*)take(sizeof(WorkItem) * (size_t)(s->n_lj_items + s->n_build_items));
   s->tasks = (ClusterTask*)take(sizeof(ClusterTask) * (size_t)s->n_cl_max);
   s->task_base = (int*)take(sizeof(int) * (size_t)s->n_lj_items);
   s->n_tasks = (int*)take(2 * sizeof(int));
@@ -1100,7 +1084,6 @@ int md_create(const md_desc* d, md_system** out) {
             up(s->tiles_int, s->t_int.data(), sizeof(Tile) * s->t_int.size()) &&
             up(s->site, site.data(), sizeof(uint16_t) * s->N) &&
             up(s->lam, lam0.data(), sizeof(double) * lam0.size()) &&
-            up(s->region_cells, s->region_cells_h.data(), sizeof(int) * s->region_cells_h.size()) &&
             (!s->generic || (up(s->mtype, s->mtype_h.data(), s->mtype_h.size()) &&
                              up((void*)s->topo.b_off, s->t_boff.data(), s->t_boff.size() * sizeof(int)) &&
                              up((void*)s->topo.b_at, s->t_bat.data(), s->t_bat.size() * sizeof(int)) &&
@@ -1112,15 +1095,19 @@ int md_create(const md_desc* d, md_system** out) {
                              up((void*)s->topo.x_at, s->t_xat.data(), s->t_xat.size() * sizeof(int)) &&
                              up((void*)s->topo.terms, s->t_terms.data(), s->t_terms.size() * sizeof(ushort4)))) &&
             up(s->shapes, s->shapes_h.data(), sizeof(RegionShape) * s->shapes_h.size()) &&
-            up(s->items, s->items_h.data(), sizeof(WorkItem) * s->items_h.size()) &&
+            up(s->runs, s->runs_h.data(), sizeof(ItemRun) * s->runs_h.size()) &&
             up(s->tiles_chain, s->t_chain.data(), sizeof(Tile) * s->t_chain.size()) &&
             cudaMemsetAsync(s->flj[0], 0, 3 * (size_t)s->Npad * sizeof(long long), s->st) == cudaSuccess &&
             cudaMemsetAsync(s->flj[1], 0, 3 * (size_t)s->Npad * sizeof(long long), s->st) == cudaSuccess &&
             cudaMemsetAsync(s->work, 0, 2 * sizeof(int), s->st) == cudaSuccess &&
             cudaMemsetAsync(s->flags, 0, sizeof(unsigned), s->st) == cudaSuccess &&
             up(s->ctl, ctl0, sizeof ctl0) &&
-            cudaMemsetAsync(s->early, 0, sizeof(unsigned long long), s->st) == cudaSuccess &&
-            cudaStreamSynchronize(s->st) == cudaSuccess;
+            cudaMemsetAsync(s->early, 0, sizeof(unsigned long long), s->st) == cudaSuccess;
+  if (ok) {
+    launch_plan(s->reps, s->n_reps, s->shapes, s->lj_region, s->n_regions, s->region_cells, s->runs,
+                (int)s->runs_h.size(), s->n_lj_items + s->n_build_items, s->items, s->st);
+    ok = cudaGetLastError() == cudaSuccess && cudaStreamSynchronize(s->st) == cudaSuccess;
+  }
   if (!ok) { fail(s, MD_ECUDA, "initial upload failed"); return bail(MD_ECUDA); }
   rc = upload_state(s, d->pos, d->vel);
   if (rc) return bail(rc);
@@ -1564,10 +1551,17 @@ int md_get_neighbors(md_system* s, int32_t* count, int32_t* entries) {
   }
   // every listed pair, both ways, by original atom index: the region tiles
   // rebuilt here exactly as the kernels stage them
+  std::vector<int> region_cells((size_t)kRegionCells * s->n_regions);
+  CU(cudaMemcpy(region_cells.data(), s->region_cells, region_cells.size() * sizeof(int), cudaMemcpyDeviceToHost));
   std::vector<std::vector<int>> nb(N);
-  for (size_t r = 0; r < s->regions_h.size(); ++r) {
-    const RegionShape& S = s->shapes_h[s->regions_h[r].shape];
-    const int* cell = s->region_cells_h.data() + kRegionCells * r;
+  const int G = s->lj_region;
+  int rep = 0;
+  for (int r = 0; r < s->n_regions; ++r) {
+    while (rep + 1 < s->n_reps && s->reps_h[rep + 1].region_off <= r) ++rep;
+    const RepDev& q = s->reps_h[rep];
+    const int nx = (q.M + G - 1) / G, x = (r - q.region_off) % nx * G, y = (r - q.region_off) / nx % nx * G;
+    const RegionShape& S = s->shapes_h[std::min(G, q.M - x) - 1 + G * (std::min(G, q.M - y) - 1)];
+    const int* cell = region_cells.data() + (size_t)kRegionCells * r;
     int start[kMaxTileCells], off[kMaxTileCells + 1];
     off[0] = 0;
     for (int k = 0; k < S.n_tile; ++k) {

@@ -66,6 +66,7 @@ struct RepDev {
   int M, cell_base, atom_off, n_atoms;
   int n_chains, chain_off, tile_off, n_tiles;
   int ctile_off, n_ctiles;      // chain tiles (blocks of the fused step kernel)
+  int region_off, pad3;         // first region (region_of)
   double T0, dof;
   // thermostats: T = t_scale sum(m v^2 / m_0); weak coupling lam^2 = 1 - dt/tau
   // + vr_num / sum; Nose-Hoover dxi = nh_rate (T - T0), V_com = com_scale sum(m v / m_0)
@@ -102,6 +103,11 @@ struct __align__(16) WorkItem {
   unsigned char h0, h1, part, parts;
   int pad[2];
 };
+// Items first, first + 1, ... are those of the regions of one shape in a replica,
+// from the region0-th on: each region's home cells in groups of `step`, each
+// group's clusters over `parts` blocks.  (Runs, not items, are what the host
+// makes: a box of few atoms can have more regions than atoms.)
+struct ItemRun { int first, rep, shape, region0, step, parts; };
 constexpr int kSMs = 152;             // streaming multiprocessors of a GB300
 // global cell ids of a region's tile cells: cells[kRegionCells * region + k]
 constexpr int kRegionCells = 48;
@@ -395,6 +401,10 @@ void launch_cell_sort(bool mixed, const void* x, int N, const int* cell_start, c
                       const int* cellc, const uint16_t* site, const RepDev* reps, int n_reps, int C,
                       int sites, int* perm, int* inv_perm, float4* pos, int* tag, float4* ref, unsigned* flags,
                       bool dep, cudaStream_t st);
+// the tile cells of every region (region r of a replica: z, y, x with x
+// fastest, ceil(M / G) a side in x and y) and the work items, made once per system
+void launch_plan(const RepDev* reps, int n_reps, const RegionShape* shapes, int G, int n_regions, int* cells,
+                 const ItemRun* runs, int n_runs, int n_items, WorkItem* items, cudaStream_t st);
 // ---------------------------------------------------------------- forces
 // cluster lists and LJ forces by regions (k_lj.cu), a block per work item.
 // The build writes each cluster's list (up to cap entries, ncl[cl] of them);

@@ -51,6 +51,7 @@ int fake_ran() { return (int)ran.size(); }
 const char* fake_kernel(int i) { return ran[i].kernel.c_str(); }
 long long fake_smem(int i) { return (long long)ran[i].smem; }
 int fake_block(int i) { return (int)ran[i].block; }
+int fake_grid(int i) { return (int)ran[i].grid; }
 long long fake_opt_in(const char* kernel) { return opt_in.count(kernel) ? (long long)opt_in[kernel] : -1; }
 
 // ---------------------------------------------------------------- kernels
