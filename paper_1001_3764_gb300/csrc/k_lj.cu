@@ -396,6 +396,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_cl_build(const float4* __rest
     const int h = threadIdx.x / 5, run = threadIdx.x % 5;
     runs[threadIdx.x] = make_int2(T.off[S.nb[h][3 * run + 1]], T.off[S.nb[h][min(3 * run + 3, 13)] + 1]);
   }
+  if (q_first >= q_end) return;   // no cluster: a sparse box's usual region
   stage_build_tile<NT>(T, item.need, pos, tag, B);
   const float rl2 = R.rlist2u;
   const float rl = sqrtf(rl2);
@@ -1002,7 +1003,10 @@ __global__ void __launch_bounds__(kRankThreads) k_cl_rank(const float4* __restri
   const WorkItem item = items[blockIdx.x];
   region_setup(T, item, shapes[item.shape], cells, cell_start, cl_start);
   const int q_first = T.ncl[item.h0], nq = T.ncl[item.h1] - q_first;
-  if (T.ncl[T.n_home] > kRegionClusterCap) return;   // reported by the force kernel
+  if (nq == 0 || T.ncl[T.n_home] > kRegionClusterCap) {   // nothing to do; too many: reported by the force kernel
+    if (threadIdx.x == 0) task_base[blockIdx.x] = nq == 0 ? -1 : 0;
+    return;
+  }
   if (threadIdx.x == 0) {
     task_base[blockIdx.x] = base = atomicAdd(n_tasks, nq);
     if (T.off[T.n_tile] > lj_cap) big[atomicAdd(n_tasks + 1, 1)] = blockIdx.x;
@@ -1090,14 +1094,21 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_cl_force(
     const RegionShape& S = shapes[item.shape];
     const RepDev& R = reps[item.rep];
     const int t_base = task_base[r];
-    if (!persistent && it == 0) {
-      // (read together with the item, whose loads are asked for here, not after the branch)
-      const bool off = lj_off(gate);
-      asm volatile("" ::"r"(item.region), "r"(t_base));
-      if (off) {
-        wait_for_predecessor();
-        return;
-      }
+    // An item without home atoms (most of them in a sparse box: 12 chains in 60 /
+    // 150 nm, 210 / 3,786 us a launch with its tables read and its tasks copied,
+    // 66 / 993 now) or a launch that is off: nothing to do.  The gate is read
+    // together with the item, whose loads are asked for here, not after the branch.
+    const bool off = !persistent && it == 0 && lj_off(gate);
+    asm volatile("" ::"r"(item.region), "r"(t_base));
+    if (off || t_base < 0) {
+      if (ENERGY)
+        for (int k = threadIdx.x; k < kEnergyVals * (item.h1 - item.h0); k += NT) {
+          const int cell = __ldg(cells + kRegionCells * item.region + S.nb[item.h0 + k / kEnergyVals][0]);
+          epart[(size_t)cell * kEnergyVals + k % kEnergyVals] = 0.0;
+        }
+      if (persistent) continue;
+      wait_for_predecessor();
+      return;
     }
     __syncthreads();   // the previous item's tables are no longer read
     region_setup(T, item, S, cells, cell_start, cl_start);

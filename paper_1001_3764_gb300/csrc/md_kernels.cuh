@@ -420,9 +420,9 @@ void launch_cl_build(const float4* pos, const int* tag, const int* cell_start, c
                      const RepDev* reps, unsigned* list, int* ncl, int cap, int tile_cap, unsigned* flags,
                      int* n_tasks, const TopoDev* topo, bool dep, cudaStream_t st);
 // after the build (which clears *n_tasks): each LJ item's clusters in the
-// order the force kernel takes them, tasks[task_base[item] + rank]; an item
-// claims its place in the table (as many entries as there are clusters) by
-// n_tasks[0]; items with tiles of more than lj_cap atoms are listed in big[0 .. n_tasks[1])
+// order the force kernel takes them, tasks[task_base[item] + rank] (task_base
+// -1: an item without clusters); an item claims its place in the table (as many
+// entries as there are clusters) by n_tasks[0]; items with tiles of more than lj_cap atoms are listed in big[0 .. n_tasks[1])
 void launch_cl_rank(const float4* pos, const int* cell_start, const int* cl_start, const int* cells,
                     const WorkItem* items, int n_items, const RegionShape* shapes, const int* ncl, ClusterTask* tasks,
                     int* task_base, int* n_tasks, int lj_cap, int* big, bool dep, cudaStream_t st);
