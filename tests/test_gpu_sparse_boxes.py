@@ -9,7 +9,7 @@ import paper_1001_3764_gb300 as md
 pytestmark = pytest.mark.gpu
 
 
-# 7, 16 and 48 cells a side for 600 atoms; regions of 3 and 2 cells, and the fixed grid
+# 7, 16 and 48 cells a side for 600 atoms (the last: cells ordered 32 to a block); regions of 3 and 2 cells, and the fixed grid
 @pytest.mark.parametrize("L", [8.0, 18.0, 53.0])
 @pytest.mark.parametrize("fields", [{}, dict(lj_region=2), dict(schedule=md.MD_SCHED_PERSISTENT), dict(precision=md.MD_PLAIN_FP32)])
 def test_sparse_boxes_match_the_oracle_wherever_the_atoms_are(L, fields):
