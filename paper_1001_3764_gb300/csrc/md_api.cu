@@ -1575,8 +1575,7 @@ int md_get_neighbors(md_system* s, int32_t* count, int32_t* entries) {
         for (int e = 0; e < nc[cl]; ++e) {
           const unsigned E = lst[(size_t)cl * s->cap + e];
           const int t = (int)(E & 0xffffu);
-          int kc = 0;
-          while (kc + 1 < S.n_tile && off[kc + 1] <= t) ++kc;
+          const int kc = (int)(std::upper_bound(off + 1, off + S.n_tile, t) - (off + 1));   // its tile cell
           const int j = pm[start[kc] + (t - off[kc])];
           for (int u = 0; u < 4; ++u)
             if ((E >> (16 + u)) & 1u) {
