@@ -1094,21 +1094,21 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_cl_force(
     const RegionShape& S = shapes[item.shape];
     const RepDev& R = reps[item.rep];
     const int t_base = task_base[r];
-    // An item without home atoms (most of them in a sparse box: 12 chains in 60 /
-    // 150 nm, 210 / 3,786 us a launch with its tables read and its tasks copied,
-    // 66 / 993 now) or a launch that is off: nothing to do.  The gate is read
-    // together with the item, whose loads are asked for here, not after the branch.
-    const bool off = !persistent && it == 0 && lj_off(gate);
-    asm volatile("" ::"r"(item.region), "r"(t_base));
-    if (off || t_base < 0) {
-      if (ENERGY)
-        for (int k = threadIdx.x; k < kEnergyVals * (item.h1 - item.h0); k += NT) {
-          const int cell = __ldg(cells + kRegionCells * item.region + S.nb[item.h0 + k / kEnergyVals][0]);
-          epart[(size_t)cell * kEnergyVals + k % kEnergyVals] = 0.0;
-        }
-      if (persistent) continue;
-      wait_for_predecessor();
-      return;
+    // A launch that is off, or an item without home atoms (most of them in a
+    // sparse box: 12 chains in 60 / 150 nm, 210 / 3,786 us a launch with its tables
+    // read and its tasks copied, 66 / 993 now): nothing to do.  A fixed grid and the
+    // launch for large tiles take such an item through the empty loops below.
+    if (!persistent && it == 0) {
+      const bool off = lj_off(gate) || t_base < 0;
+      if (off) {
+        if (ENERGY)
+          for (int k = threadIdx.x; k < kEnergyVals * (item.h1 - item.h0); k += NT) {
+            const int cell = __ldg(cells + kRegionCells * item.region + S.nb[item.h0 + k / kEnergyVals][0]);
+            epart[(size_t)cell * kEnergyVals + k % kEnergyVals] = 0.0;
+          }
+        wait_for_predecessor();
+        return;
+      }
     }
     __syncthreads();   // the previous item's tables are no longer read
     region_setup(T, item, S, cells, cell_start, cl_start);
