@@ -26,6 +26,7 @@
 // store holds the C + 1 positions of the segment being reversed.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstdlib>
@@ -164,7 +165,7 @@ struct AdjDev {
   double rc, rc2, irc6, irc12;   // cutoff and the shift terms (1/r_c)^6, (1/r_c)^12
   double irc7, irc13;            // force-shifted variant: (1/r_c)^7, (1/r_c)^13
   int sf;                        // 1 = force-shifted variant (not the paper's potential)
-  float pre2;                    // FP32 prefilter: (r_c + 1e-4 nm)^2; a candidate beyond it is out in FP64 too
+  float pre2;                    // FP32 prefilter: (r_c + margin)^2; a candidate beyond it is out in FP64 too
   double c6[3], c12[3];       // pair types 0 = C32-C32, 1 = C32-C33, 2 = C33-C33
   double kb, b0, ka, theta0, kphi, phis;
   int n_mult;
@@ -459,7 +460,7 @@ __global__ void __launch_bounds__(32 * kLjWarps) k_adj_lj(const double* __restri
       const int dj = (int)(cb & 0x7fffffffu) - i;
       // itself and its 1-2 and 1-3 neighbours (Sec. 3.1): |i - j| <= 2 on one chain
       const bool excl = (unsigned)(dj + 2) <= 4u && (unsigned)(si + dj) < (unsigned)P.sites;
-      // FP32 prefilter on the wrapped copies (error ~1e-6 nm against a 1e-4 nm margin)
+      // FP32 prefilter on the wrapped copies (error ~1e-6 nm in a melt's box against a margin of 1e-4)
       float ex = sh.x - c.x, ey = sh.y - c.y, ez = sh.z - c.z;
       if (!cells) {
         ex -= Lf * rintf(ex * iLf); ey -= Lf * rintf(ey * iLf); ez -= Lf * rintf(ez * iLf);
@@ -1002,7 +1003,10 @@ extern "C" int md_adj_create(const md_adj_desc* d, md_adj** out) {
     return adj_fail(MD_EINVAL, "hvp_precision must be 0 (FP64) or 1 (FP32)");
   }
   a->hvp32 = d->hvp_precision == 1;
-  P.pre2 = (float)((d->rc + 1e-4) * (d->rc + 1e-4));
+  // margin over the FP32 roundings of two wrapped coordinates, L and the image's
+  // sum: 2.5 spacings of L per axis, 5.2e-7 L in r (1e-4 nm up to 166 nm)
+  const double margin = std::max(1e-4, 6e-7 * d->box);
+  P.pre2 = (float)((d->rc + margin) * (d->rc + margin));
   P.kb = p.kb; P.b0 = p.b0; P.ka = p.ka; P.theta0 = p.theta0; P.phis = p.phis; P.n_mult = p.n_mult;
   P.inv_mass[0] = 1.0 / p.mass[0];
   P.inv_mass[1] = 1.0 / p.mass[1];

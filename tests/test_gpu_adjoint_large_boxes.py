@@ -32,3 +32,36 @@ def test_gradient_and_means_in_boxes_of_many_cells(n_chains, L):
     assert np.linalg.norm(h - fd) < 1e-6 * np.linalg.norm(fd)
     assert a.forward() == pytest.approx(ref.traj_means(x, m["vel"], 0.001, 3), rel=1e-9)
     a.close()
+
+
+def test_pairs_just_inside_the_cutoff_are_found_in_boxes_of_hundreds_of_nm():
+    """Dimers whose first sites lie 2e-6 nm inside r_c of another's, over a box of 1,800 nm and across its faces: an FP32
+    coordinate there is known to 6e-5 nm.  Each such site feels the truncated force of its one pair."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    rng = np.random.default_rng(5)
+    L, rc, n = 1800.0, 1.0, 4000
+    p = md.default_params()
+    a = rng.uniform(0.0, L, (n, 3))
+    a[::4, 0] = rng.uniform(-0.5, 0.5, n // 4)          # pairs across a face
+    u = rng.standard_normal((n, 3))
+    u /= np.linalg.norm(u, axis=1)[:, None]
+    b = a + (rc - 2e-6) * u
+    x = np.empty((2 * n, 2, 3))
+    x[0::2, 0], x[1::2, 0] = a, b
+    x[0::2, 1], x[1::2, 1] = a - p["b0"] * u, b + p["b0"] * u     # the second sites point away: out of range
+    x = x.reshape(-1, 3)
+    m = dict(pos=x, vel=np.zeros_like(x), L=L, n_chains=2 * n, sites=2)
+    adj = md.Adjoint(m, n_steps=0, rc=rc, params=dict(p, kb=0.0))
+    g, _, _, _ = adj.tangent(x, np.zeros_like(x))
+    adj.close()
+    d = b - a
+    r = np.linalg.norm(d, axis=1)
+    eps, sig = p["eps"][1], p["sigma"][1]               # all sites are chain ends
+    dEdr = 4 * eps * (6 * sig ** 6 / r ** 7 - 12 * sig ** 12 / r ** 13)
+    want = -(dEdr / r)[:, None] * d                      # on a; r itself is rounded by 2^-53 L / r_c in x
+    got = g.reshape(-1, 2, 3)
+    assert np.abs(got[0::2, 0] - want).max() <= 1e-9 * np.abs(want).max()
+    assert np.abs(got[1::2, 0] + want).max() <= 1e-9 * np.abs(want).max()
+    assert np.abs(got[:, 1]).max() == 0.0
