@@ -1122,6 +1122,10 @@ int md_create(const md_desc* d, md_system** out) {
 int md_step_async(md_system* s, int64_t n) {
   if (!s || n < 0) return fail(s, MD_EINVAL, "bad arguments");
   const int64_t full = n / s->R, rem = n % s->R;
+  if (full && (!s->cycle || !s->cycle_fresh)) {   // a capture failed in an earlier call, which said so
+    const int rc = capture_cycle(s);
+    if (rc) return rc;
+  }
   for (int64_t c = 0; c < full; ++c) {
     const bool skip_rebin = c == 0 && s->fresh && !s->profile;
     s->fresh = false;
