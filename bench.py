@@ -578,7 +578,7 @@ def run_gpu(args):
             print(json.dumps({"ncu_region": True, "ms_per_step": m["ms"] / args.steps, "sites": n_atoms,
                               "launches": int(m["launches"])}), flush=True)
         return
-    # the same loop with the default policy (a conditional early rebuild per step)
+    # the same loop with the default policy (a conditional early rebuild per group of steps)
     if not args.ncu_region:
         s = md.System(melt, precision=md.MD_MIXED)
         st = torch.cuda.ExternalStream(md.md_stream(s.h))
@@ -636,7 +636,7 @@ def run_gpu(args):
             "ms_per_step": results["rebuild_policy"]["ms"] / args.steps,
             "early_rebuilds": results["rebuild_policy"]["early"],
             "note": "same loop with the default MD_DISP_REBUILD policy (a displacement check in every step, "
-                    "one conditional rebuild per block of steps); the headline uses MD_DISP_ERROR, whose graphs ncu can "
+                    "one conditional rebuild per group of steps); the headline uses MD_DISP_ERROR, whose graphs ncu can "
                     "profile, with the same work on this melt"},
         "roofline": {"kernel": "k_cl_force (LJ force, Eq. 2)", "bound": "alu", "achieved": achieved,
                      "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": achieved / FP32_PEAK_TFLOPS,

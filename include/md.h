@@ -203,7 +203,7 @@ int md_create(const md_desc *desc, md_system **out);
  * steps and of every call (the paper rebuilds it every 10 steps, Sec. 5),
  * and also before the force evaluation of any step in which an atom has
  * moved more than skin/2 since the last rebuild (a device-side check that
- * opens the conditional node of the block's graph; md_early_rebins counts
+ * opens a conditional node of the block's graph; md_early_rebins counts
  * them), so every force comes from a list that holds all pairs within rc;
  * with MD_DISP_ERROR such a step is reported as MD_EUNSTABLE instead.
  * Synchronises and reports device flags. */

@@ -19,12 +19,6 @@
 
 namespace mdg {
 
-__device__ __forceinline__ float rcp_approx(float x) {
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 // Block reduction of NV FP32 per-thread values into out[NV] (FP64; thread 0
 // holds the result): each warp adds its 32 lanes in FP32 by a fixed shuffle
 // tree (an FP64 tree per lane would load this GPU's narrow FP64 pipe), lane 0

@@ -19,7 +19,7 @@
 // 3.4): per replica xi_k, 1 - c_k, 1/(1 + c_k), V_com (kNhDoubles in
 // md_kernels.cuh), c_k = dt xi_k / 2.  A step closes v_k = (v_{k-1/2} - V_com + dt F/(2m)) /
 // (1 + c_k), opens v_{k+1/2} = (1 - c_k) v_k + dt F/(2m) and drifts; the
-// last block takes T_{k+1/2} and the momentum of v_{k+1/2} and leaves
+// replica's block of the LJ launch takes T_{k+1/2} and the momentum of v_{k+1/2} and leaves
 // xi_{k+1} = xi_k + dt (T_{k+1/2} - T0)/Q, Q = tau^2 T0/(4 pi^2), and the
 // centre-of-mass velocity that the next step subtracts.  This is the
 // leap-frog update v_{k+1/2} = [v_{k-1/2}(1 - c_k) + dt F/m]/(1 + c_k).
