@@ -757,18 +757,24 @@ constexpr int kGroupSteps = 10, kOneGroup = 16;
 // is counted), instead of the run stopping.
 static cudaError_t enqueue_group(md_system* s, int first, int last, int k) {
   MoveReport mr{};
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  const cudaGraphNode_t* deps = nullptr;
+  const cudaGraphEdgeData* ed = nullptr;
+  size_t nd = 0;
   cudaGraph_t g = nullptr;
-  cudaError_t e = cudaStreamGetCaptureInfo(s->st, &cs, nullptr, &g, nullptr, nullptr, nullptr);
+  // the graph being captured and where it ends (there is none once a launch, or
+  // another thread's call, has invalidated the capture)
+  auto captured = [&] {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const cudaError_t q = cudaStreamGetCaptureInfo(s->st, &cs, nullptr, &g, &deps, &ed, &nd);
+    return q != cudaSuccess ? q : cs == cudaStreamCaptureStatusActive && g ? cudaSuccess : cudaErrorStreamCaptureInvalidated;
+  };
+  cudaError_t e = captured();
   if (e != cudaSuccess) return e;
   if ((e = cudaGraphConditionalHandleCreate(&mr.handle, g, 0, cudaGraphCondAssignDefault)) != cudaSuccess) return e;
   mr.ctl = s->ctl;
   mr.events = s->early;
   enqueue_steps(s, first, last, k, false, mr);
-  const cudaGraphNode_t* deps = nullptr;
-  const cudaGraphEdgeData* ed = nullptr;
-  size_t nd = 0;
-  if ((e = cudaStreamGetCaptureInfo(s->st, &cs, nullptr, &g, &deps, &ed, &nd)) != cudaSuccess) return e;
+  if ((e = captured()) != cudaSuccess) return e;
   cudaGraphNodeParams p{};
   p.type = cudaGraphNodeTypeConditional;
   p.conditional.handle = mr.handle;

@@ -21,6 +21,8 @@ std::string fail_call;
 int fail_nth = 0;
 cudaError_t last = cudaSuccess;
 int open_captures = 0;
+int null_graphs = 0;                                 // calls on no graph
+std::map<cudaStream_t, bool> invalid;                // captures that another thread's call has invalidated
 char pool[4096];
 size_t handles = 0;
 
@@ -43,7 +45,8 @@ cudaError_t launch(const std::string& k, dim3 g, dim3 b, size_t smem, cudaStream
 
 extern "C" {
 // ---------------------------------------------------------------- for the test
-void fake_reset() { ran.clear(); calls.clear(); fail_call.clear(); fail_nth = 0; last = cudaSuccess; }
+void fake_reset() { ran.clear(); calls.clear(); fail_call.clear(); fail_nth = 0; last = cudaSuccess; null_graphs = 0; }
+int fake_null_graphs() { return null_graphs; }
 void fake_fail(const char* what, int nth) { calls.clear(); fail_call = what; fail_nth = nth; }
 int fake_calls(const char* what) { return calls[what]; }
 int fake_open_captures() { return open_captures; }
@@ -168,9 +171,12 @@ cudaError_t cudaStreamBeginCaptureToGraph(cudaStream_t st, cudaGraph_t g, const 
 cudaError_t cudaStreamEndCapture(cudaStream_t st, cudaGraph_t* g) {
   *g = nullptr;
   if (!capture.count(st)) { last = cudaErrorIllegalState; return last; }
-  *g = (cudaGraph_t)capture[st];
+  const bool bad = invalid[st];
+  *g = bad ? nullptr : (cudaGraph_t)capture[st];
+  invalid[st] = false;
   capture.erase(st);
   --open_captures;
+  if (bad) return last = cudaErrorStreamCaptureInvalidated;
   return call("cudaStreamEndCapture", cudaErrorStreamCaptureInvalidated);
 }
 cudaError_t cudaStreamIsCapturing(cudaStream_t st, cudaStreamCaptureStatus* s) {
@@ -180,7 +186,9 @@ cudaError_t cudaStreamIsCapturing(cudaStream_t st, cudaStreamCaptureStatus* s) {
 cudaError_t cudaStreamGetCaptureInfo(cudaStream_t st, cudaStreamCaptureStatus* s, unsigned long long*, cudaGraph_t* g,
                                      const cudaGraphNode_t** deps, const cudaGraphEdgeData** ed, size_t* n) {
   cudaStreamIsCapturing(st, s);
-  if (g) *g = capture.count(st) ? (cudaGraph_t)capture[st] : nullptr;
+  if (call("invalidated") != cudaSuccess) { invalid[st] = true; last = cudaSuccess; }
+  if (invalid[st]) *s = cudaStreamCaptureStatusInvalidated;
+  if (g) *g = capture.count(st) && !invalid[st] ? (cudaGraph_t)capture[st] : nullptr;
   if (deps) *deps = nullptr;
   if (ed) *ed = nullptr;
   if (n) *n = 0;
@@ -189,12 +197,14 @@ cudaError_t cudaStreamGetCaptureInfo(cudaStream_t st, cudaStreamCaptureStatus* s
 cudaError_t cudaStreamUpdateCaptureDependencies(cudaStream_t, cudaGraphNode_t*, const cudaGraphEdgeData*, size_t, unsigned) {
   return call("cudaStreamUpdateCaptureDependencies");
 }
-cudaError_t cudaGraphConditionalHandleCreate(cudaGraphConditionalHandle* h, cudaGraph_t, unsigned, unsigned) {
+cudaError_t cudaGraphConditionalHandleCreate(cudaGraphConditionalHandle* h, cudaGraph_t g, unsigned, unsigned) {
   *h = ++handles;
+  if (!g) ++null_graphs;
   return call("cudaGraphConditionalHandleCreate");
 }
-cudaError_t cudaGraphAddNode(cudaGraphNode_t* n, cudaGraph_t, const cudaGraphNode_t*, const cudaGraphEdgeData*, size_t,
+cudaError_t cudaGraphAddNode(cudaGraphNode_t* n, cudaGraph_t g, const cudaGraphNode_t*, const cudaGraphEdgeData*, size_t,
                              cudaGraphNodeParams* p) {
+  if (!g) ++null_graphs;
   *n = handle<cudaGraphNode_t>();
   cudaGraph_t* body = new cudaGraph_t((cudaGraph_t) new Graph());   // kept: a test's few
   p->conditional.phGraph_out = body;

@@ -10,7 +10,8 @@ from fake_cudart import Fake, lattice, link
 
 GRAPH_CALLS = ["cudaStreamBeginCapture", "cudaStreamGetCaptureInfo", "cudaGraphConditionalHandleCreate", "cudaGraphAddNode",
                "cudaStreamUpdateCaptureDependencies", "cudaStreamBeginCaptureToGraph", "cudaStreamEndCapture",
-               "cudaGraphInstantiate", "cudaGraphLaunch"]
+               "cudaGraphInstantiate", "cudaGraphLaunch",
+               "invalidated"]    # the capture is found invalidated by another thread's call: no graph to add to
 
 
 @pytest.fixture(scope="module")
@@ -76,7 +77,7 @@ def test_every_refused_launch_fails_its_call(lib, kind):
                 call = calls(lib, fresh)[name]
                 lib.fake_fail(what.encode(), k)
                 assert call() == md.MD_ECUDA, (name, what, k)
-                assert lib.fake_open_captures() == 0
+                assert lib.fake_open_captures() == 0 and lib.fake_null_graphs() == 0
                 lib.fake_fail(b"", 0)
                 assert lib.md_get_state(s.h, *[a.ctypes.data for a in s.out]) == md.MD_OK   # another system's call
                 assert lib.md_step(fresh.h, 13) == md.MD_OK, (name, what, k)   # graphs that a failed capture left out are made
@@ -87,7 +88,7 @@ def test_every_refused_launch_fails_its_call(lib, kind):
             fresh = system(lib, kind)
             lib.fake_fail(what.encode(), k)
             assert fresh.create() == md.MD_ECUDA and not fresh.h, (what, k)
-            assert lib.fake_open_captures() == 0
+            assert lib.fake_open_captures() == 0 and lib.fake_null_graphs() == 0
             lib.fake_fail(b"", 0)
             assert lib.md_rebin(s.h) == md.MD_OK
     s.close()
