@@ -446,7 +446,9 @@ class System:
             d.workspace = (addr + 255) // 256 * 256
             d.workspace_bytes = nbytes
         self.desc = d
-        torch.cuda.synchronize(self.device)
+        # the workspace may be memory that work on the current stream still uses (a wait for the whole device would
+        # break a graph capture that another thread's system is in)
+        self.stream.wait_stream(torch.cuda.current_stream(self.device))
         self.h = md_create(d)
         self.info = md_info(self.h)
         self.dt, self.rebin_every = dt, d.rebin_every
